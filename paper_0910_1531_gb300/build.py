@@ -20,6 +20,7 @@ LIB_NAME = "libgb300dft.so"
 CT_SIZES = (0, 32, 48, 64, 96, 128, 256)
 SOURCES = ([("api.cu", "api", []), ("bulk.cpp", "bulk", []), ("noalloc.cu", "noalloc", []),
             ("dispatch.cu", "dispatch", []), ("newton.cu", "newton", [])]
+           + [("colfft.cu", f"colfft_{r}", [f"-DDFT_INST_REAL={r}"]) for r in ("float", "double")]
            + [("kinst.cu", f"kinst_{r}_{n}", [f"-DDFT_INST_REAL={r}", f"-DDFT_INST_N={n}"])
               for r in ("float", "double") for n in CT_SIZES])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

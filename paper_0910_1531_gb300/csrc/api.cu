@@ -297,7 +297,8 @@ template <typename Real> struct Ops {
             LAUNCH(p, K_ZFFT, 2.0 * p->S * CB(p),
                    P::zfft(p->stream, false, p->g, p->S, W, &p->ctl->status, tw(p, 2), p->wait_polls));
             LAUNCH(p, K_ZMUL, (p->S + DFT_NSPEC + p->S) * CB(p),
-                   P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), W, slot_n(slot), slot_es(p, slot)));
+                   P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), 0, W, slot_n(slot), slot_es(p, slot),
+                           nullptr));
             LAUNCH(p, K_ZFFT, 2.0 * DFT_NSPEC * CB(p),
                    P::zfft(p->stream, true, p->g, DFT_NSPEC, slot_n(slot), &p->ctl->status, tw(p, 2), p->wait_polls));
         } else {
@@ -367,8 +368,8 @@ template <typename Real> struct Ops {
             // one z pass for both samples (the ES tiles read once; sample 2's results after sample
             // 1's, at T1 components S .. 2 S - 1), then one y inverse over the 2 S components
             LAUNCH(p, K_ZBWD, (2.0 * DFT_NSPEC + 4.0 * p->S) * CB(p),
-                   P::zconv_bwd_pair(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), p->S, p->ctl + 1, T1(p), esA,
-                                     esB, tw(p, 2)));
+                   P::zconv_bwd_pair(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), p->S, p->ctl + 1,
+                                     T1(p), esA, esB, tw(p, 2)));
             LAUNCH(p, K_YFFT, 2.0 * (2 * p->S) * CB(p),
                    P::yfft(p->stream, true, p->g, p->ay, p->Ty, 2 * p->S, T1(p), &p->ctl->status, tw(p, 1),
                            p->wait_polls));
@@ -614,7 +615,7 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
     using P = Passes<Real>;
     const SpeciesDesc<Real>& sp = species<Real>(p);
     const int S = p->S;
-    const long long n_zk = ceil_div(p->g.nxh, p->Tz) * p->g.ny;
+    const long long n_zk = P::energy_blocks(p->g);
     const long long n_phi = p->blocks_x(p->LRphi);
     const long long n_g = p->blocks_x(p->LRupd);
     const size_t need = size_t(2 * n_zk + n_phi + n_g * (S + 1));
@@ -880,7 +881,8 @@ std::vector<AxisPlan> radix_orders(int n) {
             if (a.radix[s] != b.radix[s]) return false;
         return true;
     };
-    auto add = [&](const AxisPlan& a) {
+    auto add = [&](AxisPlan a) {
+        dft_finish_plan(&a);
         for (const AxisPlan& o : out)
             if (same(o, a)) return;
         out.push_back(a);
@@ -888,7 +890,8 @@ std::vector<AxisPlan> radix_orders(int n) {
     add(r);
     if ((n & (n - 1)) == 0) {
         for (int big : {8, 4}) {
-            AxisPlan q{n, 0, {}};
+            AxisPlan q{};
+            q.n = n;
             int m = n;
             while (m % big == 0 && q.nstages < DFT_MAXSTAGES) { q.radix[q.nstages++] = big; m /= big; }
             if (m > 1 && q.nstages < DFT_MAXSTAGES) q.radix[q.nstages++] = m;
@@ -925,10 +928,12 @@ void describe_tuning(dft_plan* p) {
     t += "; y: ";
     t += (!g.yrt && dft_is_ct_size(g.ny)) ? "TMA persistent, " + std::to_string(p->precision == DFT_FP64 ? 8 : 16) +
                                                 "-column tiles"
-                                          : "run-time column kernel, " + std::to_string(p->Ty) + "-column tiles";
+                                          : "run-time column kernel, " + std::to_string(p->Ty) + "-column tiles, radix " +
+                                                radix_text(p->ay);
     t += "; z: ";
     t += dft_is_ct_size(g.nz) ? (g.zgrp ? std::string("grouped, one tile per CTA") : std::string("TMA persistent"))
-                              : "run-time column kernel, " + std::to_string(p->Tz) + "-column tiles";
+                              : "run-time column kernel, " + std::to_string(p->Tz) + "-column tiles, radix " +
+                                    radix_text(p->az);
     if (dft_is_ct_size(g.nz) && g.zsplit) t += ", first half as z transforms and a k-space products pass";
     t += p->pdl_on ? "; launches: programmatic dependent" : "; launches: stream order";
     p->tuning = t;
@@ -1121,8 +1126,8 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
             p->g.zsplit = v;
             if (v) {
                 P::zfft(p->stream, false, p->g, p->S, O::T1(p), &p->ctl->status, O::tw(p, 2), p->wait_polls);
-                P::zmul(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), O::T1(p), O::slot_n(p->slotB),
-                        O::slot_es(p, p->slotB));
+                P::zmul(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p), O::slot_n(p->slotB),
+                        O::slot_es(p, p->slotB), nullptr);
                 P::zfft(p->stream, true, p->g, DFT_NSPEC, O::slot_n(p->slotB), &p->ctl->status, O::tw(p, 2),
                         p->wait_polls);
             } else {
@@ -1285,7 +1290,7 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     p->kf[0] = two_pi / (g.nx * g.hx);
     p->kf[1] = two_pi / (g.ny * g.hy);
     p->kf[2] = two_pi / (g.nz * g.hz);
-    if (!dft_radix_plan(g.nx, &p->ax) || !dft_radix_plan(g.ny, &p->ay) || !dft_radix_plan(g.nz, &p->az)) {
+    if (!dft_radix_plan(g.nx, &p->ax) || !dft_mixed_plan(g.ny, &p->ay) || !dft_mixed_plan(g.nz, &p->az)) {
         delete p;
         return fail(nullptr, DFT_EINVAL, "no radix plan for the grid sizes");
     }
@@ -1294,17 +1299,8 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     const bool f64 = prm->precision == DFT_FP64;
     p->csize = f64 ? sizeof(double2) : sizeof(float2);
     p->rsize = f64 ? sizeof(double) : sizeof(float);
-    p->Ty = f64 ? Passes<double>::tile_y(g.ny, 100 * 1024) : Passes<float>::tile_y(g.ny, 100 * 1024);
-    p->Tz = f64 ? Passes<double>::tile_z(g.nz, 112 * 1024) : Passes<float>::tile_z(g.nz, 112 * 1024);
-    {   // run-time lengths: narrower column tiles while a column pass would have fewer than two
-        // CTAs per SM (small grids)
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess || sms < 1) sms = 1;
-        if (!dft_is_ct_size(g.ny))
-            while (p->Ty > 1 && ceil_div(g.nxh, p->Ty) * g.nz < 2LL * sms) p->Ty /= 2;
-        if (!dft_is_ct_size(g.nz))
-            while (p->Tz > 1 && ceil_div(g.nxh, p->Tz) * g.ny < 2LL * sms) p->Tz /= 2;
-    }
+    p->Ty = f64 ? Passes<double>::tile_y(g) : Passes<float>::tile_y(g);
+    p->Tz = f64 ? Passes<double>::tile_z(g) : Passes<float>::tile_z(g);
     p->LX = pick_lines(g.nx, p->csize, 1, env_budget("DFT_XFWD_SMEM", 48 * 1024), 32);
     p->LRphi = pick_lines(g.nx, p->csize, 5, env_budget("DFT_XPHI_SMEM", 32 * 1024), 16);
     p->LRupd = pick_lines(g.nx, p->csize, (S + 1) / 2, env_budget("DFT_XUPD_SMEM", 48 * 1024), 16);
@@ -1365,38 +1361,39 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         dft_plan_destroy(p);
         return fail(nullptr, DFT_ENOMEM, "cudaMalloc failed: normalisation sums");
     }
-    // On a cubic box |k| = kf sqrt(mx^2 + my^2 + mz^2) takes one value per integer m2, so the
-    // compile-time z passes read the FMT weights and bulk-fluid kernels from per-m2 tables
-    // instead of evaluating them at every point.
-    if (dft_is_ct_size(g.nz) && p->kf[0] == p->kf[1] && p->kf[1] == p->kf[2]) {
+    // The z passes read the FMT weights and bulk-fluid kernels, functions of |k| alone, from tables
+    // instead of evaluating them at every point: on a cubic box, |k| = kf sqrt(mx^2 + my^2 + mz^2),
+    // one record per integer m2; on others one per (kx, |ky|, |kz|), N / 8 records.  21 x 21 x 161,
+    // S = 2, FP64: 16 us for the first half's products, where evaluating the sines and cosines on the
+    // FP64 pipe made that z pass 277.  A plan that cannot have the second kind (memory) evaluates per point.
+    {
+        const bool cubic = p->kf[0] == p->kf[1] && p->kf[1] == p->kf[2];
         const long long m2max = (long long)(g.nx / 2) * (g.nx / 2) + (long long)(g.ny / 2) * (g.ny / 2) +
                                 (long long)(g.nz / 2) * (g.nz / 2);
         const long long P = (long long)S * (S + 1) / 2;
-        const long long rows = m2max + 1;
+        const long long rows = cubic ? m2max + 1 : (long long)g.nxh * (g.ny / 2 + 1) * (g.nz / 2 + 1);
         // records padded to 16 bytes (read with 16-byte loads)
         const long long V = 16 / (long long)p->rsize;
         const long long ws = (2 * S + V - 1) / V * V, ks = (P + V - 1) / V * V;
-        if (cudaMalloc(&p->ktab, size_t(rows * (ws + 2 * ks)) * p->rsize) != cudaSuccess) {
+        const bool have = cudaMalloc(&p->ktab, size_t(rows * (ws + 2 * ks)) * p->rsize) == cudaSuccess;
+        if (!have) {
             cudaGetLastError();
-            dft_plan_destroy(p);
-            return fail(nullptr, DFT_ENOMEM, "cudaMalloc failed: |k| tables");
+            p->ktab = nullptr;
+            if (cubic) {
+                dft_plan_destroy(p);
+                return fail(nullptr, DFT_ENOMEM, "cudaMalloc failed: |k| tables");
+            }
         }
-        cudaError_t te;
-        if (f64) {
-            SpeciesDesc<double>& sp = p->spd;
-            double* base = static_cast<double*>(p->ktab);
+        auto fill = [&](auto* base, auto& sp) -> cudaError_t {
+            using Real = std::remove_reference_t<decltype(*base)>;
             sp.tab_w = base; sp.tab_k = base + rows * ws; sp.tab_dk = base + rows * (ws + ks);
-            sp.tab_m2max = (int)m2max;
+            sp.tab_oct = cubic ? 0 : 1;
             sp.tab_ws = (int)ws; sp.tab_ks = (int)ks;
-            te = Passes<double>::build_ktab(nullptr, sp, p->kf[0]);
-        } else {
-            SpeciesDesc<float>& sp = p->spf;
-            float* base = static_cast<float*>(p->ktab);
-            sp.tab_w = base; sp.tab_k = base + rows * ws; sp.tab_dk = base + rows * (ws + ks);
-            sp.tab_m2max = (int)m2max;
-            sp.tab_ws = (int)ws; sp.tab_ks = (int)ks;
-            te = Passes<float>::build_ktab(nullptr, sp, p->kf[0]);
-        }
+            return Passes<Real>::build_ktab(nullptr, g, sp, p->kf[0], Real(p->kf[0]), Real(p->kf[1]), Real(p->kf[2]),
+                                            rows);
+        };
+        cudaError_t te = cudaSuccess;
+        if (have) te = f64 ? fill(static_cast<double*>(p->ktab), p->spd) : fill(static_cast<float*>(p->ktab), p->spf);
         if (te != cudaSuccess) {
             dft_plan_destroy(p);
             return fail(nullptr, DFT_ECUDA, std::string("|k| tables: ") + cudaGetErrorString(te));

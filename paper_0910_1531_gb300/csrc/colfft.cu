@@ -1,0 +1,74 @@
+// Launchers of the run-time column transform, compiled once per precision (DFT_INST_REAL).
+#include "kernels.cuh"
+#include "launch.cuh"
+#include "passes.h"
+
+namespace {
+template <typename Real, bool INV, int T, bool BIG>
+cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool zax, int ncomp,
+                   typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw, long long polls) {
+    using C = typename Cplx<Real>::type;
+    constexpr int E = int(sizeof(C) / 8);
+    dftk::ColBox cb;
+    cb.n = pa.n;
+    cb.nbox = pa.n <= 256 ? 1 : 2;
+    cb.rows = dft_col_box_rows(pa.n);
+    cb.elems = dft_col_elems<Real>(pa.n, T);
+    CUtensorMap map;
+    const unsigned long long dims[4] = {(unsigned long long)g.nxh * E, (unsigned long long)g.ny,
+                                        (unsigned long long)g.nz, (unsigned long long)ncomp};
+    const unsigned long long strides[3] = {(unsigned long long)g.pxh * sizeof(C),
+                                           (unsigned long long)g.ny * g.pxh * sizeof(C),
+                                           (unsigned long long)g.nc * sizeof(C)};
+    const unsigned box[4] = {unsigned(T * E), zax ? 1u : unsigned(cb.rows), zax ? unsigned(cb.rows) : 1u, 1u};
+    cudaError_t e = tma_encode_4d(&map, data, dims, strides, box);
+    if (e != cudaSuccess) return e;
+    const int ntx = (int)ceil_div(g.nxh, T), other = zax ? g.ny : g.nz;
+    const int ntiles = ntx * other * ncomp;
+    const size_t sm = dft_col_smem<Real>(pa.n, T, pa.nstages);
+    auto kern = dftk::k_colfft<Real, INV, T, BIG>;
+    const int fit = resident_blocks(kern, dftk::kThreads, sm);
+    return launch_k(kern, ntiles < fit ? ntiles : fit, dftk::kThreads, sm, st, g.pdl, map, pa, cb, zax ? 1 : 0, ntx,
+                    other, ntiles, status, tw, polls);
+}
+
+template <typename Real, int T>
+cudaError_t launch_t(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int ncomp,
+                     typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw,
+                     long long polls) {
+    const bool big = dft_has_big_prime(pa.n);
+    if (inv)
+        return big ? launch<Real, true, T, true>(st, g, pa, zax, ncomp, data, status, tw, polls)
+                   : launch<Real, true, T, false>(st, g, pa, zax, ncomp, data, status, tw, polls);
+    return big ? launch<Real, false, T, true>(st, g, pa, zax, ncomp, data, status, tw, polls)
+               : launch<Real, false, T, false>(st, g, pa, zax, ncomp, data, status, tw, polls);
+}
+
+template <typename Real, int T> cudaError_t init_t() {
+    cudaError_t e = cudaSuccess, r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, false, T, false>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, true, T, false>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, false, T, true>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, true, T, true>)) != cudaSuccess) e = r;
+    return e;
+}
+}  // namespace
+
+template <typename Real>
+cudaError_t ColFft<Real>::init() {
+    cudaError_t e = init_t<Real, 8>(), r = init_t<Real, 4>();
+    if constexpr (sizeof(Real) == 4)
+        if (r == cudaSuccess) r = init_t<Real, 16>();
+    return e != cudaSuccess ? e : r;
+}
+
+template <typename Real>
+cudaError_t ColFft<Real>::run(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int T,
+                              int ncomp, C* data, int* status, const C* tw, long long polls) {
+    if constexpr (sizeof(Real) == 4)
+        if (T >= 16) return launch_t<Real, 16>(st, inv, g, pa, zax, ncomp, data, status, tw, polls);
+    return T >= 8 ? launch_t<Real, 8>(st, inv, g, pa, zax, ncomp, data, status, tw, polls)
+                  : launch_t<Real, 4>(st, inv, g, pa, zax, ncomp, data, status, tw, polls);
+}
+
+template struct ColFft<DFT_INST_REAL>;

@@ -38,17 +38,48 @@ template <typename C> __device__ __forceinline__ C cconj(C a) { return cmake<C>(
 template <typename C> __device__ __forceinline__ C cmul_i(C a) { return cmake<C>(-a.y, a.x); }
 template <typename C> __device__ __forceinline__ C cmul_mi(C a) { return cmake<C>(a.y, -a.x); }
 
-// Radix decomposition of one axis length: n = prod radix[s]; radices 2, 3, 4, 8, 16 and the
-// odd primes 5..DFT_MAX_PRIME (run-time transforms only; see dft_radix_plan).
+// Division by a positive run-time constant d: floor(x / d) = hi32(x ceil(2^32 / d)) for
+// 0 <= x with x d < 2^32 (the tasks and items of one block: both factors below 2^16).
+struct FastDiv {
+    unsigned mul;   // 0 for d = 1
+    int d;
+    FastDiv() = default;
+    __host__ __device__ explicit FastDiv(int dd) : mul(dd > 1 ? 0xffffffffu / (unsigned)dd + 1u : 0u), d(dd) {}
+    __device__ __forceinline__ int div(int x) const { return mul ? (int)__umulhi((unsigned)x, mul) : x; }
+};
+
+// Radix decomposition of one axis length: n = prod radix[s]; the radices of dft_small and the
+// primes up to DFT_MAX_PRIME (run-time transforms only; see dft_radix_plan, dft_mixed_plan).
+// Stage s: ns = product of the earlier radices, m = n / radix butterflies per line, twiddle step
+// n / (ns radix).
 struct AxisPlan {
     int n;
     int nstages;
     int radix[DFT_MAXSTAGES];
+    int m[DFT_MAXSTAGES];
+    int tws[DFT_MAXSTAGES];
+    FastDiv ns[DFT_MAXSTAGES];
 };
 
-// Largest prime factor an axis length may have.  Factors 5..31 take a direct odd-radix stage
-// (the R-point DFT by its definition) in the run-time transforms.
+// Fill the per-stage constants from n and the radices.
+inline void dft_finish_plan(AxisPlan* p) {
+    int ns = 1;
+    for (int s = 0; s < p->nstages; ++s) {
+        p->m[s] = p->n / p->radix[s];
+        p->tws[s] = p->n / (ns * p->radix[s]);
+        p->ns[s] = FastDiv(ns);
+        ns *= p->radix[s];
+    }
+}
+
+// Largest prime factor an axis length may have.  Factors 11..31 take a stage of their own
+// (rt_stage_prime); lengths with one of 17..31 ("big" primes) run kernels compiled for them.
 #define DFT_MAX_PRIME 31
+inline bool dft_has_big_prime(int n) {
+    for (int p : {17, 19, 23, 29, 31})
+        if (n % p == 0) return true;
+    return false;
+}
 
 // Radix plan of an axis length: the 3s, then the other odd primes up to DFT_MAX_PRIME, then
 // 16s and one of 2 / 4 / 8.  False if n has a larger prime factor or needs more than
@@ -67,7 +98,47 @@ inline bool dft_radix_plan(int n, AxisPlan* out) {
         while (m % p == 0) { if (!push(p)) return false; m /= p; }
     while (m >= 16 && m % 16 == 0) { if (!push(16)) return false; m /= 16; }
     if (m == 2 || m == 4 || m == 8) { if (!push(m)) return false; m = 1; }
+    dft_finish_plan(out);
     return m == 1 && out->nstages > 0;
+}
+
+// Radix plan of the run-time transforms: the factorisation into the radices 2..10, 12, 14, 15, 16
+// and the primes 11..31 with the least estimated work, larger radices first (a first stage takes
+// no twiddles).  A stage of radix R costs its threads R (memory and index work + flops of an
+// R-point DFT, per element) for every wave of a block's 256 threads over the m T butterflies of a
+// 16-column tile, averaged with the same without the rounding to whole waves (other tiles of the
+// SM fill it), and a barrier.  Two stages of near-equal radices win for most lengths (160 =
+// 16 x 10, 120 = 12 x 10, 84 = 12 x 7), three above 256.
+inline bool dft_mixed_plan(int n, AxisPlan* out) {
+    static const struct { int r; double flops; } kR[] = {
+        {31, 55}, {29, 52}, {23, 44}, {19, 39}, {17, 36}, {13, 27}, {11, 24}, {16, 10.5}, {15, 10}, {14, 11},
+        {12, 7.5}, {10, 7.5}, {9, 8.5}, {8, 6.5}, {7, 9}, {6, 5}, {5, 6.5}, {4, 4}, {3, 4}, {2, 2}};
+    AxisPlan cur{}, best{};
+    double best_cost = 1e30;
+    cur.n = n;
+    auto search = [&](auto&& self, int rem, int from, double cost) -> void {
+        if (cost >= best_cost) return;
+        if (rem == 1) {
+            best = cur;
+            best_cost = cost;
+            return;
+        }
+        if (cur.nstages == DFT_MAXSTAGES) return;
+        for (int i = from; i < int(sizeof(kR) / sizeof(kR[0])); ++i) {
+            const int r = kR[i].r;
+            if (rem % r) continue;
+            const double waves = double(n / r) * 16.0 / 256.0;
+            const double whole = double((n / r * 16 + 255) / 256);
+            cur.radix[cur.nstages++] = r;
+            self(self, rem / r, i, cost + 0.5 * (waves + whole) * r * (7.0 + kR[i].flops) + 40.0);
+            --cur.nstages;
+        }
+    };
+    search(search, n, 0, 0.0);
+    if (best.nstages == 0) return false;
+    *out = best;
+    dft_finish_plan(out);
+    return true;
 }
 
 // Axis lengths a plan accepts: 4 <= n <= 512 with a radix plan.
@@ -157,12 +228,13 @@ struct SpeciesDesc {
     Real es_dc[DFT_MAXS][DFT_MAXS];     // d es_c / d Gamma
     Real inv_n;                         // 1 / N
     int coulomb_limit;                  // Gamma == 0: kernel is lambda_B z_i z_j / r inside R_ij
-    // Optional tables of the |k|-only factors on a cubic box, indexed by the integer
-    // m2 = mx^2 + my^2 + mz^2 (|k| = kf sqrt(m2)); null: the kernels evaluate them per point.
-    const Real* tab_w;                  // [m2][tab_ws]: w0_s at 2 s, j3_s at 2 s + 1
-    const Real* tab_k;                  // [m2][tab_ks]: DC_ij_hat at j (j + 1) / 2 + i, i <= j
-    const Real* tab_dk;                 // [m2][tab_ks]: d DC_ij_hat / d Gamma, same order
-    int tab_m2max;
+    // Optional tables of the |k|-only factors: on a cubic box by the integer m2 = mx^2 + my^2 + mz^2
+    // (|k| = kf sqrt(m2)), else (tab_oct) by (kx, |ky|, |kz|); null: the kernels evaluate them per
+    // point.
+    const Real* tab_w;                  // [row][tab_ws]: w0_s at 2 s, j3_s at 2 s + 1
+    const Real* tab_k;                  // [row][tab_ks]: DC_ij_hat at j (j + 1) / 2 + i, i <= j
+    const Real* tab_dk;                 // [row][tab_ks]: d DC_ij_hat / d Gamma, same order
+    int tab_oct;
     int tab_ws, tab_ks;                 // record lengths: 2 S and S (S + 1) / 2 rounded up to 16 bytes
     // Optional per-axis terms of the discrete Laplacian, sin^2(k_d h_d / 2) / h_d^2 by FFT index:
     // x indices at 0, y at nx, z at nx + ny (k_laptab); null: the kernels evaluate them per point.

@@ -57,10 +57,11 @@ cudaError_t Passes<Real>::canon_scale(cudaStream_t st, Ctl* ctl, const SpeciesDe
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::build_ktab(cudaStream_t st, const SpeciesDesc<Real>& sp, double kf) {
-    const int n = sp.tab_m2max + 1;
-    dftk::k_ktab<Real><<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(sp, kf, sp.tab_m2max, const_cast<Real*>(sp.tab_w),
-                                                                  const_cast<Real*>(sp.tab_k), const_cast<Real*>(sp.tab_dk));
+cudaError_t Passes<Real>::build_ktab(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, double kf,
+                                     Real kfx, Real kfy, Real kfz, long long rows) {
+    dftk::k_ktab<Real><<<(unsigned)ceil_div(rows, 256), 256, 0, st>>>(
+        g, sp, kf, kfx, kfy, kfz, rows, const_cast<Real*>(sp.tab_w), const_cast<Real*>(sp.tab_k),
+        const_cast<Real*>(sp.tab_dk));
     return cudaGetLastError();
 }
 
@@ -72,19 +73,13 @@ cudaError_t Passes<Real>::build_laptab(cudaStream_t st, const GridDesc& g, Real 
 }
 
 template <typename Real>
-int Passes<Real>::tile_y(int n, size_t budget) {
-    if (dft_is_ct_size(n)) return dft_tile_y<Real>(n);
-    for (int T = 16; T >= 1; T /= 2)
-        if (smem_col(n, T, 2) <= budget) return T;
-    return 1;
+int Passes<Real>::tile_y(const GridDesc& g) {
+    return dft_is_ct_size(g.ny) ? dft_tile_y<Real>(g.ny) : dft_tile_rt<Real>(g.ny, g.nxh);
 }
 
 template <typename Real>
-int Passes<Real>::tile_z(int n, size_t budget) {
-    if (dft_is_ct_size(n)) return dft_tile_z<Real>(n);
-    for (int T = 16; T >= 1; T /= 2)
-        if (smem_col(n, T, 7) <= budget) return T;
-    return 1;
+int Passes<Real>::tile_z(const GridDesc& g) {
+    return dft_is_ct_size(g.nz) ? dft_tile_z<Real>(g.nz) : dft_tile_rt<Real>(g.nz, g.nxh);
 }
 
 template <typename Real>
@@ -121,10 +116,11 @@ cudaError_t Passes<Real>::zconv_bwd(cudaStream_t st, const GridDesc& g, const Ax
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
-                                         Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
-                                         const C* esB, const C* tw) {
-    DFT_SWITCH_Z(g.nz, zconv_bwd_pair(st, g, sp, kfx, kfy, kfz, ncomp_out, ctl, phi, esA, esB, tw))
+cudaError_t Passes<Real>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
+                                         const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz,
+                                         int ncomp_out, const Ctl* ctl, C* phi, const C* esA, const C* esB,
+                                         const C* tw) {
+    DFT_SWITCH_Z(g.nz, zconv_bwd_pair(st, g, pz, sp, T, kfx, kfy, kfz, ncomp_out, ctl, phi, esA, esB, tw))
 }
 
 template <typename Real>
@@ -138,19 +134,43 @@ cudaError_t Passes<Real>::zfft(cudaStream_t st, bool inv, const GridDesc& g, int
     DFT_SWITCH_Z(g.nz, zfft(st, inv, g, ncomp, data, status, tw, polls))
 }
 
+namespace {
+// blocks of the k-space products passes: every k point once, at most 16 blocks per SM
+unsigned zmul_blocks(const GridDesc& g) {
+    static const int sms = [] {
+        int dev = 0, n = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return n;
+    }();
+    const long long want = ceil_div((long long)g.nz * g.ny * g.nxh, dftk::kThreads), cap = (long long)sms * 16;
+    return (unsigned)(want < cap ? want : cap);
+}
+}  // namespace
+
 template <typename Real>
 cudaError_t Passes<Real>::zmul(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
-                               Real kfz, const C* in, C* slot_n, C* slot_es) {
-    const long long npt = (long long)g.nz * g.ny * g.nxh;
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    const long long want = ceil_div(npt, dftk::kThreads), cap = (long long)sms * 16;
-    return launch_k(dftk::k_zmul<Real>, (unsigned)(want < cap ? want : cap), dftk::kThreads, 0, st, g.pdl, g, sp, kfx,
-                    kfy, kfz, in, slot_n, slot_es);
+                               Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, double* red_energy) {
+    const unsigned grid = zmul_blocks(g);
+    if (red_energy)
+        return launch_k(dftk::k_zmul<Real, true>, grid, dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, want_psi,
+                        in, slot_n, slot_es, red_energy);
+    return launch_k(dftk::k_zmul<Real, false>, grid, dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, want_psi, in,
+                    slot_n, slot_es, red_energy);
+}
+
+template <typename Real>
+cudaError_t Passes<Real>::zmul_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                   Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi,
+                                   const C* esA, const C* esB, C* es_mat) {
+    return launch_k(dftk::k_zmul_bwd<Real>, zmul_blocks(g), dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, flags,
+                    ncomp_out, samples, ctl, phi, esA, esB, es_mat);
+}
+
+template <typename Real>
+long long Passes<Real>::energy_blocks(const GridDesc& g) {
+    if (dft_is_ct_size(g.nz)) return ceil_div(g.nxh, dft_tile_z<Real>(g.nz)) * g.ny;
+    return zmul_blocks(g);
 }
 
 template <typename Real>
@@ -228,17 +248,33 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 }  // namespace
 
-cudaError_t tma_encode_3d(CUtensorMap* map, void* base, unsigned long long d0, unsigned long long d1,
-                          unsigned long long d2, unsigned long long stride1_bytes, unsigned long long stride2_bytes,
-                          unsigned b0, unsigned b1, unsigned b2) {
+namespace {
+cudaError_t tma_encode(CUtensorMap* map, int rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                       const cuuint32_t* box) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
-    const cuuint64_t dims[3] = {d0, d1, d2};
-    const cuuint64_t strides[2] = {stride1_bytes, stride2_bytes};
-    const cuuint32_t box[3] = {b0, b1, b2};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, base, dims, strides, box, estr,
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, rank, base, dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+}  // namespace
+
+cudaError_t tma_encode_4d(CUtensorMap* map, void* base, const unsigned long long dims[4],
+                          const unsigned long long stride_bytes[3], const unsigned box[4]) {
+    cuuint64_t d[4], st[3];
+    cuuint32_t b[4];
+    for (int i = 0; i < 4; ++i) { d[i] = dims[i]; b[i] = box[i]; }
+    for (int i = 0; i < 3; ++i) st[i] = stride_bytes[i];
+    return tma_encode(map, 4, base, d, st, b);
+}
+
+cudaError_t tma_encode_3d(CUtensorMap* map, void* base, unsigned long long d0, unsigned long long d1,
+                          unsigned long long d2, unsigned long long stride1_bytes, unsigned long long stride2_bytes,
+                          unsigned b0, unsigned b1, unsigned b2) {
+    const cuuint64_t dims[3] = {d0, d1, d2};
+    const cuuint64_t strides[2] = {stride1_bytes, stride2_bytes};
+    const cuuint32_t box[3] = {b0, b1, b2};
+    return tma_encode(map, 3, base, dims, strides, box);
 }

@@ -15,6 +15,8 @@
 // exp(-2 pi i m / n), m < n, computed in double on the host.
 #pragma once
 
+#include <utility>
+
 #include "common.cuh"
 
 template <bool INV, typename C> __device__ __forceinline__ void dft2(C* v) {
@@ -97,12 +99,262 @@ template <bool INV, typename C> __device__ __forceinline__ void dft16(C* v) {
     }
 }
 
+// cos(2 pi p / q) and sin(2 pi p / q) in double at compile time: the angle reduced to [0, pi/4]
+// by symmetry, then the Taylor series.
+__host__ __device__ constexpr double ct_taylor(double x, int first) {
+    double term = first ? x : 1.0, sum = term;
+    for (int k = first + 1; k < 30; k += 2) {
+        term *= -x * x / (double(k) * double(k + 1));
+        sum += term;
+    }
+    return sum;
+}
+__host__ __device__ constexpr double ct_sin2pi(int p, int q);
+__host__ __device__ constexpr double ct_cos2pi(int p, int q) {
+    p = ((p % q) + q) % q;
+    if (2 * p > q) p = q - p;
+    if (4 * p > q) return -ct_cos2pi(q - 2 * p, 2 * q);
+    if (8 * p > q) return ct_sin2pi(q - 4 * p, 4 * q);
+    return ct_taylor(6.28318530717958647692 * double(p) / double(q), 0);
+}
+__host__ __device__ constexpr double ct_sin2pi(int p, int q) {
+    p = ((p % q) + q) % q;
+    if (2 * p > q) return -ct_sin2pi(q - p, q);
+    if (4 * p > q) return ct_sin2pi(q - 2 * p, 2 * q);
+    if (8 * p > q) return ct_cos2pi(q - 4 * p, 4 * q);
+    return ct_taylor(6.28318530717958647692 * double(p) / double(q), 1);
+}
+
+template <int... I, typename F> __device__ __forceinline__ void ct_for_impl(std::integer_sequence<int, I...>, F&& f) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, typename F> __device__ __forceinline__ void ct_for(F&& f) {
+    ct_for_impl(std::make_integer_sequence<int, N>{}, f);
+}
+
+// DFT of odd prime length R by pairs: with a_r = v_r + v_(R-r), b_r = v_r - v_(R-r), r = 1..(R-1)/2,
+// X_q, X_(R-q) = v_0 + sum_r a_r cos(2 pi r q / R) -+ i sum_r b_r sin(2 pi r q / R).
+template <int R, bool INV, typename C> __device__ __forceinline__ void dft_odd(C* v) {
+    using T = decltype(C().x);
+    constexpr int H = (R - 1) / 2;
+    C a[H], b[H];
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+        a[r] = cadd(v[r + 1], v[R - 1 - r]);
+        b[r] = csub(v[r + 1], v[R - 1 - r]);
+    }
+    const C v0 = v[0];
+#pragma unroll
+    for (int r = 0; r < H; ++r) v[0] = cadd(v[0], a[r]);
+    ct_for<H>([&](auto qc) {
+        constexpr int q = decltype(qc)::value + 1;
+        C m = v0, t = cmake<C>(T(0), T(0));
+        ct_for<H>([&](auto rc) {
+            constexpr int r = decltype(rc)::value + 1;
+            constexpr double c = ct_cos2pi(r * q, R), s = ct_sin2pi(r * q, R);
+            m = cmake<C>(m.x + a[r - 1].x * T(c), m.y + a[r - 1].y * T(c));
+            t = cmake<C>(t.x + b[r - 1].x * T(s), t.y + b[r - 1].y * T(s));
+        });
+        const C it = rot<INV>(t);
+        v[q] = cadd(m, it);
+        v[R - q] = csub(m, it);
+    });
+}
+
+template <int R, bool INV, typename C> __device__ __forceinline__ void dft_small(C* v);
+
+// DFT of length N1 N2 (coprime) without twiddles (Good-Thomas): inputs taken at N2 n1 + N1 n2 mod N,
+// outputs at the index congruent to k1 mod N1 and k2 mod N2.
+template <int N1, int N2, bool INV, typename C> __device__ __forceinline__ void dft_coprime(C* v) {
+    constexpr int N = N1 * N2;
+    C y[N];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) {
+        C u[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) u[n1] = v[(N2 * n1 + N1 * n2) % N];
+        dft_small<N1, INV>(u);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) y[k1 * N2 + n2] = u[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) {
+        C u[N2];
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) u[n2] = y[k1 * N2 + n2];
+        dft_small<N2, INV>(u);
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (k % N1 == k1) v[k] = u[k % N2];
+    }
+}
+
+// DFT of length 9 as three by three with the twiddles W9^(n2 k1).
+template <bool INV, typename C> __device__ __forceinline__ void dft9(C* v) {
+    using T = decltype(C().x);
+    C y[9];
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+        C u[3] = {v[n2], v[n2 + 3], v[n2 + 6]};
+        dft3<INV>(u);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) y[k1 * 3 + n2] = u[k1];
+    }
+    ct_for<2>([&](auto kc) {
+        ct_for<2>([&](auto nc) {
+            constexpr int k1 = decltype(kc)::value + 1, n2 = decltype(nc)::value + 1;
+            constexpr double c = ct_cos2pi(k1 * n2, 9), s = ct_sin2pi(k1 * n2, 9);
+            y[k1 * 3 + n2] = cmul(y[k1 * 3 + n2], cmake<C>(T(c), T(INV ? s : -s)));
+        });
+    });
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        C u[3] = {y[k1 * 3], y[k1 * 3 + 1], y[k1 * 3 + 2]};
+        dft3<INV>(u);
+#pragma unroll
+        for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = u[k2];
+    }
+}
+
 template <int R, bool INV, typename C> __device__ __forceinline__ void dft_small(C* v) {
     if constexpr (R == 2) dft2<INV>(v);
     else if constexpr (R == 3) dft3<INV>(v);
     else if constexpr (R == 4) dft4<INV>(v);
+    else if constexpr (R == 5 || R == 7) dft_odd<R, INV>(v);
+    else if constexpr (R == 6) dft_coprime<2, 3, INV>(v);
     else if constexpr (R == 8) dft8<INV>(v);
+    else if constexpr (R == 9) dft9<INV>(v);
+    else if constexpr (R == 10) dft_coprime<2, 5, INV>(v);
+    else if constexpr (R == 12) dft_coprime<4, 3, INV>(v);
+    else if constexpr (R == 14) dft_coprime<2, 7, INV>(v);
+    else if constexpr (R == 15) dft_coprime<3, 5, INV>(v);
     else dft16<INV>(v);
+}
+
+// ------------------------------------------------------------------------------------
+// Run-time transforms: the Stockham stages of an AxisPlan.  Lines are the columns of a tile T
+// wide (T > 0: element e of line t at e T + t, a thread keeps its column), or rows (T == 0:
+// element e of line l at e + l ls, ls odd, line index fastest across threads, so that the
+// butterflies of a half-warp fall into distinct banks).  NT: threads of the block.
+// Divisions by run-time constants are multiplications (FastDiv).
+// ------------------------------------------------------------------------------------
+template <int T> __device__ __forceinline__ void rt_split(int task, int lines, const FastDiv& dl, int& line, int& j) {
+    if constexpr (T > 0) {
+        line = task % T;
+        j = task / T;
+    } else {
+        j = dl.div(task);
+        line = task - j * lines;
+    }
+}
+
+template <int R, bool INV, int T, int NT, typename C>
+__device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
+                                         int lines, const FastDiv& dl, int ls, const C* __restrict__ tw) {
+    constexpr int ES = T > 0 ? T : 1;
+    const int m = p.m[s], ns = p.ns[s].d, tws = p.tws[s];
+    const FastDiv dns = p.ns[s];
+    const int total = m * (T > 0 ? T : lines);
+    for (int task = threadIdx.x; task < total; task += NT) {
+        int line, j;
+        rt_split<T>(task, lines, dl, line, j);
+        const int off = T > 0 ? line : line * ls;
+        const int q = dns.div(j), k = j - q * ns;
+        const C* s0 = src + off + j * ES;
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = s0[r * m * ES];
+        if (ns > 1) {
+            const C* w0 = tw + k * tws;
+#pragma unroll
+            for (int r = 1; r < R; ++r) {
+                C w = w0[(r - 1) * k * tws];
+                if (INV) w.y = -w.y;
+                v[r] = cmul(v[r], w);
+            }
+        }
+        dft_small<R, INV>(v);
+        C* d0 = dst + off + (q * ns * R + k) * ES;
+#pragma unroll
+        for (int r = 0; r < R; ++r) d0[r * ns * ES] = v[r];
+    }
+}
+
+// Stage of a prime radix R >= 11 (the pairs of dft_odd), its outputs spread over threads: a thread
+// forms X_q and X_(R-q) of QG consecutive q of one butterfly (and X_0 with the first ones).  The
+// roots W_R^(r q) = tw[(r q mod R) m] are the same for a whole butterfly and mostly for a warp.
+template <int R, bool INV, int T, int NT, typename C>
+__device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
+                                            int lines, const FastDiv& dl, int ls, const C* __restrict__ tw) {
+    using F = decltype(C().x);
+    constexpr int ES = T > 0 ? T : 1;
+    constexpr int H = (R - 1) / 2, QG = 4, NG = (H + QG - 1) / QG;
+    const int m = p.m[s], ns = p.ns[s].d, tws = p.tws[s];
+    const FastDiv dns = p.ns[s];
+    const int per = m * (T > 0 ? T : lines);
+    for (int task = threadIdx.x; task < per * NG; task += NT) {
+        int grp = 0, rem = task;
+        while (rem >= per) { rem -= per; ++grp; }
+        int line, j;
+        rt_split<T>(rem, lines, dl, line, j);
+        const int off = T > 0 ? line : line * ls;
+        const int q = dns.div(j), k = j - q * ns;
+        const C* s0 = src + off + j * ES;
+        const C v0 = s0[0];
+        C a[H], b[H], x0 = v0;
+#pragma unroll
+        for (int r = 1; r <= H; ++r) {
+            C u = s0[r * m * ES], w = s0[(R - r) * m * ES];
+            if (ns > 1) {
+                C t = tw[r * k * tws], t2 = tw[(R - r) * k * tws];
+                if (INV) { t.y = -t.y; t2.y = -t2.y; }
+                u = cmul(u, t);
+                w = cmul(w, t2);
+            }
+            a[r - 1] = cadd(u, w);
+            b[r - 1] = csub(u, w);
+            x0 = cadd(x0, a[r - 1]);
+        }
+        C* d0 = dst + off + (q * ns * R + k) * ES;
+        if (grp == 0) d0[0] = x0;
+        const int q1 = grp * QG + QG < H ? grp * QG + QG : H;
+#pragma unroll 1
+        for (int o = grp * QG + 1; o <= q1; ++o) {
+            C c = v0, t = cmake<C>(F(0), F(0));
+            int e = 0;
+#pragma unroll
+            for (int r = 0; r < H; ++r) {
+                e += o;
+                if (e >= R) e -= R;
+                const C w = tw[e * m];         // (cos, -sin)
+                c = cmake<C>(c.x + a[r].x * w.x, c.y + a[r].y * w.x);
+                t = cmake<C>(t.x - b[r].x * w.y, t.y - b[r].y * w.y);
+            }
+            const C it = rot<INV>(t);
+            d0[o * ns * ES] = cadd(c, it);
+            d0[(R - o) * ns * ES] = csub(c, it);
+        }
+    }
+}
+
+// Stage s of a plan.  BIG: lengths with a prime factor of 17..31 (kernels of their own, whose
+// register budget the other lengths do not pay).
+template <bool INV, int T, int NT, bool BIG, typename C>
+__device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPlan& p, int s, int lines,
+                                             const FastDiv& dl, int ls, const C* tw) {
+#define DFT_RT(R) case R: rt_stage<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw); break;
+#define DFT_RTP(R) case R: rt_stage_prime<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw); break;
+    switch (p.radix[s]) {
+        DFT_RT(2) DFT_RT(3) DFT_RT(4) DFT_RT(5) DFT_RT(6) DFT_RT(7) DFT_RT(8) DFT_RT(9) DFT_RT(10) DFT_RT(12)
+        DFT_RT(14) DFT_RT(15) DFT_RT(16)
+        DFT_RTP(11) DFT_RTP(13)
+        default:
+            if constexpr (BIG) {
+                switch (p.radix[s]) { DFT_RTP(17) DFT_RTP(19) DFT_RTP(23) DFT_RTP(29) DFT_RTP(31) }
+            }
+    }
+#undef DFT_RT
+#undef DFT_RTP
 }
 
 template <int R, bool INV, typename C>

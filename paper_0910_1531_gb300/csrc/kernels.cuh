@@ -5,20 +5,21 @@
 //
 //   first half  (rho -> weighted densities of eq. nDef, bulk-fluid + Poisson spectra)
 //     k_xfwd     x R2C of the S densities
-//     k_yfft     y forward
-//     k_zconv_fwd  z forward, the analytic weights of App. B (n_hat_alpha), the
+//     k_yfft_tma   y forward (k_colfft for lengths without compile-time kernels)
+//     k_zconv_fwd_*  z forward, the analytic weights of App. B (n_hat_alpha), the
 //                bulk-fluid kernel (eq. CplusPsiHat) and the Poisson symbol
 //                (eq. potentialSolution) applied in k space, z inverse of the nine
-//                weighted-density spectra (the x derivatives are formed in k_xphi)
-//     k_yfft     y inverse of the nine spectra
+//                weighted-density spectra (the x derivatives are formed in k_xphi); or as three
+//                passes (k_colfft / k_yfft_tma, k_zmul)
+//     k_yfft_tma   y inverse of the nine spectra
 //   second half (weighted densities -> c1 -> G)
 //     k_xphi     x C2R to the ten n, dPhi/dn_alpha of eq. Phi (|nV2| <= n2 bound,
 //                FP64 log(1-n3) and 1/(1-n3)^m; or another hard-sphere form), x R2C back
 //                to nine spectra
-//     k_yfft     y forward
-//     k_zconv_bwd  z forward, adjoint weights (eq. muHS), + bulk-fluid/Poisson spectra,
-//                z inverse of the S one-body correlations
-//     k_yfft     y inverse
+//     k_yfft_tma   y forward
+//     k_zconv_bwd_*  z forward, adjoint weights (eq. muHS), + bulk-fluid/Poisson spectra,
+//                z inverse of the S one-body correlations; or as three passes (k_zmul_bwd)
+//     k_yfft_tma   y inverse
 //     k_xupdate  x C2R and the update G_i = rho_bath_i exp(mu_HS_bath_i - V_i + c1_i)
 //                (eq. rhoEquation), mixing of rho for the line search, residual sums
 //
@@ -190,54 +191,6 @@ template <typename C> __device__ __forceinline__ C* align_ptr(unsigned char* p) 
     return reinterpret_cast<C*>(u);
 }
 
-// Copy a column tile (n rows of T complex, global row stride rs, columns t < valid) between
-// global and shared memory ([e][t] layout).  TT/NN > 0: compile-time tile, loads batched in
-// registers so that all of a thread's loads are in flight together.
-template <int TT, int NN, typename C>
-__device__ __forceinline__ void tile_load(C* __restrict__ dst, const C* __restrict__ src, long long rs, int valid,
-                                          int T, int n) {
-    if constexpr (TT > 0 && NN > 0) {
-        constexpr int TOTAL = TT * NN;
-        constexpr int PER = (TOTAL + kThreads - 1) / kThreads;
-        C tmp[PER];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int idx = threadIdx.x + i * kThreads;
-            const int e = idx / TT, t = idx % TT;
-            tmp[i] = cmake<C>(0, 0);
-            if ((TOTAL % kThreads == 0 || idx < TOTAL) && t < valid) tmp[i] = src[e * rs + t];
-        }
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int idx = threadIdx.x + i * kThreads;
-            if (TOTAL % kThreads == 0 || idx < TOTAL) dst[idx] = tmp[i];
-        }
-    } else {
-        for (int idx = threadIdx.x; idx < T * n; idx += blockDim.x) {
-            const int e = idx / T, t = idx - (idx / T) * T;
-            dst[idx] = (t < valid) ? src[e * rs + t] : cmake<C>(0, 0);
-        }
-    }
-}
-
-template <int TT, int NN, typename C>
-__device__ __forceinline__ void tile_store(C* __restrict__ dst, const C* __restrict__ src, long long rs, int valid,
-                                           int T, int n) {
-    if constexpr (TT > 0 && NN > 0) {
-        constexpr int TOTAL = TT * NN;
-#pragma unroll
-        for (int idx = threadIdx.x; idx < TOTAL; idx += kThreads) {
-            const int e = idx / TT, t = idx % TT;
-            if (t < valid) dst[e * rs + t] = src[idx];
-        }
-    } else {
-        for (int idx = threadIdx.x; idx < T * n; idx += blockDim.x) {
-            const int e = idx / T, t = idx - (idx / T) * T;
-            if (t < valid) dst[e * rs + t] = src[idx];
-        }
-    }
-}
-
 // ------------------------------------------------------------------------------------
 // x pass, forward: S real fields -> half spectra.  Two real rows a, b are packed as a + i b
 // into one complex transform of length nx and separated afterwards:
@@ -293,32 +246,6 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(GridDesc g, AxisPlan px, int 
         if (ra < rows) out[ra * g.pxh + k] = cmake<C>(Real(0.5) * s.x, Real(0.5) * s.y);
         if (rb < rows) out[rb * g.pxh + k] = cmake<C>(Real(0.5) * d.y, Real(-0.5) * d.x);
     }
-}
-
-// ------------------------------------------------------------------------------------
-// y pass: in-place transform of ncomp half spectra along y, tiles of T kx columns.
-// grid (ceil(nxh/T), nz, ncomp)
-// ------------------------------------------------------------------------------------
-template <typename Real, bool INV, int NY, int TY>
-__global__ void __launch_bounds__(kThreads) k_yfft(GridDesc g, AxisPlan py, int Trt,
-                                                   typename Cplx<Real>::type* __restrict__ data,
-                                                   const typename Cplx<Real>::type* __restrict__ twy) {
-    dep_launch();
-    dep_wait();
-    using C = typename Cplx<Real>::type;
-    extern __shared__ unsigned char smem_raw[];
-    const int ny = NY > 0 ? NY : g.ny, nxh = g.nxh, pxh = g.pxh;
-    const int T = TY > 0 ? TY : Trt;
-    C* tw = align_ptr<C>(smem_raw);
-    C* A = tw + ny;
-    C* B = A + T * ny;
-    for (int i = threadIdx.x; i < ny; i += blockDim.x) tw[i] = twy[i];
-    const int kx0 = blockIdx.x * T;
-    C* base = data + (long long)blockIdx.z * g.nc + (long long)blockIdx.y * ny * pxh + kx0;
-    tile_load<TY, NY>(A, base, pxh, nxh - kx0, T, ny);
-    __syncthreads();
-    C* R = any_fft<NY, INV, true, TY>(A, B, py, T, T, 1, tw);
-    tile_store<TY, NY>(base, R, pxh, nxh - kx0, T, ny);
 }
 
 // ------------------------------------------------------------------------------------
@@ -431,6 +358,105 @@ __global__ void __launch_bounds__(kThreads) k_yfft_tma(const __grid_constant__ C
     if (threadIdx.x == 0) tma::wait_all();
 }
 
+// ------------------------------------------------------------------------------------
+// Column transform of a run-time length along y or z, in place, of every component: the
+// persistent TMA pipeline of k_yfft_tma with the stages of an AxisPlan.  The tensor map views the
+// half spectra as (x: nxh E, y, z, component) 8-byte elements; a tile is T kx columns of the whole
+// axis at one index of the other axis (`other` of them) of one component, moved as nbox boxes of
+// boxrows rows (a box has at most 256; rows past the axis read as zero and are not written).
+// Memory-bound in FP32: at 160^3 8.9 us a component (3.8 TB/s; a column pass of plain tile loads,
+// divisions by run-time integers and odd primes by their R^2 terms took 44).  FP64 is bound by the
+// FP64 pipe: 21 x 21 x 161, z forward, nine components 75 us.
+// Shared memory: stage 0 | stage 1 | X | Y (only with two or more stages) | twiddles | 2 mbarriers.
+// ------------------------------------------------------------------------------------
+struct ColBox {
+    int n, nbox, rows;      // axis length; boxes of a tile and rows of a box
+    int elems;              // shared-memory elements of one tile buffer (nbox boxes, 128-byte multiple)
+};
+
+template <typename Real, bool INV, int T, bool BIG>
+__global__ void __launch_bounds__(kThreads, BIG ? 1 : 2) k_colfft(const __grid_constant__ CUtensorMap map, AxisPlan pa,
+                                                                  ColBox cb, int zax, int ntiles_x, int other,
+                                                                  int ntiles, int* __restrict__ status,
+                                                                  const typename Cplx<Real>::type* __restrict__ twd,
+                                                                  long long polls) {
+    dep_launch();
+    dep_wait();
+    using C = typename Cplx<Real>::type;
+    constexpr int E = int(sizeof(C) / 8);
+    extern __shared__ unsigned char smem_raw[];
+    const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127);
+    C* const stage0 = reinterpret_cast<C*>(base);
+    C* const X = stage0 + 2 * cb.elems;
+    C* const Y = X + cb.elems;
+    C* const tw = pa.nstages > 1 ? Y + cb.elems : Y;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + ((cb.n + 1) & ~1));
+    const uint32_t bytes = uint32_t(cb.nbox) * uint32_t(cb.rows) * uint32_t(T * sizeof(C));
+    const FastDiv one(1);
+    if (threadIdx.x == 0) {
+        tma::mbar_init(&bar[0], 1);
+        tma::mbar_init(&bar[1], 1);
+        tma::fence_mbar_init();
+    }
+    for (int i = threadIdx.x; i < cb.n; i += kThreads) tw[i] = twd[i];
+    __syncthreads();
+    auto issue = [&](int tile, int s) {
+        const int x = tile % ntiles_x, rest = tile / ntiles_x, o = rest % other, c = rest / other;
+        tma::mbar_expect_tx(&bar[s], bytes);
+        for (int b = 0; b < cb.nbox; ++b)
+            tma::load_4d(stage0 + s * cb.elems + b * cb.rows * T, &map, x * T * E, zax ? o : b * cb.rows,
+                         zax ? b * cb.rows : o, c, &bar[s]);
+    };
+    int issued = 0, consumed = 0;   // per stage, packed (stage 1 << 16) | stage 0; thread 0
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) {
+            const int tile = blockIdx.x + s * gridDim.x;
+            if (tile < ntiles) { issue(tile, s); issued += 1 << (16 * s); }
+        }
+    }
+    int it = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+        const int cur = it & 1;
+        C* st = stage0 + cur * cb.elems;
+        const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1, polls);
+        // the previous tile's store has finished reading X or Y
+        if (threadIdx.x == 0) tma::wait_read_all();
+        if (__syncthreads_or(!ok)) {
+            if (threadIdx.x == 0) {
+                atomicOr(status, DEV_TIMEOUT);
+                for (int s = 0; s < 2; ++s) {
+                    const int n_is = (issued >> (16 * s)) & 0xffff, n_co = (consumed >> (16 * s)) & 0xffff;
+                    if (n_is > n_co) tma::mbar_wait(&bar[s], (n_is - 1) & 1);
+                }
+            }
+            break;
+        }
+        consumed += 1 << (16 * cur);
+        rt_stage_any<INV, T, kThreads, BIG>(st, X, pa, 0, T, one, 1, tw);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int next = tile + 2 * gridDim.x;
+            if (next < ntiles) { issue(next, cur); issued += 1 << (16 * cur); }
+        }
+        C* a = X;
+        C* b = Y;
+        for (int s = 1; s < pa.nstages; ++s) {
+            rt_stage_any<INV, T, kThreads, BIG>(a, b, pa, s, T, one, 1, tw);
+            C* t = a; a = b; b = t;
+            if (s + 1 < pa.nstages) __syncthreads();
+        }
+        tma::fence_proxy_async();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int x = tile % ntiles_x, rest = tile / ntiles_x, o = rest % other, c = rest / other;
+            for (int q = 0; q < cb.nbox; ++q)
+                tma::store_4d(&map, x * T * E, zax ? o : q * cb.rows, zax ? q * cb.rows : o, c, a + q * cb.rows * T);
+            tma::commit();
+        }
+    }
+    if (threadIdx.x == 0) tma::wait_all();
+}
+
 // Wave vector components of tile point (kz index, t) in a z-pass tile at (kx0, ky index)
 template <typename Real> struct KPoint {
     Real kx, ky, kz, kmag;
@@ -501,150 +527,20 @@ __global__ void k_laptab(GridDesc g, Real kfx, Real kfy, Real kfz, Real* __restr
 }
 
 // ------------------------------------------------------------------------------------
-// z pass of the first half.  grid (ceil(nxh/T), ny)
-//   in:      S half spectra after x, y forward  (kx, ky, z)
-//   slot_n:  10 weighted densities, 1/N applied, after z inverse (kx, ky, z)
+// The z passes.  First half: the S half spectra of the densities after x, y forward (kx, ky, z) ->
+//   slot_n:  the nine weighted-density spectra, 1/N applied, after z inverse (kx, ky, z)
 //   slot_es: S (+1 with psi) unnormalised bulk-fluid/Poisson spectra sum_j K_ij drho_hat_j (kx, ky, kz)
-// Shared pool of 7 tiles of T x nz.
+// Second half: the nine Phi' spectra after x, y forward (kx, ky, z) ->
+//   the S one-body correlation spectra after z inverse, 1/N applied (kx, ky, z), in their place.
+//   mu_hat_i = sum_alpha Phi_hat_alpha w_hat_i^alpha(+k) (eq. muHS): with the vector weights
+//   w_hat^V2 = -i k w_hat^3 and w_hat^V1 = w_hat^V2/(4 pi R) the k-space sum needs only the five
+//   species-independent spectra Phi0, Phi1, Phi2, Phi3 + div(PhiV2), div(PhiV1).
+//   c_hat_i = (-mu_hat_i + wA es_A_i + wB es_B_i) / N.
+//   flags: 1 = hard-sphere part, 2 = electrostatic part; ncomp_out = S (or S + 1 for psi).
+// Compile-time lengths do a half in one pass (below); run-time lengths, and compile-time ones
+// where it is faster, as a z transform (k_colfft / k_yfft_tma), a k-space products pass (k_zmul,
+// k_zmul_bwd) and another z transform.
 // ------------------------------------------------------------------------------------
-template <typename Real, int NZ, int TZ, bool GRAD>
-__global__ void __launch_bounds__(kThreads) k_zconv_fwd(GridDesc g, AxisPlan pz, SpeciesDesc<Real> sp, int Trt,
-                                                        Real kfx, Real kfy, Real kfz, int want_psi,
-                                                        const typename Cplx<Real>::type* __restrict__ in,
-                                                        typename Cplx<Real>::type* __restrict__ slot_n,
-                                                        typename Cplx<Real>::type* __restrict__ slot_es,
-                                                        double* __restrict__ red_energy,
-                                                        const typename Cplx<Real>::type* __restrict__ twz) {
-    dep_launch();
-    dep_wait();
-    using C = typename Cplx<Real>::type;
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ double scratch_d[32];
-    const int nz = NZ > 0 ? NZ : g.nz, ny = g.ny, nxh = g.nxh, S = sp.S;
-    // red_energy (optional): per block, [0] = sum_k w Re(conj(drho_hat_i) es_hat_i) and
-    // [1] = sum_k w Re(conj(drho_hat_i) dK_ij/dGamma drho_hat_j), w = 1 on the kx = 0 and Nyquist
-    // planes and 2 elsewhere (the half spectrum standing for the full one)
-    double e_acc = 0.0, q_acc = 0.0;
-    const int T = TZ > 0 ? TZ : Trt;
-    const int tile = T * nz;
-    C* tw = align_ptr<C>(smem_raw);
-    C* pool[7];
-    for (int i = 0; i < 7; ++i) pool[i] = tw + nz + i * tile;
-    for (int i = threadIdx.x; i < nz; i += blockDim.x) tw[i] = twz[i];
-    const int kx0 = blockIdx.x * T;
-    const int kyi = blockIdx.y;
-    const long long zstride = (long long)ny * g.pxh;
-    const long long col0 = (long long)kyi * g.pxh + kx0;
-
-    // phase 1: forward z transform of each species tile; results end in pool[0..S-1]
-    for (int s = 0; s < S; ++s) {
-        C* b = pool[s];
-        tile_load<TZ, NZ>(b, in + (long long)s * g.nc + col0, zstride, nxh - kx0, T, nz);
-        __syncthreads();
-        C* r = any_fft<NZ, false, true, TZ>(b, pool[6], pz, T, T, 1, tw);
-        if (r != b) { pool[6] = b; pool[s] = r; }
-    }
-
-    // phase 2: k-space products at each tile point
-    const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
-    const Real fourpi = Real(4.0 * CUDART_PI);
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        const int kzi = idx / T, t = idx - (idx / T) * T;
-        const int kxi = kx0 + t;
-        const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-        C v[DFT_MAXS];
-        for (int s = 0; s < S; ++s) v[s] = pool[s][idx];
-        C acc[5];
-        for (int a = 0; a < 5; ++a) acc[a] = cmake<C>(Real(0), Real(0));
-        for (int s = 0; s < S; ++s) {
-            Real w0, j3;
-            fmt_weights<Real>(p.kmag, sp.R[s], &w0, &j3);
-            const Real R = sp.R[s];
-            acc[0] = cadd(acc[0], cscale(v[s], w0));
-            acc[1] = cadd(acc[1], cscale(v[s], R * w0));
-            acc[2] = cadd(acc[2], cscale(v[s], fourpi * R * R * w0));
-            acc[3] = cadd(acc[3], cscale(v[s], fourpi * R * R * R * j3));
-            acc[4] = cadd(acc[4], cscale(v[s], R * R * j3));       // w3 / (4 pi R)
-        }
-        if (kxi < nxh) {
-            const Real inv_lap = inverse_laplacian<Real>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
-            C dv[DFT_MAXS];
-            for (int s = 0; s < S; ++s) {
-                dv[s] = v[s];
-                if (p.zero) dv[s].x -= sp.n_rho_b[s];       // DFT(rho - rho_bath) at k = 0
-            }
-            C es[DFT_MAXS];
-            for (int s = 0; s < S; ++s) es[s] = cmake<C>(Real(0), Real(0));
-            const double wk = GRAD ? ((kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? 1.0 : 2.0) : 0.0;
-            for (int i = 0; i < S; ++i) {
-                for (int j = i; j < S; ++j) {
-                    Real dK = Real(0);
-                    const Real K = es_kernel<Real>(sp, i, j, p, inv_lap, GRAD ? &dK : nullptr);
-                    es[i] = cadd(es[i], cscale(dv[j], K));
-                    if (j != i) es[j] = cadd(es[j], cscale(dv[i], K));
-                    if constexpr (GRAD) {
-                        const double re = double(dv[i].x) * dv[j].x + double(dv[i].y) * dv[j].y;
-                        q_acc += wk * double(dK) * re * (j != i ? 2.0 : 1.0);
-                    }
-                }
-            }
-            if constexpr (GRAD)
-                for (int i = 0; i < S; ++i) e_acc += wk * (double(dv[i].x) * es[i].x + double(dv[i].y) * es[i].y);
-            const long long o = (long long)kzi * zstride + col0 + t;
-            for (int s = 0; s < S; ++s) slot_es[(long long)s * g.nc + o] = es[s];
-            if (want_psi) {
-                C q = cmake<C>(Real(0), Real(0));
-                for (int s = 0; s < S; ++s) q = cadd(q, cscale(v[s], sp.z[s]));
-                // psi_hat = 4 pi lambda_B q_hat / lap; pois[s][s] / z_s^2 = 4 pi lambda_B
-                Real flb = Real(0);
-                for (int s = 0; s < S; ++s)
-                    if (sp.z[s] != Real(0)) { flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]); break; }
-                slot_es[(long long)S * g.nc + o] = cscale(q, flb * inv_lap);
-            }
-        }
-        for (int a = 0; a < 5; ++a) pool[a][idx] = cscale(acc[a], sp.inv_n);
-    }
-    if constexpr (GRAD) {
-        const double be = block_sum(e_acc, scratch_d);
-        const double bq = block_sum(q_acc, scratch_d);
-        if (threadIdx.x == 0) {
-            const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
-            red_energy[2 * b] = be;
-            red_energy[2 * b + 1] = bq;
-        }
-    }
-    __syncthreads();
-
-    // phase 3: inverse z of the nine weighted-density spectra: n0..n3, m, then i k_y m, i k_z m,
-    // i k_y n3, i k_z n3 (zero on the Nyquist index of their axis); the derived ones first,
-    // while m and n3 are still in k space.
-    const int order[DFT_NSPEC] = {5, 6, 7, 8, 4, 3, 0, 1, 2};
-    for (int oi = 0; oi < DFT_NSPEC; ++oi) {
-        const int a = order[oi];
-        C* r;
-        if (a >= 5) {
-            const C* src = (a < 7) ? pool[4] : pool[3];
-            const int d = (a == 5 || a == 7) ? 1 : 2;
-            C* W = pool[5];
-            for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-                const int kzi = idx / T;
-                Real kd;
-                bool nyq;
-                if (d == 1) { kd = kval<Real>(kyi, g.ny, kfy); nyq = (g.ny % 2 == 0) && (2 * kyi == g.ny); }
-                else { kd = kval<Real>(kzi, g.nz, kfz); nyq = (g.nz % 2 == 0) && (2 * kzi == g.nz); }
-                const C u = src[idx];
-                W[idx] = nyq ? cmake<C>(Real(0), Real(0)) : cmake<C>(-kd * u.y, kd * u.x);
-            }
-            __syncthreads();
-            r = any_fft<NZ, true, true, TZ>(W, pool[6], pz, T, T, 1, tw);
-        } else {
-            r = any_fft<NZ, true, true, TZ>(pool[a], pool[5], pz, T, T, 1, tw);
-        }
-        tile_store<TZ, NZ>(slot_n + (long long)a * g.nc + col0, r, zstride, nxh - kx0, T, nz);
-        __syncthreads();
-    }
-}
-
 // ------------------------------------------------------------------------------------
 // Grouped z passes (compile-time length NZ, tile width TZ), grid (ceil(nxh/TZ), ny).  All
 // components of a column tile are loaded in one batch of in-flight loads and transformed by
@@ -816,41 +712,52 @@ __device__ __forceinline__ void load_record(Real (&dst)[MAXN], const Real* __res
     }
 }
 
-// Tables of the |k|-only factors for a cubic box (kf equal on the three axes): the FMT weights
-// w0, j3 of each species and the bulk-fluid kernel DC_ij_hat with its Gamma derivative, at
-// |k| = kf sqrt(m2) for every integer m2 in [0, m2max].  Evaluated once per plan with the same
-// functions the z passes call per point.
+__device__ __forceinline__ int signed_index(int j, int n) { return (2 * j <= n) ? j : j - n; }
+
+// Tables of the |k|-only factors: the FMT weights w0, j3 of each species and the bulk-fluid kernel
+// DC_ij_hat with its Gamma derivative.  On a cubic box (kf equal on the three axes) one record per
+// integer m2 = mx^2 + my^2 + mz^2, |k| = kf sqrt(m2); on other boxes (sp.tab_oct) one per (kx, |ky|,
+// |kz|), |k| as kpoint forms it.  Evaluated once per plan with the functions the z passes call
+// where there is no table.
 template <typename Real>
-__global__ void k_ktab(SpeciesDesc<Real> sp, double kf, int m2max, Real* tab_w, Real* tab_k, Real* tab_dk) {
-    const int m2 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m2 > m2max) return;
+__global__ void k_ktab(GridDesc g, SpeciesDesc<Real> sp, double kf, Real kfx, Real kfy, Real kfz, long long rows,
+                       Real* tab_w, Real* tab_k, Real* tab_dk) {
+    const long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= rows) return;
     const int S = sp.S;
-    const Real kmag = Real(kf * sqrt(double(m2)));
+    Real kmag;
+    if (sp.tab_oct) {
+        const int ix = int(row % g.nxh), rest = int(row / g.nxh), nyh = g.ny / 2 + 1;
+        const int iy = rest % nyh, iz = rest / nyh;
+        kmag = kpoint<Real>(g, ix, iy, iz, kfx, kfy, kfz).kmag;
+    } else {
+        kmag = Real(kf * sqrt(double(row)));
+    }
     for (int s = 0; s < S; ++s) {
         Real w0, j3;
         fmt_weights<Real>(kmag, sp.R[s], &w0, &j3);
-        tab_w[(long long)m2 * sp.tab_ws + 2 * s] = w0;
-        tab_w[(long long)m2 * sp.tab_ws + 2 * s + 1] = j3;
+        tab_w[row * sp.tab_ws + 2 * s] = w0;
+        tab_w[row * sp.tab_ws + 2 * s + 1] = j3;
     }
     for (int j = 0; j < S; ++j)
         for (int i = 0; i <= j; ++i) {
             Real dG = Real(0);
             const Real K = delta_c_hat<Real>(kmag, sp.es_R[i][j], sp.es_pref[i][j], sp.es_a[i][j], sp.es_b[i][j],
                                              sp.es_c[i][j], &dG, sp.es_da[i][j], sp.es_db[i][j], sp.es_dc[i][j]);
-            tab_k[(long long)m2 * sp.tab_ks + dft_pair(i, j)] = K;
-            tab_dk[(long long)m2 * sp.tab_ks + dft_pair(i, j)] = dG;
+            tab_k[row * sp.tab_ks + dft_pair(i, j)] = K;
+            tab_dk[row * sp.tab_ks + dft_pair(i, j)] = dG;
         }
 }
 
-__device__ __forceinline__ int signed_index(int j, int n) { return (2 * j <= n) ? j : j - n; }
-// m^2 = mx^2 + my^2 + mz^2 of a cubic box's mode (the |k| table index) from kx index kxi >= 0,
-// signed y index my and z index kzi
-__device__ __forceinline__ int kmode2(int kxi, int my, int kzi, int nz) {
-    const int mz = signed_index(kzi, nz);
+// Table row of the mode (kx index kxi >= 0, signed y index my, z index kzi).
+template <typename Real>
+__device__ __forceinline__ long long tab_row(const SpeciesDesc<Real>& sp, const GridDesc& g, int kxi, int my, int kzi) {
+    const int mz = signed_index(kzi, g.nz);
+    if (sp.tab_oct) return ((long long)abs(mz) * (g.ny / 2 + 1) + abs(my)) * g.nxh + kxi;
     return kxi * kxi + my * my + mz * mz;
 }
 
-// First-half z pass (same contract as k_zconv_fwd): S species spectra in, the ten weighted
+// First-half z pass: S species spectra in, the nine weighted
 // densities (z inverse, 1/N applied) and the bulk-fluid/Poisson spectra out.  Per-species loops
 // run to DFT_MAXS with guards so that every per-point array stays in registers.
 template <typename Real, int NZ, int TZ, bool GRAD>
@@ -897,15 +804,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
         const int kxi = kx0 + t;
         const bool live = kxi < nxh;
         const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-        int m2 = 0;
-        if (tab && live) { const int mz = signed_index(kzi, g.nz); m2 = kxi * kxi + my * my + mz * mz; }
+        const long long row = tab && live ? tab_row(sp, g, kxi, my, kzi) : 0;
         Real wr[DFT_TAB_W];
         Real kr[DFT_TAB_K], dkr[DFT_TAB_K];
         if (tab) {
-            load_record(wr, sp.tab_w + (long long)m2 * sp.tab_ws, 2 * S);
+            load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
             if (live) {
-                load_record(kr, sp.tab_k + (long long)m2 * sp.tab_ks, Pn);
-                if (GRAD) load_record(dkr, sp.tab_dk + (long long)m2 * sp.tab_ks, Pn);
+                load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
+                if (GRAD) load_record(dkr, sp.tab_dk + row * sp.tab_ks, Pn);
             }
         }
         C v[DFT_MAXS];
@@ -994,7 +900,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
     tiles_store_grouped<TZ, NZ>(slot_n + col0, Q, g.nc, DFT_NSPEC, zstride, nxh - kx0);
 }
 
-// Second-half z pass (same contract as k_zconv_bwd): the ten Phi' spectra in (flags & 1), the
+// Second-half z pass: the nine Phi' spectra in (flags & 1), the
 // bulk-fluid/Poisson spectra mixed in (flags & 2), ncomp_out one-body correlation spectra out.
 // The points of a thread are handled together so that all of their global and table loads are
 // in flight at once.
@@ -1058,9 +964,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
             }
         }
         if (hs && tab) {
-            int m2 = 0;
-            if (live) { const int mz = signed_index(kzi, g.nz); m2 = kxi * kxi + my * my + mz * mz; }
-            load_record(wr[i], sp.tab_w + (long long)m2 * sp.tab_ws, 2 * S);
+            load_record(wr[i], sp.tab_w + (live ? tab_row(sp, g, kxi, my, kzi) : 0) * sp.tab_ws, 2 * S);
         }
     }
 #pragma unroll
@@ -1109,8 +1013,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
 }
 
 // ------------------------------------------------------------------------------------
-// First-half z pass with TMA tiles (same contract as k_zconv_fwd without the grand-potential
-// sums), persistent like k_zconv_bwd_tma: two stages of S species tiles are filled by TMA loads
+// First-half z pass with TMA tiles (without the grand-potential sums), persistent like k_zconv_bwd_tma: two stages of S species tiles are filled by TMA loads
 // while the previous tile is transformed; seven weighted-density spectra are transformed back
 // (zgroup order), the two y derivatives formed from m and n3 after that, and the nine leave
 // through TMA stores, the bulk-fluid/Poisson spectra through plain stores.  A tensor map views a half-spectrum
@@ -1194,9 +1097,10 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
         Real kr[SM <= 3 ? 8 : DFT_TAB_K];
         auto load_tab = [&](int idx) {
             const int kxi = kx0 + idx % TZ;
-            const int m2 = (((TILE % NT == 0) || idx < TILE) && kxi < nxh) ? kmode2(kxi, my, idx / TZ, g.nz) : 0;
-            load_record(wr, sp.tab_w + (long long)m2 * sp.tab_ws, 2 * S);
-            load_record(kr, sp.tab_k + (long long)m2 * sp.tab_ks, Pn);
+            const long long row =
+                (((TILE % NT == 0) || idx < TILE) && kxi < nxh) ? tab_row(sp, g, kxi, my, idx / TZ) : 0;
+            load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
+            load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
         };
         if (tab) load_tab(threadIdx.x);
         const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1);
@@ -1314,11 +1218,16 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
 // bulk-fluid/Poisson spectra into slot_es, both in (kx, ky, kz); the same arithmetic per point as
 // k_zconv_fwd_tma.  One thread per k point, kx fastest.
 // ------------------------------------------------------------------------------------
-template <typename Real>
-__global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy, Real kfz,
+// GRAD: also the two grand-potential sums per block, red_energy[2 b] = sum_k w Re(conj(drho_hat_i)
+// es_hat_i) and red_energy[2 b + 1] = sum_k w Re(conj(drho_hat_i) dK_ij/dGamma drho_hat_j), w = 1 on
+// the kx = 0 and Nyquist planes and 2 elsewhere (the half spectrum standing for the full one).
+template <typename Real, bool GRAD>
+__global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) k_zmul(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy, Real kfz,
+                                                   int want_psi,
                                                    const typename Cplx<Real>::type* __restrict__ in,
                                                    typename Cplx<Real>::type* __restrict__ slot_n,
-                                                   typename Cplx<Real>::type* __restrict__ slot_es) {
+                                                   typename Cplx<Real>::type* __restrict__ slot_es,
+                                                   double* __restrict__ red_energy) {
     dep_launch();
     dep_wait();
     using C = typename Cplx<Real>::type;
@@ -1328,20 +1237,21 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul(Gr
     const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
     const Real fourpi = Real(4.0 * CUDART_PI);
     const bool tab = sp.tab_w != nullptr;
+    double e_acc = 0.0, q_acc = 0.0;
     for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < npt; q += (long long)gridDim.x * kThreads) {
         const int kxi = int(q % nxh);
         const long long rz = q / nxh;
         const int kyi = int(rz % g.ny), kzi = int(rz / g.ny);
         const long long o = rz * g.pxh + kxi;
         const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-        const int m2 = tab ? kmode2(kxi, signed_index(kyi, g.ny), kzi, g.nz) : 0;
+        const long long row = tab ? tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) : 0;
         C v[DFT_MAXS];
 #pragma unroll
         for (int s = 0; s < DFT_MAXS; ++s)
             if (s < S) v[s] = in[(long long)s * g.nc + o];
         {   // the nine weighted-density spectra, 1/N applied (DFT_NSPEC order), as store_wd_spectra
             Real wr[DFT_TAB_W];
-            if (tab) load_record(wr, sp.tab_w + (long long)m2 * sp.tab_ws, 2 * S);
+            if (tab) load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
             C acc[5];
 #pragma unroll
             for (int a = 0; a < 5; ++a) acc[a] = cmake<C>(Real(0), Real(0));
@@ -1362,8 +1272,24 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul(Gr
         }
         // the bulk-fluid/Poisson spectra
         Real kr[DFT_TAB_K];
-        if (tab) load_record(kr, sp.tab_k + (long long)m2 * sp.tab_ks, Pn);
+        Real dkr[GRAD ? DFT_TAB_K : 4];
+        if (tab) {
+            load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
+            if constexpr (GRAD) load_record(dkr, sp.tab_dk + row * sp.tab_ks, Pn);
+        }
         const Real inv_lap = inverse_laplacian<Real>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
+        if (want_psi) {
+            C ps = cmake<C>(Real(0), Real(0));
+            Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
+#pragma unroll
+            for (int s = 0; s < DFT_MAXS; ++s) {
+                if (s >= S) break;
+                ps = cadd(ps, cscale(v[s], sp.z[s]));
+                if (flb == Real(0) && sp.z[s] != Real(0)) flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]);
+            }
+            slot_es[(long long)S * g.nc + o] = cscale(ps, flb * inv_lap);   // psi_hat = 4 pi lambda_B q_hat / lap
+        }
+        const double wk = GRAD ? ((kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? 1.0 : 2.0) : 0.0;
         C es[DFT_MAXS];
 #pragma unroll
         for (int s = 0; s < DFT_MAXS; ++s) {
@@ -1375,25 +1301,127 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul(Gr
 #pragma unroll
             for (int i2 = 0; i2 <= j; ++i2) {
                 if (j >= S) continue;
-                Real K;
+                Real K, dK = Real(0);
                 if (tab) {
                     K = kr[dft_pair(i2, j)];
                     if (!p.zero) K -= sp.pois[i2][j] * inv_lap;
+                    if constexpr (GRAD) dK = dkr[dft_pair(i2, j)];
                 } else {
-                    K = es_kernel<Real>(sp, i2, j, p, inv_lap, nullptr);
+                    K = es_kernel<Real>(sp, i2, j, p, inv_lap, GRAD ? &dK : nullptr);
                 }
                 es[i2] = cadd(es[i2], cscale(v[j], K));
                 if (j != i2) es[j] = cadd(es[j], cscale(v[i2], K));
+                if constexpr (GRAD) {
+                    const double re = double(v[i2].x) * v[j].x + double(v[i2].y) * v[j].y;
+                    q_acc += wk * double(dK) * re * (j != i2 ? 2.0 : 1.0);
+                }
             }
         }
 #pragma unroll
-        for (int s = 0; s < DFT_MAXS; ++s)
-            if (s < S) slot_es[(long long)s * g.nc + o] = es[s];
+        for (int s = 0; s < DFT_MAXS; ++s) {
+            if (s >= S) break;
+            if constexpr (GRAD) e_acc += wk * (double(v[s].x) * es[s].x + double(v[s].y) * es[s].y);
+            slot_es[(long long)s * g.nc + o] = es[s];
+        }
+    }
+    if constexpr (GRAD) {
+        __shared__ double scratch_d[32];
+        const double be = block_sum(e_acc, scratch_d);
+        const double bq = block_sum(q_acc, scratch_d);
+        if (threadIdx.x == 0) {
+            red_energy[2 * (long long)blockIdx.x] = be;
+            red_energy[2 * (long long)blockIdx.x + 1] = bq;
+        }
     }
 }
 
 // ------------------------------------------------------------------------------------
-// Second-half z pass with TMA tiles (same contract as k_zconv_bwd), persistent: CTA b handles
+// The k-space products of the second half as a pass of their own (between the z transforms of a
+// run-time length): at each k point the nine Phi' spectra and the mixed bulk-fluid/Poisson spectra
+// into the ncomp_out correlation spectra, 1/N applied.  `samples` 2: the line search's two samples,
+// sample m's Phi' spectra at components 9 m .., its weights in ctl[m], its results at components
+// m ncomp_out ..; the ES spectra are read once for both.  One thread per k point, kx fastest; a
+// thread reads a sample's components before it writes, and a second sample's results end before
+// that sample's own Phi' or inside what the same thread has read (2 ncomp_out <= 12 < 18).
+// ------------------------------------------------------------------------------------
+template <typename Real>
+__global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bwd(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy, Real kfz,
+                                                       int flags, int ncomp_out, int samples,
+                                                       const Ctl* __restrict__ ctl, typename Cplx<Real>::type* phi,
+                                                       const typename Cplx<Real>::type* esA,
+                                                       const typename Cplx<Real>::type* esB,
+                                                       typename Cplx<Real>::type* es_mat) {
+    dep_launch();
+    dep_wait();
+    using C = typename Cplx<Real>::type;
+    constexpr int EMAX = DFT_MAXS + 1;
+    const int S = sp.S, nxh = g.nxh;
+    const long long npt = (long long)g.nz * g.ny * nxh;
+    const bool hs = (flags & 1) != 0, es_on = (flags & 2) != 0;
+    const Real fourpi = Real(4.0 * CUDART_PI);
+    const bool tab = sp.tab_w != nullptr;
+    for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < npt; q += (long long)gridDim.x * kThreads) {
+        const int kxi = int(q % nxh);
+        const long long rz = q / nxh;
+        const int kyi = int(rz % g.ny), kzi = int(rz / g.ny);
+        const long long o = rz * g.pxh + kxi;
+        Real wr[DFT_TAB_W];
+        if (hs && tab) load_record(wr, sp.tab_w + tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) * sp.tab_ws, 2 * S);
+        C ea[EMAX], eb[EMAX];
+#pragma unroll
+        for (int s = 0; s < EMAX; ++s) {
+            ea[s] = eb[s] = cmake<C>(Real(0), Real(0));
+            if (es_on && s < ncomp_out) {
+                ea[s] = esA[(long long)s * g.nc + o];
+                if (esB) eb[s] = esB[(long long)s * g.nc + o];
+            }
+        }
+#pragma unroll 1
+        for (int m = 0; m < samples; ++m) {
+            C* const ph = phi + (long long)m * DFT_NSPEC * g.nc;
+            const Real wA = CtlW<Real>::wA(ctl + m), wB = CtlW<Real>::wB(ctl + m);
+            C out[EMAX];
+#pragma unroll
+            for (int s = 0; s < EMAX; ++s) {
+                out[s] = cscale(ea[s], wA);
+                if (esB) out[s] = cadd(out[s], cscale(eb[s], wB));
+            }
+            if (es_mat) {
+#pragma unroll
+                for (int s = 0; s < EMAX; ++s)
+                    if (s < ncomp_out) es_mat[(long long)s * g.nc + o] = out[s];
+            }
+            if (hs) {
+                C x[DFT_NSPEC];
+#pragma unroll
+                for (int c = 0; c < DFT_NSPEC; ++c) x[c] = ph[(long long)c * g.nc + o];
+                const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
+                C a[5];
+                bwd_sums<Real>(x, 1, 0, p, a);
+#pragma unroll
+                for (int s = 0; s < DFT_MAXS; ++s) {
+                    if (s >= S) break;
+                    Real w0, j3;
+                    const Real Rs = sp.R[s];
+                    if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
+                    else fmt_weights<Real>(p.kmag, Rs, &w0, &j3);
+                    C mu = cscale(a[0], w0);
+                    mu = cadd(mu, cscale(a[1], Rs * w0));
+                    mu = cadd(mu, cscale(a[2], fourpi * Rs * Rs * w0));
+                    mu = cadd(mu, cscale(a[3], fourpi * Rs * Rs * Rs * j3));
+                    mu = cadd(mu, cscale(a[4], Rs * Rs * j3));
+                    out[s] = cmake<C>(out[s].x - mu.x, out[s].y - mu.y);
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < EMAX; ++s)
+                if (s < ncomp_out) phi[(long long)(m * ncomp_out + s) * g.nc + o] = cscale(out[s], sp.inv_n);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------
+// Second-half z pass with TMA tiles, persistent: CTA b handles
 // tiles b, b + gridDim.x, ...  Two shared-memory stages, each holding one tile's nine Phi'
 // spectra (in zgroup order), are filled by TMA loads (one cp.async.bulk.tensor per component,
 // completing on the stage's mbarrier) while the previous tile is transformed (seven groups: the
@@ -1526,8 +1554,9 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
         if (hs && tab) {
             const int idx = threadIdx.x;
             const int kxi = kx0 + idx % TZ;
-            const int m2 = (((TILE % NT == 0) || idx < TILE) && kxi < nxh) ? kmode2(kxi, my, idx / TZ, g.nz) : 0;
-            load_record(wr, sp.tab_w + (long long)m2 * sp.tab_ws, 2 * S);
+            const long long row =
+                (((TILE % NT == 0) || idx < TILE) && kxi < nxh) ? tab_row(sp, g, kxi, my, idx / TZ) : 0;
+            load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
         }
         C* const st = stage0 + cur * stage_elems;
         C* X = st;
@@ -1572,8 +1601,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
             }
             if (hs) {
                 if (i > 0 && tab)
-                    load_record(wr, sp.tab_w + (long long)(kxi < nxh ? kmode2(kxi, my, kzi, g.nz) : 0) * sp.tab_ws,
-                                2 * S);
+                    load_record(wr, sp.tab_w + (kxi < nxh ? tab_row(sp, g, kxi, my, kzi) : 0) * sp.tab_ws, 2 * S);
                 const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
                 C asum[5];
                 bwd_sums_folded<Real>(X, GS, pos, p, asum);
@@ -2344,114 +2372,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 1) k_xphi_cp
         __syncthreads();   // the line buffers are rewritten by the next block
     }
     if (bad) atomicOr(status, DEV_N3BOUND);
-}
-
-// ------------------------------------------------------------------------------------
-// z pass of the second half.  grid (ceil(nxh/T), ny)
-//   phi:  in  10 dPhi/dn_alpha spectra after x, y forward (kx, ky, z)
-//         out S one-body correlation spectra after z inverse, 1/N applied (kx, ky, z)
-//   mu_hat_i = sum_alpha Phi_hat_alpha w_hat_i^alpha(+k) (eq. muHS): with the vector weights
-//   w_hat^V2 = -i k w_hat^3 and w_hat^V1 = w_hat^V2/(4 pi R) the k-space sum needs only the five
-//   species-independent spectra Phi0, Phi1, Phi2, Phi3 + div(PhiV2), div(PhiV1).
-//   c_hat_i = (-mu_hat_i + wA es_A_i + wB es_B_i) / N.
-// flags: 1 = hard-sphere part, 2 = electrostatic part; ncomp_out = S (or S + 1 for psi).
-// ------------------------------------------------------------------------------------
-template <typename Real, int NZ, int TZ>
-__global__ void __launch_bounds__(kThreads) k_zconv_bwd(GridDesc g, AxisPlan pz, SpeciesDesc<Real> sp, int Trt,
-                                                        Real kfx, Real kfy, Real kfz, int flags, int ncomp_out,
-                                                        const Ctl* __restrict__ ctl,
-                                                        typename Cplx<Real>::type* phi,
-                                                        const typename Cplx<Real>::type* esA,
-                                                        const typename Cplx<Real>::type* esB,
-                                                        typename Cplx<Real>::type* es_mat,
-                                                        const typename Cplx<Real>::type* __restrict__ twz) {
-    dep_launch();
-    dep_wait();
-    using C = typename Cplx<Real>::type;
-    extern __shared__ unsigned char smem_raw[];
-    const int nz = NZ > 0 ? NZ : g.nz, ny = g.ny, nxh = g.nxh, S = sp.S;
-    const int T = TZ > 0 ? TZ : Trt;
-    const int tile = T * nz;
-    C* tw = align_ptr<C>(smem_raw);
-    C* pool[7];
-    for (int i = 0; i < 7; ++i) pool[i] = tw + nz + i * tile;
-    for (int i = threadIdx.x; i < nz; i += blockDim.x) tw[i] = twz[i];
-    const int kx0 = blockIdx.x * T;
-    const int kyi = blockIdx.y;
-    const long long zstride = (long long)ny * g.pxh;
-    const long long col0 = (long long)kyi * g.pxh + kx0;
-    const bool hs = (flags & 1) != 0, es_on = (flags & 2) != 0;
-    const Real wA = CtlW<Real>::wA(ctl), wB = CtlW<Real>::wB(ctl);
-
-    if (hs) {
-        // nine Phi' spectra (DFT_NSPEC order): 0..3 transform into accumulators 0..3, B4 into
-        // accumulator 4; -i k_y / -i k_z of Phi_V1y, Phi_V1z add to accumulator 4 and of Phi_V2y,
-        // Phi_V2z to accumulator 3 (Nyquist components of their axis dropped)
-        for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) pool[4][idx] = cmake<C>(Real(0), Real(0));
-        for (int a = 0; a < DFT_NSPEC; ++a) {
-            C* dst = (a < 4) ? pool[a] : pool[5];
-            tile_load<TZ, NZ>(dst, phi + (long long)a * g.nc + col0, zstride, nxh - kx0, T, nz);
-            __syncthreads();
-            C* r = any_fft<NZ, false, true, TZ>(dst, pool[6], pz, T, T, 1, tw);
-            if (a < 4) {
-                if (r != dst) { pool[6] = dst; pool[a] = r; }
-                continue;
-            }
-            C* acc = (a < 7) ? pool[4] : pool[3];
-            const int d = (a == 4) ? 0 : ((a == 5 || a == 7) ? 1 : 2);
-            for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-                const int kzi = idx / T;
-                const C u = r[idx];
-                if (d == 0) { acc[idx] = cadd(acc[idx], u); continue; }
-                Real kd;
-                bool nyq;
-                if (d == 1) { kd = kval<Real>(kyi, g.ny, kfy); nyq = (g.ny % 2 == 0) && (2 * kyi == g.ny); }
-                else { kd = kval<Real>(kzi, g.nz, kfz); nyq = (g.nz % 2 == 0) && (2 * kzi == g.nz); }
-                if (!nyq) acc[idx] = cadd(acc[idx], cmake<C>(kd * u.y, -kd * u.x));    // -i k_d u
-            }
-            __syncthreads();
-        }
-    }
-
-    const Real fourpi = Real(4.0 * CUDART_PI);
-    for (int idx = threadIdx.x; idx < tile; idx += blockDim.x) {
-        const int kzi = idx / T, t = idx - (idx / T) * T;
-        const int kxi = kx0 + t;
-        C out[DFT_MAXS + 1];
-        for (int s = 0; s < DFT_MAXS + 1; ++s) out[s] = cmake<C>(Real(0), Real(0));
-        if (hs) {
-            const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-            const C a0 = pool[0][idx], a1 = pool[1][idx], a2 = pool[2][idx], a3 = pool[3][idx], a4 = pool[4][idx];
-            for (int s = 0; s < S; ++s) {
-                Real w0, j3;
-                const Real R = sp.R[s];
-                fmt_weights<Real>(p.kmag, R, &w0, &j3);
-                C mu = cscale(a0, w0);
-                mu = cadd(mu, cscale(a1, R * w0));
-                mu = cadd(mu, cscale(a2, fourpi * R * R * w0));
-                mu = cadd(mu, cscale(a3, fourpi * R * R * R * j3));
-                mu = cadd(mu, cscale(a4, R * R * j3));
-                out[s] = cmake<C>(-mu.x, -mu.y);
-            }
-        }
-        if (es_on && kxi < nxh) {
-            const long long o = (long long)kzi * zstride + col0 + t;
-            for (int s = 0; s < ncomp_out; ++s) {
-                C e = cscale(esA[(long long)s * g.nc + o], wA);
-                if (esB) e = cadd(e, cscale(esB[(long long)s * g.nc + o], wB));
-                if (es_mat) es_mat[(long long)s * g.nc + o] = e;
-                out[s] = cadd(out[s], e);
-            }
-        }
-        for (int s = 0; s < ncomp_out; ++s) pool[s][idx] = cscale(out[s], sp.inv_n);
-    }
-    __syncthreads();
-
-    for (int s = 0; s < ncomp_out; ++s) {
-        C* r = any_fft<NZ, true, true, TZ>(pool[s], pool[5 + (s & 1)], pz, T, T, 1, tw);
-        tile_store<TZ, NZ>(phi + (long long)s * g.nc + col0, r, zstride, nxh - kx0, T, nz);
-        __syncthreads();
-    }
 }
 
 // ------------------------------------------------------------------------------------

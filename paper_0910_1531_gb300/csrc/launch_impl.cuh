@@ -2,26 +2,15 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "passes.h"
 
 namespace {
-// Allow each kernel the device's opt-in shared memory per block minus its static shared memory.
-template <typename K> cudaError_t set_max_smem(K kernel) {
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncAttributes fa;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 // x pass: twiddles (nx) + two buffers of `lines` rows at the kernel's row pitch
 template <typename C, int N> size_t smem_x_of(int nx, int lines) {
     const int pitch = N > 0 ? ct_row_pitch(N) : nx + 1;
     return (size_t(nx) + 2 * size_t(lines) * pitch) * sizeof(C) + 16;
 }
-template <typename C> size_t smem_col_of(int n, int T, int nbuf) { return (size_t(n) + size_t(nbuf) * T * n) * sizeof(C) + 16; }
 }  // namespace
 
 // ---------------------------------------------------------------------------------- x
@@ -198,8 +187,7 @@ cudaError_t LaunchY<Real, N>::init() {
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY>)) != cudaSuccess) e = r;
     } else {
-        if ((r = set_max_smem(dftk::k_yfft<Real, false, 0, 0>)) != cudaSuccess) e = r;
-        if ((r = set_max_smem(dftk::k_yfft<Real, true, 0, 0>)) != cudaSuccess) e = r;
+        if ((r = ColFft<Real>::init()) != cudaSuccess) e = r;
     }
     return e;
 }
@@ -235,18 +223,12 @@ cudaError_t LaunchY<Real, N>::yfft(cudaStream_t st, bool inv, const GridDesc& g,
         else launch_k(dftk::k_yfft_tma<Real, false, N, TY>, grid, dftk::kThreads, sm, st, g.pdl, map, ntx, ntiles, status, tw, polls, 1);
         return cudaSuccess;
     } else {
-        dim3 grid((unsigned)ceil_div(g.nxh, T), (unsigned)g.nz, (unsigned)ncomp);
-        const size_t sm = smem_col_of<C>(g.ny, T, 2);
-        if (inv) launch_k(dftk::k_yfft<Real, true, 0, 0>, grid, dftk::kThreads, sm, st, g.pdl, g, py, T, data, tw);
-        else launch_k(dftk::k_yfft<Real, false, 0, 0>, grid, dftk::kThreads, sm, st, g.pdl, g, py, T, data, tw);
-        (void)status;
-        (void)polls;
-        return cudaSuccess;
+        return ColFft<Real>::run(st, inv, g, py, false, T, ncomp, data, status, tw, polls);
     }
 }
 
 // ---------------------------------------------------------------------------------- z
-// N > 0: grouped kernels (all components of a tile in one transform); N == 0: run-time path.
+// N > 0: a half in one pass; N == 0 (run-time lengths): z transform, k-space products, z transform.
 template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::init() {
     cudaError_t e = cudaSuccess, r;
@@ -268,11 +250,8 @@ cudaError_t LaunchZ<Real, N>::init() {
         constexpr int TY = dft_tile_y<Real>(N);
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY, true>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY, true>)) != cudaSuccess) e = r;
-    } else {
-        if ((r = set_max_smem(dftk::k_zconv_fwd<Real, 0, 0, false>)) != cudaSuccess) e = r;
-        if ((r = set_max_smem(dftk::k_zconv_fwd<Real, 0, 0, true>)) != cudaSuccess) e = r;
-        if ((r = set_max_smem(dftk::k_zconv_bwd<Real, 0, 0>)) != cudaSuccess) e = r;
     }
+    (void)r;
     return e;
 }
 
@@ -368,14 +347,13 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
             launch_k(dftk::k_zconv_fwd_g<Real, N, TZ, false>, grid, dftk::kThreads, sm, st, g.pdl,
                 g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, nullptr, tw);
     } else {
-        dim3 grid((unsigned)ceil_div(g.nxh, T), (unsigned)g.ny);
-        const size_t sm = smem_col_of<C>(g.nz, T, 7);
-        if (red_energy)
-            launch_k(dftk::k_zconv_fwd<Real, 0, 0, true>, grid, dftk::kThreads, sm, st, g.pdl,
-                g, pz, sp, T, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy, tw);
-        else
-            launch_k(dftk::k_zconv_fwd<Real, 0, 0, false>, grid, dftk::kThreads, sm, st, g.pdl,
-                g, pz, sp, T, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, nullptr, tw);
+        C* const w = const_cast<C*>(in);
+        cudaError_t e = ColFft<Real>::run(st, false, g, pz, true, T, sp.S, w, status, tw, DFT_WAIT_POLLS);
+        if (e == cudaSuccess)
+            e = Passes<Real>::zmul(st, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy);
+        if (e == cudaSuccess)
+            e = ColFft<Real>::run(st, true, g, pz, true, T, DFT_NSPEC, slot_n, status, tw, DFT_WAIT_POLLS);
+        return e;
     }
     return cudaSuccess;
 }
@@ -434,6 +412,24 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
         return true;
     }
 }
+
+// The second half of a run-time z length for one sample or the line search's two: the Phi' spectra
+// transformed (only where the hard-sphere part is wanted), the products, the correlations
+// transformed back.
+template <typename Real, typename C>
+cudaError_t zbwd_rt(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T, Real kfx,
+                    Real kfy, Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi, const C* esA,
+                    const C* esB, C* es_mat, const C* tw) {
+    int* status = const_cast<int*>(&ctl->status);
+    cudaError_t e = cudaSuccess;
+    if (flags & 1)
+        e = ColFft<Real>::run(st, false, g, pz, true, T, samples * DFT_NSPEC, phi, status, tw, DFT_WAIT_POLLS);
+    if (e == cudaSuccess)
+        e = Passes<Real>::zmul_bwd(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, samples, ctl, phi, esA, esB, es_mat);
+    if (e == cudaSuccess)
+        e = ColFft<Real>::run(st, true, g, pz, true, T, samples * ncomp_out, phi, status, tw, DFT_WAIT_POLLS);
+    return e;
+}
 }  // namespace
 
 template <typename Real, int N>
@@ -449,17 +445,19 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, cons
         launch_k(dftk::k_zconv_bwd_g<Real, N, TZ>, grid, dftk::kThreads, sm, st, g.pdl,
             g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
     } else {
-        dim3 grid((unsigned)ceil_div(g.nxh, T), (unsigned)g.ny);
-        launch_k(dftk::k_zconv_bwd<Real, 0, 0>, grid, dftk::kThreads, smem_col_of<C>(g.nz, T, 7), st, g.pdl,
-            g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
+        return zbwd_rt<Real>(st, g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, 1, ctl, phi, esA, esB, es_mat, tw);
     }
     return cudaSuccess;
 }
 
 template <typename Real, int N>
-cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
-                                             Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
-                                             const C* esB, const C* tw) {
+cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
+                                             const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz,
+                                             int ncomp_out, const Ctl* ctl, C* phi, const C* esA, const C* esB,
+                                             const C* tw) {
+    if constexpr (N == 0)
+        return zbwd_rt<Real>(st, g, pz, sp, T, kfx, kfy, kfz, 3, ncomp_out, 2, ctl, phi, esA, esB,
+                             static_cast<C*>(nullptr), tw);
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, 3, ncomp_out, 1, ctl, phi, esA, esB,
                                  static_cast<C*>(nullptr), tw))
         return cudaSuccess;
@@ -469,7 +467,9 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g,
 template <typename Real, int N>
 bool LaunchZ<Real, N>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
     constexpr int TB = N > 0 ? dft_tile_zb<Real>(N) : 1;
-    if constexpr (N > 0 && (TB * sizeof(C)) % 16 == 0) {
+    if constexpr (N == 0) {
+        return true;
+    } else if constexpr ((TB * sizeof(C)) % 16 == 0) {
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

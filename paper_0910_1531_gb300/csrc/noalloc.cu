@@ -112,7 +112,7 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     g.nc = (long long)g.nz * g.ny * g.pxh;
     g.hx = prm->hx; g.hy = prm->hy; g.hz = prm->hz;
     AxisPlan ax, ay, az;
-    if (!dft_radix_plan(g.nx, &ax) || !dft_radix_plan(g.ny, &ay) || !dft_radix_plan(g.nz, &az))
+    if (!dft_radix_plan(g.nx, &ax) || !dft_mixed_plan(g.ny, &ay) || !dft_mixed_plan(g.nz, &az))
         FAIL(DFT_EINVAL, "no radix plan for the grid sizes");
 
     // scratch layout (float2 elements): status word | twiddles x, y, z | S spectra | 10 weighted
@@ -147,7 +147,7 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     const double two_pi = 6.28318530717958647692;
     const float kfx = float(two_pi / (g.nx * g.hx)), kfy = float(two_pi / (g.ny * g.hy)),
                 kfz = float(two_pi / (g.nz * g.hz));
-    const int Ty = Passes<float>::tile_y(g.ny, 100 * 1024), Tz = Passes<float>::tile_z(g.nz, 112 * 1024);
+    const int Ty = Passes<float>::tile_y(g), Tz = Passes<float>::tile_z(g);
     const int LX = lines_for(g.nx, 1, 48 * 1024, 32);
     const int LR = lines_for(g.nx, DFT_NCOMP / 2, 48 * 1024, 16);
 

@@ -52,6 +52,35 @@ template <typename Real> __host__ __device__ constexpr int dft_tile_zf(int n) {
 #endif
 }
 
+// Tile buffer of the run-time column transform (k_colfft) in elements: the axis in boxes of at most
+// 256 rows (a second one starts at a multiple of four rows, so that every box lands on a 128-byte
+// boundary), rounded up to 128 bytes.
+inline int dft_col_box_rows(int n) { return n <= 256 ? n : ((n + 1) / 2 + 3) & ~3; }
+template <typename Real> inline int dft_col_elems(int n, int T) {
+    const int e = (n <= 256 ? 1 : 2) * dft_col_box_rows(n) * T, q = 128 / int(2 * sizeof(Real));
+    return (e + q - 1) / q * q;
+}
+// Shared memory of k_colfft: two TMA stages, X and (from two radix stages) Y, twiddles, mbarriers.
+template <typename Real> inline size_t dft_col_smem(int n, int T, int nstages) {
+    return (size_t(nstages > 1 ? 4 : 3) * dft_col_elems<Real>(n, T) + ((n + 1) & ~1)) * 2 * sizeof(Real) +
+           2 * sizeof(uint64_t) + 128;
+}
+// Tile width of a run-time column transform (128-, 64- or 32-byte rows in FP32, 128 or 64 in
+// FP64): of the widths that leave two blocks on an SM, the one with the least work per column in
+// use, where a narrower tile's shorter rows and fewer butterflies per block count as 2 / T columns
+// (FP64, bound by its arithmetic: 1 / T) and columns past nxh as work.
+template <typename Real> inline int dft_tile_rt(int n, int nxh) {
+    constexpr bool f32 = sizeof(Real) == 4;
+    int best = 4;
+    double best_cost = 1e30;
+    for (int T = f32 ? 16 : 8; T >= 4; T /= 2) {
+        if (T > 4 && dft_col_smem<Real>(n, T, 2) > 113 * 1024) continue;
+        const double cost = double((nxh + T - 1) / T * T) * (1.0 + (f32 ? 2.0 : 1.0) / T);
+        if (cost < best_cost) { best_cost = cost; best = T; }
+    }
+    return best;
+}
+
 // Threads of the persistent TMA z passes and the resident CTAs per SM their register budget
 // is sized for.  First half: 256 threads, two CTAs per SM, up to length 128; 512 threads, one
 // CTA, at 256.  Second half: 256 threads, three CTAs per SM (FP32; two in FP64, whose
@@ -148,24 +177,33 @@ struct LaunchZ {
     static cudaError_t zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
                           Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
                           const C* esA, const C* esB, C* es_mat, const C* tw);
-    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
-                                      Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
-                                      const C* esB, const C* tw);
+    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
+                                      const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz, int ncomp_out,
+                                      const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
     static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
                             const C* tw, long long polls);
+};
+
+// Column transform of a run-time length in place (k_colfft; colfft.cu): along z (zax) or y, tiles of
+// T columns (16, 8, 4; FP64 8, 4).
+template <typename Real>
+struct ColFft {
+    using C = typename Cplx<Real>::type;
+    static cudaError_t init();
+    static cudaError_t run(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int T, int ncomp,
+                           C* data, int* status, const C* tw, long long polls);
 };
 
 template <typename Real>
 struct Passes {
     using C = typename Cplx<Real>::type;
     static cudaError_t init_attributes();
-    // dynamic shared memory of an x pass with `lines` lines and of a column pass with nbuf tiles
+    // dynamic shared memory of an x pass with `lines` lines
     static size_t smem_x(int nx, int lines) { return (size_t(nx) + 2 * size_t(lines) * (nx + 1)) * sizeof(C) + 16; }
-    static size_t smem_col(int n, int T, int nbuf) { return (size_t(n) + size_t(nbuf) * T * n) * sizeof(C) + 16; }
-    // tile widths: the compile-time value for specialised lengths, else the largest that fits `budget`
-    static int tile_y(int n, size_t budget);
-    static int tile_z(int n, size_t budget);
+    // column tile widths of the y and z passes
+    static int tile_y(const GridDesc& g);
+    static int tile_z(const GridDesc& g);
 
     static cudaError_t xfwd(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int ncomp, int lx, const Real* in,
                      C* out, const C* tw);
@@ -184,10 +222,10 @@ struct Passes {
     // The two line-search samples' second-half z passes in one launch (both hard-sphere and ES
     // parts): phi holds sample 1's nine Phi' spectra then sample 2's, ctl[0] / ctl[1] their
     // weights; sample m's ncomp_out results go to phi components m ncomp_out ...  Only where
-    // has_zbwd_pair (the persistent TMA pass); cudaErrorNotSupported otherwise.
-    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
-                                      Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
-                                      const C* esB, const C* tw);
+    // has_zbwd_pair (the persistent TMA pass, run-time lengths); cudaErrorNotSupported otherwise.
+    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
+                                      const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz, int ncomp_out,
+                                      const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
     // The split first-half z stage (compile-time lengths): zfft = the persistent TMA z transform
     // of ncomp components in place (tiles of the y pass's width; cudaErrorNotSupported for other
@@ -196,7 +234,13 @@ struct Passes {
     static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
                             const C* tw, long long polls);
     static cudaError_t zmul(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
-                            Real kfz, const C* in, C* slot_n, C* slot_es);
+                            Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, double* red_energy);
+    // the second half's products between its z transforms (run-time lengths): one sample or two
+    static cudaError_t zmul_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi, const C* esA,
+                                const C* esB, C* es_mat);
+    // pairs of partial sums zconv_fwd writes to red_energy
+    static long long energy_blocks(const GridDesc& g);
     // rho_lo (or nullptr): low part of an extended iterate rho0 + rho_lo, read
     // with rho0 and, when rho_out is written, replaced by the low part of the new iterate;
     // gspec_out (or nullptr): also the x half spectra of G (S components, the layout of xfwd's
@@ -227,9 +271,10 @@ struct Passes {
                               int LR, const C* cspec, const Real* V, double* red, const C* tw);
     static cudaError_t canon_scale(cudaStream_t st, Ctl* ctl, const SpeciesDesc<Real>& sp, const double* red,
                                    int nblocks, int pdl);
-    // fill the |k| tables of sp (tab_w, tab_k, tab_dk, tab_m2max set by the caller) for wave
-    // number kf of a cubic box
-    static cudaError_t build_ktab(cudaStream_t st, const SpeciesDesc<Real>& sp, double kf);
+    // fill the `rows` rows of the |k| tables of sp (tab_w, tab_k, tab_dk, tab_oct set by the caller);
+    // kf: the wave number of a cubic box
+    static cudaError_t build_ktab(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, double kf, Real kfx,
+                                  Real kfy, Real kfz, long long rows);
     // fill out[nx + ny + nz] with the per-axis Laplacian terms of grid g (SpeciesDesc::lap1d)
     static cudaError_t build_laptab(cudaStream_t st, const GridDesc& g, Real kfx, Real kfy, Real kfz, Real* out);
 };

@@ -60,6 +60,14 @@ __device__ __forceinline__ void load_3d(void* dst, const CUtensorMap* map, int x
         : "memory");
 }
 
+// The same for a 4D tensor.
+__device__ __forceinline__ void load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int c, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(c), "r"(smem_u32(bar))
+        : "memory");
+}
+
 // 1D bulk copy global -> shared of `bytes` (a multiple of 16; both addresses 16-byte aligned);
 // completes `bar`'s transaction count.
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -84,6 +92,12 @@ __device__ __forceinline__ void store_3d(const CUtensorMap* map, int x, int y, i
                  : "memory");
 }
 
+__device__ __forceinline__ void store_4d(const CUtensorMap* map, int x, int y, int z, int c, const void* src) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
+                 ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(c), "r"(smem_u32(src))
+                 : "memory");
+}
+
 __device__ __forceinline__ void commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // the bulk stores committed so far have finished reading shared memory
 __device__ __forceinline__ void wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -97,3 +111,7 @@ __device__ __forceinline__ void wait_all() { asm volatile("cp.async.bulk.wait_gr
 cudaError_t tma_encode_3d(CUtensorMap* map, void* base, unsigned long long d0, unsigned long long d1,
                           unsigned long long d2, unsigned long long stride1_bytes, unsigned long long stride2_bytes,
                           unsigned b0, unsigned b1, unsigned b2);
+
+// The same for a 4D tensor (strides of the dimensions past the innermost).
+cudaError_t tma_encode_4d(CUtensorMap* map, void* base, const unsigned long long dims[4],
+                          const unsigned long long stride_bytes[3], const unsigned box[4]);

@@ -1,0 +1,53 @@
+"""Column transforms of run-time lengths (k_colfft and the z stage of three passes around it): G and
+the weighted densities against the oracle at the lengths where they can go wrong.
+
+Lengths: one radix stage (4, 14, 15), every composite radix and prime stage (11..31; two of them in
+one length, so that the second takes twiddles), three stages (343 = 7^3), 256 rows (one TMA box) and
+more (two boxes, of an odd length the second partly past the axis), column counts that leave a tile
+partly empty.  FP32 is held to 1e-5 and FP64 to 1e-10 per field, the library's stated bounds
+(about 30 transform passes of log2(N) roundings each are 4e-7 in FP32).
+"""
+import numpy as np
+import pytest
+
+from oracle import functional as F
+from paper_0910_1531_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TOL = {"fp32": 1e-5, "fp64": 1e-10}
+FIELDS = [[0], [1], [2], [3], [4, 5, 6], [7, 8, 9]]
+SPECIES = ([0.095, 0.099, 0.181], [1.0, 2.0, -1.0], [0.1, 0.01, 0.12])
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_0910_1531_gb300 import build
+    build.build()
+
+
+def relerr(a, b):
+    scale = np.max(np.abs(b))
+    return float(np.max(np.abs(np.asarray(a) - b)) / (scale if scale > 0 else 1.0))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("shape", [
+    (4, 5, 6), (14, 15, 16), (9, 10, 4), (7, 512, 6), (261, 6, 8), (323, 8, 4), (6, 343, 5), (289, 4, 34), (22, 26, 12),
+    (38, 46, 10), (58, 62, 36), (256, 20, 6), (12, 275, 8), (160, 9, 33), (100, 36, 70), (17, 23, 130)])
+def test_runtime_lengths_match_the_oracle(shape, precision):
+    from paper_0910_1531_gb300 import binding
+    prob = F.Problem(shape, (0.11, 0.1, 0.09), *SPECIES)
+    rho = workloads.random_density(shape, 3, prob.bath.rho, 0.3, seed=61)
+    V = np.zeros_like(rho)
+    V[1, : shape[0] // 3] = np.inf
+    rho[1, : shape[0] // 3] = 0.0
+    plan = binding.Plan(shape, prob.h, *SPECIES, precision=precision)
+    dev = lambda x: torch.tensor(np.ascontiguousarray(x), dtype=plan.dtype, device="cuda")
+    n, n_ref = plan.weighted_densities(dev(rho)).double().cpu().numpy(), F.weighted_densities(prob, rho)
+    for f in FIELDS:
+        assert relerr(n[f], n_ref[f]) < TOL[precision], (f, plan.tuning())
+    g, _ = plan.picard_map(dev(rho), dev(V))
+    assert relerr(g.double().cpu().numpy(), F.picard_map(prob, rho, V)) < TOL[precision], plan.tuning()
+    plan.close()
