@@ -228,8 +228,9 @@ dft_status dft_iter_run(dft_plan* plan, void* rho_inout, const void* V, int iter
  *    bulk copies two blocks ahead, or by per-thread cp.async copies one block ahead (each with
  *    its own rows per block);
  *  - the x transform: the compile-time kernels (where the length has them) against the
- *    run-time ones under each candidate radix order (the default plan -- 3s, other odd primes,
- *    16s, then 2/4/8 --, its reverse, and for powers of two a plan of 8s and one of 4s);
+ *    run-time ones under each candidate radix order (the default plan of mixed radices 2..16
+ *    and primes, the reverse of one of 3s, other odd primes, 16s, then 2/4/8, and for powers of two
+ *    a plan of 8s and one of 4s);
  *  - the y transform: the persistent TMA pass against the run-time column kernel;
  *  - the z passes: the persistent TMA passes against the grouped one-tile-per-CTA kernels;
  *    then the first half's z stage as one pass against three (z transform, products, z

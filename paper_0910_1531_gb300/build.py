@@ -17,7 +17,8 @@ BUILD = os.path.join(HERE, "_build")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_NAME = "libgb300dft.so"
 # (source, object name, extra defines); kinst.cu is compiled once per (precision, axis length)
-CT_SIZES = (0, 32, 48, 64, 96, 128, 256)
+# (0: run-time lengths; -1: the x passes of run-time lengths with a prime factor of 17..31)
+CT_SIZES = (-1, 0, 32, 48, 64, 96, 128, 256)
 SOURCES = ([("api.cu", "api", []), ("bulk.cpp", "bulk", []), ("noalloc.cu", "noalloc", []),
             ("dispatch.cu", "dispatch", []), ("newton.cu", "newton", [])]
            + [("colfft.cu", f"colfft_{r}", [f"-DDFT_INST_REAL={r}"]) for r in ("float", "double")]

@@ -865,9 +865,9 @@ struct TuneResult {
 };
 std::map<TuneKey, TuneResult> g_tune_cache;
 
-// Candidate radix orders of a run-time transform of length n: the default plan (3s, other odd
-// primes, 16s, then 2/4/8), its reverse, and for powers of two one of 8s (then 4 or 2) and one of
-// 4s (then 2).
+// Candidate radix orders of a run-time transform of length n: the default plan (dft_mixed_plan), and
+// beside it the reverse of the plan of 3s, other odd primes, 16s, then 2/4/8 (where that is another
+// order), and for powers of two one of 8s (then 4 or 2) and one of 4s (then 2).
 std::vector<AxisPlan> radix_orders(int n) {
     std::vector<AxisPlan> out;
     AxisPlan d;
@@ -898,6 +898,7 @@ std::vector<AxisPlan> radix_orders(int n) {
             if (m <= 16 && q.nstages <= DFT_MAXSTAGES) add(q);
         }
     }
+    dft_mixed_plan(n, &out[0]);
     return out;
 }
 
@@ -1290,7 +1291,7 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     p->kf[0] = two_pi / (g.nx * g.hx);
     p->kf[1] = two_pi / (g.ny * g.hy);
     p->kf[2] = two_pi / (g.nz * g.hz);
-    if (!dft_radix_plan(g.nx, &p->ax) || !dft_mixed_plan(g.ny, &p->ay) || !dft_mixed_plan(g.nz, &p->az)) {
+    if (!dft_mixed_plan(g.nx, &p->ax) || !dft_mixed_plan(g.ny, &p->ay) || !dft_mixed_plan(g.nz, &p->az)) {
         delete p;
         return fail(nullptr, DFT_EINVAL, "no radix plan for the grid sizes");
     }
@@ -2023,7 +2024,7 @@ dft_status dft_set_variants(dft_plan* p, int x_variant, int x_persistent, int y_
     p->g.xrt = x_variant > 0 ? 1 : 0;
     p->g.xpers = x_persistent;
     if (x_variant > 0) p->ax = orders[x_variant - 1];
-    else dft_radix_plan(p->g.nx, &p->ax);
+    else dft_mixed_plan(p->g.nx, &p->ax);
     p->g.yrt = y_variant;
     p->g.zgrp = z_variant & 1;
     p->g.zsplit = (z_variant >> 1) & 1;

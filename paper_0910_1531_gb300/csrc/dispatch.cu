@@ -13,9 +13,12 @@
     extern template struct LaunchZ<double, N>;
 DFT_CT_SIZES(DFT_DECLARE_EXTERN)
 DFT_DECLARE_EXTERN(0)
+extern template struct LaunchX<float, -1>;
+extern template struct LaunchX<double, -1>;
 
 #define DFT_CASE(N, L, call) case N: L<Real, N>::call; break;
-#define DFT_SWITCH_X(n, call) if (g.xrt) return LaunchX<Real, 0>::call; switch (n) { \
+#define DFT_SWITCH_X(n, call) if (dft_has_big_prime(n)) return LaunchX<Real, -1>::call; \
+    if (g.xrt) return LaunchX<Real, 0>::call; switch (n) { \
     case 32: return LaunchX<Real, 32>::call; case 48: return LaunchX<Real, 48>::call; \
     case 64: return LaunchX<Real, 64>::call; case 96: return LaunchX<Real, 96>::call; \
     case 128: return LaunchX<Real, 128>::call; case 256: return LaunchX<Real, 256>::call; \
@@ -40,6 +43,7 @@ cudaError_t Passes<Real>::init_attributes() {
     if ((r = LaunchZ<Real, N>::init()) != cudaSuccess) e = r;
     DFT_CT_SIZES(DFT_INIT)
     DFT_INIT(0)
+    if ((r = LaunchX<Real, -1>::init()) != cudaSuccess) e = r;
 #undef DFT_INIT
     return e;
 }

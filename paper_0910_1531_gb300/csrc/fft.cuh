@@ -3,8 +3,8 @@
 // A CTA holds `lines` transforms of length n in shared memory; element e of
 // line l sits at buf[e * es + l * ls].  Tiles of columns of the y / z axes use
 // es = T (tile width), ls = 1 so that consecutive threads touch consecutive
-// addresses; rows of the x axis use es = 1, ls = n + 1 (odd line pitch, free
-// of bank conflicts for 8-byte elements).
+// addresses; rows of the x axis use es = 1 and an odd line pitch (free of bank
+// conflicts for 8-byte elements).
 //
 // Stage with radix R and Ns = product of the earlier radices (self-sorting,
 // out of place):  for butterfly j of n/R,
@@ -357,87 +357,16 @@ __device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPla
 #undef DFT_RTP
 }
 
-template <int R, bool INV, typename C>
-__device__ __forceinline__ void stockham_stage(const C* __restrict__ src, C* __restrict__ dst, int n, int ns,
-                                               int lines, int es, int ls, const C* __restrict__ tw) {
-    const int m = n / R;
-    const int twstep = n / (ns * R);
-    const int total = m * lines;
-    for (int task = threadIdx.x; task < total; task += blockDim.x) {
-        const int line = task % lines;
-        const int j = task / lines;
-        const int k = j % ns;
-        C v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = src[(j + r * m) * es + line * ls];
-        if (ns > 1) {
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                C w = tw[k * r * twstep];
-                if (INV) w.y = -w.y;
-                v[r] = cmul(v[r], w);
-            }
-        }
-        dft_small<R, INV>(v);
-        const int base = (j / ns) * ns * R + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) dst[(base + r * ns) * es + line * ls] = v[r];
-    }
-}
-
-// Stage of an odd prime radix R without a dedicated butterfly (5 <= R <= DFT_MAX_PRIME): the
-// R-point DFT by its definition, out_q = sum_r v_r W_R^(r q), W_R = exp(-+2 pi i / R).  The stage
-// twiddle of v_r and W_R^(r q) are both powers of exp(-+2 pi i / n), so each term takes one
-// table entry, tw[(k r n/(Ns R) + (r q mod R) n/R) mod n].  R^2 terms per butterfly, one output
-// per thread.
-template <bool INV, typename C>
-__device__ __forceinline__ void stockham_stage_odd(const C* __restrict__ src, C* __restrict__ dst, int n, int ns,
-                                                   int R, int lines, int es, int ls, const C* __restrict__ tw) {
-    const int m = n / R;
-    const int twstep = n / (ns * R);
-    const int total = m * lines * R;
-    // one output q of one butterfly per task (R times the tasks of a butterfly per thread)
-    for (int task = threadIdx.x; task < total; task += blockDim.x) {
-        const int q = task % R;
-        const int bt = task / R;
-        const int line = bt % lines;
-        const int j = bt / lines;
-        const int k = j % ns;
-        const int base = (j / ns) * ns * R + k;
-        C acc = cmake<C>(0, 0);
-        int rq = 0;   // r q mod R
-        for (int r = 0; r < R; ++r) {
-            int e = k * r * twstep + rq * m;
-            if (e >= n) e -= n;
-            C w = tw[e];
-            if (INV) w.y = -w.y;
-            acc = cadd(acc, cmul(src[(j + r * m) * es + line * ls], w));
-            rq += q;
-            if (rq >= R) rq -= R;
-        }
-        dst[(base + q * ns) * es + line * ls] = acc;
-    }
-}
-
-// Transform all lines held in `a` (b is scratch of the same size).  The caller must
-// __syncthreads() before the call (data in a visible).  Returns the buffer holding
+// Transform the `lines` rows held in `a` (b is scratch of the same size) by the stages of a plan.
+// The caller must __syncthreads() before the call (data in a visible).  Returns the buffer holding
 // the result; all threads see it on return.
-template <bool INV, typename C>
-__device__ C* smem_fft(C* a, C* b, const AxisPlan& p, int lines, int es, int ls, const C* tw) {
-    int ns = 1;
+template <bool INV, bool BIG, int NT, typename C>
+__device__ C* rt_fft_rows(C* a, C* b, const AxisPlan& p, int lines, int ls, const C* tw) {
+    const FastDiv dl(lines);
     for (int s = 0; s < p.nstages; ++s) {
-        const int R = p.radix[s];
-        switch (R) {
-            case 2: stockham_stage<2, INV>(a, b, p.n, ns, lines, es, ls, tw); break;
-            case 3: stockham_stage<3, INV>(a, b, p.n, ns, lines, es, ls, tw); break;
-            case 4: stockham_stage<4, INV>(a, b, p.n, ns, lines, es, ls, tw); break;
-            case 8: stockham_stage<8, INV>(a, b, p.n, ns, lines, es, ls, tw); break;
-            case 16: stockham_stage<16, INV>(a, b, p.n, ns, lines, es, ls, tw); break;
-            default: stockham_stage_odd<INV>(a, b, p.n, ns, R, lines, es, ls, tw); break;
-        }
+        rt_stage_any<INV, 0, NT, BIG>(a, b, p, s, lines, dl, ls, tw);
         __syncthreads();
         C* t = a; a = b; b = t;
-        ns *= R;
     }
     return a;
 }
@@ -568,7 +497,7 @@ __device__ __forceinline__ void ct_stages(C*& a, C*& b, int lines, int ls, const
     }
 }
 
-// Compile-time counterpart of smem_fft (same contract).  COLS with tile width T, or rows
+// Compile-time counterpart of rt_fft_rows (same contract).  COLS with tile width T, or rows
 // with `lines` rows of pitch ls.
 template <int N, bool INV, bool COLS, int T, typename C>
 __device__ __forceinline__ C* ct_fft(C* a, C* b, int lines, int ls, const C* tw) {
@@ -576,11 +505,12 @@ __device__ __forceinline__ C* ct_fft(C* a, C* b, int lines, int ls, const C* tw)
     return a;
 }
 
-// Length-generic front end: N > 0 uses the compile-time stages, N == 0 the run-time plan.
-template <int N, bool INV, bool COLS, int T, typename C>
-__device__ __forceinline__ C* any_fft(C* a, C* b, const AxisPlan& p, int lines, int es, int ls, const C* tw) {
-    if constexpr (N > 0) return ct_fft<N, INV, COLS, T>(a, b, lines, ls, tw);
-    else return smem_fft<INV>(a, b, p, lines, es, ls, tw);
+// Rows of a length N > 0 by the compile-time stages, of any length (N = 0; N = -1 with a prime
+// factor of 17..31) by those of the plan.
+template <int N, bool INV, typename C>
+__device__ __forceinline__ C* any_fft(C* a, C* b, const AxisPlan& p, int lines, int ls, const C* tw) {
+    if constexpr (N > 0) return ct_fft<N, INV, false, 0>(a, b, lines, ls, tw);
+    else return rt_fft_rows<INV, (N < 0), kFftThreads>(a, b, p, lines, ls, tw);
 }
 
 // ------------------------------------------------------------------------------------

@@ -30,6 +30,8 @@
 
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "tma.cuh"
@@ -182,8 +184,23 @@ __device__ __forceinline__ float block_max(float v, float* scratch) {
     return r;
 }
 
-// Position of element e within an x-pass row: padded in the compile-time passes (see ct_xpad).
+// The x passes are compiled for a length NX > 0 or for any length: NX = 0, and NX = -1 for lengths
+// with a prime factor of 17..31.  Position of element e within a row (padded in the compile-time
+// passes, see ct_xpad) and row pitch (odd in the run-time ones, see rt_split).
 template <int NX> __device__ __forceinline__ int xo(int e) { return NX > 0 ? ct_xpad(e) : e; }
+template <int NX> __host__ __device__ __forceinline__ int x_pitch(int nx) { return NX > 0 ? ct_row_pitch(NX) : nx | 1; }
+
+// Division of a block's item index by a length that may be known at compile time (D > 0).
+template <int D> struct QDiv {
+    FastDiv f;
+    __device__ __forceinline__ explicit QDiv(int d) : f(D > 0 ? 1 : d) {}
+    __device__ __forceinline__ int operator()(int x) const {
+        if constexpr (D > 0) return x / D;
+        else return f.div(x);
+    }
+};
+template <int NX> using QRow = QDiv<NX>;                              // by nx
+template <int NX> using QHalf = QDiv<(NX > 0 ? NX / 2 + 1 : 0)>;      // by nx / 2 + 1
 
 template <typename C> __device__ __forceinline__ C* align_ptr(unsigned char* p) {
     uintptr_t u = reinterpret_cast<uintptr_t>(p);
@@ -205,7 +222,9 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(GridDesc g, AxisPlan px, int 
     dep_wait();
     using C = typename Cplx<Real>::type;
     extern __shared__ unsigned char smem_raw[];
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QRow<NX> qx(nx);
+    const QHalf<NX> qh(nxh);
     C* tw = align_ptr<C>(smem_raw);
     C* A = tw + nx;
     C* B = A + lx * pitch;
@@ -221,7 +240,7 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(GridDesc g, AxisPlan px, int 
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             const int idx = base + u * kThreads;
-            const int l = idx / nx, x = idx - (idx / nx) * nx;
+            const int l = qx(idx), x = idx - l * nx;
             const long long ra = 2 * (pair0 + l), rb = ra + 1;
             av[u] = (idx < total && ra < rows) ? in[ra * nx + x] : Real(0);
             bv[u] = (idx < total && rb < rows) ? in[rb * nx + x] : Real(0);
@@ -230,14 +249,14 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(GridDesc g, AxisPlan px, int 
         for (int u = 0; u < kU; ++u) {
             const int idx = base + u * kThreads;
             if (idx >= total) break;
-            const int l = idx / nx, x = idx - (idx / nx) * nx;
+            const int l = qx(idx), x = idx - l * nx;
             A[l * pitch + xo<NX>(x)] = cmake<C>(av[u], bv[u]);
         }
     }
     __syncthreads();
-    C* R = any_fft<NX, false, false, 0>(A, B, px, lx, 1, pitch, tw);
+    C* R = any_fft<NX, false>(A, B, px, lx, pitch, tw);
     for (int idx = threadIdx.x; idx < lx * nxh; idx += blockDim.x) {
-        const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
+        const int l = qh(idx), k = idx - l * nxh;
         const long long ra = 2 * (pair0 + l), rb = ra + 1;
         const C zk = R[l * pitch + xo<NX>(k)];
         const C znk = R[l * pitch + xo<NX>(k == 0 ? 0 : nx - k)];
@@ -1784,14 +1803,29 @@ __host__ __device__ constexpr int wd_slot(int c) { return (c == 1 || c == 5 || c
 #define DFT_XUPD_BATCH 1
 #endif
 
-// 16 bytes of consecutive real values (four floats or two doubles), for 16-byte loads and stores.
+// One real value, or 16 bytes of consecutive ones (four floats or two doubles), as a thread's unit
+// of global loads and stores.
+template <typename Real> struct Vec1 {
+    using type = Real;
+    static constexpr int n = 1;
+    static __device__ __forceinline__ type load(const Real* p) { return *p; }
+    static __device__ __forceinline__ void store(Real* p, type v) { *p = v; }
+};
 template <typename Real> struct Vec16;
-template <> struct Vec16<float> { using type = float4; static constexpr int n = 4; };
-template <> struct Vec16<double> { using type = double2; static constexpr int n = 2; };
-__device__ __forceinline__ float4 ld16(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ double2 ld16(const double* p) { return *reinterpret_cast<const double2*>(p); }
-__device__ __forceinline__ void st16(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ void st16(double* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }
+template <> struct Vec16<float> {
+    using type = float4;
+    static constexpr int n = 4;
+    static __device__ __forceinline__ type load(const float* p) { return *reinterpret_cast<const float4*>(p); }
+    static __device__ __forceinline__ void store(float* p, type v) { *reinterpret_cast<float4*>(p) = v; }
+};
+template <> struct Vec16<double> {
+    using type = double2;
+    static constexpr int n = 2;
+    static __device__ __forceinline__ type load(const double* p) { return *reinterpret_cast<const double2*>(p); }
+    static __device__ __forceinline__ void store(double* p, type v) { *reinterpret_cast<double2*>(p) = v; }
+};
+__device__ __forceinline__ float& vel(float& v, int) { return v; }
+__device__ __forceinline__ double& vel(double& v, int) { return v; }
 __device__ __forceinline__ float& vel(float4& v, int e) { return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)); }
 __device__ __forceinline__ double& vel(double2& v, int e) { return e == 0 ? v.x : v.y; }
 template <typename V> __device__ __forceinline__ V vzero() { V v; memset(&v, 0, sizeof(V)); return v; }
@@ -1807,7 +1841,9 @@ __device__ __forceinline__ void load_pair_rows(const GridDesc& g, int lines, int
                                                typename Cplx<Real>::type* dst) {
     using C = typename Cplx<Real>::type;
     constexpr int kBatch = 4;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
+    const FastDiv ql(lines_per_row);
     const bool even = (nx % 2) == 0;
     const int total = lines * nxh;
     for (int base = threadIdx.x; base < total; base += kBatch * kThreads) {
@@ -1817,9 +1853,10 @@ __device__ __forceinline__ void load_pair_rows(const GridDesc& g, int lines, int
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
-            const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
-            const long long row = row0 + l / lines_per_row;
-            const int ca = 2 * (l % lines_per_row), cb = ca + 1;
+            const int l = qh(idx), k = idx - l * nxh;
+            const int lr = ql.div(l);
+            const long long row = row0 + lr;
+            const int ca = 2 * (l - lr * lines_per_row), cb = ca + 1;
             live[j] = idx < total && row < nrows;
             hasb[j] = cb < ncomp;
             oa[j] = (long long)ca * g.nc + row * g.pxh + k;
@@ -1838,7 +1875,7 @@ __device__ __forceinline__ void load_pair_rows(const GridDesc& g, int lines, int
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
             if (idx >= total) continue;
-            const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
+            const int l = qh(idx), k = idx - l * nxh;
             C a = cadd(cscale(av[j], wA), cscale(aB[j], wB));
             C b = cadd(cscale(bv[j], wA), cscale(bB[j], wB));
             if (k == 0 || (even && 2 * k == nx)) { a.y = Real(0); b.y = Real(0); }
@@ -1863,9 +1900,11 @@ __device__ __forceinline__ void load_species_rows(const GridDesc& g, int rows, l
                                                   typename Cplx<Real>::type* dst) {
     using C = typename Cplx<Real>::type;
     constexpr int kBatch = 4;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
     const bool even = (nx % 2) == 0;
     const int lpr = (S + 1) / 2;
+    const FastDiv ql(lpr);
     const int lines = rows * lpr;                 // lines of one set
     const int total = NM * lines * nxh;
     for (int base = threadIdx.x; base < total; base += kBatch * kThreads) {
@@ -1873,10 +1912,11 @@ __device__ __forceinline__ void load_species_rows(const GridDesc& g, int rows, l
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
-            const int ml = idx / nxh, k = idx - (idx / nxh) * nxh;
-            const int m = NM == 1 ? 0 : ml / lines, l = ml - m * lines;
-            const long long row = row0 + l / lpr;
-            const int ca = 2 * (l % lpr), cb = ca + 1;
+            const int ml = qh(idx), k = idx - ml * nxh;
+            const int m = NM == 1 ? 0 : (ml >= lines ? 1 : 0), l = ml - m * lines;
+            const int lr = ql.div(l);
+            const long long row = row0 + lr;
+            const int ca = 2 * (l - lr * lpr), cb = ca + 1;
             const C* src = (NM == 2 && m == 1) ? spec2 : spec;
             const long long o = row * g.pxh + k;
             av[j] = bv[j] = cmake<C>(Real(0), Real(0));
@@ -1889,7 +1929,7 @@ __device__ __forceinline__ void load_species_rows(const GridDesc& g, int rows, l
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
             if (idx >= total) continue;
-            const int ml = idx / nxh, k = idx - (idx / nxh) * nxh;
+            const int ml = qh(idx), k = idx - ml * nxh;
             C a = av[j], b = bv[j];
             const bool edge = k == 0 || (even && 2 * k == nx);
             if (edge) { a.y = Real(0); b.y = Real(0); }
@@ -1906,7 +1946,8 @@ __device__ __forceinline__ void load_row_pairs(const GridDesc& g, int rows, long
                                                const typename Cplx<Real>::type* __restrict__ spec,
                                                typename Cplx<Real>::type* dst) {
     using C = typename Cplx<Real>::type;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
     const bool even = (nx % 2) == 0;
     const int lines = (rows + 1) / 2;
     const int total = lines * nxh;
@@ -1917,7 +1958,7 @@ __device__ __forceinline__ void load_row_pairs(const GridDesc& g, int rows, long
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
-            const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
+            const int l = qh(idx), k = idx - l * nxh;
             const int ra = 2 * l, rb = 2 * l + 1;
             av[j] = bv[j] = cmake<C>(Real(0), Real(0));
             if (idx < total) {
@@ -1929,7 +1970,7 @@ __device__ __forceinline__ void load_row_pairs(const GridDesc& g, int rows, long
         for (int j = 0; j < kBatch; ++j) {
             const int idx = base + j * kThreads;
             if (idx >= total) continue;
-            const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
+            const int l = qh(idx), k = idx - l * nxh;
             C a = av[j], b = bv[j];
             const bool edge = k == 0 || (even && 2 * k == nx);
             if (edge) { a.y = Real(0); b.y = Real(0); }
@@ -1955,10 +1996,11 @@ __device__ __forceinline__ void load_wd_rows(const GridDesc& g, int rows, long l
                                              typename Cplx<Real>::type* dst,
                                              const typename Cplx<Real>::type* stage = nullptr, int cstride = 0) {
     using C = typename Cplx<Real>::type;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
     const bool even = (nx % 2) == 0;
     for (int idx = threadIdx.x; idx < rows * nxh; idx += blockDim.x) {
-        const int r = idx / nxh, k = idx - (idx / nxh) * nxh;
+        const int r = qh(idx), k = idx - r * nxh;
         const long long row = row0 + r;
         const bool live = row < nrows;
         const long long o = row * g.pxh + k;
@@ -2011,12 +2053,15 @@ __device__ __forceinline__ void store_pair_rows(const GridDesc& g, int lines, in
                                                 long long nrows, int ncomp, const typename Cplx<Real>::type* R,
                                                 typename Cplx<Real>::type* out) {
     using C = typename Cplx<Real>::type;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
+    const FastDiv ql(lines_per_row);
     for (int idx = threadIdx.x; idx < lines * nxh; idx += blockDim.x) {
-        const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
-        const long long row = row0 + l / lines_per_row;
+        const int l = qh(idx), k = idx - l * nxh;
+        const int lr = ql.div(l);
+        const long long row = row0 + lr;
         if (row >= nrows) continue;
-        const int ca = 2 * (l % lines_per_row), cb = ca + 1;
+        const int ca = 2 * (l - lr * lines_per_row), cb = ca + 1;
         const C zk = R[l * pitch + xo<NX>(k)];
         const C znk = R[l * pitch + xo<NX>(k == 0 ? 0 : nx - k)];
         const C s = cadd(zk, cconj(znk));
@@ -2037,10 +2082,11 @@ __device__ __forceinline__ void store_phi_spectra(const GridDesc& g, int rows, l
                                                   Real kfx, const typename Cplx<Real>::type* R,
                                                   typename Cplx<Real>::type* out0) {
     using C = typename Cplx<Real>::type;
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx);
+    const QHalf<NX> qh(nxh);
     const bool even = (nx % 2) == 0;
     for (int idx = threadIdx.x; idx < rows * NM * nxh; idx += blockDim.x) {
-        const int rr = idx / nxh, k = idx - (idx / nxh) * nxh;
+        const int rr = qh(idx), k = idx - rr * nxh;
         const int r = rr / NM;
         const long long row = row0 + r;
         if (row >= nrows) continue;
@@ -2091,7 +2137,8 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
     __shared__ float scratch_f[32];
     __shared__ double scratch_d[32];
     double phi_acc = 0.0;   // sum of Phi(n) over the block's points (grand potential only)
-    const int nx = NX > 0 ? NX : g.nx, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, pitch = x_pitch<NX>(nx);
+    const QRow<NX> qx(nx);
     const int lines = 5 * NM * LR;
     C* tw = align_ptr<C>(smem_raw);
     C* A = tw + nx;
@@ -2108,11 +2155,11 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
     }
     load_wd_rows<Real, NX, NM>(g, LR, row0, nrows, slotA, slotB, wA, wB, mat_out, kfx, A);
     __syncthreads();
-    C* R = any_fft<NX, true, false, 0>(A, B, px, lines, 1, pitch, tw);
+    C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
     float mx = -CUDART_INF_F;
     bool bad = false;
     for (int idx = threadIdx.x; idx < LR * NM * nx; idx += blockDim.x) {
-        const int rr = idx / nx, x = idx - (idx / nx) * nx;
+        const int rr = qx(idx), x = idx - rr * nx;
         const int r = rr / NM;
         C* base = R + (rr * 5) * pitch + xo<NX>(x);
         Real n[DFT_NCOMP];
@@ -2134,7 +2181,7 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
     if (bad) atomicOr(status, DEV_N3BOUND);
     __syncthreads();
     C* other = (R == A) ? B : A;
-    C* F = any_fft<NX, false, false, 0>(R, other, px, lines, 1, pitch, tw);
+    C* F = any_fft<NX, false>(R, other, px, lines, pitch, tw);
     store_phi_spectra<Real, NX, NM>(g, LR, row0, nrows, kfx, F, phi_out);
     const float bm = block_max(mx, scratch_f);
     if (threadIdx.x == 0 && red_max) red_max[blockIdx.x] = bm;
@@ -2391,7 +2438,9 @@ __global__ void __launch_bounds__(kThreads) k_xcanon(GridDesc g, AxisPlan px, Sp
     using C = typename Cplx<Real>::type;
     extern __shared__ unsigned char smem_raw[];
     __shared__ double scratch_d[32];
-    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1, S = sp.S;
+    const int nx = NX > 0 ? NX : g.nx, nxh = nx / 2 + 1, pitch = x_pitch<NX>(nx), S = sp.S;
+    const QRow<NX> qx(nx);
+    const QHalf<NX> qh(nxh);
     const bool even = (nx % 2) == 0;
     const int lines = nl * LR;
     C* tw = align_ptr<C>(smem_raw);
@@ -2401,9 +2450,10 @@ __global__ void __launch_bounds__(kThreads) k_xcanon(GridDesc g, AxisPlan px, Sp
     const long long nrows = (long long)g.ny * g.nz;
     const long long row0 = (long long)blockIdx.x * LR;
     const int line_of[3] = {line0, line1, line2};
+    const FastDiv ql(nl);
     for (int idx = threadIdx.x; idx < lines * nxh; idx += blockDim.x) {
-        const int l = idx / nxh, k = idx - (idx / nxh) * nxh;
-        const int r = l / nl, j = l - (l / nl) * nl;
+        const int l = qh(idx), k = idx - l * nxh;
+        const int r = ql.div(l), j = l - r * nl;
         const long long row = row0 + r;
         const int ca = 2 * line_of[j], cb = ca + 1;
         C a = cmake<C>(Real(0), Real(0)), b = a;
@@ -2417,12 +2467,12 @@ __global__ void __launch_bounds__(kThreads) k_xcanon(GridDesc g, AxisPlan px, Sp
         if (!edge) A[l * pitch + xo<NX>(nx - k)] = cmake<C>(a.x + b.y, b.x - a.y);
     }
     __syncthreads();
-    C* R = any_fft<NX, true, false, 0>(A, B, px, lines, 1, pitch, tw);
+    C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
     Real acc[DFT_MAXS], comp[DFT_MAXS];
 #pragma unroll
     for (int s = 0; s < DFT_MAXS; ++s) acc[s] = comp[s] = Real(0);
     for (int idx = threadIdx.x; idx < LR * nx; idx += blockDim.x) {
-        const int r = idx / nx, x = idx - (idx / nx) * nx;
+        const int r = qx(idx), x = idx - r * nx;
         const long long row = row0 + r;
         if (row >= nrows) continue;
 #pragma unroll
@@ -2488,7 +2538,7 @@ __global__ void __launch_bounds__(kThreads) k_canon_scale(Ctl* ctl, SpeciesDesc<
 // cspec2 (m = 1), weights from ctl[1 + m], rho0, rho1, V (and the low part) read once for both;
 // the residual sums of sample m go to red_sum / red_sum2; nothing is written to rho or G.
 template <typename Real, int NX, int NM = 1>
-__global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate(GridDesc g, AxisPlan px, SpeciesDesc<Real> sp, int LR,
+__global__ void __launch_bounds__(kThreads, NX < 0 ? 1 : (sizeof(Real) == 4 ? 3 : 2)) k_xupdate(GridDesc g, AxisPlan px, SpeciesDesc<Real> sp, int LR,
                                                       const Ctl* __restrict__ ctl,
                                                       const typename Cplx<Real>::type* __restrict__ cspec,
                                                       const typename Cplx<Real>::type* __restrict__ cspec2,
@@ -2503,7 +2553,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
     using C = typename Cplx<Real>::type;
     extern __shared__ unsigned char smem_raw[];
     __shared__ double scratch_d[32];
-    const int nx = NX > 0 ? NX : g.nx, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1, S = sp.S;
+    const int nx = NX > 0 ? NX : g.nx, pitch = x_pitch<NX>(nx), S = sp.S;
+    const QRow<NX> qx(nx);
     const int lpr = (S + 1) / 2;
     const int lines = NM * lpr * LR;
     C* tw = align_ptr<C>(smem_raw);
@@ -2525,7 +2576,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
         s_irb[s] = sp.inv_rho_b[s];
     }
     __syncthreads();
-    C* R = any_fft<NX, true, false, 0>(A, B, px, lines, 1, pitch, tw);
+    C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
     Real w0[NM], w1[NM];
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
@@ -2566,14 +2617,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
     };
     // rho_out / g_out / rho_lo may alias rho0 / rho1 / the low part read: every value is read
     // before the same thread writes that element, and the threads' elements are distinct
-    if constexpr (NX > 0) {
-        // compile-time lengths: items (species, group of VW consecutive points of a row),
-        // KB items per thread with their 16-byte loads of rho0, rho1, V (and the low part)
-        // issued before any is used, results stored 16 bytes at a time
-        using V16 = typename Vec16<Real>::type;
-        constexpr int VW = Vec16<Real>::n;
-        constexpr int KB = DFT_XUPD_BATCH;
-        static_assert(NX % VW == 0, "row length a multiple of the vector width");
+    // items (species, group of VW consecutive points of the block's rows), KB items per thread with
+    // their loads of rho0, rho1, V (and the low part) issued before any is used: 16-byte accesses
+    // for compile-time lengths (KB 2 measured 144 us per 128^3 iteration against 133), single values
+    // for run-time ones, whose rows need not start on a 16-byte boundary
+    {
+        using VT = typename std::conditional<(NX > 0), Vec16<Real>, Vec1<Real>>::type;
+        using V16 = typename VT::type;
+        constexpr int VW = VT::n;
+        constexpr int KB = NX > 0 ? DFT_XUPD_BATCH : 4;
+        static_assert(NX <= 0 || NX % VW == 0, "row length a multiple of the vector width");
         const int groups = total / VW;
         const int items = S * groups;
         // item it = s groups + gi, kept as (s, gi) and advanced without dividing
@@ -2591,14 +2644,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
                 }
                 const int it = base + j * kThreads;
                 const int s = sj[j], gi = gj[j];
-                const bool live = it < items && row0 + (gi * VW) / NX < nrows;
-                const long long o = (long long)s * g.n + row0 * NX + (long long)gi * VW;
+                const bool live = it < items && row0 + qx(gi * VW) < nrows;
+                const long long o = (long long)s * g.n + row0 * nx + (long long)gi * VW;
                 a0[j] = a1[j] = av[j] = al[j] = vzero<V16>();
                 if (live) {
-                    a0[j] = ld16(rho0 + o);
-                    if (rho1) a1[j] = ld16(rho1 + o);
-                    av[j] = ld16(V + o);
-                    if (rho_lo) al[j] = ld16(rho_lo + o);
+                    a0[j] = VT::load(rho0 + o);
+                    if (rho1) a1[j] = VT::load(rho1 + o);
+                    av[j] = VT::load(V + o);
+                    if (rho_lo) al[j] = VT::load(rho_lo + o);
                 }
             }
             gi_b += KB * kThreads;
@@ -2607,9 +2660,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
             for (int j = 0; j < KB; ++j) {
                 const int it = base + j * kThreads;
                 const int s = sj[j], gi = gj[j];
-                const int idx = gi * VW, r = idx / NX, x = idx - (idx / NX) * NX;
+                const int idx = gi * VW, r = qx(idx), x = idx - r * nx;
                 if (!(it < items && row0 + r < nrows)) continue;
-                const long long o = (long long)s * g.n + row0 * NX + idx;
+                const long long o = (long long)s * g.n + row0 * nx + idx;
 #pragma unroll
                 for (int m = 0; m < NM; ++m) {
                     C* Rl = R + (m * lpr * LR + r * lpr + s / 2) * pitch;
@@ -2624,65 +2677,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
                         if (NM == 1 && gspec_out) *hp = vel(og, e);
                     }
                     if (NM == 1 && rho_out) {
-                        st16(rho_out + o, orho);
-                        if (rho_lo) st16(rho_lo + o, olo);
+                        VT::store(rho_out + o, orho);
+                        if (rho_lo) VT::store(rho_lo + o, olo);
                     }
-                    if (NM == 1 && g_out) st16(g_out + o, og);
+                    if (NM == 1 && g_out) VT::store(g_out + o, og);
                 }
-            }
-        }
-    } else {
-        // run-time lengths: one point per thread at a time, its rho0, rho1, V (and low part)
-        // loaded one point ahead of their use
-        Real r0[DFT_MAXS], r1[DFT_MAXS], vv[DFT_MAXS], rl[DFT_MAXS];
-        auto load_point = [&](int idx, Real* a0, Real* a1, Real* av, Real* al) {
-            const long long row = row0 + idx / nx;
-            const bool live = idx < total && row < nrows;
-            const long long pt = row0 * nx + idx;
-#pragma unroll
-            for (int s = 0; s < DFT_MAXS; ++s) {
-                a0[s] = a1[s] = av[s] = al[s] = Real(0);
-                if (s < S && live) {
-                    const long long o = (long long)s * g.n + pt;
-                    a0[s] = rho0[o];
-                    a1[s] = rho1 ? rho1[o] : Real(0);
-                    av[s] = V[o];
-                    if (rho_lo) al[s] = rho_lo[o];
-                }
-            }
-        };
-        load_point(threadIdx.x, r0, r1, vv, rl);
-        for (int idx = threadIdx.x; idx < total; idx += kThreads) {
-            Real n0[DFT_MAXS], n1[DFT_MAXS], nv[DFT_MAXS], nl[DFT_MAXS];
-            load_point(idx + kThreads, n0, n1, nv, nl);
-            const int r = idx / nx, x = idx - (idx / nx) * nx;
-            if (row0 + r < nrows) {
-                const long long pt = row0 * nx + idx;
-#pragma unroll
-                for (int s = 0; s < DFT_MAXS; ++s) {
-                    if (s >= S) continue;
-                    const long long o = (long long)s * g.n + pt;
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) {
-                        Real* hp = reinterpret_cast<Real*>(R + (m * lpr * LR + r * lpr + s / 2) * pitch + xo<NX>(x)) +
-                                   (s & 1);
-                        Real rho, lo, gval;
-                        point(m, s, *hp, r0[s], r1[s], vv[s], rl[s], rho, lo, gval);
-                        if (NM == 1 && gspec_out) *hp = gval;
-                        if (NM == 1 && rho_out) {
-                            rho_out[o] = rho;
-                            if (rho_lo) rho_lo[o] = lo;
-                        }
-                        if (NM == 1 && g_out) g_out[o] = gval;
-                    }
-                }
-            }
-#pragma unroll
-            for (int s = 0; s < DFT_MAXS; ++s) {
-                r0[s] = n0[s];
-                r1[s] = n1[s];
-                vv[s] = nv[s];
-                rl[s] = nl[s];
             }
         }
     }
@@ -2692,7 +2691,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_xupdate
         // now hold G in place of c1, two species per complex line
         __syncthreads();
         C* other = (R == A) ? B : A;
-        C* F = any_fft<NX, false, false, 0>(R, other, px, lines, 1, pitch, tw);
+        C* F = any_fft<NX, false>(R, other, px, lines, pitch, tw);
         store_pair_rows<Real, NX>(g, lines, lpr, row0, nrows, S, F, gspec_out);
     }
 #pragma unroll
@@ -2723,7 +2722,8 @@ __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, Spe
     using C = typename Cplx<Real>::type;
     extern __shared__ unsigned char smem_raw[];
     __shared__ double scratch_d[32];
-    const int nx = NX > 0 ? NX : g.nx, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1, S = sp.S;
+    const int nx = NX > 0 ? NX : g.nx, pitch = x_pitch<NX>(nx), S = sp.S;
+    const QRow<NX> qx(nx);
     const int lpr = (S + 1) / 2;
     const int lines = lpr * LR;
     C* tw = align_ptr<C>(smem_raw);
@@ -2734,11 +2734,11 @@ __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, Spe
     const long long row0 = (long long)blockIdx.x * LR;
     load_pair_rows<Real, NX>(g, lines, lpr, row0, nrows, S, cspec, nullptr, Real(1), Real(0), nullptr, A);
     __syncthreads();
-    C* R = any_fft<NX, true, false, 0>(A, B, px, lines, 1, pitch, tw);
+    C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
     double acc[DFT_MAXS + 1];
     for (int s = 0; s <= DFT_MAXS; ++s) acc[s] = 0.0;
     for (int idx = threadIdx.x; idx < LR * nx; idx += blockDim.x) {
-        const int r = idx / nx, x = idx - (idx / nx) * nx;
+        const int r = qx(idx), x = idx - r * nx;
         const long long row = row0 + r;
         if (row >= nrows) continue;
         for (int s = 0; s < S; ++s) {
@@ -2781,7 +2781,8 @@ __global__ void __launch_bounds__(kThreads) k_xinv(GridDesc g, AxisPlan px, int 
     using C = typename Cplx<Real>::type;
     extern __shared__ unsigned char smem_raw[];
     __shared__ float scratch_f[32];
-    const int nx = NX > 0 ? NX : g.nx, pitch = NX > 0 ? ct_row_pitch(NX) : nx + 1;
+    const int nx = NX > 0 ? NX : g.nx, pitch = x_pitch<NX>(nx);
+    const QRow<NX> qx(nx);
     // one component without outputs (the maximum only): two grid rows per complex line
     const bool rows2 = ncomp == 1 && !wd && !out && !out_last;
     const int lpr = (ncomp + 1) / 2;
@@ -2797,10 +2798,10 @@ __global__ void __launch_bounds__(kThreads) k_xinv(GridDesc g, AxisPlan px, int 
     else if (rows2) load_row_pairs<Real, NX>(g, LR, row0, nrows, spec, A);
     else load_pair_rows<Real, NX>(g, lines, lpr, row0, nrows, ncomp, spec, nullptr, Real(1), Real(0), nullptr, A);
     __syncthreads();
-    C* R = any_fft<NX, true, false, 0>(A, B, px, lines, 1, pitch, tw);
+    C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
     float mx = -CUDART_INF_F;
     for (int idx = threadIdx.x; idx < LR * nx; idx += blockDim.x) {
-        const int r = idx / nx, x = idx - (idx / nx) * nx;
+        const int r = qx(idx), x = idx - r * nx;
         const long long row = row0 + r;
         if (row >= nrows) continue;
         if (rows2) {

@@ -8,7 +8,7 @@
 namespace {
 // x pass: twiddles (nx) + two buffers of `lines` rows at the kernel's row pitch
 template <typename C, int N> size_t smem_x_of(int nx, int lines) {
-    const int pitch = N > 0 ? ct_row_pitch(N) : nx + 1;
+    const int pitch = dftk::x_pitch<N>(nx);
     return (size_t(nx) + 2 * size_t(lines) * pitch) * sizeof(C) + 16;
 }
 }  // namespace
@@ -50,7 +50,7 @@ namespace {
 template <typename Real, int N, int NM, typename C>
 bool launch_xphi_tma(cudaStream_t st, const GridDesc& g, int LR, const Ctl* ctl, const C* A, const C* B, C* mat,
                      C* phi, float* red_max, int* status, Real kfx, const C* tw) {
-    if constexpr (N == 0) {
+    if constexpr (N <= 0) {
         return false;
     } else {
         if (!g.xpers || !status) return false;

@@ -112,7 +112,7 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     g.nc = (long long)g.nz * g.ny * g.pxh;
     g.hx = prm->hx; g.hy = prm->hy; g.hz = prm->hz;
     AxisPlan ax, ay, az;
-    if (!dft_radix_plan(g.nx, &ax) || !dft_mixed_plan(g.ny, &ay) || !dft_mixed_plan(g.nz, &az))
+    if (!dft_mixed_plan(g.nx, &ax) || !dft_mixed_plan(g.ny, &ay) || !dft_mixed_plan(g.nz, &az))
         FAIL(DFT_EINVAL, "no radix plan for the grid sizes");
 
     // scratch layout (float2 elements): status word | twiddles x, y, z | S spectra | 10 weighted
