@@ -374,15 +374,16 @@ __device__ C* rt_fft_rows(C* a, C* b, const AxisPlan& p, int lines, int ls, cons
 // ------------------------------------------------------------------------------------
 // Compile-time transforms.  The same Stockham stages with the length, the radix plan and
 // (for column tiles) the tile width known at compile time, so that index arithmetic is by
-// constants and every loop unrolls.  Radix plan of n: the factors 3 first, then 16s, then
-// one of 2/4/8 -- the same order as the run-time AxisPlan.
+// constants and every loop unrolls.  Radix plans: two stages of near-equal radices, the larger
+// first, so that both stages have butterflies for a block's threads (64 as 8 x 8 has eight per
+// line in both, as 16 x 4 four, which leaves most lanes of a small block's warps idle; FP64, bound
+// by whole warps on its pipe, most of all).  Line-search iteration, two species, against 16 first:
+// 96^3 FP32 492 -> 369 us (there were three stages), 64^3 145 -> 139, 48^3 113 -> 99, 32^3 81 -> 75;
+// FP64 32^3 408 -> 307, 48^3 1026 -> 714, 64^3 1856 -> 1566, 96^3 6254 -> 4952.
 // ------------------------------------------------------------------------------------
 __host__ __device__ constexpr int ct_radix_at(int n, int s) {
-    int m = n, k = 0;
-    while (m % 3 == 0) { if (k == s) return 3; m /= 3; ++k; }
-    while (m >= 16 && m % 16 == 0) { if (k == s) return 16; m /= 16; ++k; }
-    if (m > 1) { if (k == s) return m; ++k; }
-    return 0;
+    const int r0 = n == 32 ? 8 : n == 48 ? 8 : n == 64 ? 8 : n == 96 ? 12 : 16;
+    return s == 0 ? r0 : (s == 1 ? n / r0 : 0);
 }
 __host__ __device__ constexpr int ct_nstages(int n) { int s = 0; while (ct_radix_at(n, s) != 0) ++s; return s; }
 __host__ __device__ constexpr int ct_ns_at(int n, int s) { int p = 1; for (int i = 0; i < s; ++i) p *= ct_radix_at(n, i); return p; }
@@ -401,7 +402,7 @@ __host__ __device__ constexpr int ct_row_pitch(int n) {
     int msmall = 0;
     for (int s = 0; s < ct_nstages(n); ++s) {
         const int m = n / ct_radix_at(n, s);
-        if (m < 16) msmall = m;
+        if (m < 16 && (msmall == 0 || m < msmall)) msmall = m;
     }
     const int len = ct_xpad(n - 1) + 1;
     if (msmall == 0) return len | 1;
@@ -413,10 +414,10 @@ __host__ __device__ constexpr int ct_row_pitch(int n) {
 // Rows: the padded position ct_xpad(a + r s) of the r-th element a butterfly touches splits
 // into a per-thread part and a compile-time part when s is a multiple of 16 (then (a + r s) >> 4
 // = (a >> 4) + r s / 16), or when every a + r s stays inside one block of 16 positions past a
-// multiple of 16 (loads: a < M, 16 % M == 0; stores: NS R == 16).  The butterfly then addresses
-// its elements at one base pointer plus constants.
+// multiple of 16 (loads: a < M, 16 % M == 0; stores: 16 % (NS R) == 0).  The butterfly then
+// addresses its elements at one base pointer plus constants.
 template <int M, int R> __host__ __device__ constexpr bool ct_split_loads() { return M % 16 == 0 || 16 % M == 0; }
-template <int NS, int R> __host__ __device__ constexpr bool ct_split_stores() { return NS % 16 == 0 || NS * R == 16; }
+template <int NS, int R> __host__ __device__ constexpr bool ct_split_stores() { return NS % 16 == 0 || 16 % (NS * R) == 0; }
 
 template <int N, int R, int NS, bool INV, bool COLS, int T, typename C>
 __device__ __forceinline__ void ct_stage(const C* __restrict__ src, C* __restrict__ dst, int lines, int ls,
@@ -445,7 +446,7 @@ __device__ __forceinline__ void ct_stage(const C* __restrict__ src, C* __restric
             }
             dft_small<R, INV>(v);
             // stores: element b + r NS, b = (j / NS) NS R + k, at pad(b) + r (NS + NS / 16) (NS a
-            // multiple of 16), or at b + b / 16 + r NS (NS R = 16: b a multiple of 16 plus k < NS)
+            // multiple of 16), or at b + b / 16 + r NS (b a multiple of NS R, a divisor of 16, plus k < NS)
             const int b = (j / NS) * (NS * R) + k;
             C* d0 = dst + line * ls + ct_xpad(b);
 #pragma unroll
