@@ -72,7 +72,7 @@ struct dft_plan {
     Ctl* ctl_host = nullptr;
     int Ty = 1, Tz = 1, LX = 1, LRphi = 1, LRupd = 1;
     int LRphi2 = 1, LRupd2 = 1;     // rows per block of the paired-sample x passes
-    int LRn3 = 0;                   // rows per block of the n3-maximum x pass (0: from the budget)
+    int LRn3 = 2;                   // rows per block of the n3-maximum x pass
     SpeciesDesc<float> spf{};
     SpeciesDesc<double> spd{};
     bool prof = false;
@@ -129,6 +129,33 @@ int pick_lines(int nx, size_t csize, int lines_per_unit, size_t budget, int cap)
     if (L < 1) L = 1;
     if (L > cap) L = cap;
     return (int)L;
+}
+
+// Rows (or row pairs) per block of an x pass over `rows` of them, `lines` complex lines each: of the
+// counts up to 16 whose line buffers fit `budget`, the one with the least time for the SM that gets
+// the most blocks, each block costing its rows and (two rows' worth in FP32, half a one in FP64) its
+// start.  FP64, bound by its pipe, counts rows as the whole warps their butterflies take.  45^3
+// takes seven rows, 290 blocks on 152 SMs, in FP64 733 us an iteration; six, 338 blocks, 871.
+int spread_rows(const dft_plan* p, long long rows, int lines, size_t budget) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess || sms < 1) sms = 1;
+    const bool f64 = p->precision == DFT_FP64;
+    const int most = pick_lines(p->g.nx, p->csize, lines, budget, 16);
+    int best = 1;
+    double best_cost = 1e300;
+    for (int L = 1; L <= most; ++L) {
+        double fill = 1.0;
+        if (f64) {
+            fill = 0.0;
+            for (int s = 0; s < p->ax.nstages; ++s) {
+                const double tasks = double(L) * lines * p->ax.m[s];
+                fill += std::ceil(tasks / 32.0) * 32.0 / tasks / p->ax.nstages;
+            }
+        }
+        const double cost = double(ceil_div(ceil_div(rows, L), sms)) * (L * fill + (f64 ? 0.5 : 2.0));
+        if (cost < best_cost * 0.999) { best_cost = cost; best = L; }
+    }
+    return best;
 }
 
 template <typename Real> SpeciesDesc<Real>& species(dft_plan* p);
@@ -394,7 +421,8 @@ template <typename Real> struct Ops {
     static dft_status xinv(dft_plan* p, int ncomp, const C* spec, Real* out, Real* out_last, const double* offs,
                            int cmax, float* red_max, int* blocks_out) {
         const int lpr = (ncomp + 1) / 2;
-        const int LR = (ncomp == 1 && p->LRn3 > 0) ? p->LRn3 : pick_lines(p->g.nx, sizeof(C), lpr, 48 * 1024, 16);
+        // the maximum alone takes two grid rows per line
+        const int LR = (ncomp == 1 && !out && !out_last) ? p->LRn3 : pick_lines(p->g.nx, sizeof(C), lpr, 48 * 1024, 16);
         Offsets<Real> off;
         for (int c = 0; c < DFT_NCOMP + 2; ++c) off.v[c] = Real(0);
         if (offs)
@@ -1302,11 +1330,24 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     p->rsize = f64 ? sizeof(double) : sizeof(float);
     p->Ty = f64 ? Passes<double>::tile_y(g) : Passes<float>::tile_y(g);
     p->Tz = f64 ? Passes<double>::tile_z(g) : Passes<float>::tile_z(g);
-    p->LX = pick_lines(g.nx, p->csize, 1, env_budget("DFT_XFWD_SMEM", 48 * 1024), 32);
-    p->LRphi = pick_lines(g.nx, p->csize, 5, env_budget("DFT_XPHI_SMEM", 32 * 1024), 16);
-    p->LRupd = pick_lines(g.nx, p->csize, (S + 1) / 2, env_budget("DFT_XUPD_SMEM", 48 * 1024), 16);
-    p->LRphi2 = pick_lines(g.nx, p->csize, 10, env_budget("DFT_XPHI_SMEM", 32 * 1024), 16);
-    p->LRupd2 = pick_lines(g.nx, p->csize, 2 * ((S + 1) / 2), env_budget("DFT_XUPD_SMEM", 48 * 1024), 16);
+    // Rows per block of the x passes (dft_autotune refines them): see spread_rows.  Budgets from sweeps of
+    // 32 to 114 KB, two species, line search: Phi' passes FP32 64 KB (32 KB: 160^3 2.08 -> 1.88 ms an
+    // iteration, 100^3 780 -> 687 us, 128^3 701 -> 670; 98 KB: 96^3 369 -> 393), FP64 98 KB (32 KB: 100^3
+    // 7.30 -> 6.60 ms, 128^3 12.0 -> 11.1); update passes 64 KB (48: 160^3 three species 2.30 -> 2.29 ms,
+    // 128^3 795 -> 788 us).
+    {
+        const size_t phi_budget = env_budget("DFT_XPHI_SMEM", (f64 ? 98 : 64) * 1024);
+        const size_t upd_budget = env_budget("DFT_XUPD_SMEM", 64 * 1024);
+        const size_t fwd_budget = env_budget("DFT_XFWD_SMEM", 48 * 1024);
+        const long long rows = (long long)g.ny * g.nz;
+        const int lpr = (S + 1) / 2;
+        p->LX = spread_rows(p, S * rows / 2, 1, fwd_budget);
+        p->LRphi = spread_rows(p, rows, 5, phi_budget);
+        p->LRupd = spread_rows(p, rows, lpr, upd_budget);
+        p->LRphi2 = spread_rows(p, rows, 10, phi_budget);
+        p->LRupd2 = spread_rows(p, rows, 2 * lpr, upd_budget);
+        p->LRn3 = 2 * spread_rows(p, rows / 2, 1, fwd_budget);
+    }
     if (f64) fill_species<double>(p);
     else fill_species<float>(p);
 
