@@ -83,7 +83,7 @@ struct dft_plan {
     double prof_ms[K_COUNT] = {0};
     double prof_bytes[K_COUNT] = {0};
     std::string err;
-    void* ktab = nullptr;           // |k| tables of the compile-time z passes (cubic boxes)
+    void* ktab = nullptr;           // |k| tables of the z passes
     void* laptab = nullptr;         // per-axis Laplacian terms of the Poisson kernel (SpeciesDesc::lap1d)
     cudaStream_t cap = nullptr;     // capture stream of the one-iteration graph (dft_iter_run)
     cudaStream_t side = nullptr;    // copy stream of dft_picard_step_host
@@ -170,6 +170,9 @@ template <typename Real> void fill_species(dft_plan* p) {
     sp.S = p->S;
     for (int i = 0; i < p->S; ++i) {
         sp.R[i] = Real(p->R[i]);
+        sp.r2[i] = Real(p->R[i] * p->R[i]);
+        sp.a2[i] = Real(4.0 * pi * p->R[i] * p->R[i]);
+        sp.v3[i] = Real(4.0 * pi * p->R[i] * p->R[i] * p->R[i]);
         sp.z[i] = Real(p->z[i]);
         sp.rho_b[i] = Real(b.rho[i]);
         sp.inv_rho_b[i] = b.rho[i] > 0 ? Real(1.0 / b.rho[i]) : Real(0);
@@ -295,6 +298,12 @@ void collect_profile(dft_plan* p) {
         if ((p)->prof && (p)->recs.size() > kProfBatch) collect_profile(p);                   \
     } while (0)
 
+#define TRY(x)                        \
+    do {                              \
+        dft_status _s = (x);          \
+        if (_s != DFT_OK) return _s;  \
+    } while (0)
+
 // --------------------------------------------------------------------------------------
 // sequences
 // --------------------------------------------------------------------------------------
@@ -319,21 +328,33 @@ template <typename Real> struct Ops {
         if (!pre)
             LAUNCH(p, K_XFWD, p->S * (RB(p) + CB(p)), P::xfwd(p->stream, p->g, p->ax, p->S, p->LX, rho, W, tw(p, 0)));
         LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, p->S, W, &p->ctl->status, tw(p, 1), p->wait_polls));
-        if (p->g.zsplit && dft_is_ct_size(p->g.nz) && !want_psi && !red_energy) {
-            // z forward transform of the species, the k-space products, z inverse of the nine
+        if (p->g.zsplit && dft_is_ct_size(p->g.nz) && !dft_zsplit<Real>(p->g.nz) && !want_psi && !red_energy) {
+            // z forward transform of the species, the k-space products, z inverse of the seven
             LAUNCH(p, K_ZFFT, 2.0 * p->S * CB(p),
                    P::zfft(p->stream, false, p->g, p->S, W, &p->ctl->status, tw(p, 2), p->wait_polls));
-            LAUNCH(p, K_ZMUL, (p->S + DFT_NSPEC + p->S) * CB(p),
+            LAUNCH(p, K_ZMUL, (p->S + DFT_NZSPEC + p->S) * CB(p),
                    P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), 0, W, slot_n(slot), slot_es(p, slot),
                            nullptr));
-            LAUNCH(p, K_ZFFT, 2.0 * DFT_NSPEC * CB(p),
-                   P::zfft(p->stream, true, p->g, DFT_NSPEC, slot_n(slot), &p->ctl->status, tw(p, 2), p->wait_polls));
+            LAUNCH(p, K_ZFFT, 2.0 * DFT_NZSPEC * CB(p),
+                   P::zfft(p->stream, true, p->g, 1, slot_n(slot), &p->ctl->status, tw(p, 2), p->wait_polls, COL_WD));
         } else {
-            LAUNCH(p, K_ZFWD, (p->S + DFT_NSPEC + p->S + want_psi) * CB(p),
+            LAUNCH(p, K_ZFWD, (p->S + DFT_NZSPEC + p->S + want_psi) * CB(p),
                    P::zconv_fwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W,
                                 slot_n(slot), slot_es(p, slot), red_energy, tw(p, 2), &p->ctl->status));
         }
-        LAUNCH(p, K_YFFT, 2.0 * (DFT_NSPEC) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, DFT_NSPEC, slot_n(slot), &p->ctl->status, tw(p, 1), p->wait_polls));
+        // seven spectra in, nine out (the y derivatives formed in the pass)
+        LAUNCH(p, K_YFFT, (DFT_NZSPEC + DFT_NSPEC) * CB(p),
+               P::yfft(p->stream, true, p->g, p->ay, p->Ty, 1, slot_n(slot), &p->ctl->status, tw(p, 1), p->wait_polls,
+                       COL_DERIV, kf(p, 1)));
+        return DFT_OK;
+    }
+
+    // y forward of the Phi' spectra in T1, one or two sets: nine spectra in, seven out (the y
+    // derivatives added in the pass)
+    static dft_status yfold(dft_plan* p, int sets) {
+        LAUNCH(p, K_YFFT, sets * (DFT_NSPEC + DFT_NZSPEC) * CB(p),
+               P::yfft(p->stream, false, p->g, p->ay, p->Ty, sets, T1(p), &p->ctl->status, tw(p, 1), p->wait_polls,
+                       COL_FOLD, kf(p, 1)));
         return DFT_OK;
     }
 
@@ -351,8 +372,8 @@ template <typename Real> struct Ops {
         LAUNCH(p, K_XPHI, ((use_B ? 2 : 1) + 1 + (materialise ? 1 : 0)) * DFT_NSPEC * CB(p),
                P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, A, B, materialise ? A : nullptr, T1(p),
                                   p->red_max, &p->ctl->status, nullptr, kf(p, 0), tw(p, 0)));
-        LAUNCH(p, K_YFFT, 2.0 * (DFT_NSPEC) * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, DFT_NSPEC, T1(p), &p->ctl->status, tw(p, 1), p->wait_polls));
-        LAUNCH(p, K_ZBWD, (DFT_NSPEC + p->S * ((use_B ? 2 : 1) + 1 + (materialise ? 1 : 0))) * CB(p),
+        TRY(yfold(p, 1));
+        LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S * ((use_B ? 2 : 1) + 1 + (materialise ? 1 : 0))) * CB(p),
                P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), 3, p->S,
                                        p->ctl, T1(p), esA, esB, materialise ? esA : nullptr, tw(p, 2)));
         LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, p->S, T1(p), &p->ctl->status, tw(p, 1), p->wait_polls));
@@ -374,7 +395,7 @@ template <typename Real> struct Ops {
 
     // The two line-search samples rho0 + a_m (rho1 - rho0), a_1 = alpha_s / 2, a_2 = alpha_s (weights
     // in ctl[1], ctl[2], set by FIN_AMAX), evaluated together: one Phi' x pass for both mixtures of
-    // the slots (one read of slots A and B), one y pass over the 18 Phi' spectra, one z pass for
+    // the slots (one read of slots A and B), one y pass over the 18 Phi' spectra (14 out), one z pass for
     // both (the persistent TMA pass; else one per sample), one y pass over the 2 S correlation
     // spectra (else one per sample), and one update pass reading rho0, rho1, V (and the low part)
     // once for both residual sums (red_sum, red_sum2).  Nothing is written to rho or G.
@@ -387,14 +408,12 @@ template <typename Real> struct Ops {
         C* T2 = T1(p) + (long long)DFT_NSPEC * p->g.nc;   // the second sample's spectra
         LAUNCH(p, K_XPHI, 4.0 * DFT_NSPEC * CB(p),
                P::xphi2(p->stream, p->g, p->ax, p->LRphi2, p->ctl, A, B, T1(p), &p->ctl->status, kf(p, 0), tw(p, 0)));
-        LAUNCH(p, K_YFFT, 2.0 * (2 * DFT_NSPEC) * CB(p),
-               P::yfft(p->stream, false, p->g, p->ay, p->Ty, 2 * DFT_NSPEC, T1(p), &p->ctl->status, tw(p, 1),
-                       p->wait_polls));
+        TRY(yfold(p, 2));
         C* c2 = T2;   // the second sample's correlation spectra
         if (P::has_zbwd_pair(p->g, p->S)) {
             // one z pass for both samples (the ES tiles read once; sample 2's results after sample
             // 1's, at T1 components S .. 2 S - 1), then one y inverse over the 2 S components
-            LAUNCH(p, K_ZBWD, (2.0 * DFT_NSPEC + 4.0 * p->S) * CB(p),
+            LAUNCH(p, K_ZBWD, (2.0 * DFT_NZSPEC + 4.0 * p->S) * CB(p),
                    P::zconv_bwd_pair(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), p->S, p->ctl + 1,
                                      T1(p), esA, esB, tw(p, 2)));
             LAUNCH(p, K_YFFT, 2.0 * (2 * p->S) * CB(p),
@@ -404,7 +423,7 @@ template <typename Real> struct Ops {
         } else {
             for (int m = 0; m < 2; ++m) {
                 C* phi = m == 0 ? T1(p) : T2;
-                LAUNCH(p, K_ZBWD, (DFT_NSPEC + p->S * 3) * CB(p),
+                LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S * 3) * CB(p),
                        P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), 3, p->S,
                                     p->ctl + 1 + m, phi, esA, esB, nullptr, tw(p, 2)));
                 LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p),
@@ -463,12 +482,6 @@ dft_status reset_status(dft_plan* p) {
     if (e != cudaSuccess) return fail(p, DFT_ECUDA, std::string("memset: ") + cudaGetErrorString(e));
     return DFT_OK;
 }
-
-#define TRY(x)                        \
-    do {                              \
-        dft_status _s = (x);          \
-        if (_s != DFT_OK) return _s;  \
-    } while (0)
 
 // v_ready (optional): an event the second half (the first use of V) waits for
 template <typename Real> dft_status iter_begin_t(dft_plan* p, Real* rho, const Real* V, cudaEvent_t v_ready = nullptr) {
@@ -541,8 +554,8 @@ template <typename Real> dft_status c1_hs_t(dft_plan* p, const Real* rho, Real* 
     TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     LAUNCH(p, K_XPHI, 2.0 * DFT_NSPEC * CB(p), P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, O::slot_n(p->slotA), nullptr, nullptr,
                               O::T1(p), p->red_max, &p->ctl->status, nullptr, O::kf(p, 0), O::tw(p, 0)));
-    LAUNCH(p, K_YFFT, 2.0 * (DFT_NSPEC) * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, DFT_NSPEC, O::T1(p), &p->ctl->status, O::tw(p, 1), p->wait_polls));
-    LAUNCH(p, K_ZBWD, (DFT_NSPEC + p->S) * CB(p), P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 1, p->S,
+    TRY(O::yfold(p, 1));
+    LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S) * CB(p), P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 1, p->S,
                                    p->ctl, O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
     LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, p->S, O::T1(p), &p->ctl->status, O::tw(p, 1), p->wait_polls));
     TRY(O::xinv(p, p->S, O::T1(p), c1, nullptr, nullptr, -1, nullptr, nullptr));
@@ -667,9 +680,8 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
     LAUNCH(p, K_XPHI, 2.0 * DFT_NSPEC * CB(p), P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, O::slot_n(p->slotA),
                                                         nullptr, nullptr, O::T1(p), p->red_max, &p->ctl->status,
                                                         r_phi, O::kf(p, 0), O::tw(p, 0)));
-    LAUNCH(p, K_YFFT, 2.0 * DFT_NSPEC * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, DFT_NSPEC, O::T1(p),
-                                                        &p->ctl->status, O::tw(p, 1), p->wait_polls));
-    LAUNCH(p, K_ZBWD, (DFT_NSPEC + 2 * S) * CB(p),
+    TRY(O::yfold(p, 1));
+    LAUNCH(p, K_ZBWD, (DFT_NZSPEC + 2 * S) * CB(p),
            P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, S, p->ctl,
                         O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
     LAUNCH(p, K_YFFT, 2.0 * S * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, S, O::T1(p), &p->ctl->status,
@@ -960,10 +972,12 @@ void describe_tuning(dft_plan* p) {
                                           : "run-time column kernel, " + std::to_string(p->Ty) + "-column tiles, radix " +
                                                 radix_text(p->ay);
     t += "; z: ";
-    t += dft_is_ct_size(g.nz) ? (g.zgrp ? std::string("grouped, one tile per CTA") : std::string("TMA persistent"))
+    const bool zsplit = p->precision == DFT_FP64;
+    t += dft_is_ct_size(g.nz) ? (zsplit ? std::string("TMA z transforms around k-space products passes")
+                                 : g.zgrp ? std::string("grouped, one tile per CTA") : std::string("TMA persistent"))
                               : "run-time column kernel, " + std::to_string(p->Tz) + "-column tiles, radix " +
                                     radix_text(p->az);
-    if (dft_is_ct_size(g.nz) && g.zsplit) t += ", first half as z transforms and a k-space products pass";
+    if (dft_is_ct_size(g.nz) && g.zsplit && !zsplit) t += ", first half as z transforms and a k-space products pass";
     t += p->pdl_on ? "; launches: programmatic dependent" : "; launches: stream order";
     p->tuning = t;
 }
@@ -1128,14 +1142,14 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
         for (int v = 0; v < 2; ++v) {
             p->g.yrt = v;
             ms[v] = time_it([&] {
-                P::yfft(p->stream, false, p->g, p->ay, p->Ty, DFT_NSPEC, O::T1(p), &p->ctl->status, O::tw(p, 1),
-                        p->wait_polls);
+                P::yfft(p->stream, false, p->g, p->ay, p->Ty, 1, O::T1(p), &p->ctl->status, O::tw(p, 1),
+                        p->wait_polls, COL_FOLD, O::kf(p, 1));
             });
         }
         p->g.yrt = ms[1] < ms[0] ? 1 : 0;
     }
     // z: the persistent TMA passes against the grouped one-tile-per-CTA kernels (both halves)
-    if (dft_is_ct_size(p->g.nz)) {
+    if (dft_is_ct_size(p->g.nz) && !dft_zsplit<Real>(p->g.nz)) {
         float ms[2];
         for (int v = 0; v < 2; ++v) {
             p->g.zgrp = v;
@@ -1157,8 +1171,8 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
                 P::zfft(p->stream, false, p->g, p->S, O::T1(p), &p->ctl->status, O::tw(p, 2), p->wait_polls);
                 P::zmul(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p), O::slot_n(p->slotB),
                         O::slot_es(p, p->slotB), nullptr);
-                P::zfft(p->stream, true, p->g, DFT_NSPEC, O::slot_n(p->slotB), &p->ctl->status, O::tw(p, 2),
-                        p->wait_polls);
+                P::zfft(p->stream, true, p->g, 1, O::slot_n(p->slotB), &p->ctl->status, O::tw(p, 2),
+                        p->wait_polls, COL_WD);
             } else {
                 P::zconv_fwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p),
                              O::slot_n(p->slotB), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2), &p->ctl->status);
@@ -1442,10 +1456,10 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         }
     }
     // The Poisson kernel's lap(k) is a sum of one term per axis: tabulated by FFT index once, with
-    // the expression the z passes would evaluate at every point.
+    // the expression the z passes would evaluate at every point; after it the axes' wave numbers.
     {
         const size_t nl = size_t(g.nx) + g.ny + g.nz;
-        if (cudaMalloc(&p->laptab, nl * p->rsize) != cudaSuccess) {
+        if (cudaMalloc(&p->laptab, 2 * nl * p->rsize) != cudaSuccess) {
             cudaGetLastError();
             dft_plan_destroy(p);
             return fail(nullptr, DFT_ENOMEM, "cudaMalloc failed: Laplacian table");
@@ -1453,9 +1467,11 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         cudaError_t te;
         if (f64) {
             p->spd.lap1d = static_cast<const double*>(p->laptab);
+            p->spd.kax = p->spd.lap1d + nl;
             te = Passes<double>::build_laptab(nullptr, g, p->kf[0], p->kf[1], p->kf[2], static_cast<double*>(p->laptab));
         } else {
             p->spf.lap1d = static_cast<const float*>(p->laptab);
+            p->spf.kax = p->spf.lap1d + nl;
             te = Passes<float>::build_laptab(nullptr, g, float(p->kf[0]), float(p->kf[1]), float(p->kf[2]),
                                              static_cast<float*>(p->laptab));
         }

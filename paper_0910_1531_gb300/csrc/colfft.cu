@@ -4,9 +4,10 @@
 #include "passes.h"
 
 namespace {
-template <typename Real, bool INV, int T, bool BIG>
+template <typename Real, bool INV, int T, bool BIG, int MODE>
 cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool zax, int ncomp,
-                   typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw, long long polls) {
+                   typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw, long long polls,
+                   int mode, Real kf) {
     using C = typename Cplx<Real>::type;
     constexpr int E = int(sizeof(C) / 8);
     dftk::ColBox cb;
@@ -16,7 +17,8 @@ cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool 
     cb.elems = dft_col_elems<Real>(pa.n, T);
     CUtensorMap map;
     const unsigned long long dims[4] = {(unsigned long long)g.nxh * E, (unsigned long long)g.ny,
-                                        (unsigned long long)g.nz, (unsigned long long)ncomp};
+                                        (unsigned long long)g.nz,
+                                        (unsigned long long)(mode == COL_PLAIN ? ncomp : ncomp * DFT_NSPEC)};
     const unsigned long long strides[3] = {(unsigned long long)g.pxh * sizeof(C),
                                            (unsigned long long)g.ny * g.pxh * sizeof(C),
                                            (unsigned long long)g.nc * sizeof(C)};
@@ -24,33 +26,48 @@ cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool 
     cudaError_t e = tma_encode_4d(&map, data, dims, strides, box);
     if (e != cudaSuccess) return e;
     const int ntx = (int)ceil_div(g.nxh, T), other = zax ? g.ny : g.nz;
-    const int ntiles = ntx * other * ncomp;
+    const int ntiles = ntx * other * (mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC);
     const size_t sm = dft_col_smem<Real>(pa.n, T, pa.nstages);
-    auto kern = dftk::k_colfft<Real, INV, T, BIG>;
+    auto kern = dftk::k_colfft<Real, INV, T, BIG, MODE>;
     const int fit = resident_blocks(kern, dftk::kThreads, sm);
     return launch_k(kern, ntiles < fit ? ntiles : fit, dftk::kThreads, sm, st, g.pdl, map, pa, cb, zax ? 1 : 0, ntx,
-                    other, ntiles, status, tw, polls);
+                    other, ntiles, mode != COL_PLAIN ? 1 : 0, status, tw, kf, polls);
+}
+
+template <typename Real, bool INV, int T>
+cudaError_t launch_m(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool zax, int ncomp,
+                     typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw,
+                     long long polls, int mode, Real kf) {
+    constexpr int kDual = INV ? COL_DERIV : COL_FOLD;
+    const bool big = dft_has_big_prime(pa.n);
+    if (mode == kDual)
+        return big ? launch<Real, INV, T, true, kDual>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf)
+                   : launch<Real, INV, T, false, kDual>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
+    return big ? launch<Real, INV, T, true, COL_PLAIN>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf)
+               : launch<Real, INV, T, false, COL_PLAIN>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
+}
+
+template <typename Real, bool INV, int T> cudaError_t init_m() {
+    constexpr int kDual = INV ? COL_DERIV : COL_FOLD;
+    cudaError_t e = cudaSuccess, r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, INV, T, false, COL_PLAIN>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, INV, T, true, COL_PLAIN>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, INV, T, false, kDual>)) != cudaSuccess) e = r;
+    if ((r = set_max_smem(dftk::k_colfft<Real, INV, T, true, kDual>)) != cudaSuccess) e = r;
+    return e;
 }
 
 template <typename Real, int T>
 cudaError_t launch_t(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int ncomp,
                      typename Cplx<Real>::type* data, int* status, const typename Cplx<Real>::type* tw,
-                     long long polls) {
-    const bool big = dft_has_big_prime(pa.n);
-    if (inv)
-        return big ? launch<Real, true, T, true>(st, g, pa, zax, ncomp, data, status, tw, polls)
-                   : launch<Real, true, T, false>(st, g, pa, zax, ncomp, data, status, tw, polls);
-    return big ? launch<Real, false, T, true>(st, g, pa, zax, ncomp, data, status, tw, polls)
-               : launch<Real, false, T, false>(st, g, pa, zax, ncomp, data, status, tw, polls);
+                     long long polls, int mode, Real kf) {
+    return inv ? launch_m<Real, true, T>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf)
+               : launch_m<Real, false, T>(st, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
 }
 
 template <typename Real, int T> cudaError_t init_t() {
-    cudaError_t e = cudaSuccess, r;
-    if ((r = set_max_smem(dftk::k_colfft<Real, false, T, false>)) != cudaSuccess) e = r;
-    if ((r = set_max_smem(dftk::k_colfft<Real, true, T, false>)) != cudaSuccess) e = r;
-    if ((r = set_max_smem(dftk::k_colfft<Real, false, T, true>)) != cudaSuccess) e = r;
-    if ((r = set_max_smem(dftk::k_colfft<Real, true, T, true>)) != cudaSuccess) e = r;
-    return e;
+    const cudaError_t e = init_m<Real, false, T>(), r = init_m<Real, true, T>();
+    return e != cudaSuccess ? e : r;
 }
 }  // namespace
 
@@ -64,11 +81,11 @@ cudaError_t ColFft<Real>::init() {
 
 template <typename Real>
 cudaError_t ColFft<Real>::run(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int T,
-                              int ncomp, C* data, int* status, const C* tw, long long polls) {
+                              int ncomp, C* data, int* status, const C* tw, long long polls, int mode, Real kf) {
     if constexpr (sizeof(Real) == 4)
-        if (T >= 16) return launch_t<Real, 16>(st, inv, g, pa, zax, ncomp, data, status, tw, polls);
-    return T >= 8 ? launch_t<Real, 8>(st, inv, g, pa, zax, ncomp, data, status, tw, polls)
-                  : launch_t<Real, 4>(st, inv, g, pa, zax, ncomp, data, status, tw, polls);
+        if (T >= 16) return launch_t<Real, 16>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
+    return T >= 8 ? launch_t<Real, 8>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf)
+                  : launch_t<Real, 4>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
 }
 
 template struct ColFft<DFT_INST_REAL>;

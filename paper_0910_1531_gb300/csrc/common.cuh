@@ -17,6 +17,12 @@
 // the x pass that takes the spectra to real space (and the divergence terms of the back
 // convolution in the x pass that leaves it), so the y and z passes carry nine components.
 #define DFT_NSPEC 9
+// Of these the z passes carry seven: i k_y m and i k_y n3 (and on the way back the -i k_y terms) are
+// formed in the y pass, whose tiles hold all k_y.  Component of the q-th of them:
+#define DFT_NZSPEC 7
+__host__ __device__ constexpr int dft_zcomp(int q) { return q < 5 ? q : 2 * q - 4; }
+// Modes of the column passes (k_yfft_tma, k_colfft)
+enum { COL_PLAIN = 0, COL_WD = 1, COL_DERIV = 2, COL_FOLD = 3 };
 // Polls of a TMA tile wait before it gives up (the plans' default; dft_set_wait_polls)
 #define DFT_WAIT_POLLS (1LL << 24)
 
@@ -239,6 +245,10 @@ struct SpeciesDesc {
     // Optional per-axis terms of the discrete Laplacian, sin^2(k_d h_d / 2) / h_d^2 by FFT index:
     // x indices at 0, y at nx, z at nx + ny (k_laptab); null: the kernels evaluate them per point.
     const Real* lap1d;
+    // Optional wave numbers by FFT index, same layout, zero on the Nyquist index (k_laptab); null:
+    // evaluated per point.
+    const Real* kax;
+    Real r2[DFT_MAXS], a2[DFT_MAXS], v3[DFT_MAXS];   // R^2, 4 pi R^2, 4 pi R^3
     // fixed-number species (canonical form of eq. rhoEquation): canon[i] != 0, target sum of G_i
     // over the grid N_i / h^3; ncanon of them
     int canon[DFT_MAXS];

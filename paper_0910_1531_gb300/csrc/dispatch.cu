@@ -94,8 +94,8 @@ cudaError_t Passes<Real>::xfwd(cudaStream_t st, const GridDesc& g, const AxisPla
 
 template <typename Real>
 cudaError_t Passes<Real>::yfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& py, int T, int ncomp,
-                               C* data, int* status, const C* tw, long long polls) {
-    DFT_SWITCH_Y(g.ny, yfft(st, inv, g, py, T, ncomp, data, status, tw, polls))
+                               C* data, int* status, const C* tw, long long polls, int mode, Real kfy) {
+    DFT_SWITCH_Y(g.ny, yfft(st, inv, g, py, T, ncomp, data, status, tw, polls, mode, kfy))
 }
 
 template <typename Real>
@@ -134,8 +134,8 @@ bool Passes<Real>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
 
 template <typename Real>
 cudaError_t Passes<Real>::zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                               const C* tw, long long polls) {
-    DFT_SWITCH_Z(g.nz, zfft(st, inv, g, ncomp, data, status, tw, polls))
+                               const C* tw, long long polls, int mode) {
+    DFT_SWITCH_Z(g.nz, zfft(st, inv, g, ncomp, data, status, tw, polls, mode))
 }
 
 namespace {
@@ -152,28 +152,46 @@ unsigned zmul_blocks(const GridDesc& g) {
 }
 }  // namespace
 
+namespace {
+// The instance of a products kernel for a plan's species count and tables.
+template <bool GRAD, typename Real> auto zmul_kernel(const SpeciesDesc<Real>& sp) {
+    if (!sp.tab_w) return dftk::k_zmul<Real, GRAD, false, DFT_MAXS>;
+    switch (sp.S) {
+        case 1: case 2: return dftk::k_zmul<Real, GRAD, true, 2>;
+        case 3: return dftk::k_zmul<Real, GRAD, true, 3>;
+        case 4: return dftk::k_zmul<Real, GRAD, true, 4>;
+        default: return dftk::k_zmul<Real, GRAD, true, DFT_MAXS>;
+    }
+}
+template <typename Real> auto zmul_bwd_kernel(const SpeciesDesc<Real>& sp) {
+    if (!sp.tab_w) return dftk::k_zmul_bwd<Real, false, DFT_MAXS>;
+    switch (sp.S) {
+        case 1: case 2: return dftk::k_zmul_bwd<Real, true, 2>;
+        case 3: return dftk::k_zmul_bwd<Real, true, 3>;
+        case 4: return dftk::k_zmul_bwd<Real, true, 4>;
+        default: return dftk::k_zmul_bwd<Real, true, DFT_MAXS>;
+    }
+}
+}  // namespace
+
 template <typename Real>
 cudaError_t Passes<Real>::zmul(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
                                Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, double* red_energy) {
-    const unsigned grid = zmul_blocks(g);
-    if (red_energy)
-        return launch_k(dftk::k_zmul<Real, true>, grid, dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, want_psi,
-                        in, slot_n, slot_es, red_energy);
-    return launch_k(dftk::k_zmul<Real, false>, grid, dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, want_psi, in,
-                    slot_n, slot_es, red_energy);
+    auto kern = red_energy ? zmul_kernel<true>(sp) : zmul_kernel<false>(sp);
+    return launch_k(kern, zmul_blocks(g), dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, want_psi, in, slot_n,
+                    slot_es, red_energy);
 }
 
 template <typename Real>
 cudaError_t Passes<Real>::zmul_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
                                    Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi,
                                    const C* esA, const C* esB, C* es_mat) {
-    return launch_k(dftk::k_zmul_bwd<Real>, zmul_blocks(g), dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, flags,
+    return launch_k(zmul_bwd_kernel(sp), zmul_blocks(g), dftk::kThreads, 0, st, g.pdl, g, sp, kfx, kfy, kfz, flags,
                     ncomp_out, samples, ctl, phi, esA, esB, es_mat);
 }
 
 template <typename Real>
 long long Passes<Real>::energy_blocks(const GridDesc& g) {
-    if (dft_is_ct_size(g.nz)) return ceil_div(g.nxh, dft_tile_z<Real>(g.nz)) * g.ny;
     return zmul_blocks(g);
 }
 

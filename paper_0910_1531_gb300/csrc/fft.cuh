@@ -231,6 +231,15 @@ template <int R, bool INV, typename C> __device__ __forceinline__ void dft_small
     else dft16<INV>(v);
 }
 
+// What a stage does with an element it loads (first stages) or stores (last ones); e: its index on
+// the axis.
+struct PreNone {
+    template <typename C> __device__ __forceinline__ void operator()(C&, int) const {}
+};
+struct PostStore {
+    template <typename C> __device__ __forceinline__ void operator()(C* p, C v, int) const { *p = v; }
+};
+
 // ------------------------------------------------------------------------------------
 // Run-time transforms: the Stockham stages of an AxisPlan.  Lines are the columns of a tile T
 // wide (T > 0: element e of line t at e T + t, a thread keeps its column), or rows (T == 0:
@@ -248,9 +257,10 @@ template <int T> __device__ __forceinline__ void rt_split(int task, int lines, c
     }
 }
 
-template <int R, bool INV, int T, int NT, typename C>
+template <int R, bool INV, int T, int NT, typename Pre, typename Post, typename C>
 __device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
-                                         int lines, const FastDiv& dl, int ls, const C* __restrict__ tw) {
+                                         int lines, const FastDiv& dl, int ls, const C* __restrict__ tw, Pre pre,
+                                         Post post) {
     constexpr int ES = T > 0 ? T : 1;
     const int m = p.m[s], ns = p.ns[s].d, tws = p.tws[s];
     const FastDiv dns = p.ns[s];
@@ -263,7 +273,10 @@ __device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restric
         const C* s0 = src + off + j * ES;
         C v[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = s0[r * m * ES];
+        for (int r = 0; r < R; ++r) {
+            v[r] = s0[r * m * ES];
+            pre(v[r], j + r * m);
+        }
         if (ns > 1) {
             const C* w0 = tw + k * tws;
 #pragma unroll
@@ -276,16 +289,17 @@ __device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restric
         dft_small<R, INV>(v);
         C* d0 = dst + off + (q * ns * R + k) * ES;
 #pragma unroll
-        for (int r = 0; r < R; ++r) d0[r * ns * ES] = v[r];
+        for (int r = 0; r < R; ++r) post(d0 + r * ns * ES, v[r], q * ns * R + k + r * ns);
     }
 }
 
 // Stage of a prime radix R >= 11 (the pairs of dft_odd), its outputs spread over threads: a thread
 // forms X_q and X_(R-q) of QG consecutive q of one butterfly (and X_0 with the first ones).  The
 // roots W_R^(r q) = tw[(r q mod R) m] are the same for a whole butterfly and mostly for a warp.
-template <int R, bool INV, int T, int NT, typename C>
+template <int R, bool INV, int T, int NT, typename Pre, typename Post, typename C>
 __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
-                                            int lines, const FastDiv& dl, int ls, const C* __restrict__ tw) {
+                                            int lines, const FastDiv& dl, int ls, const C* __restrict__ tw, Pre pre,
+                                            Post post) {
     using F = decltype(C().x);
     constexpr int ES = T > 0 ? T : 1;
     constexpr int H = (R - 1) / 2, QG = 4, NG = (H + QG - 1) / QG;
@@ -300,11 +314,14 @@ __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __rest
         const int off = T > 0 ? line : line * ls;
         const int q = dns.div(j), k = j - q * ns;
         const C* s0 = src + off + j * ES;
-        const C v0 = s0[0];
+        C v0 = s0[0];
+        pre(v0, j);
         C a[H], b[H], x0 = v0;
 #pragma unroll
         for (int r = 1; r <= H; ++r) {
             C u = s0[r * m * ES], w = s0[(R - r) * m * ES];
+            pre(u, j + r * m);
+            pre(w, j + (R - r) * m);
             if (ns > 1) {
                 C t = tw[r * k * tws], t2 = tw[(R - r) * k * tws];
                 if (INV) { t.y = -t.y; t2.y = -t2.y; }
@@ -315,8 +332,9 @@ __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __rest
             b[r - 1] = csub(u, w);
             x0 = cadd(x0, a[r - 1]);
         }
-        C* d0 = dst + off + (q * ns * R + k) * ES;
-        if (grp == 0) d0[0] = x0;
+        const int e0 = q * ns * R + k;
+        C* d0 = dst + off + e0 * ES;
+        if (grp == 0) post(d0, x0, e0);
         const int q1 = grp * QG + QG < H ? grp * QG + QG : H;
 #pragma unroll 1
         for (int o = grp * QG + 1; o <= q1; ++o) {
@@ -331,19 +349,20 @@ __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __rest
                 t = cmake<C>(t.x - b[r].x * w.y, t.y - b[r].y * w.y);
             }
             const C it = rot<INV>(t);
-            d0[o * ns * ES] = cadd(c, it);
-            d0[(R - o) * ns * ES] = csub(c, it);
+            post(d0 + o * ns * ES, cadd(c, it), e0 + o * ns);
+            post(d0 + (R - o) * ns * ES, csub(c, it), e0 + (R - o) * ns);
         }
     }
 }
 
 // Stage s of a plan.  BIG: lengths with a prime factor of 17..31 (kernels of their own, whose
 // register budget the other lengths do not pay).
-template <bool INV, int T, int NT, bool BIG, typename C>
+template <bool INV, int T, int NT, bool BIG, typename Pre = PreNone, typename Post = PostStore, typename C>
 __device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPlan& p, int s, int lines,
-                                             const FastDiv& dl, int ls, const C* tw) {
-#define DFT_RT(R) case R: rt_stage<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw); break;
-#define DFT_RTP(R) case R: rt_stage_prime<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw); break;
+                                             const FastDiv& dl, int ls, const C* tw, Pre pre = Pre{},
+                                             Post post = Post{}) {
+#define DFT_RT(R) case R: rt_stage<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw, pre, post); break;
+#define DFT_RTP(R) case R: rt_stage_prime<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw, pre, post); break;
     switch (p.radix[s]) {
         DFT_RT(2) DFT_RT(3) DFT_RT(4) DFT_RT(5) DFT_RT(6) DFT_RT(7) DFT_RT(8) DFT_RT(9) DFT_RT(10) DFT_RT(12)
         DFT_RT(14) DFT_RT(15) DFT_RT(16)
@@ -529,29 +548,13 @@ __host__ __device__ constexpr int ct_gstride(int n, int T, int csize) {
     return (ct_gtile(n, T) + 128 / csize - 1) / (128 / csize) * (128 / csize);
 }
 
-// FOLD (a first stage only): the inputs of groups 3 and 4 are taken as group g - i kf.x group
-// fold_partner(g) -- the y derivatives of the back convolution added before a z transform, where
-// the wave number k_y is one constant per tile (kf.x = 0 leaves the groups as they are).
-__host__ __device__ constexpr int fold_partner(int g) { return g == 4 ? 7 : 8; }
-
-template <bool FOLD, int T, bool SD, int GSTR, typename C>
-__device__ __forceinline__ void fold_input(C& v, const C* __restrict__ src, int e, int g, int off, C kf) {
-    if constexpr (FOLD) {
-        if ((g == 3 || g == 4) && kf.x != decltype(kf.x)(0)) {
-            const C u = src[(SD ? e * T : ct_gpos(e, T)) + off + (fold_partner(g) - g) * GSTR];
-            v.x += kf.x * u.y;
-            v.y -= kf.x * u.x;
-        }
-    }
-}
-
-template <int N, int R, int NS, bool INV, int T, int GSTR, bool SD, bool DD, int NT, bool FOLD = false, typename C>
+template <int N, int R, int NS, bool INV, int T, int GSTR, bool SD, bool DD, int NT, typename Pre = PreNone,
+          typename Post = PostStore, typename C>
 __device__ __forceinline__ void ct_stage_grouped(const C* __restrict__ src, C* __restrict__ dst, int groups,
-                                                 const C* __restrict__ tw, C kf = C{}) {
+                                                 const C* __restrict__ tw, Pre pre = Pre{}, Post post = Post{}) {
     constexpr int M = N / R;
     constexpr int TWSTEP = N / (NS * R);
     constexpr int PERG = M * T;
-    static_assert(!FOLD || NS == 1, "the fold belongs to a first stage");
     const int total = PERG * groups;
     for (int task = threadIdx.x; task < total; task += NT) {
         const int g = task / PERG;
@@ -564,7 +567,7 @@ __device__ __forceinline__ void ct_stage_grouped(const C* __restrict__ src, C* _
         for (int r = 0; r < R; ++r) {
             const int e = j + r * M;
             v[r] = src[(SD ? e * T : ct_gpos(e, T)) + off];
-            fold_input<FOLD, T, SD, GSTR>(v[r], src, e, g, off, kf);
+            pre(v[r], e);
         }
         if constexpr (NS > 1) {
 #pragma unroll
@@ -579,18 +582,18 @@ __device__ __forceinline__ void ct_stage_grouped(const C* __restrict__ src, C* _
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int e = base + r * NS;
-            dst[(DD ? e * T : ct_gpos(e, T)) + off] = v[r];
+            post(dst + (DD ? e * T : ct_gpos(e, T)) + off, v[r], e);
         }
     }
 }
 
-template <int N, bool INV, int T, int GSTR, bool SD, bool DD, int NT, int S, bool FOLD = false, typename C>
-__device__ __forceinline__ void ct_stages_grouped(C*& a, C*& b, int groups, const C* tw, C kf = C{}) {
+template <int N, bool INV, int T, int GSTR, bool SD, bool DD, int NT, int S, typename C>
+__device__ __forceinline__ void ct_stages_grouped(C*& a, C*& b, int groups, const C* tw) {
     if constexpr (S < ct_nstages(N)) {
         constexpr int R = ct_radix_at(N, S);
         constexpr int NS = ct_ns_at(N, S);
         constexpr bool last = (S + 1 == ct_nstages(N));
-        ct_stage_grouped<N, R, NS, INV, T, GSTR, SD && S == 0, DD && last, NT, FOLD && S == 0>(a, b, groups, tw, kf);
+        ct_stage_grouped<N, R, NS, INV, T, GSTR, SD && S == 0, DD && last, NT>(a, b, groups, tw);
         __syncthreads();
         C* t = a; a = b; b = t;
         ct_stages_grouped<N, INV, T, GSTR, SD, DD, NT, S + 1>(a, b, groups, tw);
@@ -598,11 +601,10 @@ __device__ __forceinline__ void ct_stages_grouped(C*& a, C*& b, int groups, cons
 }
 
 // Transform `groups` tiles held in a (b: scratch of the same size); the caller syncs before;
-// returns the buffer holding the result (synced).  FOLD: see ct_stage_grouped (kf.x = k_y).
-template <int N, bool INV, int T, int GSTR, bool SD = false, bool DD = false, int NT = kFftThreads,
-          bool FOLD = false, typename C>
-__device__ __forceinline__ C* ct_fft_grouped(C* a, C* b, int groups, const C* tw, C kf = C{}) {
-    ct_stages_grouped<N, INV, T, GSTR, SD, DD, NT, 0, FOLD>(a, b, groups, tw, kf);
+// returns the buffer holding the result (synced).
+template <int N, bool INV, int T, int GSTR, bool SD = false, bool DD = false, int NT = kFftThreads, typename C>
+__device__ __forceinline__ C* ct_fft_grouped(C* a, C* b, int groups, const C* tw) {
+    ct_stages_grouped<N, INV, T, GSTR, SD, DD, NT, 0>(a, b, groups, tw);
     return a;
 }
 
@@ -620,9 +622,8 @@ __device__ __forceinline__ void bar_sync_first(int count) {
     asm volatile("bar.sync 1, %0;" ::"r"(count) : "memory");
 }
 
-template <int N, int R, int NS, bool INV, int T, int GSTR, bool SD, bool DD, int NT, bool END_SYNC, bool FOLD = false,
-          typename C>
-__device__ __forceinline__ void ct_stage_grouped_ip(C* buf, int groups, const C* __restrict__ tw, C kf = C{}) {
+template <int N, int R, int NS, bool INV, int T, int GSTR, bool SD, bool DD, int NT, bool END_SYNC, typename C>
+__device__ __forceinline__ void ct_stage_grouped_ip(C* buf, int groups, const C* __restrict__ tw) {
     constexpr int M = N / R;
     constexpr int TWSTEP = N / (NS * R);
     constexpr int PERG = M * T;
@@ -652,8 +653,6 @@ __device__ __forceinline__ void ct_stage_grouped_ip(C* buf, int groups, const C*
             for (int r = 0; r < R; ++r) {
                 const int e = j + r * M;
                 v[r] = buf[(SD ? e * T : ct_gpos(e, T)) + off];
-                // the fold's partner groups lie past the transformed ones: never written here
-                fold_input<FOLD, T, SD, GSTR>(v[r], buf, e, g, off, kf);
             }
             if constexpr (NS > 1) {
 #pragma unroll
@@ -677,22 +676,19 @@ __device__ __forceinline__ void ct_stage_grouped_ip(C* buf, int groups, const C*
     if constexpr (END_SYNC) __syncthreads();
 }
 
-template <int N, bool INV, int T, int GSTR, bool SD, bool DD, int NT, int S, bool FOLD = false, typename C>
-__device__ __forceinline__ void ct_stages_grouped_ip(C* a, int groups, const C* tw, C kf = C{}) {
+template <int N, bool INV, int T, int GSTR, bool SD, bool DD, int NT, int S, typename C>
+__device__ __forceinline__ void ct_stages_grouped_ip(C* a, int groups, const C* tw) {
     if constexpr (S < ct_nstages(N)) {
         constexpr int R = ct_radix_at(N, S);
         constexpr int NS = ct_ns_at(N, S);
         constexpr bool last = (S + 1 == ct_nstages(N));
-        ct_stage_grouped_ip<N, R, NS, INV, T, GSTR, SD && S == 0, DD && last, NT, !last, FOLD && S == 0>(a, groups,
-                                                                                                       tw, kf);
+        ct_stage_grouped_ip<N, R, NS, INV, T, GSTR, SD && S == 0, DD && last, NT, !last>(a, groups, tw);
         ct_stages_grouped_ip<N, INV, T, GSTR, SD, DD, NT, S + 1>(a, groups, tw);
     }
 }
 
-// Transform `groups` tiles held in a, in place; the caller syncs before and after.  FOLD: see
-// ct_stage_grouped (the partner groups must lie at or past `groups`).
-template <int N, bool INV, int T, int GSTR, bool SD = false, bool DD = false, int NT = kFftThreads,
-          bool FOLD = false, typename C>
-__device__ __forceinline__ void ct_fft_grouped_ip(C* a, int groups, const C* tw, C kf = C{}) {
-    ct_stages_grouped_ip<N, INV, T, GSTR, SD, DD, NT, 0, FOLD>(a, groups, tw, kf);
+// Transform `groups` tiles held in a, in place; the caller syncs before and after.
+template <int N, bool INV, int T, int GSTR, bool SD = false, bool DD = false, int NT = kFftThreads, typename C>
+__device__ __forceinline__ void ct_fft_grouped_ip(C* a, int groups, const C* tw) {
+    ct_stages_grouped_ip<N, INV, T, GSTR, SD, DD, NT, 0>(a, groups, tw);
 }

@@ -34,6 +34,7 @@
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "passes.h"
 #include "tma.cuh"
 
 namespace dftk {
@@ -268,78 +269,143 @@ __global__ void __launch_bounds__(kThreads) k_xfwd(GridDesc g, AxisPlan px, int 
 }
 
 // ------------------------------------------------------------------------------------
+// Column transforms (y and z passes): what a pass does with the components.
+//   COL_PLAIN  every component in place
+//   COL_WD     the seven components of each set of nine that the z passes carry (dft_zcomp)
+//   COL_DERIV  inverse: those seven in place, and from the inputs of m and n3 also i k times them,
+//              transformed into the y-derivative components 5 and 7
+//   COL_FOLD   forward: those seven in place, with -i k times the transforms of the y-derivative
+//              components 5 and 7 added to components 4 and 3
+// A column holds the whole k axis, so both products cost one multiplication per element, and the z
+// passes read and write seven components instead of nine (256^3, S = 4, FP32: second-half z pass
+// 604 -> 526 us, first half's z inverse 236 -> 184, products 295 -> 265; the y passes as before).
+// k is zero on the Nyquist index.
+// ------------------------------------------------------------------------------------
+__host__ __device__ constexpr bool col_dual(int q) { return q == 3 || q == 4; }
+__host__ __device__ constexpr int col_partner(int q) { return q == 3 ? 7 : 5; }
+
+template <typename Real> struct PreDeriv {     // v -> i k v
+    const Real* k;
+    template <typename C> __device__ __forceinline__ void operator()(C& v, int e) const {
+        const Real kk = k[e];
+        v = cmake<C>(-kk * v.y, kk * v.x);
+    }
+};
+template <typename Real> struct PostFold {     // *p holds u: v - i k u
+    const Real* k;
+    template <typename C> __device__ __forceinline__ void operator()(C* p, C v, int e) const {
+        const Real kk = k[e];
+        const C u = *p;
+        *p = cmake<C>(v.x + kk * u.y, v.y - kk * u.x);
+    }
+};
+
+// Wave numbers of an axis for the two modes above, zero on the Nyquist index.
+template <typename Real> __device__ __forceinline__ void fill_axis_k(Real* k, int n, Real kf) {
+    for (int i = threadIdx.x; i < n; i += kThreads) k[i] = (2 * i == n) ? Real(0) : kval<Real>(i, n, kf);
+}
+
+// A pass's tiles, kx tile fastest, then the index on the other axis, then the item (component or, in
+// the modes with sets of nine, q-th component of set m; at most two sets).  per = kx tiles times
+// other indices; every thread needs the item, only the one that moves tiles the rest.
+struct ColItem {
+    int m, q;
+    __device__ __forceinline__ ColItem(int tile, const FastDiv& per, bool sets) {
+        int c = per.div(tile);
+        if (c * per.d > tile) --c;      // tile * per.d may exceed FastDiv's exact range
+        m = sets && c >= DFT_NZSPEC ? 1 : 0;
+        q = c - m * DFT_NZSPEC;
+    }
+    __device__ __forceinline__ int comp(bool sets) const { return sets ? m * DFT_NSPEC + dft_zcomp(q) : q; }
+    __device__ __forceinline__ int partner() const { return m * DFT_NSPEC + col_partner(q); }
+};
+
+// A persistent block's loads in order: tiles b, b + gridDim.x, ...; in COL_FOLD a tile with a
+// derivative component takes two, that component's first.
+template <int MODE> struct ColCursor {
+    int tile, sub;
+    __device__ __forceinline__ bool dual(const FastDiv& per) const {
+        return MODE == COL_FOLD && col_dual(ColItem(tile, per, true).q);
+    }
+    __device__ __forceinline__ void next(const FastDiv& per) {
+        if (MODE == COL_FOLD && sub == 0 && dual(per)) { sub = 1; return; }
+        tile += gridDim.x;
+        sub = 0;
+    }
+};
+
+// ------------------------------------------------------------------------------------
 // y pass with TMA tiles (compile-time length NY <= 256 and tile width TY).  Persistent: CTA b
 // handles tiles b, b + gridDim.x, ...  Two shared-memory stages are filled by TMA loads (one
-// cp.async.bulk.tensor per tile, completing on an mbarrier).  The first FFT stage moves a
-// tile out of its TMA stage into scratch X, so the stage is refilled with the tile after next
-// at once; the remaining stages run between X and Y (padded layout) and the last writes the
-// dense box that leaves through a TMA store, whose shared-memory reads are awaited only before
-// that buffer is written again.  The tensor map views the half spectra as (x: nxh * E, y: ny,
-// plane: nz * ncomp) 8-byte elements, E = sizeof(complex) / 8; a tile is the box (TY * E, NY,
-// 1).  A wait that runs out sets DEV_TIMEOUT and the CTA stops after draining the loads it has
-// in flight.
-// Shared memory: stage 0 | stage 1 (dense tiles) | X | Y (padded) | twiddles | 2 mbarriers.
+// cp.async.bulk.tensor per tile, completing on an mbarrier).  The first of the two FFT stages moves
+// a tile out of its TMA stage into scratch X (padded), so the stage is refilled with the tile after
+// next at once; the second writes the dense box Y that leaves through a TMA store, whose
+// shared-memory reads are awaited only before Y is written again.  The tensor map views the half
+// spectra as (x: nxh * E, y: ny, plane: nz * ncomp) 8-byte elements, E = sizeof(complex) / 8; a
+// tile is the box (TY * E, NY, 1).  A wait that runs out sets DEV_TIMEOUT and the CTA stops after
+// draining the loads it has in flight.
+// ZAX: the same pass along z (modes COL_PLAIN, COL_WD): box (TY * E, 1, NY), a tile is TY kx columns
+// of all NY z points at one ky of one component; the box lands in shared memory with the same
+// layout (element (z, t) at z TY + t).
+// Shared memory: stage 0 | stage 1 (dense tiles) | X (padded) | Y | twiddles | k | 2 mbarriers.
 // ------------------------------------------------------------------------------------
 template <typename Real, int NY, int TY> __host__ __device__ constexpr size_t yfft_tma_smem() {
     using C = typename Cplx<Real>::type;
-    return (2 * size_t(TY) * NY + 2 * size_t(ct_gstride(NY, TY, int(sizeof(C)))) + NY) * sizeof(C) +
+    return (3 * size_t(TY) * NY + size_t(ct_gstride(NY, TY, int(sizeof(C)))) + NY) * sizeof(C) + NY * sizeof(Real) +
            2 * sizeof(uint64_t) + 128;
 }
 
-// ZAX: the same pass along z.  The map is then the z passes' view (x: nxh * E, y: ny, plane:
-// nz * ncomp) with box (TY * E, 1, NY): a tile is TY kx columns of all NY z points at one ky
-// of one component, tile t = (kx tile, ky + ny c) -> coordinates (x, ky, c NY); the box lands in
-// shared memory with the same layout (element (z, t) at z TY + t) as a y tile's.
-template <typename Real, bool INV, int NY, int TY, bool ZAX = false>
-__global__ void __launch_bounds__(kThreads) k_yfft_tma(const __grid_constant__ CUtensorMap map, int ntiles_x,
-                                                       int ntiles, int* __restrict__ status,
-                                                       const typename Cplx<Real>::type* __restrict__ twy,
-                                                       long long polls, int ny_planes = 1) {
+template <typename Real, bool INV, int NY, int TY, bool ZAX = false, int MODE = COL_PLAIN>
+__global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(const __grid_constant__ CUtensorMap map, int ntiles_x, int other,
+                                                       int ntiles, int wd, int* __restrict__ status,
+                                                       const typename Cplx<Real>::type* __restrict__ twy, Real kfy,
+                                                       long long polls) {
     dep_launch();
     dep_wait();
-    static_assert(NY > 0 && NY <= 256 && TY > 0, "compile-time TMA y pass");
+    static_assert(NY > 0 && NY <= 256 && TY > 0 && ct_nstages(NY) == 2, "compile-time TMA y pass");
+    static_assert(MODE == COL_PLAIN || (MODE == (INV ? COL_DERIV : COL_FOLD) && !ZAX), "column mode");
     using C = typename Cplx<Real>::type;
     constexpr int E = int(sizeof(C) / 8);
     constexpr int TILE = TY * NY;
     constexpr int GS = ct_gstride(NY, TY, int(sizeof(C)));
-    constexpr int NST = ct_nstages(NY);
     constexpr uint32_t BYTES = uint32_t(TILE * sizeof(C));
     static_assert(BYTES % 128 == 0, "TMA stage alignment");
     extern __shared__ unsigned char smem_raw[];
     const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127);
     C* const stage0 = reinterpret_cast<C*>(base);
-    C* X = stage0 + 2 * TILE;
-    C* Y = X + GS;
-    C* tw = Y + GS;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + NY);
+    C* const Y = stage0 + 2 * TILE;
+    C* const X = Y + TILE;
+    C* const tw = X + GS;
+    Real* const kt = reinterpret_cast<Real*>(tw + NY);
+    uint64_t* const bar = reinterpret_cast<uint64_t*>(kt + NY);
+    const bool sets = MODE != COL_PLAIN || wd;
     if (threadIdx.x == 0) {
         tma::mbar_init(&bar[0], 1);
         tma::mbar_init(&bar[1], 1);
         tma::fence_mbar_init();
     }
     for (int i = threadIdx.x; i < NY; i += kThreads) tw[i] = twy[i];
+    if constexpr (MODE != COL_PLAIN) fill_axis_k<Real>(kt, NY, kfy);
     __syncthreads();
-    // tensor-map coordinates of a tile
-    auto cy = [&](int tile) { return ZAX ? (tile / ntiles_x) % ny_planes : 0; };
-    auto cz = [&](int tile) { return ZAX ? (tile / ntiles_x) / ny_planes * NY : tile / ntiles_x; };
     int issued = 0, consumed = 0;   // per stage, packed (stage 1 << 16) | stage 0; thread 0
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
-            const int tile = blockIdx.x + s * gridDim.x;
-            if (tile < ntiles) {
-                tma::mbar_expect_tx(&bar[s], BYTES);
-                tma::load_3d(stage0 + s * TILE, &map, (tile % ntiles_x) * TY * E, cy(tile), cz(tile), &bar[s]);
-                issued += 1 << (16 * s);
-            }
-        }
-    }
-    int it = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+    const FastDiv per(ntiles_x * other);
+    ColCursor<MODE> load{(int)blockIdx.x, 0};
+    auto issue = [&](int s) {       // thread 0: the next load in order into stage s
+        if (load.tile >= ntiles) return;
+        const ColItem t(load.tile, per, sets);
+        const int c = (load.sub == 0 && load.dual(per)) ? t.partner() : t.comp(sets);
+        const int x = load.tile % ntiles_x, o = load.tile / ntiles_x % other;
+        tma::mbar_expect_tx(&bar[s], BYTES);
+        tma::load_3d(stage0 + s * TILE, &map, x * TY * E, ZAX ? o : 0, ZAX ? c * NY : c * other + o, &bar[s]);
+        issued += 1 << (16 * s);
+        load.next(per);
+    };
+    if (threadIdx.x == 0) { issue(0); issue(1); }
+    ColCursor<MODE> at{(int)blockIdx.x, 0};
+    for (int it = 0; at.tile < ntiles; ++it, at.next(per)) {
         const int cur = it & 1;
-        C* st = stage0 + cur * TILE;
+        C* const st = stage0 + cur * TILE;
         const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1, polls);
-        // an odd stage count leaves the result in X, which the first stage writes next
-        if (NST % 2 == 1 && threadIdx.x == 0) tma::wait_read_all();
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0) {
                 atomicOr(status, DEV_TIMEOUT);
@@ -351,27 +417,35 @@ __global__ void __launch_bounds__(kThreads) k_yfft_tma(const __grid_constant__ C
             break;
         }
         consumed += 1 << (16 * cur);
-        ct_stage_grouped<NY, ct_radix_at(NY, 0), ct_ns_at(NY, 0), INV, TY, GS, true, NST == 1, kThreads>(st, X, 1,
-                                                                                                       tw);
-        // an even stage count leaves the result in Y, which the second stage writes next
-        if (NST % 2 == 0 && threadIdx.x == 0) tma::wait_read_all();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int next = tile + 2 * gridDim.x;
-            if (next < ntiles) {
-                tma::mbar_expect_tx(&bar[cur], BYTES);
-                tma::load_3d(st, &map, (next % ntiles_x) * TY * E, cy(next), cz(next), &bar[cur]);
-                issued += 1 << (16 * cur);
+        const ColItem t(at.tile, per, sets);
+        const bool dual = MODE != COL_PLAIN && col_dual(t.q);
+        const bool add = MODE == COL_FOLD && dual && at.sub == 1;       // Y holds the partner's transform
+        const bool hold = MODE == COL_FOLD && dual && at.sub == 0;      // keep it there
+        // COL_DERIV: the derivative first (from the same stage), then the component itself
+        for (int pass = (MODE == COL_DERIV && dual) ? 0 : 1; pass < 2; ++pass) {
+            if (MODE == COL_DERIV && pass == 0)
+                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(st, X, 1, tw,
+                                                                                              PreDeriv<Real>{kt});
+            else
+                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(st, X, 1, tw);
+            // the previous store has finished reading Y
+            if (threadIdx.x == 0 && !add) tma::wait_read_all();
+            __syncthreads();
+            if (threadIdx.x == 0 && pass == 1) issue(cur);
+            if (MODE == COL_FOLD && add)
+                ct_stage_grouped<NY, ct_radix_at(NY, 1), ct_ns_at(NY, 1), INV, TY, GS, false, true, kThreads>(
+                    X, Y, 1, tw, PreNone{}, PostFold<Real>{kt});
+            else
+                ct_stage_grouped<NY, ct_radix_at(NY, 1), ct_ns_at(NY, 1), INV, TY, GS, false, true, kThreads>(X, Y, 1,
+                                                                                                            tw);
+            tma::fence_proxy_async();
+            __syncthreads();
+            if (threadIdx.x == 0 && !hold) {
+                const int c = (MODE == COL_DERIV && pass == 0) ? t.partner() : t.comp(sets);
+                const int x = at.tile % ntiles_x, o = at.tile / ntiles_x % other;
+                tma::store_3d(&map, x * TY * E, ZAX ? o : 0, ZAX ? c * NY : c * other + o, Y);
+                tma::commit();
             }
-        }
-        C* a = X;
-        C* b = Y;
-        ct_stages_grouped<NY, INV, TY, GS, false, true, kThreads, 1>(a, b, 1, tw);
-        tma::fence_proxy_async();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            tma::store_3d(&map, (tile % ntiles_x) * TY * E, cy(tile), cz(tile), a);
-            tma::commit();
         }
     }
     if (threadIdx.x == 0) tma::wait_all();
@@ -393,14 +467,15 @@ struct ColBox {
     int elems;              // shared-memory elements of one tile buffer (nbox boxes, 128-byte multiple)
 };
 
-template <typename Real, bool INV, int T, bool BIG>
-__global__ void __launch_bounds__(kThreads, BIG ? 1 : 2) k_colfft(const __grid_constant__ CUtensorMap map, AxisPlan pa,
+template <typename Real, bool INV, int T, bool BIG, int MODE>
+__global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 16 ? 3 : 2)) k_colfft(const __grid_constant__ CUtensorMap map, AxisPlan pa,
                                                                   ColBox cb, int zax, int ntiles_x, int other,
-                                                                  int ntiles, int* __restrict__ status,
+                                                                  int ntiles, int wd, int* __restrict__ status,
                                                                   const typename Cplx<Real>::type* __restrict__ twd,
-                                                                  long long polls) {
+                                                                  Real kf, long long polls) {
     dep_launch();
     dep_wait();
+    static_assert(MODE == COL_PLAIN || MODE == (INV ? COL_DERIV : COL_FOLD), "column mode");
     using C = typename Cplx<Real>::type;
     constexpr int E = int(sizeof(C) / 8);
     extern __shared__ unsigned char smem_raw[];
@@ -409,36 +484,42 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : 2) k_colfft(const __grid_c
     C* const X = stage0 + 2 * cb.elems;
     C* const Y = X + cb.elems;
     C* const tw = pa.nstages > 1 ? Y + cb.elems : Y;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + ((cb.n + 1) & ~1));
+    Real* const kt = reinterpret_cast<Real*>(tw + cb.n);
+    uint64_t* const bar = reinterpret_cast<uint64_t*>(kt + ((cb.n + 1) & ~1));
     const uint32_t bytes = uint32_t(cb.nbox) * uint32_t(cb.rows) * uint32_t(T * sizeof(C));
     const FastDiv one(1);
+    const bool sets = MODE != COL_PLAIN || wd;
+    const int nst = pa.nstages;     // 1 to 3
     if (threadIdx.x == 0) {
         tma::mbar_init(&bar[0], 1);
         tma::mbar_init(&bar[1], 1);
         tma::fence_mbar_init();
     }
     for (int i = threadIdx.x; i < cb.n; i += kThreads) tw[i] = twd[i];
+    if constexpr (MODE != COL_PLAIN) fill_axis_k<Real>(kt, cb.n, kf);
     __syncthreads();
-    auto issue = [&](int tile, int s) {
-        const int x = tile % ntiles_x, rest = tile / ntiles_x, o = rest % other, c = rest / other;
+    int issued = 0, consumed = 0;   // per stage, packed (stage 1 << 16) | stage 0; thread 0
+    const FastDiv per(ntiles_x * other);
+    ColCursor<MODE> load{(int)blockIdx.x, 0};
+    auto issue = [&](int s) {       // thread 0: the next load in order into stage s
+        if (load.tile >= ntiles) return;
+        const ColItem t(load.tile, per, sets);
+        const int c = (load.sub == 0 && load.dual(per)) ? t.partner() : t.comp(sets);
+        const int x = load.tile % ntiles_x, o = load.tile / ntiles_x % other;
         tma::mbar_expect_tx(&bar[s], bytes);
         for (int b = 0; b < cb.nbox; ++b)
             tma::load_4d(stage0 + s * cb.elems + b * cb.rows * T, &map, x * T * E, zax ? o : b * cb.rows,
                          zax ? b * cb.rows : o, c, &bar[s]);
+        issued += 1 << (16 * s);
+        load.next(per);
     };
-    int issued = 0, consumed = 0;   // per stage, packed (stage 1 << 16) | stage 0; thread 0
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) {
-            const int tile = blockIdx.x + s * gridDim.x;
-            if (tile < ntiles) { issue(tile, s); issued += 1 << (16 * s); }
-        }
-    }
-    int it = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+    if (threadIdx.x == 0) { issue(0); issue(1); }
+    ColCursor<MODE> at{(int)blockIdx.x, 0};
+    for (int it = 0; at.tile < ntiles; ++it, at.next(per)) {
         const int cur = it & 1;
-        C* st = stage0 + cur * cb.elems;
+        C* const st = stage0 + cur * cb.elems;
         const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1, polls);
-        // the previous tile's store has finished reading X or Y
+        // the previous store has finished reading X or Y
         if (threadIdx.x == 0) tma::wait_read_all();
         if (__syncthreads_or(!ok)) {
             if (threadIdx.x == 0) {
@@ -451,26 +532,43 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : 2) k_colfft(const __grid_c
             break;
         }
         consumed += 1 << (16 * cur);
-        rt_stage_any<INV, T, kThreads, BIG>(st, X, pa, 0, T, one, 1, tw);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int next = tile + 2 * gridDim.x;
-            if (next < ntiles) { issue(next, cur); issued += 1 << (16 * cur); }
-        }
-        C* a = X;
-        C* b = Y;
-        for (int s = 1; s < pa.nstages; ++s) {
-            rt_stage_any<INV, T, kThreads, BIG>(a, b, pa, s, T, one, 1, tw);
-            C* t = a; a = b; b = t;
-            if (s + 1 < pa.nstages) __syncthreads();
-        }
-        tma::fence_proxy_async();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int x = tile % ntiles_x, rest = tile / ntiles_x, o = rest % other, c = rest / other;
-            for (int q = 0; q < cb.nbox; ++q)
-                tma::store_4d(&map, x * T * E, zax ? o : q * cb.rows, zax ? q * cb.rows : o, c, a + q * cb.rows * T);
-            tma::commit();
+        const ColItem t(at.tile, per, sets);
+        const bool dual = MODE != COL_PLAIN && col_dual(t.q);
+        const bool add = MODE == COL_FOLD && dual && at.sub == 1;       // X or Y holds the partner's transform
+        const bool hold = MODE == COL_FOLD && dual && at.sub == 0;      // keep it there
+        // The buffers: the stage, X, Y, X ...; the last one (of one to three stages X, Y, X) ends up
+        // with the result.  A tile to be added to its partner's transform must not pass through that
+        // buffer before its last stage: with three stages it goes through Y and its TMA stage.
+        C* const res = nst == 2 ? Y : X;
+        const bool spare = add && nst == 3;
+        for (int pass = (MODE == COL_DERIV && dual) ? 0 : 1; pass < 2; ++pass) {
+            if (MODE == COL_DERIV && pass == 1 && dual) {               // after the derivative's store
+                if (threadIdx.x == 0) tma::wait_read_all();
+                __syncthreads();
+            }
+            const C* src = st;
+            for (int s = 0; s < nst; ++s) {
+                C* const dst = s == nst - 1 ? res : (spare ? (s == 0 ? Y : st) : (s == 0 ? X : Y));
+                if (MODE == COL_DERIV && s == 0 && pass == 0)
+                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw, PreDeriv<Real>{kt});
+                else if (MODE == COL_FOLD && add && s == nst - 1)
+                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw, PreNone{}, PostFold<Real>{kt});
+                else
+                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw);
+                if (s == nst - 1) tma::fence_proxy_async();
+                __syncthreads();
+                // the stage is free: refill it
+                if (threadIdx.x == 0 && pass == 1 && s == (spare ? nst - 1 : 0)) issue(cur);
+                src = dst;
+            }
+            if (threadIdx.x == 0 && !hold) {
+                const int c = (MODE == COL_DERIV && pass == 0) ? t.partner() : t.comp(sets);
+                const int x = at.tile % ntiles_x, o = at.tile / ntiles_x % other;
+                for (int q = 0; q < cb.nbox; ++q)
+                    tma::store_4d(&map, x * T * E, zax ? o : q * cb.rows, zax ? q * cb.rows : o, c,
+                                  res + q * cb.rows * T);
+                tma::commit();
+            }
         }
     }
     if (threadIdx.x == 0) tma::wait_all();
@@ -478,8 +576,9 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : 2) k_colfft(const __grid_c
 
 // Wave vector components of tile point (kz index, t) in a z-pass tile at (kx0, ky index)
 template <typename Real> struct KPoint {
-    Real kx, ky, kz, kmag;
-    bool nyq_x, nyq_y, nyq_z, zero;
+    Real kx, ky, kz;
+    bool zero;
+    __device__ __forceinline__ Real kmag() const { return sqrt(kx * kx + ky * ky + kz * kz); }
 };
 
 template <typename Real>
@@ -489,10 +588,6 @@ __device__ __forceinline__ KPoint<Real> kpoint(const GridDesc& g, int kxi, int k
     p.kx = kval<Real>(kxi, g.nx, kfx);
     p.ky = kval<Real>(kyi, g.ny, kfy);
     p.kz = kval<Real>(kzi, g.nz, kfz);
-    p.kmag = sqrt(p.kx * p.kx + p.ky * p.ky + p.kz * p.kz);
-    p.nyq_x = (g.nx % 2 == 0) && (2 * kxi == g.nx);
-    p.nyq_y = (g.ny % 2 == 0) && (2 * kyi == g.ny);
-    p.nyq_z = (g.nz % 2 == 0) && (2 * kzi == g.nz);
     p.zero = (kxi == 0) && (kyi == 0) && (kzi == 0);
     return p;
 }
@@ -502,7 +597,7 @@ __device__ __forceinline__ KPoint<Real> kpoint(const GridDesc& g, int kxi, int k
 template <typename Real>
 __device__ __forceinline__ Real es_kernel(const SpeciesDesc<Real>& sp, int i, int j, const KPoint<Real>& p, Real inv_lap,
                                          Real* dGamma = nullptr) {
-    Real K = delta_c_hat<Real>(p.kmag, sp.es_R[i][j], sp.es_pref[i][j], sp.es_a[i][j], sp.es_b[i][j], sp.es_c[i][j],
+    Real K = delta_c_hat<Real>(p.kmag(), sp.es_R[i][j], sp.es_pref[i][j], sp.es_a[i][j], sp.es_b[i][j], sp.es_c[i][j],
                                dGamma, sp.es_da[i][j], sp.es_db[i][j], sp.es_dc[i][j]);
     if (!p.zero) K -= sp.pois[i][j] * inv_lap;
     return K;
@@ -523,17 +618,20 @@ __device__ __forceinline__ Real inverse_laplacian(const KPoint<Real>& p, Real hx
 
 // The same from the plan's per-axis table (sp.lap1d, the lap_term values by FFT index, evaluated
 // by k_laptab with the same expression: equal bit for bit) where it has one.
-template <typename Real>
+// ALWAYS: it has one.
+template <typename Real, bool ALWAYS = false>
 __device__ __forceinline__ Real inverse_laplacian(const SpeciesDesc<Real>& sp, const GridDesc& g, const KPoint<Real>& p,
                                                   int kxi, int kyi, int kzi, Real hx, Real hy, Real hz) {
-    if (!sp.lap1d) return inverse_laplacian<Real>(p, hx, hy, hz);
+    if constexpr (!ALWAYS)
+        if (!sp.lap1d) return inverse_laplacian<Real>(p, hx, hy, hz);
     if (p.zero) return Real(0);
     const Real lap = Real(4) * (__ldg(sp.lap1d + kxi) + __ldg(sp.lap1d + g.nx + kyi) + __ldg(sp.lap1d + g.nx + g.ny + kzi));
     return Real(1) / lap;
 }
 
 // The per-axis Laplacian terms of a grid: out[i] for x indices i < nx, out[nx + j] for y, out[nx +
-// ny + l] for z (wave numbers kval of the FFT index, as the z passes form them).
+// ny + l] for z (wave numbers kval of the FFT index, as the z passes form them); then, in the same
+// order, the wave numbers themselves, zero on the Nyquist index.
 template <typename Real>
 __global__ void k_laptab(GridDesc g, Real kfx, Real kfy, Real kfz, Real* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -543,6 +641,18 @@ __global__ void k_laptab(GridDesc g, Real kfx, Real kfy, Real kfz, Real* __restr
     else if (i < g.nx + g.ny) v = lap_term(kval<Real>(i - g.nx, g.ny, kfy), Real(g.hy));
     else v = lap_term(kval<Real>(i - g.nx - g.ny, g.nz, kfz), Real(g.hz));
     out[i] = v;
+    const int j = i < g.nx ? i : (i < g.nx + g.ny ? i - g.nx : i - g.nx - g.ny);
+    const int n = i < g.nx ? g.nx : (i < g.nx + g.ny ? g.ny : g.nz);
+    const Real kf = i < g.nx ? kfx : (i < g.nx + g.ny ? kfy : kfz);
+    out[g.nx + g.ny + g.nz + i] = 2 * j == n ? Real(0) : kval<Real>(j, n, kf);
+}
+
+// Wave number of z index kzi, zero on the Nyquist index, from the plan's table where it has one (an
+// int-to-FP64 conversion and a product otherwise, on the FP64 pipe).
+template <typename Real>
+__device__ __forceinline__ Real kz_of(const SpeciesDesc<Real>& sp, const GridDesc& g, int kzi, Real kfz) {
+    if (sp.kax) return __ldg(sp.kax + g.nx + g.ny + kzi);
+    return 2 * kzi == g.nz ? Real(0) : kval<Real>(kzi, g.nz, kfz);
 }
 
 // ------------------------------------------------------------------------------------
@@ -567,109 +677,71 @@ __global__ void k_laptab(GridDesc g, Real kfx, Real kfy, Real kfz, Real* __restr
 // costs a handful of barriers instead of a dozen transforms of one component each.
 // Shared memory: twiddles | 10 tiles | 10 tiles (ct_gstride(NZ, TZ, csize) elements each).
 // ------------------------------------------------------------------------------------
-// The nine weighted-density spectra of one k point into grouped tiles (group stride GS,
-// position pos), 1/N applied: acc = (n0, n1, n2, n3, m) spectra; i k_y and i k_z of m and n3
-// are zero on the Nyquist index of their axis.
+// One species' contribution, 1/N applied, to the spectra acc = (n0, n1, n2, n3, m) at a k point:
+// the weights are w0 (1, R, 4 pi R^2) and j3 (4 pi R^3, R^2), so v is scaled by each of w0 and j3
+// once.  These sums and the back convolution's are written for the fewest FP64 instructions: at
+// 128^3, S = 3, FP64 the second half's products pass issues 58 per k point and takes 128 us (206 and
+// 428 us with a run-time choice between tables and evaluation, wave numbers converted per point and
+// each weight formed by itself).
+template <typename Real>
+__device__ __forceinline__ void wd_add_species(typename Cplx<Real>::type* acc, const SpeciesDesc<Real>& sp, int s,
+                                               typename Cplx<Real>::type v, Real w0, Real j3) {
+    const typename Cplx<Real>::type u = cscale(v, w0 * sp.inv_n), t = cscale(v, j3 * sp.inv_n);
+    acc[0] = cadd(acc[0], u);
+    acc[1] = cadd(acc[1], cscale(u, sp.R[s]));
+    acc[2] = cadd(acc[2], cscale(u, sp.a2[s]));
+    acc[3] = cadd(acc[3], cscale(t, sp.v3[s]));
+    acc[4] = cadd(acc[4], cscale(t, sp.r2[s]));       // w3 / (4 pi R)
+}
+
+// The seven weighted-density spectra of one k point that the z passes carry into groups (group
+// stride GS, position pos; q-th of them = component dft_zcomp(q)): acc, then i k_z m and i k_z n3
+// (kz zero on the Nyquist index).  The y pass forms the y derivatives, the x pass the x derivatives.
 template <typename Real>
 __device__ __forceinline__ void store_wd_spectra(typename Cplx<Real>::type* O, int GS, int pos,
-                                                 const typename Cplx<Real>::type* acc, Real inv_n,
-                                                 const KPoint<Real>& p) {
+                                                 const typename Cplx<Real>::type* acc, Real kz) {
     using C = typename Cplx<Real>::type;
 #pragma unroll
-    for (int a = 0; a < 5; ++a) O[a * GS + pos] = cscale(acc[a], inv_n);
-    const C m = cscale(acc[4], inv_n), n3 = cscale(acc[3], inv_n);
-    const C zero = cmake<C>(Real(0), Real(0));
-    O[5 * GS + pos] = p.nyq_y ? zero : cmake<C>(-p.ky * m.y, p.ky * m.x);
-    O[6 * GS + pos] = p.nyq_z ? zero : cmake<C>(-p.kz * m.y, p.kz * m.x);
-    O[7 * GS + pos] = p.nyq_y ? zero : cmake<C>(-p.ky * n3.y, p.ky * n3.x);
-    O[8 * GS + pos] = p.nyq_z ? zero : cmake<C>(-p.kz * n3.y, p.kz * n3.x);
+    for (int a = 0; a < 5; ++a) O[a * GS + pos] = acc[a];
+    O[5 * GS + pos] = cmake<C>(-kz * acc[4].y, kz * acc[4].x);
+    O[6 * GS + pos] = cmake<C>(-kz * acc[3].y, kz * acc[3].x);
 }
 
-// Species-independent sums of the back convolution at one k point from the nine Phi' spectra
-// of the x and y passes (group stride GS, position pos): a0..a2 = Phi_0..Phi_2,
-// a3 = B3 - i k_y Phi_V2y - i k_z Phi_V2z, a4 = B4 - i k_y Phi_V1y - i k_z Phi_V1z, where the
-// x pass formed B3 = Phi_3 - i k_x Phi_V2x and B4 = -i k_x Phi_V1x (Nyquist terms dropped).
+// Species-independent sums of the back convolution at one k point from the seven Phi' spectra of
+// the y pass (groups as above): a0..a2 = Phi_0..Phi_2, a3 = B3 - i k_z Phi_V2z,
+// a4 = B4 - i k_z Phi_V1z, where the x pass formed B3 = Phi_3 - i k_x Phi_V2x, B4 = -i k_x Phi_V1x
+// and the y pass added their y terms (Nyquist terms dropped: kz zero there).
 template <typename Real>
-__device__ __forceinline__ void bwd_sums(const typename Cplx<Real>::type* X, int GS, int pos, const KPoint<Real>& p,
+__device__ __forceinline__ void bwd_sums(const typename Cplx<Real>::type* X, int GS, int pos, Real kz,
                                          typename Cplx<Real>::type* a) {
-    using C = typename Cplx<Real>::type;
-    a[0] = X[0 * GS + pos];
-    a[1] = X[1 * GS + pos];
-    a[2] = X[2 * GS + pos];
-    a[3] = X[3 * GS + pos];
-    a[4] = X[4 * GS + pos];
-    if (!p.nyq_y) {
-        const C u1 = X[5 * GS + pos], u2 = X[7 * GS + pos];
-        a[4] = cadd(a[4], cmake<C>(p.ky * u1.y, -p.ky * u1.x));
-        a[3] = cadd(a[3], cmake<C>(p.ky * u2.y, -p.ky * u2.x));
-    }
-    if (!p.nyq_z) {
-        const C u1 = X[6 * GS + pos], u2 = X[8 * GS + pos];
-        a[4] = cadd(a[4], cmake<C>(p.kz * u1.y, -p.kz * u1.x));
-        a[3] = cadd(a[3], cmake<C>(p.kz * u2.y, -p.kz * u2.x));
-    }
-}
-
-// The persistent TMA z passes transform seven of the nine spectra: the y-derivative spectra
-// (components 5 and 7: i k_y m and i k_y n3, or their Phi' counterparts) differ from the m and n3
-// spectra by the factor i k_y, which is one constant per z tile, so it is applied on the tile
-// (after the first half's z inverse, before the second half's z forward) instead of transforming
-// them.  In a tile's shared memory, component c sits at group zgroup(c): the seven transformed
-// spectra first (0..4, then i k_z m, i k_z n3), the two y-derivative spectra at 7 and 8 (the
-// fold partners of groups 4 and 3).
-constexpr int kZGroups = 7;
-__host__ __device__ constexpr int zgroup(int c) { return c < 5 ? c : (c == 5 ? 7 : c == 6 ? 5 : c == 7 ? 8 : 6); }
-
-// bwd_sums on the seven transformed groups, the y derivatives already folded into groups 3 and 4
-// (a3 = B3 - i k_y Phi_V2y, a4 = B4 - i k_y Phi_V1y): the z derivatives remain.
-template <typename Real>
-__device__ __forceinline__ void bwd_sums_folded(const typename Cplx<Real>::type* X, int GS, int pos,
-                                                const KPoint<Real>& p, typename Cplx<Real>::type* a) {
     using C = typename Cplx<Real>::type;
 #pragma unroll
     for (int q = 0; q < 5; ++q) a[q] = X[q * GS + pos];
-    if (!p.nyq_z) {
-        const C u1 = X[zgroup(6) * GS + pos], u2 = X[zgroup(8) * GS + pos];
-        a[4] = cadd(a[4], cmake<C>(p.kz * u1.y, -p.kz * u1.x));
-        a[3] = cadd(a[3], cmake<C>(p.kz * u2.y, -p.kz * u2.x));
-    }
+    const C u1 = X[5 * GS + pos], u2 = X[6 * GS + pos];
+    a[4] = cmake<C>(a[4].x + kz * u1.y, a[4].y - kz * u1.x);
+    a[3] = cmake<C>(a[3].x + kz * u2.y, a[3].y - kz * u2.x);
 }
 
-// store_wd_spectra without the y derivatives: groups 0..4 and i k_z m, i k_z n3 at zgroup(6),
-// zgroup(8); the z inverse transforms these seven and zfwd_add_y_derivatives forms the other two.
+// es - mu_hat of species s: mu_hat = w0 (a0 + R a1 + 4 pi R^2 a2) + j3 (4 pi R^3 a3 + R^2 a4).
 template <typename Real>
-__device__ __forceinline__ void store_wd_spectra_z(typename Cplx<Real>::type* O, int GS, int pos,
-                                                   const typename Cplx<Real>::type* acc, Real inv_n,
-                                                   const KPoint<Real>& p) {
+__device__ __forceinline__ typename Cplx<Real>::type bwd_species(const typename Cplx<Real>::type* a,
+                                                                 const SpeciesDesc<Real>& sp, int s, Real w0, Real j3,
+                                                                 typename Cplx<Real>::type es) {
     using C = typename Cplx<Real>::type;
-#pragma unroll
-    for (int a = 0; a < 5; ++a) O[a * GS + pos] = cscale(acc[a], inv_n);
-    const C m = cscale(acc[4], inv_n), n3 = cscale(acc[3], inv_n);
-    const C zero = cmake<C>(Real(0), Real(0));
-    O[zgroup(6) * GS + pos] = p.nyq_z ? zero : cmake<C>(-p.kz * m.y, p.kz * m.x);
-    O[zgroup(8) * GS + pos] = p.nyq_z ? zero : cmake<C>(-p.kz * n3.y, p.kz * n3.x);
-}
-
-// After the first half's z inverse (dense tiles, TILE elements per group): the y-derivative
-// spectra i k_y m -> zgroup(5), i k_y n3 -> zgroup(7), zero on the Nyquist index of y.
-template <typename Real, int TILE, int NT>
-__device__ __forceinline__ void zfwd_add_y_derivatives(typename Cplx<Real>::type* Q, int GS, Real ky) {
-    using C = typename Cplx<Real>::type;
-    for (int idx = threadIdx.x; idx < 2 * TILE; idx += NT) {
-        const int h = idx / TILE, e = idx - h * TILE;
-        const C u = Q[(h ? 3 : 4) * GS + e];
-        Q[(h ? zgroup(7) : zgroup(5)) * GS + e] = cmake<C>(-ky * u.y, ky * u.x);
-    }
+    const Real R = sp.R[s], A = sp.a2[s], V = sp.v3[s], R2 = sp.r2[s];
+    const C P = cmake<C>(a[0].x + R * a[1].x + A * a[2].x, a[0].y + R * a[1].y + A * a[2].y);
+    const C Q = cmake<C>(V * a[3].x + R2 * a[4].x, V * a[3].y + R2 * a[4].y);
+    return cmake<C>(es.x - w0 * P.x - j3 * Q.x, es.y - w0 * P.y - j3 * Q.y);
 }
 
 template <int TT, int NN> __host__ __device__ constexpr size_t zg_smem_bytes(size_t csize) {
-    return (size_t(NN) + 2 * size_t(DFT_NSPEC) * ct_gstride(NN, TT, int(csize))) * csize + 16;
+    return (size_t(NN) + 2 * size_t(DFT_NZSPEC) * ct_gstride(NN, TT, int(csize))) * csize + 16;
 }
 
-// Load `groups` column tiles (component c at src + c * cstride, global row stride rs, columns
-// t < valid, zero elsewhere) into the grouped layout; every load of a thread is issued before
-// its first shared-memory store.
-template <int TT, int NN, int GMAX, typename C>
+// Load `groups` column tiles (component c at src + c * cstride; WD: the q-th is component
+// dft_zcomp(q); global row stride rs, columns t < valid, zero elsewhere) into the grouped layout;
+// every load of a thread is issued before its first shared-memory store.
+template <int TT, int NN, int GMAX, bool WD, typename C>
 __device__ __forceinline__ void tiles_load_grouped(C* __restrict__ dst, const C* __restrict__ src, long long cstride,
                                                    int groups, long long rs, int valid) {
     constexpr int TILE = TT * NN;
@@ -684,7 +756,7 @@ __device__ __forceinline__ void tiles_load_grouped(C* __restrict__ dst, const C*
             const int e = idx / TT, t = idx % TT;
             reg[gi][i] = cmake<C>(0, 0);
             if (gi < groups && (TILE % kThreads == 0 || idx < TILE) && t < valid)
-                reg[gi][i] = src[gi * cstride + e * rs + t];
+                reg[gi][i] = src[(WD ? dft_zcomp(gi) : gi) * cstride + e * rs + t];
         }
     }
 #pragma unroll
@@ -698,7 +770,7 @@ __device__ __forceinline__ void tiles_load_grouped(C* __restrict__ dst, const C*
     }
 }
 
-template <int TT, int NN, typename C>
+template <int TT, int NN, bool WD, typename C>
 __device__ __forceinline__ void tiles_store_grouped(C* __restrict__ dst, const C* __restrict__ src, long long cstride,
                                                     int groups, long long rs, int valid) {
     constexpr int TILE = TT * NN;
@@ -707,7 +779,7 @@ __device__ __forceinline__ void tiles_store_grouped(C* __restrict__ dst, const C
 #pragma unroll
         for (int idx = threadIdx.x; idx < TILE; idx += kThreads) {
             const int e = idx / TT, t = idx % TT;
-            if (t < valid) dst[gi * cstride + e * rs + t] = src[gi * GS + ct_gpos(e, TT) + t];
+            if (t < valid) dst[(WD ? dft_zcomp(gi) : gi) * cstride + e * rs + t] = src[gi * GS + ct_gpos(e, TT) + t];
         }
     }
 }
@@ -733,6 +805,12 @@ __device__ __forceinline__ void load_record(Real (&dst)[MAXN], const Real* __res
 
 __device__ __forceinline__ int signed_index(int j, int n) { return (2 * j <= n) ? j : j - n; }
 
+// Register capacity of a table record of n entries: whole 16-byte loads.
+template <typename Real> __host__ __device__ constexpr int tab_capacity(int n) {
+    const int v = int(16 / sizeof(Real));
+    return (n + v - 1) / v * v;
+}
+
 // Tables of the |k|-only factors: the FMT weights w0, j3 of each species and the bulk-fluid kernel
 // DC_ij_hat with its Gamma derivative.  On a cubic box (kf equal on the three axes) one record per
 // integer m2 = mx^2 + my^2 + mz^2, |k| = kf sqrt(m2); on other boxes (sp.tab_oct) one per (kx, |ky|,
@@ -748,7 +826,7 @@ __global__ void k_ktab(GridDesc g, SpeciesDesc<Real> sp, double kf, Real kfx, Re
     if (sp.tab_oct) {
         const int ix = int(row % g.nxh), rest = int(row / g.nxh), nyh = g.ny / 2 + 1;
         const int iy = rest % nyh, iz = rest / nyh;
-        kmag = kpoint<Real>(g, ix, iy, iz, kfx, kfy, kfz).kmag;
+        kmag = kpoint<Real>(g, ix, iy, iz, kfx, kfy, kfz).kmag();
     } else {
         kmag = Real(kf * sqrt(double(row)));
     }
@@ -779,13 +857,12 @@ __device__ __forceinline__ long long tab_row(const SpeciesDesc<Real>& sp, const 
 // First-half z pass: S species spectra in, the nine weighted
 // densities (z inverse, 1/N applied) and the bulk-fluid/Poisson spectra out.  Per-species loops
 // run to DFT_MAXS with guards so that every per-point array stays in registers.
-template <typename Real, int NZ, int TZ, bool GRAD>
+template <typename Real, int NZ, int TZ>
 __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy,
                                                              Real kfz, int want_psi,
                                                              const typename Cplx<Real>::type* __restrict__ in,
                                                              typename Cplx<Real>::type* __restrict__ slot_n,
                                                              typename Cplx<Real>::type* __restrict__ slot_es,
-                                                             double* __restrict__ red_energy,
                                                              const typename Cplx<Real>::type* __restrict__ twz) {
     dep_launch();
     dep_wait();
@@ -793,46 +870,38 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
     constexpr int TILE = TZ * NZ;
     constexpr int GS = ct_gstride(NZ, TZ, int(sizeof(C)));
     extern __shared__ unsigned char smem_raw[];
-    __shared__ double scratch_d[32];
     const int ny = g.ny, nxh = g.nxh, S = sp.S;
     const int Pn = S * (S + 1) / 2;
     C* tw = align_ptr<C>(smem_raw);
     C* A = tw + NZ;
-    C* B = A + DFT_NSPEC * GS;
+    C* B = A + DFT_NZSPEC * GS;
     for (int i = threadIdx.x; i < NZ; i += kThreads) tw[i] = twz[i];
     const int kx0 = blockIdx.x * TZ;
     const int kyi = blockIdx.y;
     const long long zstride = (long long)ny * g.pxh;
     const long long col0 = (long long)kyi * g.pxh + kx0;
-    tiles_load_grouped<TZ, NZ, DFT_MAXS>(A, in + col0, g.nc, S, zstride, nxh - kx0);
+    tiles_load_grouped<TZ, NZ, DFT_MAXS, false>(A, in + col0, g.nc, S, zstride, nxh - kx0);
     __syncthreads();
     C* R = ct_fft_grouped<NZ, false, TZ, GS>(A, B, S, tw);
     C* O = (R == A) ? B : A;
 
     const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
     const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
     const int my = signed_index(kyi, ny);
     Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
     for (int s = 0; s < S; ++s)
         if (sp.z[s] != Real(0)) { flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]); break; }
-    double e_acc = 0.0, q_acc = 0.0;
     for (int idx = threadIdx.x; idx < TILE; idx += kThreads) {
         const int kzi = idx / TZ, t = idx % TZ;
         const int pos = ct_gpos(kzi, TZ) + t;
         const int kxi = kx0 + t;
         const bool live = kxi < nxh;
         const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-        const long long row = tab && live ? tab_row(sp, g, kxi, my, kzi) : 0;
+        const long long row = live ? tab_row(sp, g, kxi, my, kzi) : 0;
         Real wr[DFT_TAB_W];
-        Real kr[DFT_TAB_K], dkr[DFT_TAB_K];
-        if (tab) {
-            load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
-            if (live) {
-                load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
-                if (GRAD) load_record(dkr, sp.tab_dk + row * sp.tab_ks, Pn);
-            }
-        }
+        Real kr[DFT_TAB_K];
+        load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
+        if (live) load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
         C v[DFT_MAXS];
 #pragma unroll
         for (int s = 0; s < DFT_MAXS; ++s)
@@ -843,18 +912,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
 #pragma unroll
         for (int s = 0; s < DFT_MAXS; ++s) {
             if (s >= S) break;
-            Real w0, j3;
-            if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
-            else fmt_weights<Real>(p.kmag, sp.R[s], &w0, &j3);
-            const Real Rs = sp.R[s];
-            acc[0] = cadd(acc[0], cscale(v[s], w0));
-            acc[1] = cadd(acc[1], cscale(v[s], Rs * w0));
-            acc[2] = cadd(acc[2], cscale(v[s], fourpi * Rs * Rs * w0));
-            acc[3] = cadd(acc[3], cscale(v[s], fourpi * Rs * Rs * Rs * j3));
-            acc[4] = cadd(acc[4], cscale(v[s], Rs * Rs * j3));       // w3 / (4 pi R)
+            wd_add_species<Real>(acc, sp, s, v[s], wr[2 * s], wr[2 * s + 1]);
         }
         if (live) {
-            const Real inv_lap = inverse_laplacian<Real>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
+            const Real inv_lap = inverse_laplacian<Real, true>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
             C dv[DFT_MAXS], es[DFT_MAXS];
 #pragma unroll
             for (int s = 0; s < DFT_MAXS; ++s) {
@@ -864,33 +925,20 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
                 }
                 es[s] = cmake<C>(Real(0), Real(0));
             }
-            const double wk = GRAD ? ((kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? 1.0 : 2.0) : 0.0;
 #pragma unroll
             for (int j = 0; j < DFT_MAXS; ++j) {
 #pragma unroll
                 for (int i = 0; i <= j; ++i) {
                     if (j >= S) continue;
-                    Real K, dK = Real(0);
-                    if (tab) {
-                        K = kr[dft_pair(i, j)];
-                        if (!p.zero) K -= sp.pois[i][j] * inv_lap;
-                        if (GRAD) dK = dkr[dft_pair(i, j)];
-                    } else {
-                        K = es_kernel<Real>(sp, i, j, p, inv_lap, GRAD ? &dK : nullptr);
-                    }
+                    const Real K = kr[dft_pair(i, j)] - sp.pois[i][j] * inv_lap;    // inv_lap is zero at k = 0
                     es[i] = cadd(es[i], cscale(dv[j], K));
                     if (j != i) es[j] = cadd(es[j], cscale(dv[i], K));
-                    if constexpr (GRAD) {
-                        const double re = double(dv[i].x) * dv[j].x + double(dv[i].y) * dv[j].y;
-                        q_acc += wk * double(dK) * re * (j != i ? 2.0 : 1.0);
-                    }
                 }
             }
             const long long o = (long long)kzi * zstride + col0 + t;
 #pragma unroll
             for (int s = 0; s < DFT_MAXS; ++s) {
                 if (s >= S) break;
-                if constexpr (GRAD) e_acc += wk * (double(dv[s].x) * es[s].x + double(dv[s].y) * es[s].y);
                 slot_es[(long long)s * g.nc + o] = es[s];
             }
             if (want_psi) {
@@ -902,21 +950,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
                 slot_es[(long long)S * g.nc + o] = cscale(q, flb * inv_lap);
             }
         }
-        // the nine weighted-density spectra, 1/N applied (DFT_NSPEC order)
-        store_wd_spectra<Real>(O, GS, pos, acc, sp.inv_n, p);
-    }
-    if constexpr (GRAD) {
-        const double be = block_sum(e_acc, scratch_d);
-        const double bq = block_sum(q_acc, scratch_d);
-        if (threadIdx.x == 0) {
-            const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
-            red_energy[2 * b] = be;
-            red_energy[2 * b + 1] = bq;
-        }
+        store_wd_spectra<Real>(O, GS, pos, acc, kz_of(sp, g, kzi, kfz));
     }
     __syncthreads();
-    C* Q = ct_fft_grouped<NZ, true, TZ, GS>(O, R, DFT_NSPEC, tw);
-    tiles_store_grouped<TZ, NZ>(slot_n + col0, Q, g.nc, DFT_NSPEC, zstride, nxh - kx0);
+    C* Q = ct_fft_grouped<NZ, true, TZ, GS>(O, R, DFT_NZSPEC, tw);
+    tiles_store_grouped<TZ, NZ, true>(slot_n + col0, Q, g.nc, DFT_NZSPEC, zstride, nxh - kx0);
 }
 
 // Second-half z pass: the nine Phi' spectra in (flags & 1), the
@@ -943,7 +981,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
     const int ny = g.ny, nxh = g.nxh, S = sp.S;
     C* tw = align_ptr<C>(smem_raw);
     C* A = tw + NZ;
-    C* B = A + DFT_NSPEC * GS;
+    C* B = A + DFT_NZSPEC * GS;
     for (int i = threadIdx.x; i < NZ; i += kThreads) tw[i] = twz[i];
     const int kx0 = blockIdx.x * TZ;
     const int kyi = blockIdx.y;
@@ -953,13 +991,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
     const Real wA = CtlW<Real>::wA(ctl), wB = CtlW<Real>::wB(ctl);
     C* R = A;
     if (hs) {
-        tiles_load_grouped<TZ, NZ, DFT_NSPEC>(A, phi + col0, g.nc, DFT_NSPEC, zstride, nxh - kx0);
+        tiles_load_grouped<TZ, NZ, DFT_NZSPEC, true>(A, phi + col0, g.nc, DFT_NZSPEC, zstride, nxh - kx0);
         __syncthreads();
-        R = ct_fft_grouped<NZ, false, TZ, GS>(A, B, DFT_NSPEC, tw);
+        R = ct_fft_grouped<NZ, false, TZ, GS>(A, B, DFT_NZSPEC, tw);
     }
     C* O = (R == A) ? B : A;
     const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
     const int my = signed_index(kyi, ny);
 
     // loads first: bulk-fluid/Poisson spectra and table records of all of this thread's points
@@ -982,7 +1019,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
                 ea[i][s] = e;
             }
         }
-        if (hs && tab) {
+        if (hs) {
             load_record(wr[i], sp.tab_w + (live ? tab_row(sp, g, kxi, my, kzi) : 0) * sp.tab_ws, 2 * S);
         }
     }
@@ -1003,23 +1040,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
                 if (s < ncomp_out) es_mat[(long long)s * g.nc + o] = ea[i][s];
         }
         if (hs) {
-            const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
             C asum[5];
-            bwd_sums<Real>(R, GS, pos, p, asum);
-            const C a0 = asum[0], a1 = asum[1], a2 = asum[2], a3 = asum[3], a4 = asum[4];
+            bwd_sums<Real>(R, GS, pos, kz_of(sp, g, kzi, kfz), asum);
 #pragma unroll
             for (int s = 0; s < DFT_MAXS; ++s) {
                 if (s >= S) break;
-                Real w0, j3;
-                const Real Rs = sp.R[s];
-                if (tab) { w0 = wr[i][2 * s]; j3 = wr[i][2 * s + 1]; }
-                else fmt_weights<Real>(p.kmag, Rs, &w0, &j3);
-                C mu = cscale(a0, w0);
-                mu = cadd(mu, cscale(a1, Rs * w0));
-                mu = cadd(mu, cscale(a2, fourpi * Rs * Rs * w0));
-                mu = cadd(mu, cscale(a3, fourpi * Rs * Rs * Rs * j3));
-                mu = cadd(mu, cscale(a4, Rs * Rs * j3));
-                out[s] = cmake<C>(out[s].x - mu.x, out[s].y - mu.y);
+                out[s] = bwd_species<Real>(asum, sp, s, wr[i][2 * s], wr[i][2 * s + 1], out[s]);
             }
         }
 #pragma unroll
@@ -1028,24 +1054,23 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
     }
     __syncthreads();
     C* Q = ct_fft_grouped<NZ, true, TZ, GS>(O, R, ncomp_out, tw);
-    tiles_store_grouped<TZ, NZ>(phi + col0, Q, g.nc, ncomp_out, zstride, nxh - kx0);
+    tiles_store_grouped<TZ, NZ, false>(phi + col0, Q, g.nc, ncomp_out, zstride, nxh - kx0);
 }
 
 // ------------------------------------------------------------------------------------
 // First-half z pass with TMA tiles (without the grand-potential sums), persistent like k_zconv_bwd_tma: two stages of S species tiles are filled by TMA loads
-// while the previous tile is transformed; seven weighted-density spectra are transformed back
-// (zgroup order), the two y derivatives formed from m and n3 after that, and the nine leave
-// through TMA stores, the bulk-fluid/Poisson spectra through plain stores.  A tensor map views a half-spectrum
+// while the previous tile is transformed; the seven weighted-density spectra are transformed back
+// and leave through TMA stores, the bulk-fluid/Poisson spectra through plain stores.  A tensor map views a half-spectrum
 // array as (x: nxh * E, y: ny, plane: nz * ncomp) 8-byte elements; a tile is the box
 // (TZ * E, 1, NZ) at plane c * nz.  A wait that runs out sets DEV_TIMEOUT and the CTA stops
 // after draining the loads it has in flight.
-// Shared memory: stage 0 | stage 1 (S padded groups each) | W | V (nine padded groups each) |
+// Shared memory: stage 0 | stage 1 (S padded groups each) | W | V (seven padded groups each) |
 // twiddles | two mbarriers.
 // ------------------------------------------------------------------------------------
 template <typename Real, int NZ, int TZ> __host__ __device__ constexpr size_t zfwd_tma_smem(int S) {
     using C = typename Cplx<Real>::type;
     constexpr size_t GS = size_t(ct_gstride(NZ, TZ, int(sizeof(C))));
-    return ((2 * size_t(S) + 2 * DFT_NSPEC) * GS + NZ) * sizeof(C) + 2 * sizeof(uint64_t) + 128;
+    return ((2 * size_t(S) + 2 * DFT_NZSPEC) * GS + NZ) * sizeof(C) + 2 * sizeof(uint64_t) + 128;
 }
 
 template <typename Real, int NZ, int TZ, int NT, int MINB, int SM = DFT_MAXS>
@@ -1073,8 +1098,8 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
     const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127);
     C* const stage0 = reinterpret_cast<C*>(base);
     C* W = stage0 + 2 * stage_elems;
-    C* Vb = W + DFT_NSPEC * GS;
-    C* tw = Vb + DFT_NSPEC * GS;
+    C* Vb = W + DFT_NZSPEC * GS;
+    C* tw = Vb + DFT_NZSPEC * GS;
     uint64_t* bar = reinterpret_cast<uint64_t*>(tw + NZ);
     const uint32_t tile_bytes = uint32_t(S) * BOX;
     const long long zstride = (long long)ny * g.pxh;
@@ -1101,7 +1126,6 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
     }
     const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
     const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
     Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
     for (int s = 0; s < S; ++s)
         if (sp.z[s] != Real(0)) { flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]); break; }
@@ -1112,8 +1136,8 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
         const int my = signed_index(kyi, ny);
         // table records of this thread's points, in flight while the tile arrives
         // (the first point's; a thread's later points load theirs at the top of their iteration)
-        Real wr[SM <= 3 ? 8 : DFT_TAB_W];
-        Real kr[SM <= 3 ? 8 : DFT_TAB_K];
+        Real wr[tab_capacity<Real>(2 * SM)];
+        Real kr[tab_capacity<Real>(SM * (SM + 1) / 2)];
         auto load_tab = [&](int idx) {
             const int kxi = kx0 + idx % TZ;
             const long long row =
@@ -1121,7 +1145,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
             load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
             load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
         };
-        if (tab) load_tab(threadIdx.x);
+        load_tab(threadIdx.x);
         const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1);
         // the previous tile's TMA stores have finished reading shared memory
         if (threadIdx.x == 0) tma::wait_read_all();
@@ -1142,7 +1166,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
         for (int i = 0; i < PER; ++i) {
             const int idx = threadIdx.x + i * NT;
             if ((TILE % NT != 0) && idx >= TILE) break;
-            if (tab && i > 0) load_tab(idx);
+            if (i > 0) load_tab(idx);
             const int kzi = idx / TZ, t = idx % TZ;
             const int pos = ct_gpos(kzi, TZ) + t;
             const int kxi = kx0 + t;
@@ -1158,18 +1182,10 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
 #pragma unroll
             for (int s = 0; s < SM; ++s) {
                 if (s >= S) break;
-                Real w0, j3;
-                if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
-                else fmt_weights<Real>(p.kmag, sp.R[s], &w0, &j3);
-                const Real Rs = sp.R[s];
-                acc[0] = cadd(acc[0], cscale(v[s], w0));
-                acc[1] = cadd(acc[1], cscale(v[s], Rs * w0));
-                acc[2] = cadd(acc[2], cscale(v[s], fourpi * Rs * Rs * w0));
-                acc[3] = cadd(acc[3], cscale(v[s], fourpi * Rs * Rs * Rs * j3));
-                acc[4] = cadd(acc[4], cscale(v[s], Rs * Rs * j3));       // w3 / (4 pi R)
+                wd_add_species<Real>(acc, sp, s, v[s], wr[2 * s], wr[2 * s + 1]);
             }
             if (live) {
-                const Real inv_lap = inverse_laplacian<Real>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
+                const Real inv_lap = inverse_laplacian<Real, true>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
                 C dv[SM], es[SM];
 #pragma unroll
                 for (int s = 0; s < SM; ++s) {
@@ -1184,13 +1200,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
 #pragma unroll
                     for (int i2 = 0; i2 <= j; ++i2) {
                         if (j >= S) continue;
-                        Real K;
-                        if (tab) {
-                            K = kr[dft_pair(i2, j)];
-                            if (!p.zero) K -= sp.pois[i2][j] * inv_lap;
-                        } else {
-                            K = es_kernel<Real>(sp, i2, j, p, inv_lap, nullptr);
-                        }
+                        const Real K = kr[dft_pair(i2, j)] - sp.pois[i2][j] * inv_lap;  // inv_lap is zero at k = 0
                         es[i2] = cadd(es[i2], cscale(dv[j], K));
                         if (j != i2) es[j] = cadd(es[j], cscale(dv[i2], K));
                     }
@@ -1207,8 +1217,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
                     slot_es[(long long)S * g.nc + o] = cscale(q, flb * inv_lap);
                 }
             }
-            // the weighted-density spectra but the y derivatives, 1/N applied
-            store_wd_spectra_z<Real>(W, GS, pos, acc, sp.inv_n, p);
+            store_wd_spectra<Real>(W, GS, pos, acc, kz_of(sp, g, kzi, kfz));
         }
         __syncthreads();
         // the stage is free now: refill it with the tile after next while the inverse runs
@@ -1216,13 +1225,12 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
             const int next = tile + 2 * gridDim.x;
             if (next < ntiles) { issue(next, cur); issued += 1 << (16 * cur); }
         }
-        C* Q = ct_fft_grouped<NZ, true, TZ, GS, false, true, NT>(W, Vb, kZGroups, tw);
-        const bool nyq_y = (ny % 2 == 0) && (2 * kyi == ny);
-        zfwd_add_y_derivatives<Real, TILE, NT>(Q, GS, nyq_y ? Real(0) : kval<Real>(kyi, ny, kfy));
+        C* Q = ct_fft_grouped<NZ, true, TZ, GS, false, true, NT>(W, Vb, DFT_NZSPEC, tw);
         tma::fence_proxy_async();
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int a = 0; a < DFT_NSPEC; ++a) tma::store_3d(&map_n, kx0 * E, kyi, a * NZ, Q + zgroup(a) * GS);
+            for (int q = 0; q < DFT_NZSPEC; ++q)
+                tma::store_3d(&map_n, kx0 * E, kyi, dft_zcomp(q) * NZ, Q + q * GS);
             tma::commit();
         }
     }
@@ -1240,7 +1248,9 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
 // GRAD: also the two grand-potential sums per block, red_energy[2 b] = sum_k w Re(conj(drho_hat_i)
 // es_hat_i) and red_energy[2 b + 1] = sum_k w Re(conj(drho_hat_i) dK_ij/dGamma drho_hat_j), w = 1 on
 // the kx = 0 and Nyquist planes and 2 elsewhere (the half spectrum standing for the full one).
-template <typename Real, bool GRAD>
+// TAB: the |k| factors come from the plan's tables (kernels that could also evaluate them, and that
+// carried arrays for five species, spilled 316 bytes in FP64).  SM: most species.
+template <typename Real, bool GRAD, bool TAB, int SM>
 __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) k_zmul(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy, Real kfz,
                                                    int want_psi,
                                                    const typename Cplx<Real>::type* __restrict__ in,
@@ -1250,58 +1260,54 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
     dep_launch();
     dep_wait();
     using C = typename Cplx<Real>::type;
-    const int S = sp.S, nxh = g.nxh;
+    constexpr int TW = tab_capacity<Real>(2 * SM), TK = tab_capacity<Real>(SM * (SM + 1) / 2);
+    const int S = sp.S;
+    const unsigned nxh = g.nxh, npt = (unsigned)g.nz * g.ny * nxh;
     const int Pn = S * (S + 1) / 2;
-    const long long npt = (long long)g.nz * g.ny * nxh;
-    const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
-    const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
     double e_acc = 0.0, q_acc = 0.0;
-    for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < npt; q += (long long)gridDim.x * kThreads) {
-        const int kxi = int(q % nxh);
-        const long long rz = q / nxh;
-        const int kyi = int(rz % g.ny), kzi = int(rz / g.ny);
-        const long long o = rz * g.pxh + kxi;
+    for (unsigned q = blockIdx.x * kThreads + threadIdx.x; q < npt; q += gridDim.x * kThreads) {
+        const unsigned rz = q / nxh;
+        const int kxi = int(q - rz * nxh), kzi = int(rz / (unsigned)g.ny), kyi = int(rz - kzi * g.ny);
+        const long long o = (long long)rz * g.pxh + kxi;
         const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-        const long long row = tab ? tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) : 0;
-        C v[DFT_MAXS];
+        const long long row = TAB ? tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) : 0;
+        C v[SM];
 #pragma unroll
-        for (int s = 0; s < DFT_MAXS; ++s)
+        for (int s = 0; s < SM; ++s)
             if (s < S) v[s] = in[(long long)s * g.nc + o];
-        {   // the nine weighted-density spectra, 1/N applied (DFT_NSPEC order), as store_wd_spectra
-            Real wr[DFT_TAB_W];
-            if (tab) load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
+        {   // the seven weighted-density spectra the z inverse transforms, 1/N applied
+            Real wr[TW];
+            if constexpr (TAB) load_record(wr, sp.tab_w + row * sp.tab_ws, 2 * S);
             C acc[5];
 #pragma unroll
             for (int a = 0; a < 5; ++a) acc[a] = cmake<C>(Real(0), Real(0));
 #pragma unroll
-            for (int s = 0; s < DFT_MAXS; ++s) {
+            for (int s = 0; s < SM; ++s) {
                 if (s >= S) break;
                 Real w0, j3;
-                if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
-                else fmt_weights<Real>(p.kmag, sp.R[s], &w0, &j3);
-                const Real Rs = sp.R[s];
-                acc[0] = cadd(acc[0], cscale(v[s], w0));
-                acc[1] = cadd(acc[1], cscale(v[s], Rs * w0));
-                acc[2] = cadd(acc[2], cscale(v[s], fourpi * Rs * Rs * w0));
-                acc[3] = cadd(acc[3], cscale(v[s], fourpi * Rs * Rs * Rs * j3));
-                acc[4] = cadd(acc[4], cscale(v[s], Rs * Rs * j3));       // w3 / (4 pi R)
+                if constexpr (TAB) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
+                else fmt_weights<Real>(p.kmag(), sp.R[s], &w0, &j3);
+                wd_add_species<Real>(acc, sp, s, v[s], w0, j3);
             }
-            store_wd_spectra<Real>(slot_n, int(g.nc), int(o), acc, sp.inv_n, p);
+            C wd[DFT_NZSPEC];
+            store_wd_spectra<Real>(wd, 1, 0, acc, kz_of(sp, g, kzi, kfz));
+#pragma unroll
+            for (int c = 0; c < DFT_NZSPEC; ++c) slot_n[(long long)dft_zcomp(c) * g.nc + o] = wd[c];
         }
         // the bulk-fluid/Poisson spectra
-        Real kr[DFT_TAB_K];
-        Real dkr[GRAD ? DFT_TAB_K : 4];
-        if (tab) {
+        Real kr[TK];
+        Real dkr[GRAD ? TK : 4];
+        if constexpr (TAB) {
             load_record(kr, sp.tab_k + row * sp.tab_ks, Pn);
             if constexpr (GRAD) load_record(dkr, sp.tab_dk + row * sp.tab_ks, Pn);
         }
-        const Real inv_lap = inverse_laplacian<Real>(sp, g, p, kxi, kyi, kzi, hx, hy, hz);
+        const Real inv_lap =
+            inverse_laplacian<Real, TAB>(sp, g, p, kxi, kyi, kzi, Real(g.hx), Real(g.hy), Real(g.hz));
         if (want_psi) {
             C ps = cmake<C>(Real(0), Real(0));
             Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
 #pragma unroll
-            for (int s = 0; s < DFT_MAXS; ++s) {
+            for (int s = 0; s < SM; ++s) {
                 if (s >= S) break;
                 ps = cadd(ps, cscale(v[s], sp.z[s]));
                 if (flb == Real(0) && sp.z[s] != Real(0)) flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]);
@@ -1309,21 +1315,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
             slot_es[(long long)S * g.nc + o] = cscale(ps, flb * inv_lap);   // psi_hat = 4 pi lambda_B q_hat / lap
         }
         const double wk = GRAD ? ((kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? 1.0 : 2.0) : 0.0;
-        C es[DFT_MAXS];
+        C es[SM];
 #pragma unroll
-        for (int s = 0; s < DFT_MAXS; ++s) {
+        for (int s = 0; s < SM; ++s) {
             if (s < S && p.zero) v[s].x -= sp.n_rho_b[s];       // DFT(rho - rho_bath) at k = 0
             es[s] = cmake<C>(Real(0), Real(0));
         }
 #pragma unroll
-        for (int j = 0; j < DFT_MAXS; ++j) {
+        for (int j = 0; j < SM; ++j) {
+            if (j >= S) break;
 #pragma unroll
             for (int i2 = 0; i2 <= j; ++i2) {
-                if (j >= S) continue;
                 Real K, dK = Real(0);
-                if (tab) {
-                    K = kr[dft_pair(i2, j)];
-                    if (!p.zero) K -= sp.pois[i2][j] * inv_lap;
+                if constexpr (TAB) {
+                    K = kr[dft_pair(i2, j)] - sp.pois[i2][j] * inv_lap;     // inv_lap is zero at k = 0
                     if constexpr (GRAD) dK = dkr[dft_pair(i2, j)];
                 } else {
                     K = es_kernel<Real>(sp, i2, j, p, inv_lap, GRAD ? &dK : nullptr);
@@ -1337,7 +1342,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
             }
         }
 #pragma unroll
-        for (int s = 0; s < DFT_MAXS; ++s) {
+        for (int s = 0; s < SM; ++s) {
             if (s >= S) break;
             if constexpr (GRAD) e_acc += wk * (double(v[s].x) * es[s].x + double(v[s].y) * es[s].y);
             slot_es[(long long)s * g.nc + o] = es[s];
@@ -1355,15 +1360,15 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
 }
 
 // ------------------------------------------------------------------------------------
-// The k-space products of the second half as a pass of their own (between the z transforms of a
-// run-time length): at each k point the nine Phi' spectra and the mixed bulk-fluid/Poisson spectra
-// into the ncomp_out correlation spectra, 1/N applied.  `samples` 2: the line search's two samples,
-// sample m's Phi' spectra at components 9 m .., its weights in ctl[m], its results at components
-// m ncomp_out ..; the ES spectra are read once for both.  One thread per k point, kx fastest; a
-// thread reads a sample's components before it writes, and a second sample's results end before
-// that sample's own Phi' or inside what the same thread has read (2 ncomp_out <= 12 < 18).
+// The k-space products of the second half as a pass of their own (between its z transforms): at
+// each k point the seven Phi' spectra and the mixed bulk-fluid/Poisson spectra into the ncomp_out
+// correlation spectra, 1/N applied.  `samples` 2: the line search's two samples, sample m's Phi'
+// spectra at components 9 m .., its weights in ctl[m], its results at components m ncomp_out ..; the
+// ES spectra are read once for both.  One thread per k point, kx fastest; a thread reads a sample's
+// components before it writes, and a second sample's results end before that sample's own Phi' or
+// inside what the same thread has read (2 ncomp_out <= 12 < 18).  TAB, SM as in k_zmul.
 // ------------------------------------------------------------------------------------
-template <typename Real>
+template <typename Real, bool TAB, int SM>
 __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bwd(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy, Real kfz,
                                                        int flags, int ncomp_out, int samples,
                                                        const Ctl* __restrict__ ctl, typename Cplx<Real>::type* phi,
@@ -1373,19 +1378,18 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bw
     dep_launch();
     dep_wait();
     using C = typename Cplx<Real>::type;
-    constexpr int EMAX = DFT_MAXS + 1;
-    const int S = sp.S, nxh = g.nxh;
-    const long long npt = (long long)g.nz * g.ny * nxh;
+    constexpr int EMAX = SM + 1, TW = tab_capacity<Real>(2 * SM);
+    const int S = sp.S;
+    const unsigned nxh = g.nxh, npt = (unsigned)g.nz * g.ny * nxh;
     const bool hs = (flags & 1) != 0, es_on = (flags & 2) != 0;
-    const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
-    for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < npt; q += (long long)gridDim.x * kThreads) {
-        const int kxi = int(q % nxh);
-        const long long rz = q / nxh;
-        const int kyi = int(rz % g.ny), kzi = int(rz / g.ny);
-        const long long o = rz * g.pxh + kxi;
-        Real wr[DFT_TAB_W];
-        if (hs && tab) load_record(wr, sp.tab_w + tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) * sp.tab_ws, 2 * S);
+    for (unsigned q = blockIdx.x * kThreads + threadIdx.x; q < npt; q += gridDim.x * kThreads) {
+        const unsigned rz = q / nxh;
+        const int kxi = int(q - rz * nxh), kzi = int(rz / (unsigned)g.ny), kyi = int(rz - kzi * g.ny);
+        const long long o = (long long)rz * g.pxh + kxi;
+        Real wr[TW];
+        if constexpr (TAB)
+            if (hs) load_record(wr, sp.tab_w + tab_row(sp, g, kxi, signed_index(kyi, g.ny), kzi) * sp.tab_ws, 2 * S);
+        const Real kz = kz_of(sp, g, kzi, kfz);
         C ea[EMAX], eb[EMAX];
 #pragma unroll
         for (int s = 0; s < EMAX; ++s) {
@@ -1399,53 +1403,36 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bw
         for (int m = 0; m < samples; ++m) {
             C* const ph = phi + (long long)m * DFT_NSPEC * g.nc;
             const Real wA = CtlW<Real>::wA(ctl + m), wB = CtlW<Real>::wB(ctl + m);
-            C out[EMAX];
+            C a[5];
+            if (hs) {
+                C x[DFT_NZSPEC];
+#pragma unroll
+                for (int c = 0; c < DFT_NZSPEC; ++c) x[c] = ph[(long long)dft_zcomp(c) * g.nc + o];
+                bwd_sums<Real>(x, 1, 0, kz, a);
+            }
 #pragma unroll
             for (int s = 0; s < EMAX; ++s) {
-                out[s] = cscale(ea[s], wA);
-                if (esB) out[s] = cadd(out[s], cscale(eb[s], wB));
-            }
-            if (es_mat) {
-#pragma unroll
-                for (int s = 0; s < EMAX; ++s)
-                    if (s < ncomp_out) es_mat[(long long)s * g.nc + o] = out[s];
-            }
-            if (hs) {
-                C x[DFT_NSPEC];
-#pragma unroll
-                for (int c = 0; c < DFT_NSPEC; ++c) x[c] = ph[(long long)c * g.nc + o];
-                const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
-                C a[5];
-                bwd_sums<Real>(x, 1, 0, p, a);
-#pragma unroll
-                for (int s = 0; s < DFT_MAXS; ++s) {
-                    if (s >= S) break;
+                if (s >= ncomp_out) break;
+                C out = cscale(ea[s], wA);
+                if (esB) out = cadd(out, cscale(eb[s], wB));
+                if (es_mat) es_mat[(long long)s * g.nc + o] = out;
+                if (hs && s < SM) {
                     Real w0, j3;
-                    const Real Rs = sp.R[s];
-                    if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
-                    else fmt_weights<Real>(p.kmag, Rs, &w0, &j3);
-                    C mu = cscale(a[0], w0);
-                    mu = cadd(mu, cscale(a[1], Rs * w0));
-                    mu = cadd(mu, cscale(a[2], fourpi * Rs * Rs * w0));
-                    mu = cadd(mu, cscale(a[3], fourpi * Rs * Rs * Rs * j3));
-                    mu = cadd(mu, cscale(a[4], Rs * Rs * j3));
-                    out[s] = cmake<C>(out[s].x - mu.x, out[s].y - mu.y);
+                    if constexpr (TAB) { w0 = wr[2 * (s < SM ? s : 0)]; j3 = wr[2 * (s < SM ? s : 0) + 1]; }
+                    else fmt_weights<Real>(kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz).kmag(), sp.R[s], &w0, &j3);
+                    out = bwd_species<Real>(a, sp, s, w0, j3, out);
                 }
+                phi[(long long)(m * ncomp_out + s) * g.nc + o] = cscale(out, sp.inv_n);
             }
-#pragma unroll
-            for (int s = 0; s < EMAX; ++s)
-                if (s < ncomp_out) phi[(long long)(m * ncomp_out + s) * g.nc + o] = cscale(out[s], sp.inv_n);
         }
     }
 }
 
 // ------------------------------------------------------------------------------------
 // Second-half z pass with TMA tiles, persistent: CTA b handles
-// tiles b, b + gridDim.x, ...  Two shared-memory stages, each holding one tile's nine Phi'
-// spectra (in zgroup order), are filled by TMA loads (one cp.async.bulk.tensor per component,
-// completing on the stage's mbarrier) while the previous tile is transformed (seven groups: the
-// y-derivative spectra folded into groups 3 and 4 by the first stage); the tile's bulk-fluid/Poisson
-// spectra arrive in one single-buffered area (third mbarrier), loaded while the previous tile's
+// tiles b, b + gridDim.x, ...  Two shared-memory stages, each holding one tile's seven Phi'
+// spectra, are filled by TMA loads (one cp.async.bulk.tensor per component, completing on the
+// stage's mbarrier) while the previous tile is transformed; the tile's bulk-fluid/Poisson spectra arrive in one single-buffered area (third mbarrier), loaded while the previous tile's
 // inverse and this tile's forward transform run.  The ncomp_out results are written over the
 // first groups of the transformed tile and leave through TMA stores.  At length 256 both
 // transforms run in place (ct_fft_grouped_ip), which keeps the CTA within half an SM's shared
@@ -1460,7 +1447,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bw
 // A tile's components are read and written only by the CTA that takes it, loads before stores,
 // so map_out may overlap map_phi.  A wait that runs out sets DEV_TIMEOUT and the CTA stops after
 // draining the loads it has in flight.
-// Shared memory: stage 0 | stage 1 (nine padded groups each) | W (nine padded groups, below
+// Shared memory: stage 0 | stage 1 (seven padded groups each) | W (seven padded groups, below
 // length 256) | ES (nes dense tiles) | twiddles | three mbarriers.
 // ------------------------------------------------------------------------------------
 __host__ __device__ constexpr bool zbwd_in_place(int nz) { return nz >= 256; }
@@ -1468,11 +1455,11 @@ __host__ __device__ constexpr bool zbwd_in_place(int nz) { return nz >= 256; }
 template <typename Real, int NZ, int TZ> __host__ __device__ constexpr size_t zbwd_tma_smem(int nes) {
     using C = typename Cplx<Real>::type;
     constexpr size_t GS = size_t(ct_gstride(NZ, TZ, int(sizeof(C))));
-    constexpr size_t groups = (zbwd_in_place(NZ) ? 2 : 3) * size_t(DFT_NSPEC);
+    constexpr size_t groups = (zbwd_in_place(NZ) ? 2 : 3) * size_t(DFT_NZSPEC);
     return (groups * GS + size_t(nes) * TZ * NZ + NZ) * sizeof(C) + 3 * sizeof(uint64_t) + 128;
 }
 
-template <typename Real, int NZ, int TZ, int NT, int MINB>
+template <typename Real, int NZ, int TZ, int NT, int MINB, int SM>
 __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constant__ CUtensorMap map_phi,
                                                             const __grid_constant__ CUtensorMap map_esA,
                                                             const __grid_constant__ CUtensorMap map_esB,
@@ -1490,13 +1477,13 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
     constexpr int TILE = TZ * NZ;
     constexpr int GS = ct_gstride(NZ, TZ, int(sizeof(C)));
     constexpr int PER = (TILE + NT - 1) / NT;
-    constexpr int EMAX = DFT_MAXS + 1;
+    constexpr int EMAX = SM + 1;
     constexpr uint32_t BOX = uint32_t(TILE * sizeof(C));
     static_assert(NZ > 0 && NZ <= 256 && (TZ * sizeof(C)) % 16 == 0 && BOX % 128 == 0, "z TMA tile");
     extern __shared__ unsigned char smem_raw[];
     const bool hs = (flags & 1) != 0, es_on = (flags & 2) != 0;
     const int nes = es_on ? ncomp_out * (has_esB ? 2 : 1) : 0;
-    constexpr int stage_elems = DFT_NSPEC * GS;
+    constexpr int stage_elems = DFT_NZSPEC * GS;
     constexpr bool IP = zbwd_in_place(NZ);
     const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127);
     C* const stage0 = reinterpret_cast<C*>(base);
@@ -1517,9 +1504,9 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
         C* st = stage0 + s * stage_elems;
         const int tile = item_tile(item), m = pair ? (item & 1) : 0;
         const int x = (tile % ntiles_x) * TZ * E, y = tile / ntiles_x;
-        tma::mbar_expect_tx(&bar[s], uint32_t(DFT_NSPEC) * BOX);
-        for (int c = 0; c < DFT_NSPEC; ++c)
-            tma::load_3d(st + zgroup(c) * GS, &map_phi, x, y, (m * DFT_NSPEC + c) * NZ, &bar[s]);
+        tma::mbar_expect_tx(&bar[s], uint32_t(DFT_NZSPEC) * BOX);
+        for (int q = 0; q < DFT_NZSPEC; ++q)
+            tma::load_3d(st + q * GS, &map_phi, x, y, (m * DFT_NSPEC + dft_zcomp(q)) * NZ, &bar[s]);
     };
     auto issue_es = [&](int tile) {
         const int x = (tile % ntiles_x) * TZ * E, y = tile / ntiles_x;
@@ -1556,7 +1543,6 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
         }
     };
     const Real fourpi = Real(4.0 * CUDART_PI);
-    const bool tab = sp.tab_w != nullptr;
     for (int it = 0;; ++it) {
         const int tile = item_tile(it);
         if (tile >= ntiles) break;
@@ -1569,8 +1555,8 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
         const int my = signed_index(kyi, ny);
         // the first point's table record is in flight while the tile arrives; a thread's later
         // points load theirs where they are used
-        Real wr[DFT_TAB_W];
-        if (hs && tab) {
+        Real wr[tab_capacity<Real>(2 * SM)];
+        if (hs) {
             const int idx = threadIdx.x;
             const int kxi = kx0 + idx % TZ;
             const long long row =
@@ -1583,12 +1569,8 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
             const bool ok = tma::mbar_wait(&bar[cur], (it >> 1) & 1);
             if (__syncthreads_or(!ok)) { drain(); break; }
             if (threadIdx.x == 0) consumed += 1 << (16 * cur);
-            // the y derivatives folded into groups 3 and 4 on the way into the first stage: seven
-            // groups transformed
-            const bool nyq_y = (ny % 2 == 0) && (2 * kyi == ny);
-            const C kf = cmake<C>(nyq_y ? Real(0) : kval<Real>(kyi, ny, kfy), Real(0));
-            if constexpr (IP) ct_fft_grouped_ip<NZ, false, TZ, GS, true, false, NT, true>(X, kZGroups, tw, kf);
-            else X = ct_fft_grouped<NZ, false, TZ, GS, true, false, NT, true>(st, W, kZGroups, tw, kf);
+            if constexpr (IP) ct_fft_grouped_ip<NZ, false, TZ, GS, true, false, NT>(X, DFT_NZSPEC, tw);
+            else X = ct_fft_grouped<NZ, false, TZ, GS, true, false, NT>(st, W, DFT_NZSPEC, tw);
         }
         // the ES tiles of this tile (loaded since the previous tile's pointwise phase; a pair's
         // second item reuses them); the barrier also ends the forward transform
@@ -1619,25 +1601,14 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
                     if (s < ncomp_out) es_mat[(long long)s * g.nc + o] = out[s];
             }
             if (hs) {
-                if (i > 0 && tab)
+                if (i > 0)
                     load_record(wr, sp.tab_w + (kxi < nxh ? tab_row(sp, g, kxi, my, kzi) : 0) * sp.tab_ws, 2 * S);
-                const KPoint<Real> p = kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz);
                 C asum[5];
-                bwd_sums_folded<Real>(X, GS, pos, p, asum);
-                const C a0 = asum[0], a1 = asum[1], a2 = asum[2], a3 = asum[3], a4 = asum[4];
-#pragma unroll
-                for (int s = 0; s < DFT_MAXS; ++s) {
+                bwd_sums<Real>(X, GS, pos, kz_of(sp, g, kzi, kfz), asum);
+    #pragma unroll
+                for (int s = 0; s < SM; ++s) {
                     if (s >= S) break;
-                    Real w0, j3;
-                    const Real Rs = sp.R[s];
-                    if (tab) { w0 = wr[2 * s]; j3 = wr[2 * s + 1]; }
-                    else fmt_weights<Real>(p.kmag, Rs, &w0, &j3);
-                    C mu = cscale(a0, w0);
-                    mu = cadd(mu, cscale(a1, Rs * w0));
-                    mu = cadd(mu, cscale(a2, fourpi * Rs * Rs * w0));
-                    mu = cadd(mu, cscale(a3, fourpi * Rs * Rs * Rs * j3));
-                    mu = cadd(mu, cscale(a4, Rs * Rs * j3));
-                    out[s] = cmake<C>(out[s].x - mu.x, out[s].y - mu.y);
+                    out[s] = bwd_species<Real>(asum, sp, s, wr[2 * s], wr[2 * s + 1], out[s]);
                 }
             }
             // over the first groups at this thread's own position (read above, by this thread only)

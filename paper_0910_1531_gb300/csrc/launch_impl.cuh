@@ -186,67 +186,77 @@ cudaError_t LaunchY<Real, N>::init() {
         constexpr int TY = dft_tile_y<Real>(N);
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY, false, COL_FOLD>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY, false, COL_DERIV>)) != cudaSuccess) e = r;
     } else {
         if ((r = ColFft<Real>::init()) != cudaSuccess) e = r;
     }
     return e;
 }
 
+namespace {
+// One launch of the compile-time column pass along y or (ZAX) z.
+template <typename Real, bool INV, int N, bool ZAX, int MODE, typename C>
+cudaError_t launch_col_ct(cudaStream_t st, const GridDesc& g, int ncomp, C* data, int* status, const C* tw,
+                          long long polls, int mode, Real kf) {
+    constexpr int TY = dft_tile_y<Real>(N);
+    constexpr int E = int(sizeof(C) / 8);
+    const int planes = mode == COL_PLAIN ? ncomp : ncomp * DFT_NSPEC, items = mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC;
+    CUtensorMap map;
+    cudaError_t e = tma_encode_3d(&map, data, (unsigned long long)g.nxh * E, (unsigned long long)g.ny,
+                                  (unsigned long long)g.nz * planes, (unsigned long long)g.pxh * sizeof(C),
+                                  (unsigned long long)g.ny * g.pxh * sizeof(C), TY * E, ZAX ? 1 : N, ZAX ? N : 1);
+    if (e != cudaSuccess) return e;
+    const int ntx = (int)ceil_div(g.nxh, TY), other = ZAX ? g.ny : g.nz;
+    const int ntiles = ntx * other * items;
+    const size_t sm = dftk::yfft_tma_smem<Real, N, TY>();
+    auto kern = dftk::k_yfft_tma<Real, INV, N, TY, ZAX, MODE>;
+    const int fit = resident_blocks(kern, dftk::kThreads, sm);
+    return launch_k(kern, ntiles < fit ? ntiles : fit, dftk::kThreads, sm, st, g.pdl, map, ntx, other, ntiles,
+                    mode != COL_PLAIN ? 1 : 0, status, tw, kf, polls);
+}
+}  // namespace
+
 template <typename Real, int N>
 cudaError_t LaunchY<Real, N>::yfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& py, int T, int ncomp,
-                                   C* data, int* status, const C* tw, long long polls) {
+                                   C* data, int* status, const C* tw, long long polls, int mode, Real kfy) {
     if constexpr (N > 0) {
-        // TMA path: persistent CTAs, two TMA-filled stages + one FFT scratch tile + twiddles + 2 mbarriers
-        constexpr int TY = dft_tile_y<Real>(N);
-        constexpr int E = int(sizeof(C) / 8);
-        CUtensorMap map;
-        cudaError_t e = tma_encode_3d(&map, data, (unsigned long long)g.nxh * E, (unsigned long long)g.ny,
-                                      (unsigned long long)g.nz * ncomp, (unsigned long long)g.pxh * sizeof(C),
-                                      (unsigned long long)g.ny * g.pxh * sizeof(C), TY * E, N, 1);
-        if (e != cudaSuccess) return e;
-        const int ntx = (int)ceil_div(g.nxh, TY);
-        const int ntiles = ntx * g.nz * ncomp;
-        const size_t sm = dftk::yfft_tma_smem<Real, N, TY>();
-        static int per_sm[2] = {0, 0};
-        static int sms = 0;
-        int& occ = per_sm[inv ? 1 : 0];
-        if (occ == 0) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (inv) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dftk::k_yfft_tma<Real, true, N, TY>, dftk::kThreads, sm);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dftk::k_yfft_tma<Real, false, N, TY>, dftk::kThreads, sm);
-            if (occ < 1) occ = 1;
-        }
-        const int grid = (int)(ntiles < (long long)sms * occ ? ntiles : sms * occ);
-        if (inv) launch_k(dftk::k_yfft_tma<Real, true, N, TY>, grid, dftk::kThreads, sm, st, g.pdl, map, ntx, ntiles, status, tw, polls, 1);
-        else launch_k(dftk::k_yfft_tma<Real, false, N, TY>, grid, dftk::kThreads, sm, st, g.pdl, map, ntx, ntiles, status, tw, polls, 1);
-        return cudaSuccess;
+        if (mode == COL_DERIV)
+            return launch_col_ct<Real, true, N, false, COL_DERIV>(st, g, ncomp, data, status, tw, polls, mode, kfy);
+        if (mode == COL_FOLD)
+            return launch_col_ct<Real, false, N, false, COL_FOLD>(st, g, ncomp, data, status, tw, polls, mode, kfy);
+        return inv ? launch_col_ct<Real, true, N, false, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, kfy)
+                   : launch_col_ct<Real, false, N, false, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, kfy);
     } else {
-        return ColFft<Real>::run(st, inv, g, py, false, T, ncomp, data, status, tw, polls);
+        return ColFft<Real>::run(st, inv, g, py, false, T, ncomp, data, status, tw, polls, mode, kfy);
     }
 }
 
 // ---------------------------------------------------------------------------------- z
-// N > 0: a half in one pass; N == 0 (run-time lengths): z transform, k-space products, z transform.
+// A half in one pass, or (dft_zsplit, and for the grand-potential sums) as z transform, k-space
+// products, z transform.
 template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::init() {
     cudaError_t e = cudaSuccess, r;
-    if constexpr (N > 0) {
+    if constexpr (!dft_zsplit<Real>(N)) {
         constexpr int TZ = dft_tile_z<Real>(N);
-        if ((r = set_max_smem(dftk::k_zconv_fwd_g<Real, N, TZ, false>)) != cudaSuccess) e = r;
-        if ((r = set_max_smem(dftk::k_zconv_fwd_g<Real, N, TZ, true>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_zconv_fwd_g<Real, N, TZ>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_zconv_bwd_g<Real, N, TZ>)) != cudaSuccess) e = r;
         constexpr int TB = dft_tile_zb<Real>(N), TF = dft_tile_zf<Real>(N);
         constexpr int NB = dft_zbwd_threads<Real>(N), MBB = dft_zbwd_minb<Real>(N);
         constexpr int NF = dft_zfwd_threads<Real>(N), MBF = dft_zfwd_minb<Real>(N);
         if constexpr ((TB * sizeof(typename Cplx<Real>::type)) % 16 == 0)
-            if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB>)) != cudaSuccess) e = r;
+        {
+            if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, 3>)) != cudaSuccess) e = r;
+            if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, DFT_MAXS>)) != cudaSuccess) e = r;
+        }
         if constexpr ((TF * sizeof(typename Cplx<Real>::type)) % 16 == 0) {
             constexpr int MBF3 = dft_zfwd_minb_s3<Real>(N);
             if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF, DFT_MAXS>)) != cudaSuccess) e = r;
             if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF3, 3>)) != cudaSuccess) e = r;
         }
+    }
+    if constexpr (N > 0) {
         constexpr int TY = dft_tile_y<Real>(N);
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY, true>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY, true>)) != cudaSuccess) e = r;
@@ -257,50 +267,42 @@ cudaError_t LaunchZ<Real, N>::init() {
 
 template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                                   const C* tw, long long polls) {
+                                   const C* tw, long long polls, int mode) {
     if constexpr (N > 0) {
-        // the y pass's persistent TMA kernel along z: tiles of TY kx columns x nz at one ky
-        constexpr int TY = dft_tile_y<Real>(N);
-        constexpr int E = int(sizeof(C) / 8);
-        CUtensorMap map;
-        cudaError_t e = tma_encode_3d(&map, data, (unsigned long long)g.nxh * E, (unsigned long long)g.ny,
-                                      (unsigned long long)g.nz * ncomp, (unsigned long long)g.pxh * sizeof(C),
-                                      (unsigned long long)g.ny * g.pxh * sizeof(C), TY * E, 1, N);
-        if (e != cudaSuccess) return e;
-        const int ntx = (int)ceil_div(g.nxh, TY);
-        const int ntiles = ntx * g.ny * ncomp;
-        const size_t sm = dftk::yfft_tma_smem<Real, N, TY>();
-        static int per_sm[2] = {0, 0};
-        static int sms = 0;
-        int& occ = per_sm[inv ? 1 : 0];
-        if (occ == 0) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (inv) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dftk::k_yfft_tma<Real, true, N, TY, true>, dftk::kThreads, sm);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dftk::k_yfft_tma<Real, false, N, TY, true>, dftk::kThreads, sm);
-            if (occ < 1) occ = 1;
-        }
-        const int grid = (int)(ntiles < (long long)sms * occ ? ntiles : sms * occ);
-        if (inv)
-            return launch_k(dftk::k_yfft_tma<Real, true, N, TY, true>, grid, dftk::kThreads, sm, st, g.pdl, map, ntx,
-                            ntiles, status, tw, polls, g.ny);
-        return launch_k(dftk::k_yfft_tma<Real, false, N, TY, true>, grid, dftk::kThreads, sm, st, g.pdl, map, ntx,
-                        ntiles, status, tw, polls, g.ny);
+        return inv ? launch_col_ct<Real, true, N, true, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, Real(0))
+                   : launch_col_ct<Real, false, N, true, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, Real(0));
     } else {
-        (void)st; (void)inv; (void)g; (void)ncomp; (void)data; (void)status; (void)tw; (void)polls;
+        (void)st; (void)inv; (void)g; (void)ncomp; (void)data; (void)status; (void)tw; (void)polls; (void)mode;
         return cudaErrorNotSupported;
     }
 }
+
+namespace {
+// The z transform of a split z stage: the compile-time TMA pass or the run-time one.
+template <typename Real, int N, typename C>
+cudaError_t z_axis(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp, int mode,
+                   C* data, int* status, const C* tw) {
+    if constexpr (N > 0) return LaunchZ<Real, N>::zfft(st, inv, g, ncomp, data, status, tw, DFT_WAIT_POLLS, mode);
+    else return ColFft<Real>::run(st, inv, g, pz, true, T, ncomp, data, status, tw, DFT_WAIT_POLLS, mode, Real(0));
+}
+}  // namespace
 
 template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
                                  int T, Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n,
                                  C* slot_es, double* red_energy, const C* tw, int* status) {
-    constexpr int TZ = N > 0 ? dft_tile_z<Real>(N) : 1;
-    constexpr int TB = N > 0 ? dft_tile_zf<Real>(N) : 1;
-    constexpr bool kTma = N > 0 && (TB * sizeof(C)) % 16 == 0;
-    if constexpr (kTma) {
+    constexpr bool kSplit = dft_zsplit<Real>(N);
+    if (kSplit || red_energy || !sp.tab_w) {
+        // z transform, k-space products, z transform
+        cudaError_t e = z_axis<Real, N>(st, false, g, pz, T, sp.S, COL_PLAIN, const_cast<C*>(in), status, tw);
+        if (e == cudaSuccess)
+            e = Passes<Real>::zmul(st, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy);
+        if (e == cudaSuccess) e = z_axis<Real, N>(st, true, g, pz, T, 1, COL_WD, slot_n, status, tw);
+        return e;
+    }
+    if constexpr (!kSplit) {
+        constexpr int TZ = dft_tile_z<Real>(N);
+        constexpr int TB = dft_tile_zf<Real>(N);
         static int optin = 0, sms = 0;
         if (optin == 0) {
             int dev = 0;
@@ -309,8 +311,7 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         }
         const size_t sm = dftk::zfwd_tma_smem<Real, N, TB>(sp.S);
-        if (!red_energy && status && !g.zgrp && sm <= size_t(optin)) {
-            // TMA path (the grand-potential sums keep the one-tile-per-CTA kernel below)
+        if (status && !g.zgrp && sm <= size_t(optin)) {
             constexpr int NT = dft_zfwd_threads<Real>(N), MB = dft_zfwd_minb<Real>(N);
             constexpr int E = int(sizeof(C) / 8);
             CUtensorMap map_in, map_n;
@@ -328,32 +329,14 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
             constexpr int MB3 = dft_zfwd_minb_s3<Real>(N);
             auto kern = sp.S <= 3 ? dftk::k_zconv_fwd_tma<Real, N, TB, NT, MB3, 3>
                                   : dftk::k_zconv_fwd_tma<Real, N, TB, NT, MB, DFT_MAXS>;
-            int occ = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, sm);
-            if (occ < 1) occ = 1;
-            const int grid = (int)(ntiles < (long long)sms * occ ? ntiles : sms * occ);
+            const int fit = resident_blocks(kern, NT, sm), grid = ntiles < fit ? ntiles : fit;
             launch_k(kern, grid, NT, sm, st, g.pdl, map_in, map_n, g, sp, kfx, kfy, kfz, want_psi, slot_es, ntx, ntiles,
                      status, tw);
             return cudaSuccess;
         }
-    }
-    if constexpr (N > 0) {
-        const size_t sm = dftk::zg_smem_bytes<TZ, N>(sizeof(C));
         dim3 grid((unsigned)ceil_div(g.nxh, TZ), (unsigned)g.ny);
-        if (red_energy)
-            launch_k(dftk::k_zconv_fwd_g<Real, N, TZ, true>, grid, dftk::kThreads, sm, st, g.pdl,
-                g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy, tw);
-        else
-            launch_k(dftk::k_zconv_fwd_g<Real, N, TZ, false>, grid, dftk::kThreads, sm, st, g.pdl,
-                g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, nullptr, tw);
-    } else {
-        C* const w = const_cast<C*>(in);
-        cudaError_t e = ColFft<Real>::run(st, false, g, pz, true, T, sp.S, w, status, tw, DFT_WAIT_POLLS);
-        if (e == cudaSuccess)
-            e = Passes<Real>::zmul(st, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy);
-        if (e == cudaSuccess)
-            e = ColFft<Real>::run(st, true, g, pz, true, T, DFT_NSPEC, slot_n, status, tw, DFT_WAIT_POLLS);
-        return e;
+        return launch_k(dftk::k_zconv_fwd_g<Real, N, TZ>, grid, dftk::kThreads, dftk::zg_smem_bytes<TZ, N>(sizeof(C)), st,
+                        g.pdl, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, tw);
     }
     return cudaSuccess;
 }
@@ -367,11 +350,10 @@ template <typename Real, int N, typename C>
 bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy, Real kfz,
                      int flags, int ncomp_out, int pair, const Ctl* ctl, C* phi, const C* esA, const C* esB, C* es_mat,
                      const C* tw) {
-    constexpr int TB = N > 0 ? dft_tile_zb<Real>(N) : 1;
-    constexpr bool kTma = N > 0 && (TB * sizeof(C)) % 16 == 0;
-    if constexpr (!kTma) {
+    if constexpr (dft_zsplit<Real>(N)) {
         return false;
     } else {
+        constexpr int TB = dft_tile_zb<Real>(N);
         const bool es_on = (flags & 2) != 0;
         const int nes = es_on ? ncomp_out * (esB ? 2 : 1) : 0;
         static int optin = 0, sms = 0;
@@ -382,7 +364,7 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         }
         const size_t sm = dftk::zbwd_tma_smem<Real, N, TB>(nes);
-        if (g.zgrp || sm > size_t(optin)) return false;
+        if (g.zgrp || !sp.tab_w || sm > size_t(optin)) return false;
         // persistent CTAs, two TMA-filled stages of nine Phi' tiles, one area of ES tiles
         constexpr int NT = dft_zbwd_threads<Real>(N), MB = dft_zbwd_minb<Real>(N);
         constexpr int E = int(sizeof(C) / 8);
@@ -400,34 +382,33 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
         if (e != cudaSuccess) return false;
         const int ntx = (int)ceil_div(g.nxh, TB);
         const int ntiles = ntx * g.ny;
-        int occ = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dftk::k_zconv_bwd_tma<Real, N, TB, NT, MB>, NT, sm);
-        if (occ < 1) occ = 1;
-        const int grid = (int)(ntiles < (long long)sms * occ ? ntiles : sms * occ);
+        // at most three species: the instance whose records and species loops are sized for three
+        auto kern = sp.S <= 3 ? dftk::k_zconv_bwd_tma<Real, N, TB, NT, MB, 3>
+                              : dftk::k_zconv_bwd_tma<Real, N, TB, NT, MB, DFT_MAXS>;
+        const int fit = resident_blocks(kern, NT, sm), grid = ntiles < fit ? ntiles : fit;
         // the status word of the device control block records a TMA wait that ran out
         int* status = const_cast<int*>(&ctl->status);
-        launch_k(dftk::k_zconv_bwd_tma<Real, N, TB, NT, MB>, grid, NT, sm, st, g.pdl, map_phi, map_esA, map_esB,
+        launch_k(kern, grid, NT, sm, st, g.pdl, map_phi, map_esA, map_esB,
                  map_out, g, sp, kfx, kfy, kfz, flags, ncomp_out, esB ? 1 : 0, pair, ctl, es_mat, ntx, ntiles, status,
                  tw);
         return true;
     }
 }
 
-// The second half of a run-time z length for one sample or the line search's two: the Phi' spectra
+// The second half as three passes, for one sample or the line search's two: the Phi' spectra
 // transformed (only where the hard-sphere part is wanted), the products, the correlations
 // transformed back.
-template <typename Real, typename C>
-cudaError_t zbwd_rt(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T, Real kfx,
+template <typename Real, int N, typename C>
+cudaError_t zbwd_split(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T, Real kfx,
                     Real kfy, Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi, const C* esA,
                     const C* esB, C* es_mat, const C* tw) {
     int* status = const_cast<int*>(&ctl->status);
     cudaError_t e = cudaSuccess;
     if (flags & 1)
-        e = ColFft<Real>::run(st, false, g, pz, true, T, samples * DFT_NSPEC, phi, status, tw, DFT_WAIT_POLLS);
+        e = z_axis<Real, N>(st, false, g, pz, T, samples, COL_WD, phi, status, tw);
     if (e == cudaSuccess)
         e = Passes<Real>::zmul_bwd(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, samples, ctl, phi, esA, esB, es_mat);
-    if (e == cudaSuccess)
-        e = ColFft<Real>::run(st, true, g, pz, true, T, samples * ncomp_out, phi, status, tw, DFT_WAIT_POLLS);
+    if (e == cudaSuccess) e = z_axis<Real, N>(st, true, g, pz, T, samples * ncomp_out, COL_PLAIN, phi, status, tw);
     return e;
 }
 }  // namespace
@@ -436,16 +417,16 @@ template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
                                  int T, Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
                                  const C* esA, const C* esB, C* es_mat, const C* tw) {
-    constexpr int TZ = N > 0 ? dft_tile_z<Real>(N) : 1;
+    if (dft_zsplit<Real>(N) || !sp.tab_w)
+        return zbwd_split<Real, N>(st, g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, 1, ctl, phi, esA, esB, es_mat,
+                                   tw);
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, 0, ctl, phi, esA, esB, es_mat, tw))
         return cudaSuccess;
-    if constexpr (N > 0) {
-        const size_t sm = dftk::zg_smem_bytes<TZ, N>(sizeof(C));
+    if constexpr (!dft_zsplit<Real>(N)) {
+        constexpr int TZ = dft_tile_z<Real>(N);
         dim3 grid((unsigned)ceil_div(g.nxh, TZ), (unsigned)g.ny);
-        launch_k(dftk::k_zconv_bwd_g<Real, N, TZ>, grid, dftk::kThreads, sm, st, g.pdl,
-            g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
-    } else {
-        return zbwd_rt<Real>(st, g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, 1, ctl, phi, esA, esB, es_mat, tw);
+        return launch_k(dftk::k_zconv_bwd_g<Real, N, TZ>, grid, dftk::kThreads, dftk::zg_smem_bytes<TZ, N>(sizeof(C)), st,
+                        g.pdl, g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
     }
     return cudaSuccess;
 }
@@ -455,8 +436,8 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g,
                                              const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz,
                                              int ncomp_out, const Ctl* ctl, C* phi, const C* esA, const C* esB,
                                              const C* tw) {
-    if constexpr (N == 0)
-        return zbwd_rt<Real>(st, g, pz, sp, T, kfx, kfy, kfz, 3, ncomp_out, 2, ctl, phi, esA, esB,
+    if (dft_zsplit<Real>(N) || !sp.tab_w)
+        return zbwd_split<Real, N>(st, g, pz, sp, T, kfx, kfy, kfz, 3, ncomp_out, 2, ctl, phi, esA, esB,
                              static_cast<C*>(nullptr), tw);
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, 3, ncomp_out, 1, ctl, phi, esA, esB,
                                  static_cast<C*>(nullptr), tw))
@@ -466,15 +447,13 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g,
 
 template <typename Real, int N>
 bool LaunchZ<Real, N>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
-    constexpr int TB = N > 0 ? dft_tile_zb<Real>(N) : 1;
-    if constexpr (N == 0) {
+    if constexpr (dft_zsplit<Real>(N)) {
         return true;
-    } else if constexpr ((TB * sizeof(C)) % 16 == 0) {
+    } else {
+        constexpr int TB = dft_tile_zb<Real>(N);
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         return !g.zgrp && dftk::zbwd_tma_smem<Real, N, TB>(2 * ncomp_out) <= size_t(optin);
-    } else {
-        return false;
     }
 }

@@ -142,7 +142,14 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     SpeciesDesc<float> sp;
     std::memset(&sp, 0, sizeof(sp));
     sp.S = S;
-    for (int i = 0; i < S; ++i) sp.R[i] = float(prm->radius_nm[i]);
+    const double fourpi = 12.56637061435917295385;
+    for (int i = 0; i < S; ++i) {
+        const double R = prm->radius_nm[i];
+        sp.R[i] = float(R);
+        sp.r2[i] = float(R * R);
+        sp.a2[i] = float(fourpi * R * R);
+        sp.v3[i] = float(fourpi * R * R * R);
+    }
     sp.inv_n = float(1.0 / double(g.n));
     const double two_pi = 6.28318530717958647692;
     const float kfx = float(two_pi / (g.nx * g.hx)), kfy = float(two_pi / (g.ny * g.hy)),
@@ -168,7 +175,8 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     if (e == cudaSuccess)
         e = Passes<float>::zconv_fwd(st, g, az, sp, Tz, kfx, kfy, kfz, 0, base + o_spec, base + o_n, base + o_es,
                                      nullptr, base + o_twz, status);
-    if (e == cudaSuccess) e = Passes<float>::yfft(st, true, g, ay, Ty, DFT_NSPEC, base + o_n, status, base + o_twy);
+    if (e == cudaSuccess)
+        e = Passes<float>::yfft(st, true, g, ay, Ty, 1, base + o_n, status, base + o_twy, DFT_WAIT_POLLS, COL_DERIV, kfy);
     if (e == cudaSuccess)
         e = Passes<float>::xinv(st, g, ax, LR, DFT_NCOMP, base + o_n, static_cast<float*>(n_out), nullptr, off, -1,
                                 nullptr, 1, kfx, base + o_twx);

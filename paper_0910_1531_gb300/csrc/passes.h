@@ -36,6 +36,12 @@ template <typename Real> __host__ __device__ constexpr int dft_tile_z(int n) {
     return (t >> DFT_TILE_ZG_SHIFT) > 0 ? (t >> DFT_TILE_ZG_SHIFT) : 1;
 }
 
+// The z stages that run as three passes (z transform, k-space products, z transform): run-time
+// lengths, and FP64, where the one-pass kernels' narrow tiles (one or two columns at 128) leave lanes
+// of the FP64 pipe's warps idle: three species, FP64, one line-search iteration at 128^3 12.2 ms with
+// the one-pass kernels, 11.4 with three passes (two species at 64^3 1407 -> 1323 us, 32^3 263 -> 253).
+template <typename Real> __host__ __device__ constexpr bool dft_zsplit(int n) { return n == 0 || sizeof(Real) == 8; }
+
 // Persistent TMA z passes: half the grouped width (at least 16 bytes of a row, the TMA
 // minimum).
 template <typename Real> __host__ __device__ constexpr int dft_tile_zb(int n) {
@@ -60,10 +66,11 @@ template <typename Real> inline int dft_col_elems(int n, int T) {
     const int e = (n <= 256 ? 1 : 2) * dft_col_box_rows(n) * T, q = 128 / int(2 * sizeof(Real));
     return (e + q - 1) / q * q;
 }
-// Shared memory of k_colfft: two TMA stages, X and (from two radix stages) Y, twiddles, mbarriers.
+// Shared memory of k_colfft: two TMA stages, X and (from two radix stages) Y, twiddles, wave
+// numbers, mbarriers.
 template <typename Real> inline size_t dft_col_smem(int n, int T, int nstages) {
-    return (size_t(nstages > 1 ? 4 : 3) * dft_col_elems<Real>(n, T) + ((n + 1) & ~1)) * 2 * sizeof(Real) +
-           2 * sizeof(uint64_t) + 128;
+    return (size_t(nstages > 1 ? 4 : 3) * dft_col_elems<Real>(n, T) + n) * 2 * sizeof(Real) +
+           ((n + 1) & ~1) * sizeof(Real) + 2 * sizeof(uint64_t) + 128;
 }
 // Tile width of a run-time column transform (128-, 64- or 32-byte rows in FP32, 128 or 64 in
 // FP64): of the widths that leave two blocks on an SM, the one with the least work per column in
@@ -81,12 +88,20 @@ template <typename Real> inline int dft_tile_rt(int n, int nxh) {
     return best;
 }
 
+// Resident CTAs per SM that the compile-time column pass's register budget is sized for: what its
+// shared memory allows (at 256 one), and no more than its radices' registers (FP64 radix 16: two).
+template <typename Real> __host__ __device__ constexpr int dft_yfft_minb(int n) {
+    if (n >= 256) return 1;
+    if (sizeof(Real) == 4) return n >= 128 ? 3 : 4;
+    return n >= 96 ? 2 : 3;
+}
+
 // Threads of the persistent TMA z passes and the resident CTAs per SM their register budget
 // is sized for.  First half: 256 threads, two CTAs per SM, up to length 128; 512 threads, one
 // CTA, at 256.  Second half: 256 threads, three CTAs per SM (FP32; two in FP64, whose
-// butterflies need twice the registers), up to 128; 288 threads (nine warps: one pass of the
-// threads covers the radix-16 butterflies of the nine Phi' groups of a two-column tile), two
-// CTAs per SM, at 256 (its shared memory allows no more).  DFT_ZFWD_THREADS / DFT_ZFWD_MINB / DFT_ZBWD_THREADS / DFT_ZBWD_MINB (build
+// butterflies need twice the registers), up to 128; 256 threads (one pass of them covers the
+// radix-16 butterflies of the seven Phi' groups of a two-column tile), two CTAs per SM, at 256 (its
+// shared memory allows no more).  DFT_ZFWD_THREADS / DFT_ZFWD_MINB / DFT_ZBWD_THREADS / DFT_ZBWD_MINB (build
 // flags) override.
 template <typename Real> __host__ __device__ constexpr int dft_zfwd_threads(int n) {
 #ifdef DFT_ZFWD_THREADS
@@ -108,14 +123,14 @@ template <typename Real> __host__ __device__ constexpr int dft_zfwd_minb_s3(int 
 #ifdef DFT_ZFWD_MINB_S3
     return DFT_ZFWD_MINB_S3;
 #else
-    return dft_zfwd_minb<Real>(n);
+    return n < 256 ? 3 : dft_zfwd_minb<Real>(n);
 #endif
 }
 template <typename Real> __host__ __device__ constexpr int dft_zbwd_threads(int n) {
 #ifdef DFT_ZBWD_THREADS
     return DFT_ZBWD_THREADS;
 #else
-    return n >= 256 ? 288 : 256;
+    return 256;
 #endif
 }
 template <typename Real> __host__ __device__ constexpr int dft_zbwd_minb(int n) {
@@ -164,7 +179,7 @@ struct LaunchY {
     using C = typename Cplx<Real>::type;
     static cudaError_t init();
     static cudaError_t yfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& py, int T, int ncomp, C* data,
-                     int* status, const C* tw, long long polls);
+                            int* status, const C* tw, long long polls, int mode, Real kfy);
 };
 
 template <typename Real, int N>
@@ -182,17 +197,18 @@ struct LaunchZ {
                                       const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
     static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                            const C* tw, long long polls);
+                            const C* tw, long long polls, int mode);
 };
 
 // Column transform of a run-time length in place (k_colfft; colfft.cu): along z (zax) or y, tiles of
-// T columns (16, 8, 4; FP64 8, 4).
+// T columns (16, 8, 4; FP64 8, 4).  mode: COL_*; ncomp counts components, or with the modes of sets
+// the sets of nine; kf: the axis's wave number unit (COL_DERIV, COL_FOLD).
 template <typename Real>
 struct ColFft {
     using C = typename Cplx<Real>::type;
     static cudaError_t init();
     static cudaError_t run(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pa, bool zax, int T, int ncomp,
-                           C* data, int* status, const C* tw, long long polls);
+                           C* data, int* status, const C* tw, long long polls, int mode, Real kf);
 };
 
 template <typename Real>
@@ -207,9 +223,11 @@ struct Passes {
 
     static cudaError_t xfwd(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int ncomp, int lx, const Real* in,
                      C* out, const C* tw);
-    // polls: bound of each TMA tile wait (DFT_WAIT_POLLS; the drains after a give-up keep it)
+    // polls: bound of each TMA tile wait (DFT_WAIT_POLLS; the drains after a give-up keep it);
+    // mode COL_PLAIN: ncomp components in place; COL_DERIV (inverse) / COL_FOLD (forward): ncomp sets
+    // of the nine weighted-density / Phi' spectra, with the y derivatives formed / added
     static cudaError_t yfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& py, int T, int ncomp, C* data,
-                     int* status, const C* tw, long long polls = DFT_WAIT_POLLS);
+                     int* status, const C* tw, long long polls = DFT_WAIT_POLLS, int mode = COL_PLAIN, Real kfy = 0);
     static cudaError_t zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
                           Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
                           double* red_energy, const C* tw, int* status);
@@ -228,11 +246,12 @@ struct Passes {
                                       const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
     // The split first-half z stage (compile-time lengths): zfft = the persistent TMA z transform
-    // of ncomp components in place (tiles of the y pass's width; cudaErrorNotSupported for other
-    // lengths), zmul = the k-space products from the S species spectra into the nine
-    // weighted-density spectra (slot_n, 1/N applied) and the S ES spectra (slot_es).
+    // of ncomp components (COL_WD: of the seven of ncomp sets of nine) in place (tiles of the y
+    // pass's width; cudaErrorNotSupported for other lengths), zmul = the k-space products from the
+    // S species spectra into seven weighted-density spectra (slot_n, 1/N applied) and the S ES
+    // spectra (slot_es).
     static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                            const C* tw, long long polls);
+                            const C* tw, long long polls, int mode = COL_PLAIN);
     static cudaError_t zmul(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
                             Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, double* red_energy);
     // the second half's products between its z transforms (run-time lengths): one sample or two
