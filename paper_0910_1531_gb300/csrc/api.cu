@@ -1365,7 +1365,7 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     if (f64) fill_species<double>(p);
     else fill_species<float>(p);
 
-    cudaError_t e = f64 ? Passes<double>::init_attributes() : Passes<float>::init_attributes();
+    cudaError_t e = f64 ? Passes<double>::init_attributes(&g) : Passes<float>::init_attributes(&g);
     if (e != cudaSuccess) {
         delete p;
         return fail(nullptr, DFT_ECUDA, std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e));

@@ -14,7 +14,10 @@ cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool 
     cb.n = pa.n;
     cb.nbox = pa.n <= 256 ? 1 : 2;
     cb.rows = dft_col_box_rows(pa.n);
-    cb.elems = dft_col_elems<Real>(pa.n, T);
+    const int ntx = (int)ceil_div(g.nxh, T), across = zax ? g.ny : g.nz;
+    const int items = mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC;
+    cb.planes = dft_col_planes<Real>(pa.n, g.nxh, T, across, items, sm_count());
+    cb.elems = dft_col_elems<Real>(pa.n, T, cb.planes);
     CUtensorMap map;
     const unsigned long long dims[4] = {(unsigned long long)g.nxh * E, (unsigned long long)g.ny,
                                         (unsigned long long)g.nz,
@@ -22,12 +25,13 @@ cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool 
     const unsigned long long strides[3] = {(unsigned long long)g.pxh * sizeof(C),
                                            (unsigned long long)g.ny * g.pxh * sizeof(C),
                                            (unsigned long long)g.nc * sizeof(C)};
-    const unsigned box[4] = {unsigned(T * E), zax ? 1u : unsigned(cb.rows), zax ? unsigned(cb.rows) : 1u, 1u};
+    const unsigned pl = unsigned(cb.planes), rows = unsigned(cb.rows);
+    const unsigned box[4] = {unsigned(T * E), zax ? pl : rows, zax ? rows : pl, 1u};
     cudaError_t e = tma_encode_4d(&map, data, dims, strides, box);
     if (e != cudaSuccess) return e;
-    const int ntx = (int)ceil_div(g.nxh, T), other = zax ? g.ny : g.nz;
-    const int ntiles = ntx * other * (mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC);
-    const size_t sm = dft_col_smem<Real>(pa.n, T, pa.nstages);
+    const int other = (int)ceil_div(across, cb.planes);
+    const int ntiles = ntx * other * items;
+    const size_t sm = dft_col_smem<Real>(pa.n, T, pa.nstages, cb.planes);
     auto kern = dftk::k_colfft<Real, INV, T, BIG, MODE>;
     const int fit = resident_blocks(kern, dftk::kThreads, sm);
     return launch_k(kern, ntiles < fit ? ntiles : fit, dftk::kThreads, sm, st, g.pdl, map, pa, cb, zax ? 1 : 0, ntx,
@@ -74,8 +78,7 @@ template <typename Real, int T> cudaError_t init_t() {
 template <typename Real>
 cudaError_t ColFft<Real>::init() {
     cudaError_t e = init_t<Real, 8>(), r = init_t<Real, 4>();
-    if constexpr (sizeof(Real) == 4)
-        if (r == cudaSuccess) r = init_t<Real, 16>();
+    if (r == cudaSuccess) r = init_t<Real, sizeof(Real) == 4 ? 16 : 2>();
     return e != cudaSuccess ? e : r;
 }
 
@@ -84,6 +87,10 @@ cudaError_t ColFft<Real>::run(cudaStream_t st, bool inv, const GridDesc& g, cons
                               int ncomp, C* data, int* status, const C* tw, long long polls, int mode, Real kf) {
     if constexpr (sizeof(Real) == 4)
         if (T >= 16) return launch_t<Real, 16>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
+    // FP64: half-width tiles where four columns would leave SMs without a tile (4 x 4 x 512, three columns)
+    if constexpr (sizeof(Real) == 8)
+        if (T == 4 && ceil_div(g.nxh, 4) * (zax ? g.ny : g.nz) * ncomp * (mode == COL_PLAIN ? 1 : DFT_NZSPEC) < sm_count())
+            return launch_t<Real, 2>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
     return T >= 8 ? launch_t<Real, 8>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf)
                   : launch_t<Real, 4>(st, inv, g, pa, zax, ncomp, data, status, tw, polls, mode, kf);
 }

@@ -65,6 +65,7 @@ struct AxisPlan {
     int m[DFT_MAXSTAGES];
     int tws[DFT_MAXSTAGES];
     FastDiv ns[DFT_MAXSTAGES];
+    FastDiv dm[DFT_MAXSTAGES];      // division by m
 };
 
 // Fill the per-stage constants from n and the radices.
@@ -74,6 +75,7 @@ inline void dft_finish_plan(AxisPlan* p) {
         p->m[s] = p->n / p->radix[s];
         p->tws[s] = p->n / (ns * p->radix[s]);
         p->ns[s] = FastDiv(ns);
+        p->dm[s] = FastDiv(p->m[s]);
         ns *= p->radix[s];
     }
 }

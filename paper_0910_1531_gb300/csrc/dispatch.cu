@@ -35,16 +35,19 @@ extern template struct LaunchX<double, -1>;
     default: return LaunchZ<Real, 0>::call; }
 
 template <typename Real>
-cudaError_t Passes<Real>::init_attributes() {
+cudaError_t Passes<Real>::init_attributes(const GridDesc* g) {
     cudaError_t e = cudaSuccess, r;
 #define DFT_INIT(N) \
-    if ((r = LaunchX<Real, N>::init()) != cudaSuccess) e = r; \
-    if ((r = LaunchY<Real, N>::init()) != cudaSuccess) e = r; \
-    if ((r = LaunchZ<Real, N>::init()) != cudaSuccess) e = r;
+    if ((!g || g->nx == N) && (r = LaunchX<Real, N>::init()) != cudaSuccess) e = r; \
+    if ((!g || g->ny == N) && (r = LaunchY<Real, N>::init()) != cudaSuccess) e = r; \
+    if ((!g || g->nz == N) && (r = LaunchZ<Real, N>::init()) != cudaSuccess) e = r;
     DFT_CT_SIZES(DFT_INIT)
-    DFT_INIT(0)
-    if ((r = LaunchX<Real, -1>::init()) != cudaSuccess) e = r;
 #undef DFT_INIT
+    // the run-time kernels: any length may be pinned to them
+    const bool big = g && dft_has_big_prime(g->nx);
+    if (!big && (r = LaunchX<Real, 0>::init()) != cudaSuccess) e = r;
+    if ((!g || big) && (r = LaunchX<Real, -1>::init()) != cudaSuccess) e = r;
+    if ((r = ColFft<Real>::init()) != cudaSuccess) e = r;
     return e;
 }
 

@@ -241,34 +241,55 @@ struct PostStore {
 };
 
 // ------------------------------------------------------------------------------------
-// Run-time transforms: the Stockham stages of an AxisPlan.  Lines are the columns of a tile T
-// wide (T > 0: element e of line t at e T + t, a thread keeps its column), or rows (T == 0:
-// element e of line l at e + l ls, ls odd, line index fastest across threads, so that the
-// butterflies of a half-warp fall into distinct banks).  NT: threads of the block.
-// Divisions by run-time constants are multiplications (FastDiv).
+// Run-time transforms: the Stockham stages of an AxisPlan.  NT: threads of the block.  Divisions by
+// run-time constants are multiplications (FastDiv).  Lines are the rows of RtRows or the columns of
+// RtCols; either maps a task (one butterfly of one line) to the butterfly j and the shared-memory
+// offset of the line's element 0, and gives the distance between its elements.
 // ------------------------------------------------------------------------------------
-template <int T> __device__ __forceinline__ void rt_split(int task, int lines, const FastDiv& dl, int& line, int& j) {
-    if constexpr (T > 0) {
-        line = task % T;
-        j = task / T;
-    } else {
+// `lines` rows: element e of line l at e + l ls, ls odd; line index fastest across threads, so that
+// the butterflies of a half-warp fall into distinct banks.
+struct RtRows {
+    int lines, ls;
+    FastDiv dl;
+    __device__ __forceinline__ RtRows(int n, int pitch) : lines(n), ls(pitch), dl(n) {}
+    __device__ __forceinline__ int count() const { return lines; }
+    __device__ __forceinline__ int stride() const { return 1; }
+    __device__ __forceinline__ void split(int task, const AxisPlan&, int, int& j, int& off) const {
         j = dl.div(task);
-        line = task - j * lines;
+        off = (task - j * lines) * ls;
     }
-}
+};
+// Tiles of T columns by P planes of the other axis.  Along y the planes follow one another (element
+// e of column t of plane p at (p n + e) T + t), along z they are interleaved ((e P + p) T + t): the
+// orders in which a TMA box lands.  Threads run over t, then over what is contiguous next.
+template <int T> struct RtCols {
+    int P, es, ps;
+    bool zax;
+    FastDiv dp;
+    __device__ __forceinline__ RtCols(int planes, int n, bool z)
+        : P(planes), es(z ? planes * T : T), ps(z ? T : n * T), zax(z), dp(planes) {}
+    __device__ __forceinline__ int count() const { return P * T; }
+    __device__ __forceinline__ int stride() const { return es; }
+    __device__ __forceinline__ void split(int task, const AxisPlan& a, int s, int& j, int& off) const {
+        const int t = task % T, rest = task / T;
+        int p = 0;
+        if (P == 1) j = rest;
+        else if (zax) { j = dp.div(rest); p = rest - j * P; }
+        else { p = a.dm[s].div(rest); j = rest - p * a.m[s]; }
+        off = p * ps + t;
+    }
+};
 
-template <int R, bool INV, int T, int NT, typename Pre, typename Post, typename C>
+template <int R, bool INV, int NT, typename L, typename Pre, typename Post, typename C>
 __device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
-                                         int lines, const FastDiv& dl, int ls, const C* __restrict__ tw, Pre pre,
-                                         Post post) {
-    constexpr int ES = T > 0 ? T : 1;
+                                         const L& lines, const C* __restrict__ tw, Pre pre, Post post) {
+    const int ES = lines.stride();
     const int m = p.m[s], ns = p.ns[s].d, tws = p.tws[s];
     const FastDiv dns = p.ns[s];
-    const int total = m * (T > 0 ? T : lines);
+    const int total = m * lines.count();
     for (int task = threadIdx.x; task < total; task += NT) {
-        int line, j;
-        rt_split<T>(task, lines, dl, line, j);
-        const int off = T > 0 ? line : line * ls;
+        int j, off;
+        lines.split(task, p, s, j, off);
         const int q = dns.div(j), k = j - q * ns;
         const C* s0 = src + off + j * ES;
         C v[R];
@@ -296,22 +317,20 @@ __device__ __forceinline__ void rt_stage(const C* __restrict__ src, C* __restric
 // Stage of a prime radix R >= 11 (the pairs of dft_odd), its outputs spread over threads: a thread
 // forms X_q and X_(R-q) of QG consecutive q of one butterfly (and X_0 with the first ones).  The
 // roots W_R^(r q) = tw[(r q mod R) m] are the same for a whole butterfly and mostly for a warp.
-template <int R, bool INV, int T, int NT, typename Pre, typename Post, typename C>
+template <int R, bool INV, int NT, typename L, typename Pre, typename Post, typename C>
 __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __restrict__ dst, const AxisPlan& p, int s,
-                                            int lines, const FastDiv& dl, int ls, const C* __restrict__ tw, Pre pre,
-                                            Post post) {
+                                            const L& lines, const C* __restrict__ tw, Pre pre, Post post) {
     using F = decltype(C().x);
-    constexpr int ES = T > 0 ? T : 1;
+    const int ES = lines.stride();
     constexpr int H = (R - 1) / 2, QG = 4, NG = (H + QG - 1) / QG;
     const int m = p.m[s], ns = p.ns[s].d, tws = p.tws[s];
     const FastDiv dns = p.ns[s];
-    const int per = m * (T > 0 ? T : lines);
+    const int per = m * lines.count();
     for (int task = threadIdx.x; task < per * NG; task += NT) {
         int grp = 0, rem = task;
         while (rem >= per) { rem -= per; ++grp; }
-        int line, j;
-        rt_split<T>(rem, lines, dl, line, j);
-        const int off = T > 0 ? line : line * ls;
+        int j, off;
+        lines.split(rem, p, s, j, off);
         const int q = dns.div(j), k = j - q * ns;
         const C* s0 = src + off + j * ES;
         C v0 = s0[0];
@@ -357,12 +376,11 @@ __device__ __noinline__ void rt_stage_prime(const C* __restrict__ src, C* __rest
 
 // Stage s of a plan.  BIG: lengths with a prime factor of 17..31 (kernels of their own, whose
 // register budget the other lengths do not pay).
-template <bool INV, int T, int NT, bool BIG, typename Pre = PreNone, typename Post = PostStore, typename C>
-__device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPlan& p, int s, int lines,
-                                             const FastDiv& dl, int ls, const C* tw, Pre pre = Pre{},
-                                             Post post = Post{}) {
-#define DFT_RT(R) case R: rt_stage<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw, pre, post); break;
-#define DFT_RTP(R) case R: rt_stage_prime<R, INV, T, NT>(src, dst, p, s, lines, dl, ls, tw, pre, post); break;
+template <bool INV, int NT, bool BIG, typename L, typename Pre = PreNone, typename Post = PostStore, typename C>
+__device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPlan& p, int s, const L& lines,
+                                             const C* tw, Pre pre = Pre{}, Post post = Post{}) {
+#define DFT_RT(R) case R: rt_stage<R, INV, NT>(src, dst, p, s, lines, tw, pre, post); break;
+#define DFT_RTP(R) case R: rt_stage_prime<R, INV, NT>(src, dst, p, s, lines, tw, pre, post); break;
     switch (p.radix[s]) {
         DFT_RT(2) DFT_RT(3) DFT_RT(4) DFT_RT(5) DFT_RT(6) DFT_RT(7) DFT_RT(8) DFT_RT(9) DFT_RT(10) DFT_RT(12)
         DFT_RT(14) DFT_RT(15) DFT_RT(16)
@@ -381,9 +399,9 @@ __device__ __forceinline__ void rt_stage_any(const C* src, C* dst, const AxisPla
 // the result; all threads see it on return.
 template <bool INV, bool BIG, int NT, typename C>
 __device__ C* rt_fft_rows(C* a, C* b, const AxisPlan& p, int lines, int ls, const C* tw) {
-    const FastDiv dl(lines);
+    const RtRows rows(lines, ls);
     for (int s = 0; s < p.nstages; ++s) {
-        rt_stage_any<INV, 0, NT, BIG>(a, b, p, s, lines, dl, ls, tw);
+        rt_stage_any<INV, NT, BIG>(a, b, p, s, rows, tw);
         __syncthreads();
         C* t = a; a = b; b = t;
     }

@@ -201,7 +201,7 @@ __device__ __forceinline__ float block_max(float v, float* scratch) {
 
 // The x passes are compiled for a length NX > 0 or for any length: NX = 0, and NX = -1 for lengths
 // with a prime factor of 17..31.  Position of element e within a row (padded in the compile-time
-// passes, see ct_xpad) and row pitch (odd in the run-time ones, see rt_split).
+// passes, see ct_xpad) and row pitch (odd in the run-time ones, see RtRows).
 template <int NX> __device__ __forceinline__ int xo(int e) { return NX > 0 ? ct_xpad(e) : e; }
 template <int NX> __host__ __device__ __forceinline__ int x_pitch(int nx) { return NX > 0 ? ct_row_pitch(NX) : nx | 1; }
 
@@ -469,8 +469,8 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
 // Column transform of a run-time length along y or z, in place, of every component: the
 // persistent TMA pipeline of k_yfft_tma with the stages of an AxisPlan.  The tensor map views the
 // half spectra as (x: nxh E, y, z, component) 8-byte elements; a tile is T kx columns of the whole
-// axis at one index of the other axis (`other` of them) of one component, moved as nbox boxes of
-// boxrows rows (a box has at most 256; rows past the axis read as zero and are not written).
+// axis at `planes` indices of the other axis (`other` such groups; indices past the axis read as
+// zero and are not written) of one component, moved as one box, or, past 256 rows, two.
 // Memory-bound in FP32: at 160^3 8.9 us a component (3.8 TB/s; a column pass of plain tile loads,
 // divisions by run-time integers and odd primes by their R^2 terms took 44).  FP64 is bound by the
 // FP64 pipe: 21 x 21 x 161, z forward, nine components 75 us.
@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
 // ------------------------------------------------------------------------------------
 struct ColBox {
     int n, nbox, rows;      // axis length; boxes of a tile and rows of a box
-    int elems;              // shared-memory elements of one tile buffer (nbox boxes, 128-byte multiple)
+    int planes;             // planes of the other axis in a tile (1 with two boxes)
+    int elems;              // shared-memory elements of one tile buffer (128-byte multiple)
 };
 
 template <typename Real, bool INV, int T, bool BIG, int MODE>
@@ -500,8 +501,8 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 
     C* const tw = pa.nstages > 1 ? Y + cb.elems : Y;
     Real* const kt = reinterpret_cast<Real*>(tw + cb.n);
     uint64_t* const bar = reinterpret_cast<uint64_t*>(kt + ((cb.n + 1) & ~1));
-    const uint32_t bytes = uint32_t(cb.nbox) * uint32_t(cb.rows) * uint32_t(T * sizeof(C));
-    const FastDiv one(1);
+    const uint32_t bytes = uint32_t(cb.nbox) * uint32_t(cb.rows * cb.planes) * uint32_t(T * sizeof(C));
+    const RtCols<T> cols(cb.planes, cb.n, zax != 0);
     const bool sets = MODE != COL_PLAIN || wd;
     const int nst = pa.nstages;     // 1 to 3
     if (threadIdx.x == 0) {
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 
         if (load.tile >= ntiles) return;
         const ColItem t(load.tile, per, sets);
         const int c = (load.sub == 0 && load.dual(per)) ? t.partner() : t.comp(sets);
-        const int x = load.tile % ntiles_x, o = load.tile / ntiles_x % other;
+        const int x = load.tile % ntiles_x, o = load.tile / ntiles_x % other * cb.planes;
         tma::mbar_expect_tx(&bar[s], bytes);
         for (int b = 0; b < cb.nbox; ++b)
             tma::load_4d(stage0 + s * cb.elems + b * cb.rows * T, &map, x * T * E, zax ? o : b * cb.rows,
@@ -564,11 +565,11 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 
             for (int s = 0; s < nst; ++s) {
                 C* const dst = s == nst - 1 ? res : (spare ? (s == 0 ? Y : st) : (s == 0 ? X : Y));
                 if (MODE == COL_DERIV && s == 0 && pass == 0)
-                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw, PreDeriv<Real>{kt});
+                    rt_stage_any<INV, kThreads, BIG>(src, dst, pa, s, cols, tw, PreDeriv<Real>{kt});
                 else if (MODE == COL_FOLD && add && s == nst - 1)
-                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw, PreNone{}, PostFold<Real>{kt});
+                    rt_stage_any<INV, kThreads, BIG>(src, dst, pa, s, cols, tw, PreNone{}, PostFold<Real>{kt});
                 else
-                    rt_stage_any<INV, T, kThreads, BIG>(src, dst, pa, s, T, one, 1, tw);
+                    rt_stage_any<INV, kThreads, BIG>(src, dst, pa, s, cols, tw);
                 if (s == nst - 1) tma::fence_proxy_async();
                 __syncthreads();
                 // the stage is free: refill it
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 
             }
             if (threadIdx.x == 0 && !hold) {
                 const int c = (MODE == COL_DERIV && pass == 0) ? t.partner() : t.comp(sets);
-                const int x = at.tile % ntiles_x, o = at.tile / ntiles_x % other;
+                const int x = at.tile % ntiles_x, o = at.tile / ntiles_x % other * cb.planes;
                 for (int q = 0; q < cb.nbox; ++q)
                     tma::store_4d(&map, x * T * E, zax ? o : q * cb.rows, zax ? q * cb.rows : o, c,
                                   res + q * cb.rows * T);

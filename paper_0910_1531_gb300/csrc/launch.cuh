@@ -17,6 +17,14 @@ template <typename K> cudaError_t set_max_smem(K kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
+// SMs of the current device.
+inline int sm_count() {
+    int dev = 0, n = 1;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+    return n;
+}
+
 // Blocks of a persistent kernel that fit on the GPU at once (at least one per SM).  The answers for
 // the kernels a thread launched last are kept: a plan launches few kernels, each with one
 // shared-memory size, many times.

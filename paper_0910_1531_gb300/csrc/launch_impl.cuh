@@ -188,9 +188,8 @@ cudaError_t LaunchY<Real, N>::init() {
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, false, N, TY, false, COL_FOLD>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_yfft_tma<Real, true, N, TY, false, COL_DERIV>)) != cudaSuccess) e = r;
-    } else {
-        if ((r = ColFft<Real>::init()) != cudaSuccess) e = r;
     }
+    (void)r;
     return e;
 }
 

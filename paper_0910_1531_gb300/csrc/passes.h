@@ -62,18 +62,17 @@ template <typename Real> __host__ __device__ constexpr int dft_tile_zf(int n) {
 // 256 rows (a second one starts at a multiple of four rows, so that every box lands on a 128-byte
 // boundary), rounded up to 128 bytes.
 inline int dft_col_box_rows(int n) { return n <= 256 ? n : ((n + 1) / 2 + 3) & ~3; }
-template <typename Real> inline int dft_col_elems(int n, int T) {
-    const int e = (n <= 256 ? 1 : 2) * dft_col_box_rows(n) * T, q = 128 / int(2 * sizeof(Real));
+template <typename Real> inline int dft_col_elems(int n, int T, int planes = 1) {
+    const int e = (n <= 256 ? 1 : 2) * dft_col_box_rows(n) * T * planes, q = 128 / int(2 * sizeof(Real));
     return (e + q - 1) / q * q;
 }
 // Shared memory of k_colfft: two TMA stages, X and (from two radix stages) Y, twiddles, wave
 // numbers, mbarriers.
-template <typename Real> inline size_t dft_col_smem(int n, int T, int nstages) {
-    return (size_t(nstages > 1 ? 4 : 3) * dft_col_elems<Real>(n, T) + n) * 2 * sizeof(Real) +
+template <typename Real> inline size_t dft_col_smem(int n, int T, int nstages, int planes = 1) {
+    return (size_t(nstages > 1 ? 4 : 3) * dft_col_elems<Real>(n, T, planes) + n) * 2 * sizeof(Real) +
            ((n + 1) & ~1) * sizeof(Real) + 2 * sizeof(uint64_t) + 128;
 }
-// Tile width of a run-time column transform (128-, 64- or 32-byte rows in FP32, 128 or 64 in
-// FP64): of the widths that leave two blocks on an SM, the one with the least work per column in
+// Tile width of a run-time column transform (128-, 64- or 32-byte rows): of the widths that leave two blocks on an SM, the one with the least work per column in
 // use, where a narrower tile's shorter rows and fewer butterflies per block count as 2 / T columns
 // (FP64, bound by its arithmetic: 1 / T) and columns past nxh as work.
 template <typename Real> inline int dft_tile_rt(int n, int nxh) {
@@ -94,6 +93,20 @@ template <typename Real> __host__ __device__ constexpr int dft_yfft_minb(int n) 
     if (n >= 256) return 1;
     if (sizeof(Real) == 4) return n >= 128 ? 3 : 4;
     return n >= 96 ? 2 : 3;
+}
+
+// Planes of the other axis (`other` of them) in a tile of a run-time column transform of `items`
+// components: as many as a buffer of 2048 elements (FP64 1024) takes, while four tiles per SM remain, so
+// that short axes do not pay a tile's latency (a few us) for some hundred elements.  One plane against this:
+// 21 x 21 x 161, FP64, S = 2, a y forward pass 69 -> 37 us, an iteration 979 -> 752; 4 x 4 x 512, FP64, a y
+// pass 19 -> 13; 100^3 FP32 an iteration 644 -> 537.
+template <typename Real> inline int dft_col_planes(int n, int nxh, int T, int other, int items, int sms) {
+    if (n > 256) return 1;
+    const int most = (sizeof(Real) == 4 ? 2048 : 1024) / (n * T);
+    const long long tiles = (long long)((nxh + T - 1) / T) * other * items;
+    const long long spread = tiles / (4LL * sms);
+    const long long p = spread < most ? spread : most;
+    return p < 1 ? 1 : (p > 256 ? 256 : (int)p);
 }
 
 // Threads of the persistent TMA z passes and the resident CTAs per SM their register budget
@@ -214,7 +227,8 @@ struct ColFft {
 template <typename Real>
 struct Passes {
     using C = typename Cplx<Real>::type;
-    static cudaError_t init_attributes();
+    // allow the kernels of a grid's lengths (nullptr: of every length) their shared memory
+    static cudaError_t init_attributes(const GridDesc* g = nullptr);
     // dynamic shared memory of an x pass with `lines` lines
     static size_t smem_x(int nx, int lines) { return (size_t(nx) + 2 * size_t(lines) * (nx + 1)) * sizeof(C) + 16; }
     // column tile widths of the y and z passes

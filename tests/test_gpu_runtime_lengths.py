@@ -4,7 +4,8 @@ the weighted densities against the oracle at the lengths where they can go wrong
 Lengths: one radix stage (4, 14, 15), every composite radix and prime stage (11..31; two of them in
 one length, so that the second takes twiddles), three stages (343 = 7^3), 256 rows (one TMA box) and
 more (two boxes, of an odd length the second partly past the axis), column counts that leave a tile
-partly empty.  FP32 is held to 1e-5 and FP64 to 1e-10 per field, the library's stated bounds
+partly empty, short axes whose tiles take several planes (133 of them, the last tile partly past the
+end).  FP32 is held to 1e-5 and FP64 to 1e-10 per field, the library's stated bounds
 (about 30 transform passes of log2(N) roundings each are 4e-7 in FP32).
 """
 import numpy as np
@@ -35,7 +36,7 @@ def relerr(a, b):
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("shape", [
     (4, 5, 6), (14, 15, 16), (9, 10, 4), (7, 512, 6), (261, 6, 8), (323, 8, 4), (6, 343, 5), (289, 4, 34), (22, 26, 12),
-    (38, 46, 10), (58, 62, 36), (256, 20, 6), (12, 275, 8), (160, 9, 33), (100, 36, 70), (17, 23, 130)])
+    (38, 46, 10), (58, 62, 36), (256, 20, 6), (12, 275, 8), (160, 9, 33), (100, 36, 70), (17, 23, 130), (10, 133, 100), (133, 10, 60)])
 def test_runtime_lengths_match_the_oracle(shape, precision):
     from paper_0910_1531_gb300 import binding
     prob = F.Problem(shape, (0.11, 0.1, 0.09), *SPECIES)
