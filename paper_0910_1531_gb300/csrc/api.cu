@@ -475,11 +475,9 @@ dft_status read_ctl(dft_plan* p) {
     return DFT_OK;
 }
 
+// The control blocks at the start of an evaluation (before the passes that may record a status).
 dft_status reset_status(dft_plan* p) {
-    // the iteration's status word and those of the two samples' blocks
-    cudaError_t e = cudaSuccess;
-    for (int m = 0; m < 3 && e == cudaSuccess; ++m) e = cudaMemsetAsync(&p->ctl[m].status, 0, sizeof(int), p->stream);
-    if (e != cudaSuccess) return fail(p, DFT_ECUDA, std::string("memset: ") + cudaGetErrorString(e));
+    LAUNCH(p, K_FIN, 0.0, launch_ctl_reset(p->stream, p->ctl, p->g.pdl));
     return DFT_OK;
 }
 
@@ -492,7 +490,6 @@ template <typename Real> dft_status iter_begin_t(dft_plan* p, Real* rho, const R
     if (p->rho_lo && cudaMemsetAsync(p->rho_lo, 0, size_t(p->S) * p->g.n * sizeof(Real), p->stream) != cudaSuccess)
         return fail(p, DFT_ECUDA, "memset of the iterate's low part");
     TRY(O::first_half(p, rho, p->slotA, 0));
-    TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     if (v_ready && cudaStreamWaitEvent(p->stream, v_ready, 0) != cudaSuccess)
         return fail(p, DFT_ECUDA, "stream wait");
     TRY(O::second_half(p, false, false, rho, nullptr, V, nullptr, static_cast<Real*>(p->gbuf), nullptr,
@@ -551,7 +548,6 @@ template <typename Real> dft_status c1_hs_t(dft_plan* p, const Real* rho, Real* 
     using P = Passes<Real>;
     const SpeciesDesc<Real>& sp = species<Real>(p);
     TRY(O::first_half(p, rho, p->slotA, 0));
-    TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     LAUNCH(p, K_XPHI, 2.0 * DFT_NSPEC * CB(p), P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, O::slot_n(p->slotA), nullptr, nullptr,
                               O::T1(p), p->red_max, &p->ctl->status, nullptr, O::kf(p, 0), O::tw(p, 0)));
     TRY(O::yfold(p, 1));
@@ -569,7 +565,6 @@ template <typename Real> dft_status c1_es_t(dft_plan* p, const Real* rho, Real* 
     const int want_psi = psi ? 1 : 0;
     const int nout = p->S + want_psi;
     TRY(O::first_half(p, rho, p->slotA, want_psi));
-    TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     LAUNCH(p, K_ZBWD, 2.0 * nout * CB(p), P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 2, nout,
                                    p->ctl, O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
     LAUNCH(p, K_YFFT, 2.0 * (nout) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, nout, O::T1(p), &p->ctl->status, O::tw(p, 1), p->wait_polls));
@@ -583,7 +578,6 @@ template <typename Real> dft_status picard_map_t(dft_plan* p, const Real* rho, c
     using O = Ops<Real>;
     TRY(reset_status(p));
     TRY(O::first_half(p, rho, p->slotA, 0));
-    TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     TRY(O::second_half(p, false, false, rho, nullptr, V, nullptr, g));
     TRY(finalize(p, FIN_F0 | FIN_N3CUR, (int)p->blocks_x(p->LRupd), (int)p->blocks_x(p->LRphi), -1.0));
     return DFT_OK;
@@ -676,7 +670,6 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
     const double dv = p->g.hx * p->g.hy * p->g.hz;
     TRY(reset_status(p));
     TRY(O::first_half(p, rho, p->slotA, 0, r_energy));
-    TRY(finalize(p, FIN_IDENTITY, 0, 0, -1.0));
     LAUNCH(p, K_XPHI, 2.0 * DFT_NSPEC * CB(p), P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, O::slot_n(p->slotA),
                                                         nullptr, nullptr, O::T1(p), p->red_max, &p->ctl->status,
                                                         r_phi, O::kf(p, 0), O::tw(p, 0)));
@@ -1573,6 +1566,7 @@ dft_status dft_c1_es(dft_plan* p, const void* rho, void* c1_out, void* psi_out) 
     if (!rho || !c1_out) return fail(p, DFT_EINVAL, "NULL field pointer");
     if (psi_out && p->S > DFT_MAX_SPECIES - 1) return fail(p, DFT_EINVAL, "psi_out needs nspecies <= 4");
     p->iter_ready = false;
+    TRY(reset_status(p));
     if (is_fp64(p))
         return c1_es_t<double>(p, static_cast<const double*>(rho), static_cast<double*>(c1_out),
                                static_cast<double*>(psi_out));

@@ -60,7 +60,7 @@ cudaError_t Passes<Real>::xcanon(cudaStream_t st, const GridDesc& g, const AxisP
 template <typename Real>
 cudaError_t Passes<Real>::canon_scale(cudaStream_t st, Ctl* ctl, const SpeciesDesc<Real>& sp, const double* red,
                                       int nblocks, int pdl) {
-    return launch_k(dftk::k_canon_scale<Real>, 1, dftk::kThreads, 0, st, pdl, ctl, sp, red, nblocks);
+    return launch_k(dftk::k_canon_scale<Real>, 1, dftk::kFinThreads, 0, st, pdl, ctl, sp, red, nblocks);
 }
 
 template <typename Real>
@@ -238,6 +238,10 @@ cudaError_t Passes<Real>::xgrad(cudaStream_t st, const GridDesc& g, const AxisPl
 
 template struct Passes<float>;
 template struct Passes<double>;
+
+cudaError_t launch_ctl_reset(cudaStream_t st, Ctl* ctl, int pdl) {
+    return launch_k(dftk::k_ctl_reset, 1, 32, 0, st, pdl, ctl);
+}
 
 cudaError_t launch_finalize(cudaStream_t st, Ctl* ctl, const double* red_sum, const double* red_sum2, int nsum,
                             const float* red_max, int nmax, int op, double inv_count, double alpha_fixed,

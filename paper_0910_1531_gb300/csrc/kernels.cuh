@@ -2477,9 +2477,38 @@ __global__ void __launch_bounds__(kThreads) k_xcanon(GridDesc g, AxisPlan px, Sp
     C* tw = align_ptr<C>(smem_raw);
     C* A = tw + nx;
     C* B = A + lines * pitch;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) tw[i] = twx[i];
     const long long nrows = (long long)g.ny * g.nz;
     const long long row0 = (long long)blockIdx.x * LR;
+    // A confined species is excluded from most rows, whose sums are zero: only blocks with a point
+    // accessible to one transform theirs (pore at 256^3, eight ions in a hundredth of a per cent of
+    // the box: 215 us without this, 33 with, most of it reading V).
+    {
+        const int pts = (int)(nrows - row0 < LR ? nrows - row0 : LR) * nx;
+        bool open = false;
+        for (int s = 0; s < S; ++s) {
+            if (!sp.canon[s]) continue;
+            const Real* v = V + (long long)s * g.n + row0 * nx;
+            using VT = typename std::conditional<(NX > 0), Vec16<Real>, Vec1<Real>>::type;
+            constexpr int VW = VT::n, KB = 4;       // KB loads in flight per thread
+            for (int i0 = threadIdx.x * VW; i0 < pts; i0 += KB * kThreads * VW) {
+                typename VT::type x[KB];
+#pragma unroll
+                for (int u = 0; u < KB; ++u) {
+                    const int i = i0 + u * kThreads * VW;
+                    x[u] = VT::load(v + (i < pts ? i : i0));
+                }
+#pragma unroll
+                for (int u = 0; u < KB; ++u)
+#pragma unroll
+                    for (int e = 0; e < VW; ++e) open = open || !(vel(x[u], e) == Real(CUDART_INF));
+            }
+        }
+        if (!__syncthreads_or(open)) {
+            if (threadIdx.x < S && sp.canon[threadIdx.x]) red[(long long)blockIdx.x * DFT_MAXS + threadIdx.x] = 0.0;
+            return;
+        }
+    }
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) tw[i] = twx[i];
     const int line_of[3] = {line0, line1, line2};
     const FastDiv ql(nl);
     for (int idx = threadIdx.x; idx < lines * nxh; idx += blockDim.x) {
@@ -2538,18 +2567,25 @@ __global__ void __launch_bounds__(kThreads) k_xcanon(GridDesc g, AxisPlan px, Sp
     }
 }
 
-// canon_scale_i = (N_i / h^3) / sum over blocks of the k_xcanon partial sums (one block).
+// canon_scale_i = (N_i / h^3) / sum over blocks of the k_xcanon partial sums (one block, four loads
+// in flight per thread: 256^3 21 -> 9 us).
 template <typename Real>
-__global__ void __launch_bounds__(kThreads) k_canon_scale(Ctl* ctl, SpeciesDesc<Real> sp, const double* __restrict__ red,
-                                                          int nblocks) {
+__global__ void __launch_bounds__(kFinThreads) k_canon_scale(Ctl* ctl, SpeciesDesc<Real> sp, const double* __restrict__ red,
+                                                             int nblocks) {
     dep_launch();
     dep_wait();
     __shared__ double scratch_d[32];
     for (int s = 0; s < sp.S; ++s) {
         if (!sp.canon[s]) continue;
-        double t = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) t += red[(long long)b * DFT_MAXS + s];
-        const double tot = block_sum(t, scratch_d);
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = threadIdx.x; b < nblocks; b += 4 * kFinThreads) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = b + u * kFinThreads;
+                if (q < nblocks) t[u] += red[(long long)q * DFT_MAXS + s];
+            }
+        }
+        const double tot = block_sum((t[0] + t[1]) + (t[2] + t[3]), scratch_d);
         if (threadIdx.x == 0) {
             ctl->canon_scale[s] = sp.nfix_dv[s] / tot;
             if (!(tot > 0.0) || !isfinite(tot)) ctl->status |= DEV_NONFINITE;
@@ -2890,6 +2926,19 @@ __device__ __forceinline__ void set_weights(Ctl* c, double a) {
     c->wAf = float(c->wA); c->wBf = float(c->wB); c->w0f = float(c->w0); c->w1f = float(c->w1);
 }
 
+// Start of an evaluation: the status words of the three control blocks cleared and the weights of a
+// plain G evaluation (1, 0) set.  One launch of 1.5 us where three memsets and a bookkeeping kernel
+// took eight between the passes of a small grid.
+__global__ void k_ctl_reset(Ctl* ctl) {
+    dep_launch();
+    dep_wait();
+    if (threadIdx.x < 3) ctl[threadIdx.x].status = 0;
+    if (threadIdx.x == 0) {
+        set_weights(ctl, 0.0);
+        ctl->alpha = 0.5;   // no previous step: the first sampled interval is alpha_max (<= 1 = 2 * 0.5)
+    }
+}
+
 // ctl points at three control blocks: the iteration's, then the weights of the two line-search
 // samples (ctl[1], ctl[2]: wA, wB, w0, w1 only), which FIN_AMAX sets for the paired evaluation.
 template <int B>
@@ -2957,10 +3006,6 @@ __global__ void __launch_bounds__(B) k_finalize(Ctl* ctl, const double* __restri
     if (threadIdx.x != 0) return;
     Ctl* c = ctl;
     const double f = tot * inv_count;
-    if (op & FIN_IDENTITY) {
-        set_weights(c, 0.0);
-        c->alpha = 0.5;   // no previous step: the first sampled interval is alpha_max (<= 1 = 2 * 0.5)
-    }
     if (op & FIN_F0) {
         c->f[0] = f;
         c->resid = sqrt(f);

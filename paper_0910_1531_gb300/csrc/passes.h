@@ -312,6 +312,9 @@ struct Passes {
     static cudaError_t build_laptab(cudaStream_t st, const GridDesc& g, Real kfx, Real kfy, Real kfz, Real* out);
 };
 
+// The plan's three control blocks at the start of an evaluation: status cleared, weights (1, 0).
+cudaError_t launch_ctl_reset(cudaStream_t st, Ctl* ctl, int pdl);
+
 // ctl: the plan's three control blocks (iteration, sample 1 weights, sample 2 weights);
 // red_sum2 (or nullptr): the second sample's partial sums for FIN_F12_CHOOSE; pdl: launch with
 // programmatic dependent launch (GridDesc::pdl)
