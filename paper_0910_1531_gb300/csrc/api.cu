@@ -1141,26 +1141,13 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
         }
         p->g.yrt = ms[1] < ms[0] ? 1 : 0;
     }
-    // z: the persistent TMA passes against the grouped one-tile-per-CTA kernels (both halves)
+    // z: the persistent TMA passes against the grouped one-tile-per-CTA kernels, and the first half's
+    // stage as one pass of either kind or as z transforms around a k-space products pass.  Each is
+    // timed in four alternating rounds and its best round counts; the kind of the one-pass kernels and
+    // the form of the first half are chosen together, by the sum of the two halves.
     if (dft_is_ct_size(p->g.nz) && !dft_zsplit<Real>(p->g.nz)) {
-        float ms[2];
-        for (int v = 0; v < 2; ++v) {
-            p->g.zgrp = v;
-            ms[v] = time_it([&] {
-                P::zconv_fwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p),
-                             O::slot_n(p->slotB), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2), &p->ctl->status);
-                P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, p->S,
-                             p->ctl, O::T1(p), O::slot_es(p, p->slotA), O::slot_es(p, p->slotB), nullptr,
-                             O::tw(p, 2));
-            });
-        }
-        p->g.zgrp = ms[1] < ms[0] ? 1 : 0;
-        // the first-half z stage as one pass (the choice above) or split into z transforms and a
-        // k-space products pass; the two often time within a few per cent, so each is timed in
-        // four alternating rounds and its best round counts
-        auto stage_z = [&](int v) {
-            p->g.zsplit = v;
-            if (v) {
+        auto fwd = [&](int split) {
+            if (split) {
                 P::zfft(p->stream, false, p->g, p->S, O::T1(p), &p->ctl->status, O::tw(p, 2), p->wait_polls);
                 P::zmul(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p), O::slot_n(p->slotB),
                         O::slot_es(p, p->slotB), nullptr);
@@ -1171,14 +1158,22 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
                              O::slot_n(p->slotB), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2), &p->ctl->status);
             }
         };
-        float best_v[2] = {1e30f, 1e30f};
+        auto bwd = [&] {
+            P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, p->S, p->ctl,
+                         O::T1(p), O::slot_es(p, p->slotA), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2));
+        };
+        float f_one[2] = {1e30f, 1e30f}, b_one[2] = {1e30f, 1e30f}, f_split = 1e30f;
         for (int round = 0; round < 4; ++round) {
             for (int v = 0; v < 2; ++v) {
-                const float t = time_it([&] { stage_z(v); });
-                if (t < best_v[v]) best_v[v] = t;
+                p->g.zgrp = v;
+                f_one[v] = std::min(f_one[v], time_it([&] { fwd(0); }));
+                b_one[v] = std::min(b_one[v], time_it(bwd));
             }
+            f_split = std::min(f_split, time_it([&] { fwd(1); }));
         }
-        p->g.zsplit = best_v[1] < best_v[0] ? 1 : 0;
+        const float t0 = b_one[0] + std::min(f_one[0], f_split), t1 = b_one[1] + std::min(f_one[1], f_split);
+        p->g.zgrp = t1 < t0 ? 1 : 0;
+        p->g.zsplit = f_split < f_one[p->g.zgrp] ? 1 : 0;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1322,6 +1317,10 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     g.nc = (long long)g.nz * g.ny * g.pxh;
     g.hx = prm->hx; g.hy = prm->hy; g.hz = prm->hz;
     g.pdl = 1;
+    // the first half's z stage as three passes where the grid fills the GPU in each (S = 2, one
+    // iteration: 256^3 4.97 ms against 5.05 in one pass, 128^3 and 96^3 equal); on smaller grids one launch
+    // is worth more (64^3 139.6 us against 142.7; dft_autotune decides by timing)
+    g.zsplit = g.n >= (1LL << 20) ? 1 : 0;
     const double two_pi = 6.28318530717958647692;
     p->kf[0] = two_pi / (g.nx * g.hx);
     p->kf[1] = two_pi / (g.ny * g.hy);

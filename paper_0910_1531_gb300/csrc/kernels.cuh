@@ -2032,9 +2032,9 @@ __device__ __forceinline__ void load_wd_rows(const GridDesc& g, int rows, long l
     const bool even = (nx % 2) == 0;
     for (int idx = threadIdx.x; idx < rows * nxh; idx += blockDim.x) {
         const int r = qh(idx), k = idx - r * nxh;
-        const long long row = row0 + r;
-        const bool live = row < nrows;
-        const long long o = row * g.pxh + k;
+        const unsigned row = (unsigned)row0 + r;
+        const bool live = row < (unsigned)nrows;
+        const unsigned o = row * (unsigned)g.pxh + k;      // 32-bit: a component has < 2^27 elements
         C v[DFT_NSPEC], vb[DFT_NSPEC];
 #pragma unroll
         for (int c = 0; c < DFT_NSPEC; ++c) {
@@ -2044,8 +2044,8 @@ __device__ __forceinline__ void load_wd_rows(const GridDesc& g, int rows, long l
                     v[c] = stage[c * cstride + r * g.pxh + k];
                     if (Bm) vb[c] = stage[(DFT_NSPEC + c) * cstride + r * g.pxh + k];
                 } else {
-                    v[c] = A[(long long)c * g.nc + o];
-                    if (Bm) vb[c] = Bm[(long long)c * g.nc + o];
+                    v[c] = (A + (long long)c * g.nc)[o];
+                    if (Bm) vb[c] = (Bm + (long long)c * g.nc)[o];
                 }
             }
         }
@@ -2059,7 +2059,7 @@ __device__ __forceinline__ void load_wd_rows(const GridDesc& g, int rows, long l
             for (int c = 0; c < DFT_NSPEC; ++c) {
                 u[c] = cadd(cscale(v[c], wA[m]), cscale(vb[c], wB[m]));
                 if (edge) u[c].y = Real(0);
-                if (NM == 1 && mat_out && live) mat_out[(long long)c * g.nc + o] = u[c];
+                if (NM == 1 && mat_out && live) (mat_out + (long long)c * g.nc)[o] = u[c];
             }
             const C zero = cmake<C>(Real(0), Real(0));
             const C dm = nyq ? zero : cmake<C>(-kx * u[4].y, kx * u[4].x);     // i k_x m
@@ -2119,8 +2119,8 @@ __device__ __forceinline__ void store_phi_spectra(const GridDesc& g, int rows, l
     for (int idx = threadIdx.x; idx < rows * NM * nxh; idx += blockDim.x) {
         const int rr = qh(idx), k = idx - rr * nxh;
         const int r = rr / NM;
-        const long long row = row0 + r;
-        if (row >= nrows) continue;
+        const unsigned row = (unsigned)row0 + r;
+        if (row >= (unsigned)nrows) continue;
         C* out = out0 + (long long)(rr - r * NM) * DFT_NSPEC * g.nc;
         C a[5], b[5];
 #pragma unroll
@@ -2133,16 +2133,16 @@ __device__ __forceinline__ void store_phi_spectra(const GridDesc& g, int rows, l
             b[l] = cmake<C>(Real(0.5) * d.y, Real(-0.5) * d.x);
         }
         const Real kx = (even && 2 * k == nx) ? Real(0) : Real(k) * kfx;
-        const long long o = row * g.pxh + k;
-        out[0 * g.nc + o] = a[0];
-        out[1 * g.nc + o] = b[0];
-        out[2 * g.nc + o] = a[1];
-        out[5 * g.nc + o] = b[1];
-        out[3 * g.nc + o] = cadd(a[2], cmake<C>(kx * b[2].y, -kx * b[2].x));   // Phi_3 - i k_x Phi_V2x
-        out[4 * g.nc + o] = cmake<C>(kx * a[3].y, -kx * a[3].x);               // -i k_x Phi_V1x
-        out[6 * g.nc + o] = b[3];
-        out[7 * g.nc + o] = a[4];
-        out[8 * g.nc + o] = b[4];
+        const unsigned o = row * (unsigned)g.pxh + k;
+        (out + 0 * g.nc)[o] = a[0];
+        (out + 1 * g.nc)[o] = b[0];
+        (out + 2 * g.nc)[o] = a[1];
+        (out + 5 * g.nc)[o] = b[1];
+        (out + 3 * g.nc)[o] = cadd(a[2], cmake<C>(kx * b[2].y, -kx * b[2].x));   // Phi_3 - i k_x Phi_V2x
+        (out + 4 * g.nc)[o] = cmake<C>(kx * a[3].y, -kx * a[3].x);               // -i k_x Phi_V1x
+        (out + 6 * g.nc)[o] = b[3];
+        (out + 7 * g.nc)[o] = a[4];
+        (out + 8 * g.nc)[o] = b[4];
     }
 }
 

@@ -136,7 +136,7 @@ template <typename Real> __host__ __device__ constexpr int dft_zfwd_minb_s3(int 
 #ifdef DFT_ZFWD_MINB_S3
     return DFT_ZFWD_MINB_S3;
 #else
-    return n < 256 ? 3 : dft_zfwd_minb<Real>(n);
+    return n <= 64 ? 3 : dft_zfwd_minb<Real>(n);   // radix 16 at 128 spills under a budget for three
 #endif
 }
 template <typename Real> __host__ __device__ constexpr int dft_zbwd_threads(int n) {
