@@ -232,9 +232,9 @@ dft_status dft_iter_run(dft_plan* plan, void* rho_inout, const void* V, int iter
  *    and primes, the reverse of one of 3s, other odd primes, 16s, then 2/4/8, and for powers of two
  *    a plan of 8s and one of 4s);
  *  - the y transform: the persistent TMA pass against the run-time column kernel;
- *  - the z passes: the persistent TMA passes against the grouped one-tile-per-CTA kernels;
- *    then the first half's z stage as one pass against three (z transform, products, z
- *    transform).
+ *  - the z stages: the persistent TMA passes or the grouped one-tile-per-CTA kernels, and the first
+ *    half's stage as one pass or as three (z transform, products, z transform), chosen together
+ *    (FP64 and run-time lengths run three passes in both halves either way).
  * Results are cached per (grid, species count, precision) for the life of the process, so
  * later plans of the same shape reuse them without timing.  Invalidates a preceding
  * dft_iter_begin (call it again).  lines_out (may be NULL) receives the first three row
@@ -252,12 +252,12 @@ const char* dft_plan_tuning(const dft_plan* plan);
  * last); x_persistent 1 = with the compile-time kernels, the Phi' passes as the persistent
  * kernel whose row blocks arrive by bulk copies two blocks ahead, 2 = by per-thread cp.async
  * copies one block ahead (0 = one CTA per row block);
- * y_variant 0 = persistent TMA pass (run-time kernel for lengths without one), 1 = run-time
- * column kernel; z_variant bit 0: 0 = persistent TMA passes, 1 = grouped one-tile-per-CTA
- * kernels; bit 1: the first half's z stage as three passes (persistent TMA z transform of the
- * species, a k-space products pass, z transform of the nine weighted densities) instead of one
- * (lengths without compile-time kernels run the run-time ones either way).  Invalidates a
- * preceding dft_iter_begin. */
+ * y_variant 0 = persistent TMA pass of the compile-time length (lengths without one run the run-time
+ * column kernel), 1 = run-time column kernel; z_variant bit 0: 0 = persistent TMA passes, 1 =
+ * grouped one-tile-per-CTA kernels; bit 1: the first half's z stage as three passes (persistent TMA z
+ * transform of the species, a k-space products pass, z transform of seven weighted-density spectra)
+ * instead of one.  Lengths without compile-time kernels and FP64 plans run three passes either way.
+ * Invalidates a preceding dft_iter_begin. */
 dft_status dft_set_variants(dft_plan* plan, int x_variant, int x_persistent, int y_variant, int z_variant);
 
 /*
@@ -323,7 +323,7 @@ dft_status dft_batch_iterate(dft_batch* batch, int iters, double alpha_or_neg, d
 
 /*
  * Bound of the bounded device-side waits (failure detection; no counterpart in the paper).
- * The y passes move their column tiles by TMA and wait for each tile on an mbarrier; a wait
+ * The y passes and the z transforms move their column tiles by TMA and wait for each tile on an mbarrier; a wait
  * gives up after `polls` polls (default DFT_WAIT_POLLS_DEFAULT), the CTA then drains the copies
  * it still has in flight (those waits keep the default bound, so no copy outlives the CTA),
  * records the timeout in the plan's device status word and stops, and the call that queued the

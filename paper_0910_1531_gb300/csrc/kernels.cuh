@@ -8,15 +8,15 @@
 //     k_yfft_tma   y forward (k_colfft for lengths without compile-time kernels)
 //     k_zconv_fwd_*  z forward, the analytic weights of App. B (n_hat_alpha), the
 //                bulk-fluid kernel (eq. CplusPsiHat) and the Poisson symbol
-//                (eq. potentialSolution) applied in k space, z inverse of the nine
-//                weighted-density spectra (the x derivatives are formed in k_xphi); or as three
-//                passes (k_colfft / k_yfft_tma, k_zmul)
-//     k_yfft_tma   y inverse of the nine spectra
+//                (eq. potentialSolution) applied in k space, z inverse of seven
+//                weighted-density spectra; or as three passes (k_colfft / k_yfft_tma, k_zmul)
+//     k_yfft_tma   y inverse of the nine spectra (the two y derivatives formed on the way in;
+//                the x derivatives are formed in k_xphi)
 //   second half (weighted densities -> c1 -> G)
 //     k_xphi     x C2R to the ten n, dPhi/dn_alpha of eq. Phi (|nV2| <= n2 bound,
 //                FP64 log(1-n3) and 1/(1-n3)^m; or another hard-sphere form), x R2C back
 //                to nine spectra
-//     k_yfft_tma   y forward
+//     k_yfft_tma   y forward, the two y-derivative spectra added into two others: seven out
 //     k_zconv_bwd_*  z forward, adjoint weights (eq. muHS), + bulk-fluid/Poisson spectra,
 //                z inverse of the S one-body correlations; or as three passes (k_zmul_bwd)
 //     k_yfft_tma   y inverse
@@ -2103,7 +2103,7 @@ __device__ __forceinline__ void store_pair_rows(const GridDesc& g, int lines, in
 }
 
 // Half spectra of the ten dPhi/dn_alpha rows of `rows` grid rows (five complex lines each, in the
-// wd_comp arrangement of load_pair_rows) into the nine spectra the y and z passes carry:
+// wd_comp arrangement of load_pair_rows) into the nine spectra the y pass takes:
 // Phi_0..Phi_2, B3 = Phi_3 - i k_x Phi_V2x, B4 = -i k_x Phi_V1x, Phi_V1y, Phi_V1z, Phi_V2y,
 // Phi_V2z (the -i k_x terms dropped on the Nyquist index).  Each line maps to its own outputs:
 // line 2 holds Phi_3 and Phi_V2x, line 3 Phi_V1x and Phi_V1z.
