@@ -14,15 +14,17 @@ cudaError_t launch(cudaStream_t st, const GridDesc& g, const AxisPlan& pa, bool 
     cb.n = pa.n;
     cb.nbox = pa.n <= 256 ? 1 : 2;
     cb.rows = dft_col_box_rows(pa.n);
-    const int ntx = (int)ceil_div(g.nxh, T), across = zax ? g.ny : g.nz;
+    // the planes as nxh columns x ny rows; along z as chunks of T columns, or all columns as one row
+    const bool flat = zax && dft_col_flat<Real>(pa.n, g.ny, g.pxh, T), chunks = flat && g.ny * g.pxh % T == 0;
+    const int nxh = !flat ? g.nxh : (chunks ? T : g.ny * g.pxh), ny = !flat ? g.ny : (chunks ? g.ny * g.pxh / T : 1);
+    const int ntx = (int)ceil_div(nxh, T), across = zax ? ny : g.nz;
     const int items = mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC;
-    cb.planes = dft_col_planes<Real>(pa.n, g.nxh, T, across, items, sm_count());
+    cb.planes = dft_col_planes<Real>(pa.n, nxh, T, across, items, sm_count());
     cb.elems = dft_col_elems<Real>(pa.n, T, cb.planes);
     CUtensorMap map;
-    const unsigned long long dims[4] = {(unsigned long long)g.nxh * E, (unsigned long long)g.ny,
-                                        (unsigned long long)g.nz,
+    const unsigned long long dims[4] = {(unsigned long long)nxh * E, (unsigned long long)ny, (unsigned long long)g.nz,
                                         (unsigned long long)(mode == COL_PLAIN ? ncomp : ncomp * DFT_NSPEC)};
-    const unsigned long long strides[3] = {(unsigned long long)g.pxh * sizeof(C),
+    const unsigned long long strides[3] = {(unsigned long long)(flat ? T : g.pxh) * sizeof(C),
                                            (unsigned long long)g.ny * g.pxh * sizeof(C),
                                            (unsigned long long)g.nc * sizeof(C)};
     const unsigned pl = unsigned(cb.planes), rows = unsigned(cb.rows);

@@ -596,17 +596,18 @@ __host__ __device__ constexpr int ct_gstride(int n, int T, int csize) {
 template <int N, int R, int NS, bool INV, int T, int GSTR, bool SD, bool DD, int NT, typename Pre = PreNone,
           typename Post = PostStore, typename C>
 __device__ __forceinline__ void ct_stage_grouped(const C* __restrict__ src, C* __restrict__ dst, int groups,
-                                                 const C* __restrict__ tw, Pre pre = Pre{}, Post post = Post{}) {
+                                                 const C* __restrict__ tw, Pre pre = Pre{}, Post post = Post{},
+                                                 bool single = false) {
     constexpr int M = N / R;
     constexpr int TWSTEP = N / (NS * R);
     constexpr int PERG = M * T;
-    const int total = PERG * groups;
+    const int total = single ? M : PERG * groups;
     for (int task = threadIdx.x; task < total; task += NT) {
         const int g = task / PERG;
         const int rem = task - g * PERG;
-        const int t = rem % T, j = rem / T;
+        const int t = single ? 0 : rem % T, j = single ? task : rem / T;
         const int k = j % NS;
-        const int off = g * GSTR + t;
+        const int off = single ? 0 : g * GSTR + t;
         C v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {

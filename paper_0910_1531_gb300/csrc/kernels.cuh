@@ -358,9 +358,14 @@ template <int MODE> struct ColCursor {
 // spectra as (x: nxh * E, y: ny, plane: nz * ncomp) 8-byte elements, E = sizeof(complex) / 8; a
 // tile is the box (TY * E, NY, 1).  A wait that runs out sets DEV_TIMEOUT and the CTA stops after
 // draining the loads it has in flight.
-// ZAX: the same pass along z (modes COL_PLAIN, COL_WD): box (TY * E, 1, NY), a tile is TY kx columns
-// of all NY z points at one ky of one component; the box lands in shared memory with the same
-// layout (element (z, t) at z TY + t).
+// ZAX: the same pass along z (modes COL_PLAIN, COL_WD): a tile is TY of the ny pxh columns (pitch
+// padding included; nothing reads it) of all NY z points of one component; the box lands in shared
+// memory with the same layout (element (z, t) at z TY + t).  Tiles of one ky each left most of the last
+// one empty, as nx / 2 + 1 is one past a multiple: seven spectra, 128^3 FP64 258 -> 237 us, 256^3 FP32
+// 184 -> 158.
+// Along y that last tile stays (wd bit 1: it holds one column).  Bound by the FP64 pipe, FP64 from 96 on
+// runs the butterflies of that one column only (128^3, Phi' forward of nine spectra 634 -> 603 us); FP32,
+// the short lengths and COL_DERIV lose more by the branch (FP32 128^3 COL_DERIV 26 -> 79 us).
 // Shared memory: stage 0 | stage 1 (dense tiles) | X (padded) | Y | twiddles | k | 2 mbarriers.
 // ------------------------------------------------------------------------------------
 template <typename Real, int NY, int TY> __host__ __device__ constexpr size_t yfft_tma_smem() {
@@ -383,6 +388,7 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
     constexpr int TILE = TY * NY;
     constexpr int GS = ct_gstride(NY, TY, int(sizeof(C)));
     constexpr uint32_t BYTES = uint32_t(TILE * sizeof(C));
+    constexpr bool kSingle = sizeof(Real) == 8 && NY >= 96 && MODE != COL_DERIV && !ZAX;
     static_assert(BYTES % 128 == 0, "TMA stage alignment");
     extern __shared__ unsigned char smem_raw[];
     const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127);
@@ -392,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
     C* const tw = X + GS;
     Real* const kt = reinterpret_cast<Real*>(tw + NY);
     uint64_t* const bar = reinterpret_cast<uint64_t*>(kt + NY);
-    const bool sets = MODE != COL_PLAIN || wd;
+    const bool sets = MODE != COL_PLAIN || (wd & 1);
     if (threadIdx.x == 0) {
         tma::mbar_init(&bar[0], 1);
         tma::mbar_init(&bar[1], 1);
@@ -435,23 +441,25 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
         const bool dual = MODE != COL_PLAIN && col_dual(t.q);
         const bool add = MODE == COL_FOLD && dual && at.sub == 1;       // Y holds the partner's transform
         const bool hold = MODE == COL_FOLD && dual && at.sub == 0;      // keep it there
+        const bool single = kSingle && (wd & 2) && at.tile % ntiles_x == ntiles_x - 1;
         // COL_DERIV: the derivative first (from the same stage), then the component itself
         for (int pass = (MODE == COL_DERIV && dual) ? 0 : 1; pass < 2; ++pass) {
             if (MODE == COL_DERIV && pass == 0)
-                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(st, X, 1, tw,
-                                                                                              PreDeriv<Real>{kt});
+                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(
+                    st, X, 1, tw, PreDeriv<Real>{kt}, PostStore{}, single);
             else
-                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(st, X, 1, tw);
+                ct_stage_grouped<NY, ct_radix_at(NY, 0), 1, INV, TY, GS, true, false, kThreads>(
+                    st, X, 1, tw, PreNone{}, PostStore{}, single);
             // the previous store has finished reading Y
             if (threadIdx.x == 0 && !add) tma::wait_read_all();
             __syncthreads();
             if (threadIdx.x == 0 && pass == 1) issue(cur);
             if (MODE == COL_FOLD && add)
                 ct_stage_grouped<NY, ct_radix_at(NY, 1), ct_ns_at(NY, 1), INV, TY, GS, false, true, kThreads>(
-                    X, Y, 1, tw, PreNone{}, PostFold<Real>{kt});
+                    X, Y, 1, tw, PreNone{}, PostFold<Real>{kt}, single);
             else
-                ct_stage_grouped<NY, ct_radix_at(NY, 1), ct_ns_at(NY, 1), INV, TY, GS, false, true, kThreads>(X, Y, 1,
-                                                                                                            tw);
+                ct_stage_grouped<NY, ct_radix_at(NY, 1), ct_ns_at(NY, 1), INV, TY, GS, false, true, kThreads>(
+                    X, Y, 1, tw, PreNone{}, PostStore{}, single);
             tma::fence_proxy_async();
             __syncthreads();
             if (threadIdx.x == 0 && !hold) {

@@ -202,17 +202,19 @@ cudaError_t launch_col_ct(cudaStream_t st, const GridDesc& g, int ncomp, C* data
     constexpr int E = int(sizeof(C) / 8);
     const int planes = mode == COL_PLAIN ? ncomp : ncomp * DFT_NSPEC, items = mode == COL_PLAIN ? ncomp : ncomp * DFT_NZSPEC;
     CUtensorMap map;
-    cudaError_t e = tma_encode_3d(&map, data, (unsigned long long)g.nxh * E, (unsigned long long)g.ny,
+    // along z the ny rows of a plane are one row of ny pxh columns
+    const int cols = ZAX ? g.ny * g.pxh : g.nxh, rows = ZAX ? 1 : g.ny;
+    cudaError_t e = tma_encode_3d(&map, data, (unsigned long long)cols * E, (unsigned long long)rows,
                                   (unsigned long long)g.nz * planes, (unsigned long long)g.pxh * sizeof(C),
                                   (unsigned long long)g.ny * g.pxh * sizeof(C), TY * E, ZAX ? 1 : N, ZAX ? N : 1);
     if (e != cudaSuccess) return e;
-    const int ntx = (int)ceil_div(g.nxh, TY), other = ZAX ? g.ny : g.nz;
+    const int ntx = (int)ceil_div(cols, TY), other = ZAX ? 1 : g.nz;
     const int ntiles = ntx * other * items;
     const size_t sm = dftk::yfft_tma_smem<Real, N, TY>();
     auto kern = dftk::k_yfft_tma<Real, INV, N, TY, ZAX, MODE>;
     const int fit = resident_blocks(kern, dftk::kThreads, sm);
     return launch_k(kern, ntiles < fit ? ntiles : fit, dftk::kThreads, sm, st, g.pdl, map, ntx, other, ntiles,
-                    mode != COL_PLAIN ? 1 : 0, status, tw, kf, polls);
+                    (mode != COL_PLAIN ? 1 : 0) | (cols % TY == 1 ? 2 : 0), status, tw, kf, polls);
 }
 }  // namespace
 
