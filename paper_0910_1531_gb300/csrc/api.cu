@@ -754,7 +754,7 @@ dft_status newton_t(dft_plan* p, Real* rho, const Real* V, double tol, int max_n
         return static_cast<Real*>(q);
     };
     double* part_dev = nullptr;
-    std::vector<double> part_host(grid);
+    std::vector<double> part_host(2 * grid + m), hcol(m);
     struct Cleanup {
         std::vector<Real*>& b;
         double*& pd;
@@ -767,7 +767,7 @@ dft_status newton_t(dft_plan* p, Real* rho, const Real* V, double tol, int max_n
     Real* rt = alloc(n);
     Real* d = alloc(n);
     Real* basis = alloc(size_t(m + 1) * n);
-    if (!F || !Ft || !g || !gt || !rt || !d || !basis || cudaMalloc(&part_dev, sizeof(double) * grid) != cudaSuccess) {
+    if (!F || !Ft || !g || !gt || !rt || !d || !basis || cudaMalloc(&part_dev, sizeof(double) * (2 * grid + m)) != cudaSuccess) {
         cudaGetLastError();
         return fail(p, DFT_ENOMEM, "Newton-Krylov work vectors");
     }
@@ -811,16 +811,15 @@ dft_status newton_t(dft_plan* p, Real* rho, const Real* V, double tol, int max_n
         for (int j = 0; j < m; ++j) {
             // w = J v_j
             NK_CUDA(vk.step(rho, Vk(j), eps, V, rt));
-            TRY(evalG(rt, gt, nullptr));
+            ++gevals;
+            TRY(picard_map_t<Real>(p, rt, V, gt));
             NK_CUDA(vk.jv(rt, gt, F, V, eps, Vk(j + 1)));
-            for (int i = 0; i <= j; ++i) {      // modified Gram-Schmidt
-                double h = 0.0;
-                TRY(dot(Vk(j + 1), Vk(i), &h));
-                H[size_t(i) * m + j] = h;
-                NK_CUDA(vk.axpby(-h, Vk(i), 1.0, Vk(j + 1)));
-            }
+            // modified Gram-Schmidt; the host reads the evaluation's status and the column together
             double hn2 = 0.0;
-            TRY(dot(Vk(j + 1), Vk(j + 1), &hn2));
+            NK_CUDA(vk.orthogonalise(basis, j + 1, Vk(j + 1), part_dev));
+            TRY(read_ctl(p));
+            NK_CUDA(vk.read_column(j + 1, part_dev, part_host.data(), hcol.data(), &hn2));
+            for (int i = 0; i <= j; ++i) H[size_t(i) * m + j] = hcol[i];
             const double hn = std::sqrt(hn2);
             H[size_t(j + 1) * m + j] = hn;
             if (hn > 0.0) NK_CUDA(vk.axpby(1.0 / hn, Vk(j + 1), 0.0, Vk(j + 1)));

@@ -18,6 +18,11 @@ public:
     cudaError_t axpby(double alpha, const Real* x, double beta, Real* y) const;
     // <a, b> in FP64 (synchronises the stream); partial_dev / partial_host hold `grid` doubles
     cudaError_t dot(const Real* a, const Real* b, double* partial_dev, double* partial_host, double* out) const;
+    // w orthogonalised against the k basis vectors (n apart) by modified Gram-Schmidt, all of it queued;
+    // dev: 2 grid partial sums, then the k coefficients
+    cudaError_t orthogonalise(const Real* basis, int k, Real* w, double* dev) const;
+    // the coefficients and w . w after orthogonalise; host: 2 grid + k doubles.  Waits for the stream.
+    cudaError_t read_column(int k, const double* dev, double* host, double* h_out, double* ww_out) const;
 
 private:
     cudaStream_t st_;

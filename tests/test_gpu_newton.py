@@ -71,3 +71,24 @@ def test_newton_fp32_reaches_the_fp32_floor():
     g = F.picard_map(prob, got, w.V)
     assert np.sqrt(P.residual_sq(prob, got, g)) < 1e-5
     plan.close()
+
+
+@pytest.mark.parametrize("shape,krylov_dim", [((4, 4, 4), 30), ((5, 6, 7), 3), ((48, 10, 33), 30)])
+def test_newton_orthogonalisation_sizes_fp64(shape, krylov_dim):
+    # fields smaller than one block of the orthogonalisation, of an odd length, and larger than its grid;
+    # a restart at the largest basis.  r < 1e-11 on the GPU leaves the oracle's residual at the maps'
+    # difference, 1e-10 per point
+    prob = F.Problem(shape, 0.1, [0.095, 0.181], [1.0, -1.0], [1.0, 1.0])
+    V = np.stack([z * 2.0 * np.sin(2 * np.pi * np.arange(shape[0]) / shape[0])[:, None, None] * np.ones(shape)
+                  for z in (1.0, -1.0)])
+    V[:, 0, 0, 0] = np.inf
+    rho0 = np.where(np.isinf(V), 0.0, prob.bath.rho[:, None, None, None])
+    from paper_0910_1531_gb300 import binding
+    plan = binding.Plan(shape, 0.1, [0.095, 0.181], [1.0, -1.0], [1.0, 1.0], precision="fp64")
+    rho = torch.tensor(rho0, dtype=torch.float64, device="cuda")
+    its, gevals, r, ok = plan.solve_newton(rho, torch.tensor(V, device="cuda"), tol=1e-11, max_newton=40,
+                                           krylov_dim=krylov_dim)
+    assert ok and r < 1e-11, (its, gevals, r)
+    got = rho.cpu().numpy()
+    assert np.sqrt(P.residual_sq(prob, got, F.picard_map(prob, got, V))) < 2e-10
+    plan.close()
