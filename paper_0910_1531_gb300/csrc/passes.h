@@ -99,11 +99,13 @@ template <typename Real> inline int dft_tile_rt(int n, int nxh, int ny = 0, int 
 }
 
 // Resident CTAs per SM that the compile-time column pass's register budget is sized for: what its
-// shared memory allows (at 256 one), and no more than its radices' registers (FP64 radix 16: two).
+// shared memory allows (at 256 one), and no more than its radices' registers (FP64 radix 16: two).  FP64 32
+// and 64 (8 x 4, 8 x 8) at four against three: 32^3, two species, y passes of nine spectra 13.0 -> 10.7 us, z
+// transforms 7.1 -> 6.0, an iteration 250.6 -> 241.6; 64^3 1256 -> 1248; 48 (8 x 6) 598 -> 604, so three there.
 template <typename Real> __host__ __device__ constexpr int dft_yfft_minb(int n) {
     if (n >= 256) return 1;
     if (sizeof(Real) == 4) return n >= 128 ? 3 : 4;
-    return n >= 96 ? 2 : 3;
+    return n >= 96 ? 2 : (n == 48 ? 3 : 4);
 }
 
 // Planes of the other axis (`other` of them) in a tile of a run-time column transform of `items`
