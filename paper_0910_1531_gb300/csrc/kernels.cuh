@@ -33,7 +33,6 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "dsfloat.cuh"
 #include "fft.cuh"
 #include "passes.h"
 #include "tma.cuh"
@@ -171,19 +170,6 @@ __device__ __forceinline__ double block_sum_ds(float hi, float lo, double* scrat
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += scratch[i];
     return r;
 }
-
-// Accumulator of a grand-potential sum: a double, or a pair of floats for FP32 fields.
-template <typename Real> struct OmegaAcc;
-template <> struct OmegaAcc<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double x) { v += x; }
-    __device__ __forceinline__ double sum(double* scratch) const { return block_sum(v, scratch); }
-};
-template <> struct OmegaAcc<float> {
-    ds v = {0.0f, 0.0f};
-    __device__ __forceinline__ void add(ds x) { v = v + x; }
-    __device__ __forceinline__ double sum(double* scratch) const { return block_sum_ds(v.hi, v.lo, scratch); }
-};
 
 __device__ __forceinline__ float block_max(float v, float* scratch) {
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -1260,14 +1246,6 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
     if (threadIdx.x == 0) tma::wait_all();
 }
 
-// acc += f Re(conj(a) b)
-__device__ __forceinline__ void energy_add(OmegaAcc<double>& acc, double2 a, double2 b, double f) {
-    acc.add(f * (a.x * b.x + a.y * b.y));
-}
-__device__ __forceinline__ void energy_add(OmegaAcc<float>& acc, float2 a, float2 b, float f) {
-    acc.add((ds_prod2(a.x, b.x) + ds_prod2(a.y, b.y)) * f);
-}
-
 // ------------------------------------------------------------------------------------
 // The k-space products of the first half as a pass of their own (the split first-half z stage:
 // z forward transform of the S species, this pass, z inverse transform of the nine weighted
@@ -1295,7 +1273,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
     const int S = sp.S;
     const unsigned nxh = g.nxh, npt = (unsigned)g.nz * g.ny * nxh;
     const int Pn = S * (S + 1) / 2;
-    OmegaAcc<Real> e_acc, q_acc;
+    double e_acc = 0.0, q_acc = 0.0;
     for (unsigned q = blockIdx.x * kThreads + threadIdx.x; q < npt; q += gridDim.x * kThreads) {
         const unsigned rz = q / nxh;
         const int kxi = int(q - rz * nxh), kzi = int(rz / (unsigned)g.ny), kyi = int(rz - kzi * g.ny);
@@ -1345,7 +1323,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
             }
             slot_es[(long long)S * g.nc + o] = cscale(ps, flb * inv_lap);   // psi_hat = 4 pi lambda_B q_hat / lap
         }
-        const Real wk = (kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? Real(1) : Real(2);
+        const double wk = GRAD ? ((kxi == 0 || (g.nx % 2 == 0 && 2 * kxi == g.nx)) ? 1.0 : 2.0) : 0.0;
         C es[SM];
 #pragma unroll
         for (int s = 0; s < SM; ++s) {
@@ -1366,20 +1344,23 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 && !GRAD ? 3 : 2) 
                 }
                 es[i2] = cadd(es[i2], cscale(v[j], K));
                 if (j != i2) es[j] = cadd(es[j], cscale(v[i2], K));
-                if constexpr (GRAD) energy_add(q_acc, v[i2], v[j], dK * (j != i2 ? 2 * wk : wk));
+                if constexpr (GRAD) {
+                    const double re = double(v[i2].x) * v[j].x + double(v[i2].y) * v[j].y;
+                    q_acc += wk * double(dK) * re * (j != i2 ? 2.0 : 1.0);
+                }
             }
         }
 #pragma unroll
         for (int s = 0; s < SM; ++s) {
             if (s >= S) break;
-            if constexpr (GRAD) energy_add(e_acc, v[s], es[s], wk);
+            if constexpr (GRAD) e_acc += wk * (double(v[s].x) * es[s].x + double(v[s].y) * es[s].y);
             slot_es[(long long)s * g.nc + o] = es[s];
         }
     }
     if constexpr (GRAD) {
         __shared__ double scratch_d[32];
-        const double be = e_acc.sum(scratch_d);
-        const double bq = q_acc.sum(scratch_d);
+        const double be = block_sum(e_acc, scratch_d);
+        const double bq = block_sum(q_acc, scratch_d);
         if (threadIdx.x == 0) {
             red_energy[2 * (long long)blockIdx.x] = be;
             red_energy[2 * (long long)blockIdx.x + 1] = bq;
@@ -1700,7 +1681,7 @@ __device__ __forceinline__ void wb_g(Real n3, double lnD_hi, Real* g, Real* dg) 
 }
 
 // Phi itself (eq. Phi, or the form `kind`), in FP64, for the grand potential; same clamp as the
-// derivatives.
+// derivatives.  Bounds the Phi' pass of an FP32 plan where it is asked for (64^3: 52 us with it).
 template <typename Real> __device__ __forceinline__ double phi_value(const Real* n, int kind) {
     const double n0 = n[0], n1 = n[1], n2 = n[2], n3 = n[3];
     const double D = 1.0 - n3;
@@ -1717,46 +1698,6 @@ template <typename Real> __device__ __forceinline__ double phi_value(const Real*
     xi = xi < 0.0 ? 0.0 : (xi > 1.0 ? 1.0 : xi);
     const double om = 1.0 - xi;
     return base + n2 * n2 * n2 * om * om * om / (24.0 * CUDART_PI * D * D);
-}
-
-// A double as a pair (the rare terms outside the pairs' range are formed in FP64).
-__device__ __forceinline__ ds ds_from(double x) {
-    const float h = float(x);
-    return {h, float(x - double(h))};
-}
-
-// The same of FP32 fields for eq. Phi and the Rosenfeld form: the products of fields are exact as
-// pairs, D = 1 - n3 too.  About 250 FP32 instructions where FP64 takes 100, each 16 cycles of the SM's
-// FP64 pipe: 64^3, the Phi' pass with this sum 52 -> 15.6 us.  n3 outside (-1, 1) and the White Bear
-// form keep FP64.
-__device__ __forceinline__ void phi_accumulate(OmegaAcc<double>& acc, const double* n, int kind) {
-    acc.add(phi_value<double>(n, kind));
-}
-__device__ __forceinline__ void phi_accumulate(OmegaAcc<float>& acc, const float* n, int kind) {
-    const float n0 = n[0], n1 = n[1], n2 = n[2], n3 = n[3];
-    if (kind == DFT_PHI_WHITE_BEAR || !(n3 > -1.0f && n3 < 0.99999f)) {
-        acc.add(ds_from(phi_value<float>(n, kind)));
-        return;
-    }
-    const ds D = ds_sum2(1.0f, -n3), r = ds_recip(D);
-    const ds q = ds_prod2(n[7], n[7]) + ds_prod2(n[8], n[8]) + ds_prod2(n[9], n[9]);
-    const ds dot = ds_prod2(n[4], n[7]) + ds_prod2(n[5], n[8]) + ds_prod2(n[6], n[9]);
-    ds v = (ds_prod2(n1, n2) - dot) * r - ds_log(D) * n0;
-    ds t;
-    if (kind == DFT_PHI_ROSENFELD) {
-        t = (ds_prod2(n2, n2) - q * 3.0f) * n2;
-    } else {
-        // n2^3 (1 - xi)^3, xi = q / n2^2 clamped to [0, 1]; below n2 = 1e-12 it is below 1e-36
-        t = {0.0f, 0.0f};
-        if (n2 > 1e-12f) {
-            const ds xi = q * ds_recip(ds_prod2(n2, n2));
-            if (xi.hi < 1.0f) {
-                const ds u = (xi.hi > 0.0f ? ds{1.0f, 0.0f} - xi : ds{1.0f, 0.0f}) * n2;
-                t = u * u * u;
-            }
-        }
-    }
-    acc.add(v + t * (r * r) * ds_const(1.0 / (24.0 * CUDART_PI)));
 }
 
 // The derivatives of eq. Phi (kind DFT_PHI_RSLT) or of the other forms, whose last term
@@ -2175,7 +2116,7 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
     extern __shared__ unsigned char smem_raw[];
     __shared__ float scratch_f[32];
     __shared__ double scratch_d[32];
-    OmegaAcc<Real> phi_acc;   // sum of Phi(n) over the block's points (grand potential only)
+    double phi_acc = 0.0;   // sum of Phi(n) over the block's points (grand potential only)
     const int nx = NX > 0 ? NX : g.nx, pitch = x_pitch<NX>(nx);
     const QRow<NX> qx(nx);
     const int lines = 5 * NM * LR;
@@ -2208,7 +2149,7 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
             n[7] = v2.y; n[4] = v3.x; n[6] = v3.y; n[8] = v4.x; n[9] = v4.y;
         }
         if (row0 + r < nrows) mx = fmaxf(mx, float(n[3]));
-        if (red_phi && row0 + r < nrows) phi_accumulate(phi_acc, n, g.phi);
+        if (red_phi && row0 + r < nrows) phi_acc += phi_value<Real>(n, g.phi);
         const bool ok = phi_derivatives<Real>(n, g.phi);
         if (!ok && row0 + r < nrows) bad = true;
         base[0] = cmake<C>(n[0], n[1]);
@@ -2225,7 +2166,7 @@ __global__ void __launch_bounds__(kThreads) k_xphi(GridDesc g, AxisPlan px, int 
     const float bm = block_max(mx, scratch_f);
     if (threadIdx.x == 0 && red_max) red_max[blockIdx.x] = bm;
     if (red_phi) {
-        const double bp = phi_acc.sum(scratch_d);
+        const double bp = block_sum(phi_acc, scratch_d);
         if (threadIdx.x == 0) red_phi[blockIdx.x] = bp;
     }
 }
@@ -2778,39 +2719,14 @@ __global__ void __launch_bounds__(kThreads, NX < 0 ? 1 : (sizeof(Real) == 4 ? 3 
     }
 }
 
-// One accessible point of the gradient pass: adds rho (ln(rho / rho_bath) - 1) + rho (V - mu_ex) to
-// `ideal`, returns h^3 [ln(rho / rho_bath) + V - mu_hs - c].  FP32 fields in pairs of floats (a
-// logarithm in FP64 per point bound the pass: 64^3, S = 2, 53 -> 12.4 us); arguments outside the
-// pairs' range in FP64.
-__device__ __forceinline__ double grad_point(OmegaAcc<double>& ideal, double rv, double v, double c, double irb,
-                                             double mu_hs, double mu_ex, double dv) {
-    const double lr = log(rv * irb);
-    ideal.add(rv * (lr - 1.0) + rv * (v - mu_ex));
-    return dv * (lr + v - mu_hs - c);
-}
-__device__ __forceinline__ float grad_point(OmegaAcc<float>& ideal, float rv, float v, float c, float irb, float mu_hs,
-                                            float mu_ex, float dv) {
-    const ds x = ds_prod2(rv, irb);
-    if (!(x.hi > 1e-30f && x.hi < 1e30f && rv > 1e-30f && rv < 1e12f && fabsf(v) < 1e12f)) {
-        const double lr = log(double(rv) * double(irb));
-        ideal.add(ds_from(double(rv) * (lr - 1.0) + double(rv) * (double(v) - double(mu_ex))));
-        return float(dv * (lr + double(v) - double(mu_hs) - double(c)));
-    }
-    const ds lr = ds_log(x);
-    ideal.add((lr + (ds_sum2(v, -mu_ex) + ds{-1.0f, 0.0f})) * rv);
-    const ds t = lr + (ds_sum2(v, -mu_hs) + ds{-c, 0.0f});
-    return __fmaf_rn(dv, t.hi, __fmul_rn(dv, t.lo));
-}
-__device__ __forceinline__ void grad_count(OmegaAcc<double>& n, double rv) { n.add(rv); }
-__device__ __forceinline__ void grad_count(OmegaAcc<float>& n, float rv) { n.add(ds{rv, 0.0f}); }
-
 // ------------------------------------------------------------------------------------
 // Gradient pass: x inverse of the one-body correlations c_i, then at each point
 //   dOmega/drho_i = h^3 [ln(rho_i / rho_bath_i) + V_i - beta mu_HS_bath_i - c_i]   (accessible, rho > 0)
 //   dOmega/dV_i   = h^3 rho_i
 // and per-block sums red[b (S + 1) + 0] = sum_i sum_x [rho_i (ln(rho_i/rho_bath_i) - 1) + rho_i (V_i -
-// beta mu_ex_bath_i)] (accessible points), red[b (S + 1) + 1 + i] = sum_x rho_i, in FP64 or pairs of
-// floats across a block's threads, FP64 across blocks.
+// beta mu_ex_bath_i)] (accessible points), red[b (S + 1) + 1 + i] = sum_x rho_i, all in FP64.  In FP32
+// plans too, where the logarithm and products per point and species bound the pass on the FP64 pipe (64^3, two
+// species: 52 us).
 // ------------------------------------------------------------------------------------
 template <typename Real, int NX>
 __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, SpeciesDesc<Real> sp, int LR, Real dv,
@@ -2837,7 +2753,9 @@ __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, Spe
     load_pair_rows<Real, NX>(g, lines, lpr, row0, nrows, S, cspec, nullptr, Real(1), Real(0), nullptr, A);
     __syncthreads();
     C* R = any_fft<NX, true>(A, B, px, lines, pitch, tw);
-    OmegaAcc<Real> ideal, num[DFT_MAXS];
+    double ideal = 0.0, num[DFT_MAXS];
+#pragma unroll
+    for (int s = 0; s < DFT_MAXS; ++s) num[s] = 0.0;
     for (int idx = threadIdx.x; idx < LR * nx; idx += blockDim.x) {
         const int r = qx(idx), x = idx - r * nx;
         const long long row = row0 + r;
@@ -2852,8 +2770,12 @@ __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, Spe
             const Real v = V[o];
             const bool acc_ok = !(isinf(v) && v > Real(0)) && rv > Real(0);
             Real gr = Real(0);
-            if (acc_ok) gr = grad_point(ideal, rv, v, c, sp.inv_rho_b[s], sp.mu_hs_b[s], sp.mu_ex_b[s], dv);
-            grad_count(num[s], rv);
+            if (acc_ok) {
+                const double lr = log(double(rv) * double(sp.inv_rho_b[s]));
+                gr = Real(dv * (lr + double(v) - double(sp.mu_hs_b[s]) - double(c)));
+                ideal += double(rv) * (lr - 1.0) + double(rv) * (double(v) - double(sp.mu_ex_b[s]));
+            }
+            num[s] += double(rv);
             if (grad_rho) grad_rho[o] = gr;
             if (grad_V) grad_V[o] = dv * rv;
         }
@@ -2861,7 +2783,7 @@ __global__ void __launch_bounds__(kThreads) k_xgrad(GridDesc g, AxisPlan px, Spe
 #pragma unroll
     for (int s = -1; s < DFT_MAXS; ++s) {
         if (s >= S) break;
-        const double b = s < 0 ? ideal.sum(scratch_d) : num[s < 0 ? 0 : s].sum(scratch_d);
+        const double b = block_sum(s < 0 ? ideal : num[s < 0 ? 0 : s], scratch_d);
         if (threadIdx.x == 0) red[(long long)blockIdx.x * (S + 1) + 1 + s] = b;
     }
 }

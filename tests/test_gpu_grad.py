@@ -34,8 +34,10 @@ TOL = {"fp32": dict(omega=1e-5, field=1e-5, bulk=2e-3), "fp64": dict(omega=1e-10
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("obstacle", [False, True])
-def test_grad_matches_oracle(precision, obstacle):
+@pytest.mark.parametrize("h", [(0.1, 0.1, 0.1), (0.1, 0.09, 0.11)])      # |k| tables per m^2 and per octant point
+def test_grad_matches_oracle(precision, obstacle, h):
     w = workloads.smooth_field_nacl(n=16, h=0.1, molar=0.5, seed=2)
+    w.h = h
     prob = F.Problem(w.shape, w.h, w.radius, w.z, w.bulk_molar)
     V = w.V.copy()
     if obstacle:
@@ -51,6 +53,34 @@ def test_grad_matches_oracle(precision, obstacle):
     assert relerr(d_V.cpu().numpy(), F.grad_omega_v(prob, rho)) < TOL[precision]["field"]
     ref_bulk = F.grad_omega_bulk(w.shape, w.h, w.radius, w.z, w.bulk_molar, rho, V)
     assert np.allclose(d_bulk, ref_bulk, rtol=TOL[precision]["bulk"], atol=0)
+
+
+@pytest.mark.parametrize("v", [0.7, -1.3, 0.0])
+def test_omega_sums_of_fp32_plans_are_fp64(v):
+    # Neutral spheres of radius 1e-6 nm have no excess terms (Phi below 1e-16 of the ideal part), so Omega is the
+    # ideal and external sum over FP32 fields, whose FP64 value is known: each term takes at most six roundings
+    # (the product rho / rho_bath is exact, the logarithm within an ulp); a block's sums of equal terms double
+    # exactly; the sums of at most 16 blocks, added in order, are off by half a rounding each on the average of
+    # the growing sum, at most nine of the whole: 15 x 2^-53 of the terms' absolute values.  Sums or logarithms of
+    # 48 bits fail at some of the densities.
+    from paper_0910_1531_gb300 import binding
+    shape, h = (4, 4, 4), 0.1
+    plan = binding.Plan(shape, h, [1e-6], [0.0], [1.0], precision="fp32")
+    b = plan.bulk()
+    # the plan's FP32 species constants
+    irb, mu = float(np.float32(1.0 / b["rho"][0])), float(np.float32(b["mu_hs"][0] + b["mu_es"][0]))
+    V = torch.full((1,) + shape, v, dtype=torch.float32, device="cuda")
+    v32 = float(np.float32(v))
+    worst = 0.0
+    for ratio in np.geomspace(0.05, 60.0, 300):
+        rv = float(np.float32(ratio * b["rho"][0]))
+        om, _, _, _ = plan.grad(torch.full((1,) + shape, rv, dtype=torch.float32, device="cuda"), V, want_bulk=False)
+        ln = np.log(rv * irb)
+        ref = h ** 3 * 64 * (rv * (ln - 1.0) + rv * (v32 - mu))
+        size = h ** 3 * 64 * rv * (abs(ln) + 1.0 + abs(v32) + abs(mu))
+        worst = max(worst, abs(om - ref) / size)
+    assert worst <= 15 * 2.0 ** -53, worst
+    plan.close()
 
 
 def test_autograd_matches_finite_differences_fp64():
