@@ -357,7 +357,8 @@ dft_status dft_set_dependent_launch(dft_plan* plan, int enable);
  * memory traffic (bytes: every input element read once and every output
  * element written once by each launch) since the last enable; it
  * synchronises the stream.  Names: "xfwd", "yfft", "zconv_fwd", "xphi",
- * "zconv_bwd", "xupdate", "xinv", "finalize".  Any out pointer may be NULL.
+ * "zconv_bwd" (a half's z stage in one pass), "zfft", "zmul" (the z transforms and k-space products
+ * of one in three), "xupdate", "xinv", "finalize".  Any out pointer may be NULL.
  */
 dft_status dft_profile_enable(dft_plan* plan, int enable);
 dft_status dft_profile_read(dft_plan* plan, const char* name, int* launches, double* total_ms,

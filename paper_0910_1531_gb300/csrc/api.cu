@@ -328,19 +328,18 @@ template <typename Real> struct Ops {
         if (!pre)
             LAUNCH(p, K_XFWD, p->S * (RB(p) + CB(p)), P::xfwd(p->stream, p->g, p->ax, p->S, p->LX, rho, W, tw(p, 0)));
         LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, p->S, W, &p->ctl->status, tw(p, 1), p->wait_polls));
-        if (p->g.zsplit && dft_is_ct_size(p->g.nz) && !dft_zsplit<Real>(p->g.nz) && !want_psi && !red_energy) {
+        if (red_energy || P::z_three(p->g, sp) || (p->g.zsplit && !want_psi)) {
             // z forward transform of the species, the k-space products, z inverse of the seven
-            LAUNCH(p, K_ZFFT, 2.0 * p->S * CB(p),
-                   P::zfft(p->stream, false, p->g, p->S, W, &p->ctl->status, tw(p, 2), p->wait_polls));
-            LAUNCH(p, K_ZMUL, (p->S + DFT_NZSPEC + p->S) * CB(p),
-                   P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), 0, W, slot_n(slot), slot_es(p, slot),
-                           nullptr));
-            LAUNCH(p, K_ZFFT, 2.0 * DFT_NZSPEC * CB(p),
-                   P::zfft(p->stream, true, p->g, 1, slot_n(slot), &p->ctl->status, tw(p, 2), p->wait_polls, COL_WD));
+            const long long polls = red_energy || P::z_three(p->g, sp) ? DFT_WAIT_POLLS : p->wait_polls;
+            TRY(zfft(p, false, p->S, COL_PLAIN, W, polls));
+            LAUNCH(p, K_ZMUL, (p->S + DFT_NZSPEC + p->S + want_psi) * CB(p),
+                   P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W, slot_n(slot),
+                           slot_es(p, slot), red_energy));
+            TRY(zfft(p, true, 1, COL_WD, slot_n(slot), polls));
         } else {
             LAUNCH(p, K_ZFWD, (p->S + DFT_NZSPEC + p->S + want_psi) * CB(p),
-                   P::zconv_fwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W,
-                                slot_n(slot), slot_es(p, slot), red_energy, tw(p, 2), &p->ctl->status));
+                   P::zconv_fwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W, slot_n(slot),
+                                slot_es(p, slot), tw(p, 2), &p->ctl->status));
         }
         // seven spectra in, nine out (the y derivatives formed in the pass)
         LAUNCH(p, K_YFFT, (DFT_NZSPEC + DFT_NSPEC) * CB(p),
@@ -355,6 +354,40 @@ template <typename Real> struct Ops {
         LAUNCH(p, K_YFFT, sets * (DFT_NSPEC + DFT_NZSPEC) * CB(p),
                P::yfft(p->stream, false, p->g, p->ay, p->Ty, sets, T1(p), &p->ctl->status, tw(p, 1), p->wait_polls,
                        COL_FOLD, kf(p, 1)));
+        return DFT_OK;
+    }
+
+    // a z transform of a three-pass z stage: ncomp components of data, or (COL_WD) the seven of ncomp sets
+    static dft_status zfft(dft_plan* p, bool inv, int ncomp, int mode, C* data, long long polls) {
+        LAUNCH(p, K_ZFFT, 2.0 * (mode == COL_WD ? ncomp * DFT_NZSPEC : ncomp) * CB(p),
+               P::zfft(p->stream, inv, p->g, p->az, p->Tz, ncomp, data, &p->ctl->status, tw(p, 2), polls, mode));
+        return DFT_OK;
+    }
+
+    // The second half's z stage in place in T1, one or two samples (sample m: nine Phi' spectra at component
+    // 9 m, weights in ctl[m], nout results at component m nout): in three passes, the Phi' spectra transformed
+    // only where the hard-sphere part (flags bit 0) is wanted, or in one.  es_mat (or nullptr, one sample):
+    // the mixed ES spectra.
+    static dft_status z_second(dft_plan* p, int samples, int flags, int nout, const Ctl* ctl, const C* esA,
+                               const C* esB, C* es_mat) {
+        const SpeciesDesc<Real>& sp = species<Real>(p);
+        const double in = (flags & 1 ? samples * DFT_NZSPEC : 0) + (flags & 2 ? nout * (esB ? 2 : 1) : 0);
+        const double bytes = (in + samples * nout + (es_mat ? nout : 0)) * CB(p);
+        if (P::z_three(p->g, sp)) {
+            if (flags & 1) TRY(zfft(p, false, samples, COL_WD, T1(p), DFT_WAIT_POLLS));
+            LAUNCH(p, K_ZMUL, bytes,
+                   P::zmul_bwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), flags, nout, samples, ctl, T1(p), esA,
+                               esB, es_mat));
+            return zfft(p, true, samples * nout, COL_PLAIN, T1(p), DFT_WAIT_POLLS);
+        }
+        if (samples == 2)
+            LAUNCH(p, K_ZBWD, bytes,
+                   P::zconv_bwd_pair(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), nout, ctl, T1(p), esA, esB,
+                                     tw(p, 2)));
+        else
+            LAUNCH(p, K_ZBWD, bytes,
+                   P::zconv_bwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), flags, nout, ctl, T1(p), esA, esB,
+                                es_mat, tw(p, 2)));
         return DFT_OK;
     }
 
@@ -373,9 +406,7 @@ template <typename Real> struct Ops {
                P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, A, B, materialise ? A : nullptr, T1(p),
                                   p->red_max, &p->ctl->status, nullptr, kf(p, 0), tw(p, 0)));
         TRY(yfold(p, 1));
-        LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S * ((use_B ? 2 : 1) + 1 + (materialise ? 1 : 0))) * CB(p),
-               P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), 3, p->S,
-                                       p->ctl, T1(p), esA, esB, materialise ? esA : nullptr, tw(p, 2)));
+        TRY(z_second(p, 1, 3, p->S, p->ctl, esA, esB, materialise ? esA : nullptr));
         LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, p->S, T1(p), &p->ctl->status, tw(p, 1), p->wait_polls));
         if (p->ncanon > 0) {
             // fixed-number species: the sum of their Boltzmann factors first (its reciprocal
@@ -410,12 +441,10 @@ template <typename Real> struct Ops {
                P::xphi2(p->stream, p->g, p->ax, p->LRphi2, p->ctl, A, B, T1(p), &p->ctl->status, kf(p, 0), tw(p, 0)));
         TRY(yfold(p, 2));
         C* c2 = T2;   // the second sample's correlation spectra
-        if (P::has_zbwd_pair(p->g, p->S)) {
-            // one z pass for both samples (the ES tiles read once; sample 2's results after sample
+        if (P::z_three(p->g, sp) || P::has_zbwd_pair(p->g, p->S)) {
+            // one z stage for both samples (the ES tiles read once; sample 2's results after sample
             // 1's, at T1 components S .. 2 S - 1), then one y inverse over the 2 S components
-            LAUNCH(p, K_ZBWD, (2.0 * DFT_NZSPEC + 4.0 * p->S) * CB(p),
-                   P::zconv_bwd_pair(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), p->S, p->ctl + 1,
-                                     T1(p), esA, esB, tw(p, 2)));
+            TRY(z_second(p, 2, 3, p->S, p->ctl + 1, esA, esB, nullptr));
             LAUNCH(p, K_YFFT, 2.0 * (2 * p->S) * CB(p),
                    P::yfft(p->stream, true, p->g, p->ay, p->Ty, 2 * p->S, T1(p), &p->ctl->status, tw(p, 1),
                            p->wait_polls));
@@ -424,8 +453,8 @@ template <typename Real> struct Ops {
             for (int m = 0; m < 2; ++m) {
                 C* phi = m == 0 ? T1(p) : T2;
                 LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S * 3) * CB(p),
-                       P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, kf(p, 0), kf(p, 1), kf(p, 2), 3, p->S,
-                                    p->ctl + 1 + m, phi, esA, esB, nullptr, tw(p, 2)));
+                       P::zconv_bwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), 3, p->S, p->ctl + 1 + m, phi,
+                                    esA, esB, nullptr, tw(p, 2)));
                 LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p),
                        P::yfft(p->stream, true, p->g, p->ay, p->Ty, p->S, phi, &p->ctl->status, tw(p, 1),
                                p->wait_polls));
@@ -551,8 +580,7 @@ template <typename Real> dft_status c1_hs_t(dft_plan* p, const Real* rho, Real* 
     LAUNCH(p, K_XPHI, 2.0 * DFT_NSPEC * CB(p), P::xphi(p->stream, p->g, p->ax, p->LRphi, p->ctl, O::slot_n(p->slotA), nullptr, nullptr,
                               O::T1(p), p->red_max, &p->ctl->status, nullptr, O::kf(p, 0), O::tw(p, 0)));
     TRY(O::yfold(p, 1));
-    LAUNCH(p, K_ZBWD, (DFT_NZSPEC + p->S) * CB(p), P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 1, p->S,
-                                   p->ctl, O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
+    TRY(O::z_second(p, 1, 1, p->S, p->ctl, O::slot_es(p, p->slotA), nullptr, nullptr));
     LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, p->S, O::T1(p), &p->ctl->status, O::tw(p, 1), p->wait_polls));
     TRY(O::xinv(p, p->S, O::T1(p), c1, nullptr, nullptr, -1, nullptr, nullptr));
     return DFT_OK;
@@ -565,8 +593,7 @@ template <typename Real> dft_status c1_es_t(dft_plan* p, const Real* rho, Real* 
     const int want_psi = psi ? 1 : 0;
     const int nout = p->S + want_psi;
     TRY(O::first_half(p, rho, p->slotA, want_psi));
-    LAUNCH(p, K_ZBWD, 2.0 * nout * CB(p), P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 2, nout,
-                                   p->ctl, O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
+    TRY(O::z_second(p, 1, 2, nout, p->ctl, O::slot_es(p, p->slotA), nullptr, nullptr));
     LAUNCH(p, K_YFFT, 2.0 * (nout) * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, nout, O::T1(p), &p->ctl->status, O::tw(p, 1), p->wait_polls));
     double offs[DFT_NCOMP + 2] = {0};
     for (int s = 0; s < p->S; ++s) offs[s] = -p->bath.mu_es[s];
@@ -674,9 +701,7 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
                                                         nullptr, nullptr, O::T1(p), p->red_max, &p->ctl->status,
                                                         r_phi, O::kf(p, 0), O::tw(p, 0)));
     TRY(O::yfold(p, 1));
-    LAUNCH(p, K_ZBWD, (DFT_NZSPEC + 2 * S) * CB(p),
-           P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, S, p->ctl,
-                        O::T1(p), O::slot_es(p, p->slotA), nullptr, nullptr, O::tw(p, 2)));
+    TRY(O::z_second(p, 1, 3, S, p->ctl, O::slot_es(p, p->slotA), nullptr, nullptr));
     LAUNCH(p, K_YFFT, 2.0 * S * CB(p), P::yfft(p->stream, true, p->g, p->ay, p->Ty, S, O::T1(p), &p->ctl->status,
                                                 O::tw(p, 1), p->wait_polls));
     LAUNCH(p, K_XUPD, S * (CB(p) + RB(p) * (2 + (d_rho ? 1 : 0) + (d_V ? 1 : 0))),
@@ -1144,22 +1169,23 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
     // stage as one pass of either kind or as z transforms around a k-space products pass.  Each is
     // timed in four alternating rounds and its best round counts; the kind of the one-pass kernels and
     // the form of the first half are chosen together, by the sum of the two halves.
-    if (dft_is_ct_size(p->g.nz) && !dft_zsplit<Real>(p->g.nz)) {
+    if (!P::z_three(p->g, sp)) {
         auto fwd = [&](int split) {
             if (split) {
-                P::zfft(p->stream, false, p->g, p->S, O::T1(p), &p->ctl->status, O::tw(p, 2), p->wait_polls);
+                P::zfft(p->stream, false, p->g, p->az, p->Tz, p->S, O::T1(p), &p->ctl->status, O::tw(p, 2),
+                        p->wait_polls);
                 P::zmul(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p), O::slot_n(p->slotB),
                         O::slot_es(p, p->slotB), nullptr);
-                P::zfft(p->stream, true, p->g, 1, O::slot_n(p->slotB), &p->ctl->status, O::tw(p, 2),
+                P::zfft(p->stream, true, p->g, p->az, p->Tz, 1, O::slot_n(p->slotB), &p->ctl->status, O::tw(p, 2),
                         p->wait_polls, COL_WD);
             } else {
-                P::zconv_fwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p),
-                             O::slot_n(p->slotB), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2), &p->ctl->status);
+                P::zconv_fwd(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 0, O::T1(p),
+                             O::slot_n(p->slotB), O::slot_es(p, p->slotB), O::tw(p, 2), &p->ctl->status);
             }
         };
         auto bwd = [&] {
-            P::zconv_bwd(p->stream, p->g, p->az, sp, p->Tz, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, p->S, p->ctl,
-                         O::T1(p), O::slot_es(p, p->slotA), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2));
+            P::zconv_bwd(p->stream, p->g, sp, O::kf(p, 0), O::kf(p, 1), O::kf(p, 2), 3, p->S, p->ctl, O::T1(p),
+                         O::slot_es(p, p->slotA), O::slot_es(p, p->slotB), nullptr, O::tw(p, 2));
         };
         float f_one[2] = {1e30f, 1e30f}, b_one[2] = {1e30f, 1e30f}, f_split = 1e30f;
         for (int round = 0; round < 4; ++round) {

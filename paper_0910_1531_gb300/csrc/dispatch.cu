@@ -102,10 +102,10 @@ cudaError_t Passes<Real>::yfft(cudaStream_t st, bool inv, const GridDesc& g, con
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
-                             int T, Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
-                             double* red_energy, const C* tw, int* status) {
-    DFT_SWITCH_Z(g.nz, zconv_fwd(st, g, pz, sp, T, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy, tw, status))
+cudaError_t Passes<Real>::zconv_fwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                    Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, const C* tw,
+                                    int* status) {
+    DFT_SWITCH_Z(g.nz, zconv_fwd(st, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, tw, status))
 }
 
 template <typename Real>
@@ -116,18 +116,17 @@ cudaError_t Passes<Real>::xphi(cudaStream_t st, const GridDesc& g, const AxisPla
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
-                             int T, Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
-                             const C* esA, const C* esB, C* es_mat, const C* tw) {
-    DFT_SWITCH_Z(g.nz, zconv_bwd(st, g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw))
+cudaError_t Passes<Real>::zconv_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                    Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                    const C* esB, C* es_mat, const C* tw) {
+    DFT_SWITCH_Z(g.nz, zconv_bwd(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw))
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
-                                         const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz,
-                                         int ncomp_out, const Ctl* ctl, C* phi, const C* esA, const C* esB,
-                                         const C* tw) {
-    DFT_SWITCH_Z(g.nz, zconv_bwd_pair(st, g, pz, sp, T, kfx, kfy, kfz, ncomp_out, ctl, phi, esA, esB, tw))
+cudaError_t Passes<Real>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                         Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                         const C* esB, const C* tw) {
+    DFT_SWITCH_Z(g.nz, zconv_bwd_pair(st, g, sp, kfx, kfy, kfz, ncomp_out, ctl, phi, esA, esB, tw))
 }
 
 template <typename Real>
@@ -136,9 +135,9 @@ bool Passes<Real>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
 }
 
 template <typename Real>
-cudaError_t Passes<Real>::zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                               const C* tw, long long polls, int mode) {
-    DFT_SWITCH_Z(g.nz, zfft(st, inv, g, ncomp, data, status, tw, polls, mode))
+cudaError_t Passes<Real>::zfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp,
+                               C* data, int* status, const C* tw, long long polls, int mode) {
+    DFT_SWITCH_Z(g.nz, zfft(st, inv, g, pz, T, ncomp, data, status, tw, polls, mode))
 }
 
 namespace {

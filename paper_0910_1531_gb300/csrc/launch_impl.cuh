@@ -234,8 +234,7 @@ cudaError_t LaunchY<Real, N>::yfft(cudaStream_t st, bool inv, const GridDesc& g,
 }
 
 // ---------------------------------------------------------------------------------- z
-// A half in one pass, or (dft_zsplit, and for the grand-potential sums) as z transform, k-space
-// products, z transform.
+// The z transforms of any length, and the halves in one pass (FP32, compile-time lengths).
 template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::init() {
     cudaError_t e = cudaSuccess, r;
@@ -267,41 +266,21 @@ cudaError_t LaunchZ<Real, N>::init() {
 }
 
 template <typename Real, int N>
-cudaError_t LaunchZ<Real, N>::zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                                   const C* tw, long long polls, int mode) {
+cudaError_t LaunchZ<Real, N>::zfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp,
+                                   C* data, int* status, const C* tw, long long polls, int mode) {
     if constexpr (N > 0) {
         return inv ? launch_col_ct<Real, true, N, true, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, Real(0))
                    : launch_col_ct<Real, false, N, true, COL_PLAIN>(st, g, ncomp, data, status, tw, polls, mode, Real(0));
     } else {
-        (void)st; (void)inv; (void)g; (void)ncomp; (void)data; (void)status; (void)tw; (void)polls; (void)mode;
-        return cudaErrorNotSupported;
+        return ColFft<Real>::run(st, inv, g, pz, true, T, ncomp, data, status, tw, polls, mode, Real(0));
     }
 }
-
-namespace {
-// The z transform of a split z stage: the compile-time TMA pass or the run-time one.
-template <typename Real, int N, typename C>
-cudaError_t z_axis(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp, int mode,
-                   C* data, int* status, const C* tw) {
-    if constexpr (N > 0) return LaunchZ<Real, N>::zfft(st, inv, g, ncomp, data, status, tw, DFT_WAIT_POLLS, mode);
-    else return ColFft<Real>::run(st, inv, g, pz, true, T, ncomp, data, status, tw, DFT_WAIT_POLLS, mode, Real(0));
-}
-}  // namespace
 
 template <typename Real, int N>
-cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
-                                 int T, Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n,
-                                 C* slot_es, double* red_energy, const C* tw, int* status) {
-    constexpr bool kSplit = dft_zsplit<Real>(N);
-    if (kSplit || red_energy || !sp.tab_w) {
-        // z transform, k-space products, z transform
-        cudaError_t e = z_axis<Real, N>(st, false, g, pz, T, sp.S, COL_PLAIN, const_cast<C*>(in), status, tw);
-        if (e == cudaSuccess)
-            e = Passes<Real>::zmul(st, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, red_energy);
-        if (e == cudaSuccess) e = z_axis<Real, N>(st, true, g, pz, T, 1, COL_WD, slot_n, status, tw);
-        return e;
-    }
-    if constexpr (!kSplit) {
+cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                        Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
+                                        const C* tw, int* status) {
+    if constexpr (!dft_zsplit<Real>(N)) {
         constexpr int TZ = dft_tile_z<Real>(N);
         constexpr int TB = dft_tile_zf<Real>(N);
         static int optin = 0, sms = 0;
@@ -339,7 +318,7 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
         return launch_k(dftk::k_zconv_fwd_g<Real, N, TZ>, grid, dftk::kThreads, dftk::zg_smem_bytes<TZ, N>(sizeof(C)), st,
                         g.pdl, g, sp, kfx, kfy, kfz, want_psi, in, slot_n, slot_es, tw);
     }
-    return cudaSuccess;
+    return cudaErrorNotSupported;
 }
 
 namespace {
@@ -365,7 +344,7 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         }
         const size_t sm = dftk::zbwd_tma_smem<Real, N, TB>(nes);
-        if (g.zgrp || !sp.tab_w || sm > size_t(optin)) return false;
+        if (g.zgrp || sm > size_t(optin)) return false;
         // persistent CTAs, two TMA-filled stages of nine Phi' tiles, one area of ES tiles
         constexpr int NT = dft_zbwd_threads<Real>(N), MB = dft_zbwd_minb<Real>(N);
         constexpr int E = int(sizeof(C) / 8);
@@ -395,32 +374,12 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
         return true;
     }
 }
-
-// The second half as three passes, for one sample or the line search's two: the Phi' spectra
-// transformed (only where the hard-sphere part is wanted), the products, the correlations
-// transformed back.
-template <typename Real, int N, typename C>
-cudaError_t zbwd_split(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T, Real kfx,
-                    Real kfy, Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi, const C* esA,
-                    const C* esB, C* es_mat, const C* tw) {
-    int* status = const_cast<int*>(&ctl->status);
-    cudaError_t e = cudaSuccess;
-    if (flags & 1)
-        e = z_axis<Real, N>(st, false, g, pz, T, samples, COL_WD, phi, status, tw);
-    if (e == cudaSuccess)
-        e = Passes<Real>::zmul_bwd(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, samples, ctl, phi, esA, esB, es_mat);
-    if (e == cudaSuccess) e = z_axis<Real, N>(st, true, g, pz, T, samples * ncomp_out, COL_PLAIN, phi, status, tw);
-    return e;
-}
 }  // namespace
 
 template <typename Real, int N>
-cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp,
-                                 int T, Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
-                                 const C* esA, const C* esB, C* es_mat, const C* tw) {
-    if (dft_zsplit<Real>(N) || !sp.tab_w)
-        return zbwd_split<Real, N>(st, g, pz, sp, T, kfx, kfy, kfz, flags, ncomp_out, 1, ctl, phi, esA, esB, es_mat,
-                                   tw);
+cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                        Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
+                                        const C* esA, const C* esB, C* es_mat, const C* tw) {
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, 0, ctl, phi, esA, esB, es_mat, tw))
         return cudaSuccess;
     if constexpr (!dft_zsplit<Real>(N)) {
@@ -429,17 +388,13 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, cons
         return launch_k(dftk::k_zconv_bwd_g<Real, N, TZ>, grid, dftk::kThreads, dftk::zg_smem_bytes<TZ, N>(sizeof(C)), st,
                         g.pdl, g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
     }
-    return cudaSuccess;
+    return cudaErrorNotSupported;
 }
 
 template <typename Real, int N>
-cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
-                                             const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz,
-                                             int ncomp_out, const Ctl* ctl, C* phi, const C* esA, const C* esB,
-                                             const C* tw) {
-    if (dft_zsplit<Real>(N) || !sp.tab_w)
-        return zbwd_split<Real, N>(st, g, pz, sp, T, kfx, kfy, kfz, 3, ncomp_out, 2, ctl, phi, esA, esB,
-                             static_cast<C*>(nullptr), tw);
+cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                             Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                             const C* esB, const C* tw) {
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, 3, ncomp_out, 1, ctl, phi, esA, esB,
                                  static_cast<C*>(nullptr), tw))
         return cudaSuccess;
@@ -449,7 +404,7 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd_pair(cudaStream_t st, const GridDesc& g,
 template <typename Real, int N>
 bool LaunchZ<Real, N>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
     if constexpr (dft_zsplit<Real>(N)) {
-        return true;
+        return false;
     } else {
         constexpr int TB = dft_tile_zb<Real>(N);
         int dev = 0, optin = 0;

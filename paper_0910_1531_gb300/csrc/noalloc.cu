@@ -172,9 +172,13 @@ dft_status dft_weighted_densities_noalloc(const dft_params* prm, void* cuda_stre
     for (int c = 0; c < DFT_NCOMP + 2; ++c) off.v[c] = 0.f;
     e = Passes<float>::xfwd(st, g, ax, S, LX, static_cast<const float*>(rho), base + o_spec, base + o_twx);
     if (e == cudaSuccess) e = Passes<float>::yfft(st, false, g, ay, Ty, S, base + o_spec, status, base + o_twy);
+    // no |k| tables: the products pass evaluates the weights per point
     if (e == cudaSuccess)
-        e = Passes<float>::zconv_fwd(st, g, az, sp, Tz, kfx, kfy, kfz, 0, base + o_spec, base + o_n, base + o_es,
-                                     nullptr, base + o_twz, status);
+        e = Passes<float>::zfft(st, false, g, az, Tz, S, base + o_spec, status, base + o_twz, DFT_WAIT_POLLS);
+    if (e == cudaSuccess)
+        e = Passes<float>::zmul(st, g, sp, kfx, kfy, kfz, 0, base + o_spec, base + o_n, base + o_es, nullptr);
+    if (e == cudaSuccess)
+        e = Passes<float>::zfft(st, true, g, az, Tz, 1, base + o_n, status, base + o_twz, DFT_WAIT_POLLS, COL_WD);
     if (e == cudaSuccess)
         e = Passes<float>::yfft(st, true, g, ay, Ty, 1, base + o_n, status, base + o_twy, DFT_WAIT_POLLS, COL_DERIV, kfy);
     if (e == cudaSuccess)

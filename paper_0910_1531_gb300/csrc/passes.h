@@ -212,18 +212,17 @@ template <typename Real, int N>
 struct LaunchZ {
     using C = typename Cplx<Real>::type;
     static cudaError_t init();
-    static cudaError_t zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
-                          Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
-                          double* red_energy, const C* tw, int* status);
-    static cudaError_t zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
-                          Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
-                          const C* esA, const C* esB, C* es_mat, const C* tw);
-    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
-                                      const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz, int ncomp_out,
-                                      const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
+    static cudaError_t zconv_fwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                 Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, const C* tw, int* status);
+    static cudaError_t zconv_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                 Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                 const C* esB, C* es_mat, const C* tw);
+    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                      Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                      const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
-    static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                            const C* tw, long long polls, int mode);
+    static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp, C* data,
+                            int* status, const C* tw, long long polls, int mode);
 };
 
 // Column transform of a run-time length in place (k_colfft; colfft.cu): along z (zax) or y, tiles of
@@ -255,37 +254,42 @@ struct Passes {
     // of the nine weighted-density / Phi' spectra, with the y derivatives formed / added
     static cudaError_t yfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& py, int T, int ncomp, C* data,
                      int* status, const C* tw, long long polls = DFT_WAIT_POLLS, int mode = COL_PLAIN, Real kfy = 0);
-    static cudaError_t zconv_fwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
-                          Real kfx, Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
-                          double* red_energy, const C* tw, int* status);
+    // Whether a half's z stage can only run as three passes (zfft, zmul or zmul_bwd, zfft); the zconv
+    // passes, a half in one, need FP32, a compile-time length and the |k| tables, and return
+    // cudaErrorNotSupported otherwise.
+    static bool z_three(const GridDesc& g, const SpeciesDesc<Real>& sp) {
+        return dft_zsplit<Real>(dft_is_ct_size(g.nz) ? g.nz : 0) || !sp.tab_w;
+    }
+    static cudaError_t zconv_fwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                 Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, const C* tw, int* status);
     static cudaError_t xphi(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int LR, const Ctl* ctl, const C* A,
                      const C* B, C* mat, C* phi, float* red_max, int* status, double* red_phi, Real kfx,
                      const C* tw);
-    static cudaError_t zconv_bwd(cudaStream_t st, const GridDesc& g, const AxisPlan& pz, const SpeciesDesc<Real>& sp, int T,
-                          Real kfx, Real kfy, Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi,
-                          const C* esA, const C* esB, C* es_mat, const C* tw);
+    static cudaError_t zconv_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
+                                 Real kfz, int flags, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                 const C* esB, C* es_mat, const C* tw);
     // The two line-search samples' second-half z passes in one launch (both hard-sphere and ES
     // parts): phi holds sample 1's nine Phi' spectra then sample 2's, ctl[0] / ctl[1] their
     // weights; sample m's ncomp_out results go to phi components m ncomp_out ...  Only where
-    // has_zbwd_pair (the persistent TMA pass, run-time lengths); cudaErrorNotSupported otherwise.
-    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const AxisPlan& pz,
-                                      const SpeciesDesc<Real>& sp, int T, Real kfx, Real kfy, Real kfz, int ncomp_out,
-                                      const Ctl* ctl, C* phi, const C* esA, const C* esB, const C* tw);
+    // has_zbwd_pair (the persistent TMA pass); cudaErrorNotSupported otherwise.
+    static cudaError_t zconv_bwd_pair(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx,
+                                      Real kfy, Real kfz, int ncomp_out, const Ctl* ctl, C* phi, const C* esA,
+                                      const C* esB, const C* tw);
     static bool has_zbwd_pair(const GridDesc& g, int ncomp_out);
-    // The split first-half z stage (compile-time lengths): zfft = the persistent TMA z transform
-    // of ncomp components (COL_WD: of the seven of ncomp sets of nine) in place (tiles of the y
-    // pass's width; cudaErrorNotSupported for other lengths), zmul = the k-space products from the
-    // S species spectra into seven weighted-density spectra (slot_n, 1/N applied) and the S ES
-    // spectra (slot_es).
-    static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, int ncomp, C* data, int* status,
-                            const C* tw, long long polls, int mode = COL_PLAIN);
+    // The z stages in three passes: zfft = the z transform of ncomp components (COL_WD: of the seven of
+    // ncomp sets of nine) in place (k_yfft_tma or k_colfft along z), zmul = the first half's k-space
+    // products from the S species spectra into seven weighted-density spectra (slot_n, 1/N applied) and
+    // the S (want_psi: S + 1) ES spectra (slot_es); red_energy (or nullptr): energy_blocks pairs of partial
+    // sums of the grand potential.
+    static cudaError_t zfft(cudaStream_t st, bool inv, const GridDesc& g, const AxisPlan& pz, int T, int ncomp, C* data,
+                            int* status, const C* tw, long long polls, int mode = COL_PLAIN);
     static cudaError_t zmul(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
                             Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es, double* red_energy);
-    // the second half's products between its z transforms (run-time lengths): one sample or two
+    // the second half's products between its z transforms: one sample or the line search's two
     static cudaError_t zmul_bwd(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy,
                                 Real kfz, int flags, int ncomp_out, int samples, const Ctl* ctl, C* phi, const C* esA,
                                 const C* esB, C* es_mat);
-    // pairs of partial sums zconv_fwd writes to red_energy
+    // pairs of partial sums zmul writes to red_energy
     static long long energy_blocks(const GridDesc& g);
     // rho_lo (or nullptr): low part of an extended iterate rho0 + rho_lo, read
     // with rho0 and, when rho_out is written, replaced by the low part of the new iterate;

@@ -250,6 +250,32 @@ def test_profile_counts_launches():
     assert by == 2 * 9 * nc * 8     # nine weighted-density spectra in and out
     n, ms, by = plan.profile_read("yfft")
     assert n == 4
+    plan.close()
+
+
+@pytest.mark.parametrize("precision,shape", [("fp64", (32, 16, 16)), ("fp32", (20, 16, 16))])
+def test_profile_counts_the_z_stages_of_three_passes(precision, shape):
+    # FP64 and run-time z lengths: each half's z stage is a transform, the products and a transform, each
+    # counted with its own bytes; the line search's two samples share their launches
+    S = 2
+    prob, rho, V = make_case(shape, 0.1, S, seed=5)
+    plan = plan_for(prob, precision)
+    cb = shape[0] * 16 * 9 * (16 if precision == "fp64" else 8)
+    plan.profile_enable(True)
+    rd, Vd = to_dev(rho, plan), to_dev(V, plan)
+    plan.picard_map(rd, Vd)
+    assert [plan.profile_read(k)[0] for k in ("zconv_fwd", "zconv_bwd", "zmul", "zfft")] == [0, 0, 2, 4]
+    # seven of the nine weighted-density spectra; S bulk-fluid/Poisson spectra out and in
+    assert plan.profile_read("zmul")[2] == ((S + 7 + S) + (7 + S + S)) * cb
+    assert plan.profile_read("zfft")[2] == 2 * (S + 7 + 7 + S) * cb
+    plan.iter_begin(rd, Vd)
+    plan.profile_enable(True)
+    plan.iter_step(rd, Vd, -1.0)
+    assert [plan.profile_read(k)[0] for k in ("zconv_fwd", "zconv_bwd", "zmul", "zfft")] == [0, 0, 3, 6]
+    # the first half; both samples (two slots' spectra mixed); the accepted point (its mixed spectra kept)
+    assert plan.profile_read("zmul")[2] == ((S + 7 + S) + (14 + 2 * S + 2 * S) + (7 + 2 * S + S + S)) * cb
+    assert plan.profile_read("zfft")[2] == 2 * ((S + 7) + (14 + 2 * S) + (7 + S)) * cb
+    plan.close()
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
