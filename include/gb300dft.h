@@ -323,7 +323,8 @@ dft_status dft_batch_iterate(dft_batch* batch, int iters, double alpha_or_neg, d
 
 /*
  * Bound of the bounded device-side waits (failure detection; no counterpart in the paper).
- * The y passes and the z transforms move their column tiles by TMA and wait for each tile on an mbarrier; a wait
+ * The y passes and the z transforms of three-pass z stages move their column tiles by TMA and wait for
+ * each tile on an mbarrier (the one-pass z stages do too; their waits keep the default bound).  A wait
  * gives up after `polls` polls (default DFT_WAIT_POLLS_DEFAULT), the CTA then drains the copies
  * it still has in flight (those waits keep the default bound, so no copy outlives the CTA),
  * records the timeout in the plan's device status word and stops, and the call that queued the

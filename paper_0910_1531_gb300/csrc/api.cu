@@ -100,7 +100,7 @@ struct dft_plan {
     bool iter_ready = false;
     const void* iter_rho = nullptr;
     const void* iter_V = nullptr;
-    long long wait_polls = DFT_WAIT_POLLS;   // bound of the y passes' TMA tile waits
+    long long wait_polls = DFT_WAIT_POLLS;   // bound of the tile waits of the y passes and z transforms
     bool pdl_on = true;             // programmatic dependent launch of the passes (off while profiling)
 
     long long blocks_x(int LR) const { return ceil_div((long long)g.ny * g.nz, LR); }
@@ -330,12 +330,11 @@ template <typename Real> struct Ops {
         LAUNCH(p, K_YFFT, 2.0 * (p->S) * CB(p), P::yfft(p->stream, false, p->g, p->ay, p->Ty, p->S, W, &p->ctl->status, tw(p, 1), p->wait_polls));
         if (red_energy || P::z_three(p->g, sp) || (p->g.zsplit && !want_psi)) {
             // z forward transform of the species, the k-space products, z inverse of the seven
-            const long long polls = red_energy || P::z_three(p->g, sp) ? DFT_WAIT_POLLS : p->wait_polls;
-            TRY(zfft(p, false, p->S, COL_PLAIN, W, polls));
+            TRY(zfft(p, false, p->S, COL_PLAIN, W));
             LAUNCH(p, K_ZMUL, (p->S + DFT_NZSPEC + p->S + want_psi) * CB(p),
                    P::zmul(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W, slot_n(slot),
                            slot_es(p, slot), red_energy));
-            TRY(zfft(p, true, 1, COL_WD, slot_n(slot), polls));
+            TRY(zfft(p, true, 1, COL_WD, slot_n(slot)));
         } else {
             LAUNCH(p, K_ZFWD, (p->S + DFT_NZSPEC + p->S + want_psi) * CB(p),
                    P::zconv_fwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), want_psi, W, slot_n(slot),
@@ -358,9 +357,10 @@ template <typename Real> struct Ops {
     }
 
     // a z transform of a three-pass z stage: ncomp components of data, or (COL_WD) the seven of ncomp sets
-    static dft_status zfft(dft_plan* p, bool inv, int ncomp, int mode, C* data, long long polls) {
+    static dft_status zfft(dft_plan* p, bool inv, int ncomp, int mode, C* data) {
         LAUNCH(p, K_ZFFT, 2.0 * (mode == COL_WD ? ncomp * DFT_NZSPEC : ncomp) * CB(p),
-               P::zfft(p->stream, inv, p->g, p->az, p->Tz, ncomp, data, &p->ctl->status, tw(p, 2), polls, mode));
+               P::zfft(p->stream, inv, p->g, p->az, p->Tz, ncomp, data, &p->ctl->status, tw(p, 2), p->wait_polls,
+                       mode));
         return DFT_OK;
     }
 
@@ -374,11 +374,11 @@ template <typename Real> struct Ops {
         const double in = (flags & 1 ? samples * DFT_NZSPEC : 0) + (flags & 2 ? nout * (esB ? 2 : 1) : 0);
         const double bytes = (in + samples * nout + (es_mat ? nout : 0)) * CB(p);
         if (P::z_three(p->g, sp)) {
-            if (flags & 1) TRY(zfft(p, false, samples, COL_WD, T1(p), DFT_WAIT_POLLS));
+            if (flags & 1) TRY(zfft(p, false, samples, COL_WD, T1(p)));
             LAUNCH(p, K_ZMUL, bytes,
                    P::zmul_bwd(p->stream, p->g, sp, kf(p, 0), kf(p, 1), kf(p, 2), flags, nout, samples, ctl, T1(p), esA,
                                esB, es_mat));
-            return zfft(p, true, samples * nout, COL_PLAIN, T1(p), DFT_WAIT_POLLS);
+            return zfft(p, true, samples * nout, COL_PLAIN, T1(p));
         }
         if (samples == 2)
             LAUNCH(p, K_ZBWD, bytes,

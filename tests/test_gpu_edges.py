@@ -6,7 +6,8 @@ record a flag, the call returns the status, and the next call on the same plan w
 * a bath at packing fraction 0.6: the pointwise terms take the FP64 branch (n3 >= 0.5) and the
   uniform bath stays a fixed point;
 * n3 >= 1 somewhere: DFT_EN3BOUND; an infinite Boltzmann factor: DFT_ENONFINITE;
-* TMA tile waits bounded at 0 polls (each gives up at once): DFT_ETIMEOUT.
+* TMA tile waits bounded at 0 polls (each gives up at once): DFT_ETIMEOUT; the bound reaches the y
+  passes and the z transforms alike.
 """
 import numpy as np
 import pytest
@@ -130,4 +131,34 @@ def test_bounded_wait_gives_up_and_the_plan_recovers(precision):
     plan.set_wait_polls(None)
     g, _ = plan.picard_map(_dev(rho, plan), _dev(V, plan))
     assert relerr(g.cpu().numpy(), F.picard_map(prob, rho, V)) < TOL[precision]
+    plan.close()
+
+
+@pytest.mark.parametrize("precision,shape,z", [("fp64", (32, 16, 12), None), ("fp64", (20, 16, 12), None),
+                                               ("fp32", (20, 16, 12), None), ("fp32", (32, 16, 12), 2)])
+def test_wait_bound_reaches_the_z_transforms(precision, shape, z):
+    # With a bound of 0 polls no column pass transforms anything: the y passes leave the x spectra as they are,
+    # and so must the z transforms of a three-pass z stage.  The products and the x passes still run, so n0 and n1
+    # (which share a complex row and need no y derivative) are then, row by row, the x convolution of the row at
+    # (iz, iy) with the weights at that (kz, ky) index; a z transform that ignored the bound would mix the rows.
+    from oracle.weights import fmt_weights_hat
+    from oracle.fourier import kgrid
+    h = (0.1, 0.09, 0.11)
+    prob = F.Problem(shape, h, *SPECIES)
+    rho = workloads.random_density(shape, 2, prob.bath.rho, 0.3, seed=37)
+    plan = _plan(precision, shape=shape, h=h)
+    if z is not None:
+        plan.set_variants(1, 0, z)
+    plan.set_wait_polls(0)
+    n = plan.weighted_densities(_dev(rho, plan)).double().cpu().numpy()
+    plan.set_wait_polls(None)
+    nx = shape[2]
+    kz, ky, kx = np.broadcast_arrays(*kgrid(shape, h))
+    spec = np.fft.rfft(rho, axis=-1)
+    for a in (0, 1):
+        ref = 0.0
+        for s, R in enumerate(SPECIES[0]):
+            wk = fmt_weights_hat(kz, ky, kx, R)[a][..., :nx // 2 + 1]
+            ref = ref + np.fft.irfft(spec[s] * wk, n=nx, axis=-1) * nx / rho[0].size
+        assert relerr(n[a], ref) < TOL[precision], a
     plan.close()
