@@ -242,7 +242,7 @@ dft_status dft_iter_run(dft_plan* plan, void* rho_inout, const void* V, int iter
  */
 dft_status dft_autotune(dft_plan* plan, const void* rho, const void* V, int reps, int lines_out[3]);
 
-/* One line describing the plan's transform variants, radix orders and rows per block (the
+/* One line describing the plan's transform variants, radix orders, rows per block and |k| tables (the
  * defaults until dft_autotune chooses); owned by the plan, valid until its next call.  "" for NULL. */
 const char* dft_plan_tuning(const dft_plan* plan);
 

@@ -84,6 +84,8 @@ struct dft_plan {
     double prof_bytes[K_COUNT] = {0};
     std::string err;
     void* ktab = nullptr;           // |k| tables of the z passes
+    void* ktab_dk = nullptr;        // their Gamma derivatives on a non-cubic box (dft_grad's first call)
+    long long ktab_rows = 0;
     void* laptab = nullptr;         // per-axis Laplacian terms of the Poisson kernel (SpeciesDesc::lap1d)
     cudaStream_t cap = nullptr;     // capture stream of the one-iteration graph (dft_iter_run)
     cudaStream_t side = nullptr;    // copy stream of dft_picard_step_host
@@ -675,8 +677,21 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
                   double* d_bulk) {
     using O = Ops<Real>;
     using P = Passes<Real>;
-    const SpeciesDesc<Real>& sp = species<Real>(p);
+    SpeciesDesc<Real>& sp = species<Real>(p);
     const int S = p->S;
+    if (sp.tab_w && !sp.tab_dk) {
+        // the Gamma derivatives of a non-cubic box's kernels; without the memory for them the products pass
+        // evaluates its factors per point
+        if (cudaMalloc(&p->ktab_dk, size_t(p->ktab_rows) * sp.tab_ks * sizeof(Real)) == cudaSuccess) {
+            sp.tab_dk = static_cast<const Real*>(p->ktab_dk);
+            const cudaError_t e = P::build_ktab(p->stream, p->g, sp, p->kf[0], O::kf(p, 0), O::kf(p, 1), O::kf(p, 2),
+                                                p->ktab_rows, false);
+            if (e != cudaSuccess) return fail(p, DFT_ECUDA, std::string("|k| tables: ") + cudaGetErrorString(e));
+        } else {
+            cudaGetLastError();
+            p->ktab_dk = nullptr;
+        }
+    }
     const long long n_zk = P::energy_blocks(p->g);
     const long long n_phi = p->blocks_x(p->LRphi);
     const long long n_g = p->blocks_x(p->LRupd);
@@ -989,12 +1004,15 @@ void describe_tuning(dft_plan* p) {
                                           : "run-time column kernel, " + std::to_string(p->Ty) + "-column tiles, radix " +
                                                 radix_text(p->ay);
     t += "; z: ";
-    const bool zsplit = p->precision == DFT_FP64;
+    const bool tab = p->precision == DFT_FP64 ? p->spd.tab_w != nullptr : p->spf.tab_w != nullptr;
+    const bool zsplit = p->precision == DFT_FP64 || !tab;
     t += dft_is_ct_size(g.nz) ? (zsplit ? std::string("TMA z transforms around k-space products passes")
                                  : g.zgrp ? std::string("grouped, one tile per CTA") : std::string("TMA persistent"))
                               : "run-time column kernel, " + std::to_string(p->Tz) + "-column tiles, radix " +
                                     radix_text(p->az);
     if (dft_is_ct_size(g.nz) && g.zsplit && !zsplit) t += ", first half as z transforms and a k-space products pass";
+    const int oct = p->precision == DFT_FP64 ? p->spd.tab_oct : p->spf.tab_oct;
+    t += !tab ? "; |k| factors: evaluated" : oct ? "; |k| factors: table per octant point" : "; |k| factors: table per m^2";
     t += p->pdl_on ? "; launches: programmatic dependent" : "; launches: stream order";
     p->tuning = t;
 }
@@ -1438,7 +1456,11 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
     // instead of evaluating them at every point: on a cubic box, |k| = kf sqrt(mx^2 + my^2 + mz^2),
     // one record per integer m2; on others one per (kx, |ky|, |kz|), N / 8 records.  21 x 21 x 161,
     // S = 2, FP64: 16 us for the first half's products, where evaluating the sines and cosines on the
-    // FP64 pipe made that z pass 277.  A plan that cannot have the second kind (memory) evaluates per point.
+    // FP64 pipe made that z pass 277.  The second kind grows with the grid (480 x 512 x 500, S = 5, FP64:
+    // 3.2 GB beside the plan's 57), so its Gamma derivatives are left to dft_grad's first call, and a plan
+    // evaluates per point where the table would not leave the room that its own calls may ask for later:
+    // Newton's vectors for 30 directions and the staged fields of dft_picard_step_host.  Tables below 16 MB are
+    // not weighed.  DFT_KTAB_BYTES bounds the second kind further.
     {
         const bool cubic = p->kf[0] == p->kf[1] && p->kf[1] == p->kf[2];
         const long long m2max = (long long)(g.nx / 2) * (g.nx / 2) + (long long)(g.ny / 2) * (g.ny / 2) +
@@ -1448,7 +1470,17 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         // records padded to 16 bytes (read with 16-byte loads)
         const long long V = 16 / (long long)p->rsize;
         const long long ws = (2 * S + V - 1) / V * V, ks = (P + V - 1) / V * V;
-        const bool have = cudaMalloc(&p->ktab, size_t(rows * (ws + 2 * ks)) * p->rsize) == cudaSuccess;
+        const size_t bytes = size_t(rows * (ws + (cubic ? 2 : 1) * ks)) * p->rsize;
+        bool have = true;
+        if (!cubic) {
+            have = bytes <= env_budget("DFT_KTAB_BYTES", SIZE_MAX);
+            size_t room = 0, total = 0;
+            if (have && bytes >= (size_t(16) << 20))
+                have = cudaMemGetInfo(&room, &total) == cudaSuccess &&
+                       room >= bytes + size_t(31 + 6 + 2) * S * g.n * p->rsize;
+        }
+        have = have && cudaMalloc(&p->ktab, bytes) == cudaSuccess;
+        p->ktab_rows = rows;
         if (!have) {
             cudaGetLastError();
             p->ktab = nullptr;
@@ -1459,11 +1491,11 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         }
         auto fill = [&](auto* base, auto& sp) -> cudaError_t {
             using Real = std::remove_reference_t<decltype(*base)>;
-            sp.tab_w = base; sp.tab_k = base + rows * ws; sp.tab_dk = base + rows * (ws + ks);
+            sp.tab_w = base; sp.tab_k = base + rows * ws; sp.tab_dk = cubic ? base + rows * (ws + ks) : nullptr;
             sp.tab_oct = cubic ? 0 : 1;
             sp.tab_ws = (int)ws; sp.tab_ks = (int)ks;
             return Passes<Real>::build_ktab(nullptr, g, sp, p->kf[0], Real(p->kf[0]), Real(p->kf[1]), Real(p->kf[2]),
-                                            rows);
+                                            rows, true);
         };
         cudaError_t te = cudaSuccess;
         if (have) te = f64 ? fill(static_cast<double*>(p->ktab), p->spd) : fill(static_cast<float*>(p->ktab), p->spf);
@@ -1531,6 +1563,7 @@ dft_status dft_plan_destroy(dft_plan* p) {
     cudaFree(p->red_max);
     cudaFree(p->grad_red);
     cudaFree(p->ktab);
+    cudaFree(p->ktab_dk);
     cudaFree(p->laptab);
     cudaFree(p->red_canon);
     release_iter_graph(p);

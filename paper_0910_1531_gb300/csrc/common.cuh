@@ -241,7 +241,7 @@ struct SpeciesDesc {
     // point.
     const Real* tab_w;                  // [row][tab_ws]: w0_s at 2 s, j3_s at 2 s + 1
     const Real* tab_k;                  // [row][tab_ks]: DC_ij_hat at j (j + 1) / 2 + i, i <= j
-    const Real* tab_dk;                 // [row][tab_ks]: d DC_ij_hat / d Gamma, same order
+    const Real* tab_dk;                 // [row][tab_ks]: d DC_ij_hat / d Gamma, same order (or null)
     int tab_oct;
     int tab_ws, tab_ks;                 // record lengths: 2 S and S (S + 1) / 2 rounded up to 16 bytes
     // Optional per-axis terms of the discrete Laplacian, sin^2(k_d h_d / 2) / h_d^2 by FFT index:

@@ -65,10 +65,10 @@ cudaError_t Passes<Real>::canon_scale(cudaStream_t st, Ctl* ctl, const SpeciesDe
 
 template <typename Real>
 cudaError_t Passes<Real>::build_ktab(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, double kf,
-                                     Real kfx, Real kfy, Real kfz, long long rows) {
+                                     Real kfx, Real kfy, Real kfz, long long rows, bool all) {
     dftk::k_ktab<Real><<<(unsigned)ceil_div(rows, 256), 256, 0, st>>>(
-        g, sp, kf, kfx, kfy, kfz, rows, const_cast<Real*>(sp.tab_w), const_cast<Real*>(sp.tab_k),
-        const_cast<Real*>(sp.tab_dk));
+        g, sp, kf, kfx, kfy, kfz, rows, all ? const_cast<Real*>(sp.tab_w) : nullptr,
+        all ? const_cast<Real*>(sp.tab_k) : nullptr, const_cast<Real*>(sp.tab_dk));
     return cudaGetLastError();
 }
 
@@ -157,7 +157,7 @@ unsigned zmul_blocks(const GridDesc& g) {
 namespace {
 // The instance of a products kernel for a plan's species count and tables.
 template <bool GRAD, typename Real> auto zmul_kernel(const SpeciesDesc<Real>& sp) {
-    if (!sp.tab_w) return dftk::k_zmul<Real, GRAD, false, DFT_MAXS>;
+    if (!sp.tab_w || (GRAD && !sp.tab_dk)) return dftk::k_zmul<Real, GRAD, false, DFT_MAXS>;
     switch (sp.S) {
         case 1: case 2: return dftk::k_zmul<Real, GRAD, true, 2>;
         case 3: return dftk::k_zmul<Real, GRAD, true, 3>;

@@ -824,7 +824,7 @@ template <typename Real> __host__ __device__ constexpr int tab_capacity(int n) {
 // DC_ij_hat with its Gamma derivative.  On a cubic box (kf equal on the three axes) one record per
 // integer m2 = mx^2 + my^2 + mz^2, |k| = kf sqrt(m2); on other boxes (sp.tab_oct) one per (kx, |ky|,
 // |kz|), |k| as kpoint forms it.  Evaluated once per plan with the functions the z passes call
-// where there is no table.
+// where there is no table; a null table is left out.
 template <typename Real>
 __global__ void k_ktab(GridDesc g, SpeciesDesc<Real> sp, double kf, Real kfx, Real kfy, Real kfz, long long rows,
                        Real* tab_w, Real* tab_k, Real* tab_dk) {
@@ -839,19 +839,20 @@ __global__ void k_ktab(GridDesc g, SpeciesDesc<Real> sp, double kf, Real kfx, Re
     } else {
         kmag = Real(kf * sqrt(double(row)));
     }
-    for (int s = 0; s < S; ++s) {
-        Real w0, j3;
-        fmt_weights<Real>(kmag, sp.R[s], &w0, &j3);
-        tab_w[row * sp.tab_ws + 2 * s] = w0;
-        tab_w[row * sp.tab_ws + 2 * s + 1] = j3;
-    }
+    if (tab_w)
+        for (int s = 0; s < S; ++s) {
+            Real w0, j3;
+            fmt_weights<Real>(kmag, sp.R[s], &w0, &j3);
+            tab_w[row * sp.tab_ws + 2 * s] = w0;
+            tab_w[row * sp.tab_ws + 2 * s + 1] = j3;
+        }
     for (int j = 0; j < S; ++j)
         for (int i = 0; i <= j; ++i) {
             Real dG = Real(0);
             const Real K = delta_c_hat<Real>(kmag, sp.es_R[i][j], sp.es_pref[i][j], sp.es_a[i][j], sp.es_b[i][j],
                                              sp.es_c[i][j], &dG, sp.es_da[i][j], sp.es_db[i][j], sp.es_dc[i][j]);
-            tab_k[row * sp.tab_ks + dft_pair(i, j)] = K;
-            tab_dk[row * sp.tab_ks + dft_pair(i, j)] = dG;
+            if (tab_k) tab_k[row * sp.tab_ks + dft_pair(i, j)] = K;
+            if (tab_dk) tab_dk[row * sp.tab_ks + dft_pair(i, j)] = dG;
         }
 }
 

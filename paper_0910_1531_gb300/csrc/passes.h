@@ -321,10 +321,10 @@ struct Passes {
                               int LR, const C* cspec, const Real* V, double* red, const C* tw);
     static cudaError_t canon_scale(cudaStream_t st, Ctl* ctl, const SpeciesDesc<Real>& sp, const double* red,
                                    int nblocks, int pdl);
-    // fill the `rows` rows of the |k| tables of sp (tab_w, tab_k, tab_dk, tab_oct set by the caller);
-    // kf: the wave number of a cubic box
+    // fill the `rows` rows of the |k| tables of sp (tab_w and tab_k unless !all, tab_dk where it is not
+    // null; they and tab_oct set by the caller); kf: the wave number of a cubic box
     static cudaError_t build_ktab(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, double kf, Real kfx,
-                                  Real kfy, Real kfz, long long rows);
+                                  Real kfy, Real kfz, long long rows, bool all);
     // fill out[nx + ny + nz] with the per-axis Laplacian terms of grid g (SpeciesDesc::lap1d)
     static cudaError_t build_laptab(cudaStream_t st, const GridDesc& g, Real kfx, Real kfy, Real kfz, Real* out);
 };

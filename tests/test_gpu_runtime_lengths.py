@@ -14,6 +14,7 @@ import numpy as np
 import pytest
 
 from oracle import functional as F
+from oracle import picard as P
 from paper_0910_1531_gb300 import workloads
 
 pytestmark = pytest.mark.gpu
@@ -59,3 +60,47 @@ def test_runtime_lengths_match_the_oracle(shape, precision):
     g, _ = plan.picard_map(dev(rho), dev(V))
     assert relerr(g.double().cpu().numpy(), g_ref) < TOL[precision], plan.tuning()
     plan.close()
+
+
+FIVE = ([0.095, 0.099, 0.181, 0.14, 0.12], [1.0, 2.0, -1.0, -0.5, 0.0], [0.1, 0.01, 0.1, 0.04, 0.3])
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("shape,species", [((32, 12, 20), SPECIES), ((18, 32, 21), SPECIES), ((32, 12, 20), FIVE)])
+def test_plans_without_a_k_table_match_the_oracle(shape, species, precision, monkeypatch):
+    # a non-cubic box's |k| table holds one record per octant point (weights 2 S, kernels S (S + 1) / 2, each rounded
+    # up to 16 bytes, and no Gamma derivatives before dft_grad asks for them); a plan that cannot have it evaluates
+    # the factors per point, in the weighted densities, G, the line search's paired samples and the gradients
+    from paper_0910_1531_gb300 import binding
+    prob = F.Problem(shape, (0.11, 0.1, 0.09), *species)
+    S = len(species[0])
+    v = 4 if precision == "fp32" else 2
+    up = lambda n: (n + v - 1) // v * v
+    size = (shape[2] // 2 + 1) * (shape[1] // 2 + 1) * (shape[0] // 2 + 1) * (up(2 * S) + up(S * (S + 1) // 2)) * 16 // v
+    rho = workloads.random_density(shape, S, prob.bath.rho, 0.3, seed=67)
+    V = np.zeros_like(rho)
+    V[0, : shape[0] // 3] = np.inf
+    rho[0, : shape[0] // 3] = 0.0
+    g_ref, om_ref = F.picard_map(prob, rho, V), F.grand_potential(prob, rho, V)
+    d_ref = F.grad_omega_rho(prob, rho, V)
+    b_ref = F.grad_omega_bulk(shape, prob.h, *species, rho, V)
+    step_ref, _ = P.picard_step(prob, rho, V, g0=g_ref)
+    for limit, table in ((size, True), (size - 1, False)):
+        monkeypatch.setenv("DFT_KTAB_BYTES", str(limit))
+        plan = binding.Plan(shape, prob.h, *species, precision=precision)
+        assert ("table per octant point" in plan.tuning()) == table, plan.tuning()
+        dev = lambda x: torch.tensor(np.ascontiguousarray(x), dtype=plan.dtype, device="cuda")
+        n, n_ref = plan.weighted_densities(dev(rho)).double().cpu().numpy(), F.weighted_densities(prob, rho)
+        for f in FIELDS:
+            assert relerr(n[f], n_ref[f]) < TOL[precision], (f, table)
+        g, _ = plan.picard_map(dev(rho), dev(V))
+        assert relerr(g.double().cpu().numpy(), g_ref) < TOL[precision], table
+        om, d_rho, _, d_bulk = plan.grad(dev(rho), dev(V))
+        assert om == pytest.approx(om_ref, rel=TOL[precision])
+        assert relerr(d_rho.double().cpu().numpy(), d_ref) < TOL[precision], table
+        # bath derivatives: central differences of the oracle
+        assert np.allclose(d_bulk, b_ref, rtol=2e-3 if precision == "fp32" else 1e-6, atol=0), table
+        r = dev(rho)
+        plan.picard_step(r, dev(V), -1.0)
+        assert relerr(r.double().cpu().numpy(), step_ref) < TOL[precision], table
+        plan.close()
