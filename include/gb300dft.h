@@ -251,7 +251,8 @@ const char* dft_plan_tuning(const dft_plan* plan);
  * run-time ones under candidate radix order k (in dft_autotune's order; DFT_EINVAL past the
  * last); x_persistent 1 = with the compile-time kernels, the Phi' passes as the persistent
  * kernel whose row blocks arrive by bulk copies two blocks ahead, 2 = by per-thread cp.async
- * copies one block ahead (0 = one CTA per row block);
+ * copies one block ahead (0 = one CTA per row block); either takes fewer rows per block where the
+ * plan's own choice does not leave it the shared memory;
  * y_variant 0 = persistent TMA pass of the compile-time length (lengths without one run the run-time
  * column kernel), 1 = run-time column kernel; z_variant bit 0: 0 = persistent TMA passes, 1 =
  * grouped one-tile-per-CTA kernels; bit 1: the first half's z stage as three passes (persistent TMA z

@@ -72,6 +72,7 @@ struct dft_plan {
     Ctl* ctl_host = nullptr;
     int Ty = 1, Tz = 1, LX = 1, LRphi = 1, LRupd = 1;
     int LRphi2 = 1, LRupd2 = 1;     // rows per block of the paired-sample x passes
+    int rows_phi[2] = {1, 1};       // LRphi, LRphi2 as plan creation or the autotuner chose them
     int LRn3 = 2;                   // rows per block of the n3-maximum x pass
     SpeciesDesc<float> spf{};
     SpeciesDesc<double> spd{};
@@ -1118,12 +1119,13 @@ template <typename Real> dft_status autotune_t(dft_plan* p, const Real* rho, con
             int bp[2] = {p->LRphi, p->LRphi2};
             float bpm[2] = {1e30f, 1e30f};
             for (int L : cand) {
-                float ms = time_it([&] {
+                // (with more rows than fit, the per-block kernel would be timed)
+                float ms = P::xphi_rows(p->g, 1, L) < L ? 1e30f : time_it([&] {
                     P::xphi(p->stream, p->g, p->ax, L, p->ctl, A, A, nullptr, O::T1(p), p->red_max, &p->ctl->status,
                             nullptr, O::kf(p, 0), O::tw(p, 0));
                 });
                 if (ms < bpm[0]) { bpm[0] = ms; bp[0] = L; }
-                ms = time_it([&] {
+                ms = P::xphi_rows(p->g, 2, L) < L ? 1e30f : time_it([&] {
                     P::xphi2(p->stream, p->g, p->ax, L, p->ctl, A, A, O::T1(p), &p->ctl->status, O::kf(p, 0),
                              O::tw(p, 0));
                 });
@@ -1396,6 +1398,8 @@ dft_status dft_plan_create(const dft_params* prm, void* cuda_stream, dft_plan** 
         p->LRphi2 = spread_rows(p, rows, 10, phi_budget);
         p->LRupd2 = spread_rows(p, rows, 2 * lpr, upd_budget);
         p->LRn3 = 2 * spread_rows(p, rows / 2, 1, fwd_budget);
+        p->rows_phi[0] = p->LRphi;
+        p->rows_phi[1] = p->LRphi2;
     }
     if (f64) fill_species<double>(p);
     else fill_species<float>(p);
@@ -1792,6 +1796,8 @@ dft_status dft_autotune(dft_plan* p, const void* rho, const void* V, int reps, i
         g_tune_cache[key] = TuneResult{{p->LX, p->LRphi, p->LRupd, p->LRn3, p->LRphi2, p->LRupd2},
                                        p->g.xrt, p->g.xpers, p->g.yrt, p->g.zgrp, p->g.zsplit, p->ax};
     }
+    p->rows_phi[0] = p->LRphi;
+    p->rows_phi[1] = p->LRphi2;
     // the iteration state and its graph depend on the block counts and variants
     p->iter_ready = false;
     release_iter_graph(p);
@@ -2131,6 +2137,14 @@ dft_status dft_set_variants(dft_plan* p, int x_variant, int x_persistent, int y_
         return fail(p, DFT_EINVAL, "the y variant is 0 or 1, the z variant 0 to 3");
     p->g.xrt = x_variant > 0 ? 1 : 0;
     p->g.xpers = x_persistent;
+    // a pinned persistent Phi' pass takes the rows that fit its prefetch areas
+    const bool pers = x_variant == 0 && x_persistent > 0;
+    for (int m = 0; m < 2; ++m) {
+        int& rows = m == 0 ? p->LRphi : p->LRphi2;
+        rows = p->rows_phi[m];
+        if (pers)
+            rows = is_fp64(p) ? Passes<double>::xphi_rows(p->g, m + 1, rows) : Passes<float>::xphi_rows(p->g, m + 1, rows);
+    }
     if (x_variant > 0) p->ax = orders[x_variant - 1];
     else dft_mixed_plan(p->g.nx, &p->ax);
     p->g.yrt = y_variant;

@@ -213,6 +213,11 @@ cudaError_t Passes<Real>::xphi2(cudaStream_t st, const GridDesc& g, const AxisPl
 }
 
 template <typename Real>
+int Passes<Real>::xphi_rows(const GridDesc& g, int nm, int LR) {
+    DFT_SWITCH_X(g.nx, xphi_rows(g, nm, LR))
+}
+
+template <typename Real>
 cudaError_t Passes<Real>::xupdate2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, const SpeciesDesc<Real>& sp,
                                    int LR, const Ctl* ctl, const C* cspec, const C* cspec2, const Real* rho0,
                                    const Real* rho1, const Real* V, Real* rho_lo, double* red_sum, double* red_sum2,

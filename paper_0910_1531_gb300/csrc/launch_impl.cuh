@@ -96,6 +96,22 @@ cudaError_t LaunchX<Real, N>::xphi(cudaStream_t st, const GridDesc& g, const Axi
 }
 
 template <typename Real, int N>
+int LaunchX<Real, N>::xphi_rows(const GridDesc& g, int nm, int LR) {
+    if constexpr (N > 0) {
+        int dev = 0, optin = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        auto smem = [&](int L) {        // both slots read
+            return g.xpers == 2 ? dftk::xphi_cpa_smem<Real, N>(nm, L, 2 * DFT_NSPEC, g.pxh)
+                                : dftk::xphi_tma_smem<Real, N>(nm, L, 2 * DFT_NSPEC, g.pxh);
+        };
+        for (int L = LR; g.xpers && L >= 1; --L)
+            if (smem(L) <= size_t(optin)) return L;
+    }
+    return LR;
+}
+
+template <typename Real, int N>
 cudaError_t LaunchX<Real, N>::xphi2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int LR, const Ctl* ctl,
                                     const C* A, const C* B, C* phi, int* status, Real kfx, const C* tw) {
     if (launch_xphi_tma<Real, N, 2>(st, g, LR, ctl, A, B, static_cast<C*>(nullptr), phi, static_cast<float*>(nullptr),

@@ -186,6 +186,7 @@ struct LaunchX {
     // red_sum2; nothing written to rho or G)
     static cudaError_t xphi2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int LR, const Ctl* ctl,
                              const C* A, const C* B, C* phi, int* status, Real kfx, const C* tw);
+    static int xphi_rows(const GridDesc& g, int nm, int LR);
     static cudaError_t xupdate2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, const SpeciesDesc<Real>& sp,
                                 int LR, const Ctl* ctl, const C* cspec, const C* cspec2, const Real* rho0,
                                 const Real* rho1, const Real* V, Real* rho_lo, double* red_sum, double* red_sum2,
@@ -305,6 +306,9 @@ struct Passes {
     // red_sum2; nothing written to rho or G)
     static cudaError_t xphi2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, int LR, const Ctl* ctl,
                              const C* A, const C* B, C* phi, int* status, Real kfx, const C* tw);
+    // Rows per block, at most LR, with which the persistent form of g.xpers of the Phi' pass of nm mixtures
+    // fits the shared memory (LR itself where none is asked for or not even one row fits).
+    static int xphi_rows(const GridDesc& g, int nm, int LR);
     static cudaError_t xupdate2(cudaStream_t st, const GridDesc& g, const AxisPlan& px, const SpeciesDesc<Real>& sp,
                                 int LR, const Ctl* ctl, const C* cspec, const C* cspec2, const Real* rho0,
                                 const Real* rho1, const Real* V, Real* rho_lo, double* red_sum, double* red_sum2,

@@ -110,6 +110,31 @@ def test_line_search_steps_under_variants_fp64(which):
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("shape", [(64, 32, 128), (64, 64, 64), (8, 32, 256)])
+@pytest.mark.parametrize("xp", [1, 2])
+def test_a_pinned_persistent_pass_runs(precision, shape, xp):
+    # A persistent Phi' pass holds its row blocks' spectra of both slots in shared memory, twice with bulk copies
+    # (xp 1): 18 x 2 or 18 half rows of nx / 2 + 1 elements (rounded up to even) per row, beside five complex lines
+    # per mixture in two buffers.  With more rows per block than that leaves, the per-block kernel would run under the
+    # persistent one's name; the pinned form takes fewer rows, and unpinned the plan has its own again.
+    import re
+    from paper_0910_1531_gb300 import binding
+    prob, rho, V = _case(shape, (0.05, 0.06, 0.07), seed=59)
+    plan = binding.Plan(shape, prob.h, *SPECIES, precision=precision)
+    rows = lambda: tuple(int(re.search(k + r" (\d+)", plan.tuning()).group(1)) for k in (", xphi", "paired xphi"))
+    before = rows()
+    plan.set_variants(0, 0, 0, x_persistent=xp)
+    nx, pxh, c = shape[2], (shape[2] // 2 + 2) & ~1, 8 if precision == "fp32" else 16
+    for m, L in enumerate(rows(), 1):
+        assert (nx + (36 if xp == 1 else 18) * L * pxh + 10 * m * L * nx) * c <= 227 * 1024, (m, L)
+    g, _ = plan.picard_map(_dev(rho, plan), _dev(V, plan))
+    assert relerr(g.double().cpu().numpy(), F.picard_map(prob, rho, V)) < TOL[precision], plan.tuning()
+    plan.set_variants(0, 0, 0)
+    assert rows() == before
+    plan.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_autotuned_choice_matches_oracle(precision):
     from paper_0910_1531_gb300 import binding
     shape = (32, 64, 128)
