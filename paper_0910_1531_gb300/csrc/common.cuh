@@ -117,6 +117,9 @@ inline bool dft_radix_plan(int n, AxisPlan* out) {
 // 16-column tile, averaged with the same without the rounding to whole waves (other tiles of the
 // SM fill it), and a barrier.  Two stages of near-equal radices win for most lengths (160 =
 // 16 x 10, 120 = 12 x 10, 84 = 12 x 7), three above 256.
+// At most DFT_RT_STAGES of them: k_colfft's buffers rotate over three stages, and every length up to 512 with
+// prime factors up to 31 has such a plan.
+#define DFT_RT_STAGES 3
 inline bool dft_mixed_plan(int n, AxisPlan* out) {
     static const struct { int r; double flops; } kR[] = {
         {31, 55}, {29, 52}, {23, 44}, {19, 39}, {17, 36}, {13, 27}, {11, 24}, {16, 10.5}, {15, 10}, {14, 11},
@@ -131,7 +134,7 @@ inline bool dft_mixed_plan(int n, AxisPlan* out) {
             best_cost = cost;
             return;
         }
-        if (cur.nstages == DFT_MAXSTAGES) return;
+        if (cur.nstages == DFT_RT_STAGES) return;
         for (int i = from; i < int(sizeof(kR) / sizeof(kR[0])); ++i) {
             const int r = kR[i].r;
             if (rem % r) continue;

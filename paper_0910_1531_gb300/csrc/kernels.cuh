@@ -498,7 +498,8 @@ __global__ void __launch_bounds__(kThreads, BIG ? 1 : (sizeof(Real) == 4 && T < 
     const uint32_t bytes = uint32_t(cb.nbox) * uint32_t(cb.rows * cb.planes) * uint32_t(T * sizeof(C));
     const RtCols<T> cols(cb.planes, cb.n, zax != 0);
     const bool sets = MODE != COL_PLAIN || wd;
-    const int nst = pa.nstages;     // 1 to 3
+    const int nst = pa.nstages;     // 1 to DFT_RT_STAGES
+    static_assert(DFT_RT_STAGES == 3, "the buffers below rotate over three stages");
     if (threadIdx.x == 0) {
         tma::mbar_init(&bar[0], 1);
         tma::mbar_init(&bar[1], 1);

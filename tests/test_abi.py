@@ -86,3 +86,27 @@ def test_plan_create_accepts_prime_factors_up_to_31(lib, nx, ny, nz):
     if handle.value:
         lib.dft_plan_destroy(handle)
     assert st != -1, lib.dft_last_error(None)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_every_length_has_a_plan_of_three_stages(lib, axis):
+    # the run-time column transform holds plans of at most three radix stages; a length without one would be
+    # refused (DFT_EINVAL), so every length of 4..512 with prime factors up to 31 must have one, and no other
+    def factors(n):
+        p = 2
+        while p * p <= n:
+            while n % p == 0:
+                yield p
+                n //= p
+            p += 1
+        if n > 1:
+            yield n
+    for n in range(2, 516):
+        size = [8, 8, 8]
+        size[axis] = n
+        prm, keep = _params(*size)
+        handle = ctypes.c_void_p()
+        st = lib.dft_plan_create(ctypes.byref(prm), None, ctypes.byref(handle))
+        if handle.value:
+            lib.dft_plan_destroy(handle)
+        assert (st != -1) == (4 <= n <= 512 and max(factors(n)) <= 31), (n, lib.dft_last_error(None))
