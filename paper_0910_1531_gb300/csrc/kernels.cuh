@@ -1427,7 +1427,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 3 : 2) k_zmul_bw
                 C out = cscale(ea[s], wA);
                 if (esB) out = cadd(out, cscale(eb[s], wB));
                 if (es_mat) es_mat[(long long)s * g.nc + o] = out;
-                if (hs && s < SM) {
+                if (hs && s < S && s < SM) {        // a psi component (s = S) has no hard-sphere part
                     Real w0, j3;
                     if constexpr (TAB) { w0 = wr[2 * (s < SM ? s : 0)]; j3 = wr[2 * (s < SM ? s : 0) + 1]; }
                     else fmt_weights<Real>(kpoint<Real>(g, kxi, kyi, kzi, kfx, kfy, kfz).kmag(), sp.R[s], &w0, &j3);
