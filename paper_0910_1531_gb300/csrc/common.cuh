@@ -15,7 +15,7 @@
 // Weighted-density spectra kept between the passes: n0 n1 n2 n3, m (n_V1 = grad m), then
 // i k_y m, i k_z m, i k_y n3, i k_z n3.  The x components i k_x m and i k_x n3 are formed in
 // the x pass that takes the spectra to real space (and the divergence terms of the back
-// convolution in the x pass that leaves it), so the y and z passes carry nine components.
+// convolution in the x pass that leaves it), so the y passes carry nine components.
 #define DFT_NSPEC 9
 // Of these the z passes carry seven: i k_y m and i k_y n3 (and on the way back the -i k_y terms) are
 // formed in the y pass, whose tiles hold all k_y.  Component of the q-th of them:

@@ -86,7 +86,7 @@ int Passes<Real>::tile_y(const GridDesc& g) {
 
 template <typename Real>
 int Passes<Real>::tile_z(const GridDesc& g) {
-    return dft_is_ct_size(g.nz) ? dft_tile_z<Real>(g.nz) : dft_tile_rt<Real>(g.nz, g.nxh, g.ny, g.pxh);
+    return dft_tile_rt<Real>(g.nz, g.nxh, g.ny, g.pxh);
 }
 
 template <typename Real>

@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kThreads, dft_yfft_minb<Real>(NY)) k_yfft_tma(
 // zero and are not written) of one component, moved as one box, or, past 256 rows, two.
 // Memory-bound in FP32: at 160^3 8.9 us a component (3.8 TB/s; a column pass of plain tile loads,
 // divisions by run-time integers and odd primes by their R^2 terms took 44).  FP64 is bound by the
-// FP64 pipe: 21 x 21 x 161, z forward, nine components 75 us.
+// FP64 pipe: 21 x 21 x 161 (161 = 7 x 23), z forward 6.9 us a component.
 // Shared memory: stage 0 | stage 1 | X | Y (only with two or more stages) | twiddles | 2 mbarriers.
 // ------------------------------------------------------------------------------------
 struct ColBox {
@@ -667,25 +667,25 @@ __device__ __forceinline__ Real kz_of(const SpeciesDesc<Real>& sp, const GridDes
 
 // ------------------------------------------------------------------------------------
 // The z passes.  First half: the S half spectra of the densities after x, y forward (kx, ky, z) ->
-//   slot_n:  the nine weighted-density spectra, 1/N applied, after z inverse (kx, ky, z)
+//   slot_n:  seven of the nine weighted-density spectra (dft_zcomp), 1/N applied, after z inverse (kx, ky, z)
 //   slot_es: S (+1 with psi) unnormalised bulk-fluid/Poisson spectra sum_j K_ij drho_hat_j (kx, ky, kz)
-// Second half: the nine Phi' spectra after x, y forward (kx, ky, z) ->
+// Second half: seven Phi' spectra after x, y forward (kx, ky, z), the y derivatives added ->
 //   the S one-body correlation spectra after z inverse, 1/N applied (kx, ky, z), in their place.
 //   mu_hat_i = sum_alpha Phi_hat_alpha w_hat_i^alpha(+k) (eq. muHS): with the vector weights
 //   w_hat^V2 = -i k w_hat^3 and w_hat^V1 = w_hat^V2/(4 pi R) the k-space sum needs only the five
 //   species-independent spectra Phi0, Phi1, Phi2, Phi3 + div(PhiV2), div(PhiV1).
 //   c_hat_i = (-mu_hat_i + wA es_A_i + wB es_B_i) / N.
 //   flags: 1 = hard-sphere part, 2 = electrostatic part; ncomp_out = S (or S + 1 for psi).
-// Compile-time lengths do a half in one pass (below); run-time lengths, and compile-time ones
-// where it is faster, as a z transform (k_colfft / k_yfft_tma), a k-space products pass (k_zmul,
-// k_zmul_bwd) and another z transform.
+// FP32 plans do a half of a compile-time length in one pass (below); FP64 plans, run-time lengths, plans
+// without |k| tables and a first half where it is faster run a z transform (k_colfft / k_yfft_tma), a
+// k-space products pass (k_zmul, k_zmul_bwd) and another z transform.
 // ------------------------------------------------------------------------------------
 // ------------------------------------------------------------------------------------
 // Grouped z passes (compile-time length NZ, tile width TZ), grid (ceil(nxh/TZ), ny).  All
 // components of a column tile are loaded in one batch of in-flight loads and transformed by
 // one grouped FFT (ct_fft_grouped), so every stage keeps the CTA's threads busy and a tile
 // costs a handful of barriers instead of a dozen transforms of one component each.
-// Shared memory: twiddles | 10 tiles | 10 tiles (ct_gstride(NZ, TZ, csize) elements each).
+// Shared memory: twiddles | 7 tiles | 7 tiles (ct_gstride(NZ, TZ, csize) elements each).
 // ------------------------------------------------------------------------------------
 // One species' contribution, 1/N applied, to the spectra acc = (n0, n1, n2, n3, m) at a k point:
 // the weights are w0 (1, R, 4 pi R^2) and j3 (4 pi R^3, R^2), so v is scaled by each of w0 and j3
@@ -865,8 +865,8 @@ __device__ __forceinline__ long long tab_row(const SpeciesDesc<Real>& sp, const 
     return kxi * kxi + my * my + mz * mz;
 }
 
-// First-half z pass: S species spectra in, the nine weighted
-// densities (z inverse, 1/N applied) and the bulk-fluid/Poisson spectra out.  Per-species loops
+// First-half z pass: S species spectra in, seven weighted-density
+// spectra (z inverse, 1/N applied) and the bulk-fluid/Poisson spectra out.  Per-species loops
 // run to DFT_MAXS with guards so that every per-point array stays in registers.
 template <typename Real, int NZ, int TZ>
 __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, SpeciesDesc<Real> sp, Real kfx, Real kfy,
@@ -897,7 +897,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
     C* O = (R == A) ? B : A;
 
     const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
-    const Real fourpi = Real(4.0 * CUDART_PI);
     const int my = signed_index(kyi, ny);
     Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
     for (int s = 0; s < S; ++s)
@@ -968,7 +967,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_fwd_g(GridDesc g, Species
     tiles_store_grouped<TZ, NZ, true>(slot_n + col0, Q, g.nc, DFT_NZSPEC, zstride, nxh - kx0);
 }
 
-// Second-half z pass: the nine Phi' spectra in (flags & 1), the
+// Second-half z pass: seven Phi' spectra in (flags & 1), the
 // bulk-fluid/Poisson spectra mixed in (flags & 2), ncomp_out one-body correlation spectra out.
 // The points of a thread are handled together so that all of their global and table loads are
 // in flight at once.
@@ -1007,7 +1006,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_zconv_bwd_g(GridDesc g, Species
         R = ct_fft_grouped<NZ, false, TZ, GS>(A, B, DFT_NZSPEC, tw);
     }
     C* O = (R == A) ? B : A;
-    const Real fourpi = Real(4.0 * CUDART_PI);
     const int my = signed_index(kyi, ny);
 
     // loads first: bulk-fluid/Poisson spectra and table records of all of this thread's points
@@ -1136,7 +1134,6 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
         }
     }
     const Real hx = Real(g.hx), hy = Real(g.hy), hz = Real(g.hz);
-    const Real fourpi = Real(4.0 * CUDART_PI);
     Real flb = Real(0);      // 4 pi lambda_B = pois[s][s] / z_s^2 of a charged species
     for (int s = 0; s < S; ++s)
         if (sp.z[s] != Real(0)) { flb = sp.pois[s][s] / (sp.z[s] * sp.z[s]); break; }
@@ -1249,10 +1246,10 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_fwd_tma(const __grid_constan
 }
 
 // ------------------------------------------------------------------------------------
-// The k-space products of the first half as a pass of their own (the split first-half z stage:
-// z forward transform of the S species, this pass, z inverse transform of the nine weighted
-// densities).  At each k point of the S species spectra (after the x, y and z forward
-// transforms) the nine weighted-density spectra, 1/N applied, into slot_n and the S
+// The k-space products of the first half as a pass of their own (the first-half z stage in three:
+// z forward transform of the S species, this pass, z inverse transform of seven weighted-density
+// spectra).  At each k point of the S species spectra (after the x, y and z forward
+// transforms) the seven weighted-density spectra, 1/N applied, into slot_n and the S
 // bulk-fluid/Poisson spectra into slot_es, both in (kx, ky, kz); the same arithmetic per point as
 // k_zconv_fwd_tma.  One thread per k point, kx fastest.
 // ------------------------------------------------------------------------------------
@@ -1505,7 +1502,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
     const int S = sp.S, ny = g.ny, nxh = g.nxh;
     const long long zstride = (long long)ny * g.pxh;
     // Work items: tiles, or (pair) each tile twice, for the two line-search samples in turn
-    // (sample m's nine Phi' spectra at components 9 m .. 9 m + 8 of map_phi, its weights in
+    // (sample m's Phi' spectra at components 9 m + dft_zcomp(q) of map_phi, its weights in
     // ctl[m], its results to components m ncomp_out .. of map_out); the ES tiles of a tile are
     // loaded once for both.
     const int shift = pair ? 1 : 0;
@@ -1553,7 +1550,6 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
             if (es_issued > es_consumed) tma::mbar_wait(&bar[2], (es_issued - 1) & 1);
         }
     };
-    const Real fourpi = Real(4.0 * CUDART_PI);
     for (int it = 0;; ++it) {
         const int tile = item_tile(it);
         if (tile >= ntiles) break;
@@ -1616,7 +1612,7 @@ __global__ void __launch_bounds__(NT, MINB) k_zconv_bwd_tma(const __grid_constan
                     load_record(wr, sp.tab_w + (kxi < nxh ? tab_row(sp, g, kxi, my, kzi) : 0) * sp.tab_ws, 2 * S);
                 C asum[5];
                 bwd_sums<Real>(X, GS, pos, kz_of(sp, g, kzi, kfz), asum);
-    #pragma unroll
+#pragma unroll
                 for (int s = 0; s < SM; ++s) {
                     if (s >= S) break;
                     out[s] = bwd_species<Real>(asum, sp, s, wr[2 * s], wr[2 * s + 1], out[s]);
@@ -1778,8 +1774,6 @@ __host__ __device__ constexpr int wd_line(int c) {
 }
 __host__ __device__ constexpr int wd_slot(int c) { return (c == 1 || c == 5 || c == 7 || c == 6 || c == 9) ? 1 : 0; }
 
-// Load the Hermitian half rows of two components (mixed wA * A + wB * B) as Z = a + i b over the
-// full length nx (Z[nx-k] = conj(a_k) + i conj(b_k)).  Optionally stores the mixed half rows.
 // Items in flight per thread in the update pass's pointwise phase (build flag).
 #ifndef DFT_XUPD_BATCH
 #define DFT_XUPD_BATCH 1
@@ -1812,6 +1806,8 @@ __device__ __forceinline__ float& vel(float4& v, int e) { return e == 0 ? v.x : 
 __device__ __forceinline__ double& vel(double2& v, int e) { return e == 0 ? v.x : v.y; }
 template <typename V> __device__ __forceinline__ V vzero() { V v; memset(&v, 0, sizeof(V)); return v; }
 
+// Load the Hermitian half rows of two components (mixed wA * A + wB * B) as Z = a + i b over the
+// full length nx (Z[nx-k] = conj(a_k) + i conj(b_k)).  Optionally stores the mixed half rows.
 // Loads are issued in batches of kBatch elements per thread before any store, so that several
 // are in flight at once.
 template <typename Real, int NX>

@@ -255,22 +255,16 @@ template <typename Real, int N>
 cudaError_t LaunchZ<Real, N>::init() {
     cudaError_t e = cudaSuccess, r;
     if constexpr (!dft_zsplit<Real>(N)) {
-        constexpr int TZ = dft_tile_z<Real>(N);
+        constexpr int TZ = dft_tile_z(N);
         if ((r = set_max_smem(dftk::k_zconv_fwd_g<Real, N, TZ>)) != cudaSuccess) e = r;
         if ((r = set_max_smem(dftk::k_zconv_bwd_g<Real, N, TZ>)) != cudaSuccess) e = r;
-        constexpr int TB = dft_tile_zb<Real>(N), TF = dft_tile_zf<Real>(N);
-        constexpr int NB = dft_zbwd_threads<Real>(N), MBB = dft_zbwd_minb<Real>(N);
-        constexpr int NF = dft_zfwd_threads<Real>(N), MBF = dft_zfwd_minb<Real>(N);
-        if constexpr ((TB * sizeof(typename Cplx<Real>::type)) % 16 == 0)
-        {
-            if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, 3>)) != cudaSuccess) e = r;
-            if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, DFT_MAXS>)) != cudaSuccess) e = r;
-        }
-        if constexpr ((TF * sizeof(typename Cplx<Real>::type)) % 16 == 0) {
-            constexpr int MBF3 = dft_zfwd_minb_s3<Real>(N);
-            if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF, DFT_MAXS>)) != cudaSuccess) e = r;
-            if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF3, 3>)) != cudaSuccess) e = r;
-        }
+        constexpr int TB = dft_tile_zb(N), TF = dft_tile_zf(N);
+        constexpr int NB = dft_zbwd_threads(N), MBB = dft_zbwd_minb(N);
+        constexpr int NF = dft_zfwd_threads(N), MBF = dft_zfwd_minb(N), MBF3 = dft_zfwd_minb_s3(N);
+        if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, 3>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_zconv_bwd_tma<Real, N, TB, NB, MBB, DFT_MAXS>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF, DFT_MAXS>)) != cudaSuccess) e = r;
+        if ((r = set_max_smem(dftk::k_zconv_fwd_tma<Real, N, TF, NF, MBF3, 3>)) != cudaSuccess) e = r;
     }
     if constexpr (N > 0) {
         constexpr int TY = dft_tile_y<Real>(N);
@@ -297,8 +291,8 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
                                         Real kfy, Real kfz, int want_psi, const C* in, C* slot_n, C* slot_es,
                                         const C* tw, int* status) {
     if constexpr (!dft_zsplit<Real>(N)) {
-        constexpr int TZ = dft_tile_z<Real>(N);
-        constexpr int TB = dft_tile_zf<Real>(N);
+        constexpr int TZ = dft_tile_z(N);
+        constexpr int TB = dft_tile_zf(N);
         static int optin = 0, sms = 0;
         if (optin == 0) {
             int dev = 0;
@@ -308,7 +302,7 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
         }
         const size_t sm = dftk::zfwd_tma_smem<Real, N, TB>(sp.S);
         if (status && !g.zgrp && sm <= size_t(optin)) {
-            constexpr int NT = dft_zfwd_threads<Real>(N), MB = dft_zfwd_minb<Real>(N);
+            constexpr int NT = dft_zfwd_threads(N), MB = dft_zfwd_minb(N);
             constexpr int E = int(sizeof(C) / 8);
             CUtensorMap map_in, map_n;
             auto encode = [&](CUtensorMap* m, const C* data, int ncomp) {
@@ -322,7 +316,7 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
             const int ntx = (int)ceil_div(g.nxh, TB);
             const int ntiles = ntx * g.ny;
             // at most three species: the instance whose records and species loops are sized for three
-            constexpr int MB3 = dft_zfwd_minb_s3<Real>(N);
+            constexpr int MB3 = dft_zfwd_minb_s3(N);
             auto kern = sp.S <= 3 ? dftk::k_zconv_fwd_tma<Real, N, TB, NT, MB3, 3>
                                   : dftk::k_zconv_fwd_tma<Real, N, TB, NT, MB, DFT_MAXS>;
             const int fit = resident_blocks(kern, NT, sm), grid = ntiles < fit ? ntiles : fit;
@@ -338,10 +332,10 @@ cudaError_t LaunchZ<Real, N>::zconv_fwd(cudaStream_t st, const GridDesc& g, cons
 }
 
 namespace {
-// The persistent TMA second-half z pass: single (pair = 0: nine Phi' spectra at phi, results over
-// its first ncomp_out) or the two line-search samples (pair = 1: eighteen at phi, weights in
-// ctl[0], ctl[1], results at phi components 0 .. 2 ncomp_out - 1).  False if it does not apply
-// (no compile-time length, the grouped variant chosen, or too little shared memory).
+// The persistent TMA second-half z pass: single (pair = 0: a set of nine Phi' spectra at phi, seven of them
+// read, results over its first ncomp_out) or the two line-search samples (pair = 1: two sets, weights in
+// ctl[0], ctl[1], results at phi components 0 .. 2 ncomp_out - 1).  False if it does not apply (no
+// one-pass kernel, the grouped variant chosen, or too little shared memory).
 template <typename Real, int N, typename C>
 bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>& sp, Real kfx, Real kfy, Real kfz,
                      int flags, int ncomp_out, int pair, const Ctl* ctl, C* phi, const C* esA, const C* esB, C* es_mat,
@@ -349,7 +343,7 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
     if constexpr (dft_zsplit<Real>(N)) {
         return false;
     } else {
-        constexpr int TB = dft_tile_zb<Real>(N);
+        constexpr int TB = dft_tile_zb(N);
         const bool es_on = (flags & 2) != 0;
         const int nes = es_on ? ncomp_out * (esB ? 2 : 1) : 0;
         static int optin = 0, sms = 0;
@@ -361,8 +355,8 @@ bool launch_zbwd_tma(cudaStream_t st, const GridDesc& g, const SpeciesDesc<Real>
         }
         const size_t sm = dftk::zbwd_tma_smem<Real, N, TB>(nes);
         if (g.zgrp || sm > size_t(optin)) return false;
-        // persistent CTAs, two TMA-filled stages of nine Phi' tiles, one area of ES tiles
-        constexpr int NT = dft_zbwd_threads<Real>(N), MB = dft_zbwd_minb<Real>(N);
+        // persistent CTAs, two TMA-filled stages of seven Phi' tiles, one area of ES tiles
+        constexpr int NT = dft_zbwd_threads(N), MB = dft_zbwd_minb(N);
         constexpr int E = int(sizeof(C) / 8);
         CUtensorMap map_phi, map_esA, map_esB, map_out;
         auto encode = [&](CUtensorMap* m, const C* data, int ncomp) {
@@ -399,7 +393,7 @@ cudaError_t LaunchZ<Real, N>::zconv_bwd(cudaStream_t st, const GridDesc& g, cons
     if (launch_zbwd_tma<Real, N>(st, g, sp, kfx, kfy, kfz, flags, ncomp_out, 0, ctl, phi, esA, esB, es_mat, tw))
         return cudaSuccess;
     if constexpr (!dft_zsplit<Real>(N)) {
-        constexpr int TZ = dft_tile_z<Real>(N);
+        constexpr int TZ = dft_tile_z(N);
         dim3 grid((unsigned)ceil_div(g.nxh, TZ), (unsigned)g.ny);
         return launch_k(dftk::k_zconv_bwd_g<Real, N, TZ>, grid, dftk::kThreads, dftk::zg_smem_bytes<TZ, N>(sizeof(C)), st,
                         g.pdl, g, sp, kfx, kfy, kfz, flags, ncomp_out, ctl, phi, esA, esB, es_mat, tw);
@@ -422,7 +416,7 @@ bool LaunchZ<Real, N>::has_zbwd_pair(const GridDesc& g, int ncomp_out) {
     if constexpr (dft_zsplit<Real>(N)) {
         return false;
     } else {
-        constexpr int TB = dft_tile_zb<Real>(N);
+        constexpr int TB = dft_tile_zb(N);
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

@@ -25,14 +25,14 @@ __host__ __device__ constexpr bool dft_is_ct_size(int n) {
 template <typename Real> __host__ __device__ constexpr int dft_tile_y(int n) {
     return (sizeof(Real) == 4 ? 16 : 8) >> DFT_TILE_Y_SHIFT;
 }
-// The compile-time z passes transform all components of a tile together (two pools of ten
-// tiles in shared memory): the width keeps a CTA near 86 KB (FP32) so that two fit on an SM.
+// The one-pass z kernels (FP32) transform all components of a tile together (two pools of seven
+// tiles in shared memory): the width keeps a CTA near 61 KB (their register budget is for two on an SM).
 // DFT_TILE_ZG_SHIFT (build flag, default 0) narrows the tiles by that power of two.
 #ifndef DFT_TILE_ZG_SHIFT
 #define DFT_TILE_ZG_SHIFT 0
 #endif
-template <typename Real> __host__ __device__ constexpr int dft_tile_z(int n) {
-    const int t = (n <= 32 ? 16 : (n <= 64 ? 8 : (n <= 128 ? 4 : 2))) / (sizeof(Real) == 4 ? 1 : 2);
+__host__ __device__ constexpr int dft_tile_z(int n) {
+    const int t = n <= 32 ? 16 : (n <= 64 ? 8 : (n <= 128 ? 4 : 2));
     return (t >> DFT_TILE_ZG_SHIFT) > 0 ? (t >> DFT_TILE_ZG_SHIFT) : 1;
 }
 
@@ -44,17 +44,17 @@ template <typename Real> __host__ __device__ constexpr bool dft_zsplit(int n) { 
 
 // Persistent TMA z passes: half the grouped width (at least 16 bytes of a row, the TMA
 // minimum).
-template <typename Real> __host__ __device__ constexpr int dft_tile_zb(int n) {
-    const int t = dft_tile_z<Real>(n) / 2, tmin = sizeof(Real) == 4 ? 2 : 1;
-    return t > tmin ? t : tmin;
+__host__ __device__ constexpr int dft_tile_zb(int n) {
+    const int t = dft_tile_z(n) / 2;
+    return t > 2 ? t : 2;
 }
 // Tile width of the persistent TMA first-half z pass: the second half's (DFT_ZFWD_WIDE: the
 // grouped width).
-template <typename Real> __host__ __device__ constexpr int dft_tile_zf(int n) {
+__host__ __device__ constexpr int dft_tile_zf(int n) {
 #ifdef DFT_ZFWD_WIDE
-    return dft_tile_z<Real>(n);
+    return dft_tile_z(n);
 #else
-    return dft_tile_zb<Real>(n);
+    return dft_tile_zb(n);
 #endif
 }
 
@@ -81,8 +81,8 @@ template <typename Real> constexpr int dft_col_fill() { return sizeof(Real) == 4
 template <typename Real> inline bool dft_col_flat(int n, int ny, int pxh, int T) {
     return ny * pxh % T == 0 || n > 256 || dft_col_fill<Real>() / (n * T) < 2;
 }
-// Tile width of a run-time column transform (128-, 64- or 32-byte rows): of the widths that leave two blocks on an SM, the one with the least work per column in
-// use, where a narrower tile's shorter rows and fewer butterflies per block count as 2 / T columns
+// Tile width of a run-time column transform (128-, 64- or 32-byte rows): of the widths that leave two blocks on an
+// SM, the one with the least work per column in use, where a narrower tile's shorter rows and fewer butterflies per block count as 2 / T columns
 // (FP64, bound by its arithmetic: 1 / T) and columns past nxh as work.
 // Along z (ny > 0: the rows of a plane) the columns of a plane count together where dft_col_flat allows.
 template <typename Real> inline int dft_tile_rt(int n, int nxh, int ny = 0, int pxh = 0) {
@@ -124,46 +124,45 @@ template <typename Real> inline int dft_col_planes(int n, int nxh, int T, int ot
 
 // Threads of the persistent TMA z passes and the resident CTAs per SM their register budget
 // is sized for.  First half: 256 threads, two CTAs per SM, up to length 128; 512 threads, one
-// CTA, at 256.  Second half: 256 threads, three CTAs per SM (FP32; two in FP64, whose
-// butterflies need twice the registers), up to 128; 256 threads (one pass of them covers the
-// radix-16 butterflies of the seven Phi' groups of a two-column tile), two CTAs per SM, at 256 (its
+// CTA, at 256.  Second half: 256 threads, three CTAs per SM, up to 128; at 256 (one pass of the
+// threads covers the radix-16 butterflies of the seven Phi' groups of a two-column tile) two (its
 // shared memory allows no more).  DFT_ZFWD_THREADS / DFT_ZFWD_MINB / DFT_ZBWD_THREADS / DFT_ZBWD_MINB (build
 // flags) override.
-template <typename Real> __host__ __device__ constexpr int dft_zfwd_threads(int n) {
+__host__ __device__ constexpr int dft_zfwd_threads(int n) {
 #ifdef DFT_ZFWD_THREADS
     return DFT_ZFWD_THREADS;
 #else
     return n >= 256 ? 512 : 256;
 #endif
 }
-template <typename Real> __host__ __device__ constexpr int dft_zfwd_minb(int n) {
+__host__ __device__ constexpr int dft_zfwd_minb(int n) {
 #ifdef DFT_ZFWD_MINB
     return DFT_ZFWD_MINB;
 #else
-    return dft_zfwd_threads<Real>(n) <= 256 ? 2 : 1;
+    return dft_zfwd_threads(n) <= 256 ? 2 : 1;
 #endif
 }
 // The first-half pass for at most three species (its table records and species loops sized for
 // three): resident CTAs per SM its register budget is sized for (DFT_ZFWD_MINB_S3 overrides).
-template <typename Real> __host__ __device__ constexpr int dft_zfwd_minb_s3(int n) {
+__host__ __device__ constexpr int dft_zfwd_minb_s3(int n) {
 #ifdef DFT_ZFWD_MINB_S3
     return DFT_ZFWD_MINB_S3;
 #else
-    return n <= 64 ? 3 : dft_zfwd_minb<Real>(n);   // radix 16 at 128 spills under a budget for three
+    return n <= 64 ? 3 : dft_zfwd_minb(n);   // radix 16 at 128 spills under a budget for three
 #endif
 }
-template <typename Real> __host__ __device__ constexpr int dft_zbwd_threads(int n) {
+__host__ __device__ constexpr int dft_zbwd_threads(int n) {
 #ifdef DFT_ZBWD_THREADS
     return DFT_ZBWD_THREADS;
 #else
     return 256;
 #endif
 }
-template <typename Real> __host__ __device__ constexpr int dft_zbwd_minb(int n) {
+__host__ __device__ constexpr int dft_zbwd_minb(int n) {
 #ifdef DFT_ZBWD_MINB
     return DFT_ZBWD_MINB;
 #else
-    return (n < 256 && sizeof(Real) == 4) ? 3 : 2;
+    return n < 256 ? 3 : 2;
 #endif
 }
 
@@ -244,7 +243,7 @@ struct Passes {
     static cudaError_t init_attributes(const GridDesc* g = nullptr);
     // dynamic shared memory of an x pass with `lines` lines
     static size_t smem_x(int nx, int lines) { return (size_t(nx) + 2 * size_t(lines) * (nx + 1)) * sizeof(C) + 16; }
-    // column tile widths of the y and z passes
+    // column tile widths of the y passes and of a run-time length's z transforms
     static int tile_y(const GridDesc& g);
     static int tile_z(const GridDesc& g);
 

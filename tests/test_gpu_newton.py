@@ -73,10 +73,11 @@ def test_newton_fp32_reaches_the_fp32_floor():
     plan.close()
 
 
-@pytest.mark.parametrize("shape,krylov_dim", [((4, 4, 4), 30), ((5, 6, 7), 3), ((48, 10, 33), 30)])
+@pytest.mark.parametrize("shape,krylov_dim", [((4, 4, 4), 30), ((5, 6, 7), 3), ((48, 10, 33), 30), ((48, 33, 35), 30)])
 def test_newton_orthogonalisation_sizes_fp64(shape, krylov_dim):
-    # fields smaller than one block of the orthogonalisation, of an odd length, and larger than its grid;
-    # a restart at the largest basis.  r < 1e-11 on the GPU leaves the oracle's residual at the maps'
+    # fields smaller than one block of the orthogonalisation, of an odd length, of one element per thread for part of
+    # its grid, and larger than its grid (two blocks of 256 threads per SM: 77824 threads on 152 SMs; 110880
+    # elements); a restart at the largest basis.  r < 1e-11 on the GPU leaves the oracle's residual at the maps'
     # difference, 1e-10 per point
     prob = F.Problem(shape, 0.1, [0.095, 0.181], [1.0, -1.0], [1.0, 1.0])
     V = np.stack([z * 2.0 * np.sin(2 * np.pi * np.arange(shape[0]) / shape[0])[:, None, None] * np.ones(shape)

@@ -3,9 +3,9 @@
 The x passes run either as the compile-time kernels (the Phi' passes one CTA per row block, or
 persistent with bulk-copy or cp.async prefetch) or as the run-time ones under each candidate radix order
 (default, reversed, all-8 and all-4 plans); the y pass as the persistent TMA kernel or
-the run-time column kernel; the z passes as the persistent TMA kernels or the grouped
+the run-time column kernel; in FP32 the z passes as the persistent TMA kernels or the grouped
 one-tile-per-CTA ones, the first half's z stage as one pass or three (z transforms around a
-k-space products pass).  Each combination is pinned with dft_set_variants and checked against the
+k-space products pass; FP64 runs three in both halves whatever the z variant).  Each combination is pinned with dft_set_variants and checked against the
 oracle's G (FP32 1e-5, FP64 1e-10), and one line-search step under a run-time x variant against
 the oracle's step; finally dft_autotune's own choice is checked the same way.
 """
@@ -75,7 +75,7 @@ def test_every_variant_matches_oracle(precision, shape):
     for x in xs:
         for xp in ((0, 1) if x == 0 else (0,)):
             for y in (0, 1):
-                for z in (0, 1, 2, 3):
+                for z in (0, 1, 2, 3) if precision == "fp32" else (0,):
                     plan.set_variants(x, y, z, x_persistent=xp)
                     g, _ = plan.picard_map(_dev(rho, plan), _dev(V, plan))
                     assert relerr(g.double().cpu().numpy(), g_ref) < TOL[precision], (x, xp, y, z, plan.tuning())
@@ -149,16 +149,15 @@ def test_autotuned_choice_matches_oracle(precision):
     plan.close()
 
 
-@pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("shape", [(64, 32, 48), (128, 16, 32), (256, 8, 16)])
-def test_split_first_half_equals_the_single_pass(precision, shape):
+def test_split_first_half_equals_the_single_pass(shape):
     # the three-pass first-half z stage (z transform, k-space products, z transform) runs the
-    # same butterflies and the same products per point as the single pass; the compiler may
+    # same butterflies and the same products per point as FP32's single pass; the compiler may
     # contract the products differently in the two kernels, so the weighted densities and G
     # agree to rounding (a few ulp of the largest value), and with the oracle
     from paper_0910_1531_gb300 import binding
     prob, rho, V = _case(shape, (0.05, 0.06, 0.07), seed=53)
-    plan = binding.Plan(shape, prob.h, *SPECIES, precision=precision)
+    plan = binding.Plan(shape, prob.h, *SPECIES, precision="fp32")
     rd, Vd = _dev(rho, plan), _dev(V, plan)
     out = []
     xv = _x_variants(plan)[0]       # the compile-time x kernels where the length has them
@@ -167,8 +166,30 @@ def test_split_first_half_equals_the_single_pass(precision, shape):
         n = plan.weighted_densities(rd)
         g, _ = plan.picard_map(rd, Vd)
         out.append((n, g))
-    close = {"fp32": 2e-6, "fp64": 1e-13}[precision]
     for a in range(2):
-        assert relerr(out[1][a].double().cpu().numpy(), out[0][a].double().cpu().numpy()) < close, a
-    assert relerr(out[1][1].double().cpu().numpy(), F.picard_map(prob, rho, V)) < TOL[precision]
+        assert relerr(out[1][a].double().cpu().numpy(), out[0][a].double().cpu().numpy()) < 2e-6, a
+    assert relerr(out[1][1].double().cpu().numpy(), F.picard_map(prob, rho, V)) < TOL["fp32"]
+    plan.close()
+
+
+@pytest.mark.parametrize("shape", [(32, 16, 12), (64, 32, 48), (96, 8, 16), (128, 16, 32), (256, 8, 16)])
+def test_three_pass_z_stages_match_the_oracle_fp64(shape):
+    # FP64 has no single pass to compare with: weighted densities, c1 of both parts, G and a line-search step (whose
+    # two samples share the products pass) against the oracle at the compile-time z lengths
+    from paper_0910_1531_gb300 import binding
+    prob, rho, V = _case(shape, (0.05, 0.06, 0.07), seed=53)
+    plan = binding.Plan(shape, prob.h, *SPECIES, precision="fp64")
+    rd, Vd = _dev(rho, plan), _dev(V, plan)
+    n, n_ref = plan.weighted_densities(rd).cpu().numpy(), F.weighted_densities(prob, rho)
+    for f in ([0], [1], [2], [3], [4, 5, 6], [7, 8, 9]):
+        assert relerr(n[f], n_ref[f]) < TOL["fp64"], f
+    assert relerr(plan.c1_hs(rd).cpu().numpy(), F.c1_hs(prob, rho)) < TOL["fp64"]
+    c, psi = plan.c1_es(rd, want_psi=True)
+    c_ref, psi_ref = F.c1_es(prob, rho)
+    assert relerr(c.cpu().numpy(), c_ref) < TOL["fp64"] and relerr(psi.cpu().numpy(), psi_ref) < TOL["fp64"]
+    g_ref = F.picard_map(prob, rho, V)
+    g, _ = plan.picard_map(rd, Vd)
+    assert relerr(g.cpu().numpy(), g_ref) < TOL["fp64"]
+    plan.picard_step(rd, Vd, -1.0)
+    assert relerr(rd.cpu().numpy(), P.picard_step(prob, rho, V, g0=g_ref)[0]) < TOL["fp64"]
     plan.close()
