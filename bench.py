@@ -46,7 +46,7 @@ KERNELS = ("xfwd", "yfft", "zconv_fwd", "xphi", "zconv_bwd", "xupdate", "xinv", 
 # per workload and precision (the kinds the autotuned iteration ran when captured); valid
 # while the kernel sources and build flags hash to `digest`.
 NCU_TRAFFIC = {
-    "digest": "cbb15cdfc6bf6fe5",
+    "digest": "e752c05b84fa697b",
     "captures": {
         "3species_16obstacles_128^3/fp32": {"yfft": 80592512, "zconv_fwd": 61055744, "xphi": 260493312, "zconv_bwd": 158149120, "xupdate": 162504576, "xinv": 8714752, "finalize": 67925},
         "pore_slab_4species_256^3/fp32": {"xphi": 2413555200, "zconv_bwd": 1561309952, "zmul": 997430272, "yfft": 760231296, "zfft": 685547136, "xupdate": 1220790144},

@@ -687,7 +687,12 @@ dft_status grad_t(dft_plan* p, const Real* rho, const Real* V, double* omega_out
             sp.tab_dk = static_cast<const Real*>(p->ktab_dk);
             const cudaError_t e = P::build_ktab(p->stream, p->g, sp, p->kf[0], O::kf(p, 0), O::kf(p, 1), O::kf(p, 2),
                                                 p->ktab_rows, false);
-            if (e != cudaSuccess) return fail(p, DFT_ECUDA, std::string("|k| tables: ") + cudaGetErrorString(e));
+            if (e != cudaSuccess) {
+                sp.tab_dk = nullptr;
+                cudaFree(p->ktab_dk);
+                p->ktab_dk = nullptr;
+                return fail(p, DFT_ECUDA, std::string("|k| tables: ") + cudaGetErrorString(e));
+            }
         } else {
             cudaGetLastError();
             p->ktab_dk = nullptr;
